@@ -14,6 +14,7 @@
 #include <cstdio>
 #include <cstring>
 #include <memory>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -46,9 +47,7 @@ struct Geom {
     std::vector<int> prof_ch_off, plan_ch_off, plan_n, prof_plan;
     int total_prof_ch = 0, total_plan_ch = 0;
     DevBuf pieces, items, slot_items, slot_cut, prof_slot_off, plan_ch_off_d, plan_n_d, prof_ch_off_d,
-        prof_plan_d, ch_frel, ch_B, ch_alpha, ch_gamma, ch_nf, guard, zs_a, zs_b, zs_d, zs_g, item_slot, zs_gseg,
-        seg;
-    float phi_seg[3] = {0.f, 0.f, 0.f};
+        prof_plan_d, ch_frel, ch_B, ch_alpha, ch_gamma, ch_nf, guard, zs_a, zs_b, zs_d, zs_g, item_slot;
     bool has_nf = false, has_guard = false;
     // Raman-ODE profile: partner windows and gain scale per plan channel, RK4
     // steps per half z-step, largest candidate count of a piece
@@ -79,9 +78,10 @@ struct isrs_handle_s {
     std::string err;
     DevBuf paths, kapL;
     DevBuf P, pd_d, pd_f, step_d, step_f, lnrho_L, ptot, partial, counter, o_sigma, o_pnli, o_eta, o_snr,
-        o_pase, o_T, gA, gK, gPd, gVs, gY, dbg, ybar, dTdP, ab, ab_f, ode_y, gAB, gV, gAt, partial_mci, tab_rows,
+        o_pase, o_T, gA, gK, gPd, gVs, dbg, ybar, dTdP, ab, ab_f, ode_y, gAB, gV, gAt, partial_mci, tab_rows,
         tab_rowsV;
     std::vector<std::unique_ptr<Geom>> cache;   // most recent first
+    const float2 *gauss = nullptr;       // Gauss rules of the row sums on this device (gauss_rules)
     int tile_points = 0, tile_threads = 0;
     int64_t last_points = 0, last_psteps = 0;
     int last_launches = 0;
@@ -441,66 +441,8 @@ isrs_status cut_pieces(isrs_handle h, const isrs_channels *c, int plan, int i, i
 // Stored per step as FP64 {z_m, dz_m}, FP32 {z_m, dz_m} and the phase
 // positions in revolutions (z / 2 pi) as float-float pairs.
 // ----------------------------------------------------------------------------
-// Segments of the span for the segmented small-phase series: level v cuts
-// [0, L] into 2^{v+1} segments at the step edges nearest to s L / 2^{v+1}
-// (fewer where two targets share an edge).  Per segment {m0, m1, centre/2pi
-// as float-float}; per level and step the moments g_n (n <= 18) of the step
-// about its segment's centre; per level the |phi| limit 6 / (longest
-// segment), below which 19 moments truncate the series by < 2e-8.
-void segment_tables(const std::vector<double> &ze, std::vector<float4> &gseg, std::vector<int4> &seg,
-                    float *phi_seg)
-{
-    const int M = (int)ze.size() - 1;
-    const double L = ze[M];
-    gseg.assign((size_t)kSegLevels * M * 5, make_float4(0.f, 0.f, 0.f, 0.f));
-    seg.assign(kSegSlots, make_int4(0, 0, 0, 0));
-    int slot = 0;
-    for (int v = 0; v < kSegLevels; ++v) {
-        const int J = 2 << v;
-        std::vector<int> b{0};
-        for (int s = 1; s < J; ++s) {
-            int best = 0;
-            for (int e = 0; e <= M; ++e)
-                if (std::fabs(ze[e] - s * L / J) < std::fabs(ze[best] - s * L / J)) best = e;
-            if (best > b.back() && best < M) b.push_back(best);
-        }
-        b.push_back(M);
-        double lmax = 0.0;
-        const int nseg = (int)b.size() - 1;
-        for (int s = 0; s < (1 << (v + 1)); ++s, ++slot) {
-            if (s >= nseg) {                    // fewer segments than slots: an empty one
-                seg[slot] = make_int4(M, M, 0, 0);
-                continue;
-            }
-            const int m0 = b[s], m1 = b[s + 1];
-            const double c = 0.5 * (ze[m0] + ze[m1]);
-            lmax = std::max(lmax, ze[m1] - ze[m0]);
-            const double cr = c / (2.0 * 3.14159265358979323846);
-            const float hi = (float)cr, lo = (float)(cr - (double)hi);
-            int hib, lob;
-            std::memcpy(&hib, &hi, 4);
-            std::memcpy(&lob, &lo, 4);
-            seg[slot] = make_int4(m0, m1, hib, lob);
-            for (int m = m0; m < m1; ++m) {
-                const double lo2 = ze[m] - c, hi2 = ze[m + 1] - c;
-                float g[20] = {0.f};
-                double pa = lo2, pb = hi2;
-                for (int n = 0; n <= 18; ++n) {
-                    g[n] = (float)((pb - pa) / ((n + 1) * (hi2 - lo2)));
-                    pa *= lo2;
-                    pb *= hi2;
-                }
-                for (int q = 0; q < 5; ++q)
-                    gseg[((size_t)v * M + m) * 5 + q] = make_float4(g[4 * q], g[4 * q + 1], g[4 * q + 2], g[4 * q + 3]);
-            }
-        }
-        phi_seg[v] = (float)(6.0 / lmax);
-    }
-}
-
 void zgrid_tables(double L, double a, int n_edges, std::vector<float4> &za, std::vector<float4> &zb,
-                  std::vector<double2> &zd, float &dz_max, std::vector<float4> *zg = nullptr,
-                  std::vector<float4> *gseg = nullptr, std::vector<int4> *seg = nullptr, float *phi_seg = nullptr)
+                  std::vector<double2> &zd, float &dz_max, std::vector<float4> *zg = nullptr)
 {
     std::vector<double> ze(n_edges);
     const double drop = a > 0.0 ? -std::expm1(-a * L) : 0.0;
@@ -542,7 +484,6 @@ void zgrid_tables(double L, double a, int n_edges, std::vector<float4> &za, std:
                 (*zg)[5 * m + q] = make_float4(g[4 * q], g[4 * q + 1], g[4 * q + 2], g[4 * q + 3]);
         }
     }
-    if (gseg && seg && phi_seg) segment_tables(ze, *gseg, *seg, phi_seg);
 }
 
 // ----------------------------------------------------------------------------
@@ -550,6 +491,11 @@ void zgrid_tables(double L, double a, int n_edges, std::vector<float4> &za, std:
 //   cuts_per_plan[q]: CUT list of plan q (all channels if empty)
 //   prof_plan: plan of each profile; every profile evaluates its plan's CUT list
 // ----------------------------------------------------------------------------
+struct TileSplit {
+    int chunk, parts;
+};
+TileSplit tile_split(const isrs_handle_s *h, int n_ch, int cell_set, int G);
+
 isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isrs_channels *plans,
                      const std::vector<std::vector<int>> &cuts_per_plan, const std::vector<int> &prof_plan,
                      const isrs_quad *q, cudaStream_t st, Geom **out)
@@ -685,7 +631,6 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
 
     // work items, output slots
     const int tile_pts = h->tile_points > 0 ? h->tile_points : (1 << 20);
-    const int chunk = (int)std::max<int64_t>(1, tile_pts / G2);
     std::vector<DevItem> items, mitems;
     std::vector<int2> slot_items, slot_items2;
     std::vector<int> slot_cut, prof_slot_off, item_slot, mitem_slot;
@@ -699,14 +644,17 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
         g->total_prof_ch += plans[k].n_ch;
         prof_slot_off.push_back((int)slot_items.size());
         const std::vector<int> &cl = cuts_per_plan[k];
+        const TileSplit ts = tile_split(h, plans[k].n_ch, piece_cells, q->G);
         for (size_t s = 0; s < cut_range[k].size(); ++s) {
             const int i = cl.empty() ? (int)s : cl[s];
             const int it0 = (int)items.size();
             const int slot = (int)slot_items.size();
-            for (int a = cut_range[k][s].first; a < cut_range[k][s].second; a += chunk) {
-                const int b = std::min(a + chunk, cut_range[k][s].second);
-                items.push_back(DevItem{p, a, b, i});
-                item_slot.push_back(slot);
+            for (int a = cut_range[k][s].first; a < cut_range[k][s].second; a += ts.chunk) {
+                const int b = std::min(a + ts.chunk, cut_range[k][s].second);
+                for (int t = 0; t < ts.parts; ++t) {
+                    items.push_back(DevItem{p, a, b, i, t | ts.parts << 16});
+                    item_slot.push_back(slot);
+                }
             }
             for (int a = cut_range[k][s].first; a < cut_range[k][s].second; ++a) {
                 g->n_points += G2;
@@ -720,7 +668,7 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
                 const int ncell = n2 * (n2 + 1) / 2;
                 const int m0 = (int)mitems.size();
                 for (int t = 0; t < ncell; t += mchunk) {
-                    mitems.push_back(DevItem{p, t, std::min(t + mchunk, ncell), i});
+                    mitems.push_back(DevItem{p, t, std::min(t + mchunk, ncell), i, 1 << 16});
                     mitem_slot.push_back(slot);
                 }
                 slot_items2.push_back(make_int2(m0, (int)mitems.size()));
@@ -734,10 +682,9 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
     g->n_slots = (int)slot_items.size();
     g->n_mci_items = (int)mitems.size();
 
-    std::vector<float4> za, zb, zg, zgs;
-    std::vector<int4> segv;
+    std::vector<float4> za, zb, zg;
     std::vector<double2> zd;
-    zgrid_tables(fb->L_km, fb->alpha_R_per_km, q->n_edges, za, zb, zd, g->dz_max, &zg, &zgs, &segv, g->phi_seg);
+    zgrid_tables(fb->L_km, fb->alpha_R_per_km, q->n_edges, za, zb, zd, g->dz_max, &zg);
 
     // Raman-ODE profile: the partners of channel i are the k != i with
     // |f_k - f_i| <= raman_max_THz, one index window of the sorted plan; the
@@ -841,8 +788,6 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
     UP(zs_b, zb);
     UP(zs_d, zd);
     UP(zs_g, zg);
-    UP(zs_gseg, zgs);
-    UP(seg, segv);
     UP(item_slot, item_slot);
     if (mci) {
         UP(mci_items, mitems);
@@ -862,6 +807,7 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
         UP(tab_gath, gath);
     }
 #undef UP
+    CK(launch_piece_logs((DevPiece *)g->pieces.p, (int)g->n_pieces, st));
     CK(cudaStreamSynchronize(st));   // host vectors die at return
 
     h->cache.insert(h->cache.begin(), std::move(g));
@@ -882,9 +828,51 @@ void free_geom(Geom *g)
                       &g->ch_frel, &g->ch_B, &g->ch_alpha, &g->ch_gamma, &g->ch_nf,
                       &g->guard, &g->zs_a, &g->zs_b, &g->zs_d, &g->zs_g, &g->item_slot,
                       &g->win_lo, &g->win_hi, &g->ch_scale, &g->half_steps, &g->mci_items, &g->slot_items2,
-                      &g->item_slot_all, &g->tab_row_off, &g->tab_prow, &g->tab_gath_off, &g->tab_gath,
-                      &g->zs_gseg, &g->seg};
+                      &g->item_slot_all, &g->tab_row_off, &g->tab_prow, &g->tab_gath_off, &g->tab_gath};
     for (DevBuf *b : bufs) release(*b);
+}
+
+// The Gauss rules of the row sums (quad_nodes.cuh): constants of the method,
+// 0.6 MB in one array of the module per device, filled by a kernel the first
+// time a call needs them there.  The fill is waited for under the lock, so
+// every later reader, on any stream or thread, finds them complete.
+constexpr int kGaussMaxDevices = 64;
+std::mutex g_gauss_mu;
+const float2 *g_gauss_ptr[kGaussMaxDevices] = {nullptr};
+
+cudaError_t gauss_rules(int dev, cudaStream_t st, const float2 **out)
+{
+    if (dev < 0 || dev >= kGaussMaxDevices) return cudaErrorInvalidDevice;
+    std::lock_guard<std::mutex> lk(g_gauss_mu);
+    if (!g_gauss_ptr[dev]) {
+        void *p = nullptr;
+        cudaError_t e = gauss_array(&p);
+        if (e == cudaSuccess) e = launch_gauss((float2 *)p, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (e != cudaSuccess) return e;
+        g_gauss_ptr[dev] = (const float2 *)p;
+    }
+    *out = g_gauss_ptr[dev];
+    return cudaSuccess;
+}
+
+// Work tiles of a plan: `chunk` pieces per tile, each piece shared by `parts`
+// tiles.  A warp takes a tile (FP64: a block), so a small plan wants many: below
+// ~16,000 pieces every piece is its own tile, and below that its nodes are
+// shared by up to 8 (a 5-channel plan has 90 pieces for 4,864 resident warps;
+// every share repeats the piece's set-up, which only pays on an idle chip).  A
+// large plan takes up to 32 pieces a tile, ~8 tiles per resident warp, so that a
+// tile's fixed cost (queue, bucket rows) stays small and the last wave short.
+// The split depends on the plan and grid alone, never on the CUT list or the
+// number of profiles, so a CUT's tiles and the order of its sum are the same in
+// every call.
+TileSplit tile_split(const isrs_handle_s *h, int n_ch, int cell_set, int G)
+{
+    if (h && h->tile_points > 0) return {(int)std::max<int64_t>(1, h->tile_points / ((int64_t)G * G)), 1};
+    const int64_t n = n_ch;
+    const int64_t total = cell_set == ISRS_CELLS_SCI_XCI ? n * (2 * n + 1) : n * (n + 1) * (n + 3) / 2;
+    const int64_t parts = std::min<int64_t>(std::min(8, std::max(1, G / 16)), (16384 + total - 1) / total);
+    return {(int)std::max<int64_t>(1, std::min<int64_t>(32, total / 38912)), (int)parts};
 }
 
 struct Launch {
@@ -931,6 +919,7 @@ QuadParams quad_params(isrs_handle h, const isrs_fibre *fb, Geom *g)
     qp.dbg = kDebugBuild ? (unsigned *)h->dbg.p : nullptr;
     qp.G = g->G;
     qp.eps_v1 = g->eps_v1;
+    qp.ln_eps = -std::log(g->eps_v1);
     qp.n_steps = g->n_steps;
     qp.beta2 = fb->beta2;
     qp.beta3 = fb->beta3;
@@ -949,9 +938,7 @@ QuadParams quad_params(isrs_handle h, const isrs_fibre *fb, Geom *g)
     qp.zs_b = (const float4 *)g->zs_b.p;
     qp.zs_d = (const double2 *)g->zs_d.p;
     qp.zs_g = (const float4 *)g->zs_g.p;
-    qp.zs_gseg = (const float4 *)g->zs_gseg.p;
-    qp.seg = (const int4 *)g->seg.p;
-    for (int v = 0; v < 3; ++v) qp.phi_seg[v] = g->phi_seg[v];
+    qp.gauss = h->gauss;
     qp.dz_max = g->dz_max;
     qp.kap_L = (const double *)h->kapL.p;
     qp.L = (float)fb->L_km;
@@ -992,6 +979,7 @@ isrs_status run_forward(isrs_handle h, const isrs_fibre *fb, Geom *g, int precis
         return fail(h, ISRS_ERR_UNSUPPORTED, "the Raman-ODE adjoint does not cover the separate MCI grid");
     if (g->n_mci_items > 0 && (s = ensure(h, h->partial_mci, sizeof(double) * g->n_mci_items)) != ISRS_OK)
         return s;
+    if (!h->gauss) CK(gauss_rules(h->device, st, &h->gauss));
     if ((s = ensure(h, h->pd_d, sizeof(double) * g->total_prof_ch)) != ISRS_OK) return s;
     if ((s = ensure(h, h->pd_f, sizeof(float) * g->total_prof_ch)) != ISRS_OK) return s;
     if ((s = ensure(h, h->lnrho_L, sizeof(double) * g->total_prof_ch)) != ISRS_OK) return s;
@@ -1060,13 +1048,8 @@ isrs_status run_forward(isrs_handle h, const isrs_fibre *fb, Geom *g, int precis
         ap.V = (double *)h->gPd.p;
         ap.item_slot = (const int *)g->item_slot.p;
         ap.n_ch = n_ch;
-        const int per_sm = adjoint_blocks_per_sm(M, g->G, block);
-        int grid = h->num_sms * per_sm;
-        if (g->n_items < grid) grid = std::max(1, g->n_items);
-        if ((s = ensure(h, h->gY, adjoint_scratch_bytes(grid))) != ISRS_OK) return s;
-        ap.Yg = (double *)h->gY.p;
         if ((s = mark(h, 1, 0, st)) != ISRS_OK) return s;
-        if (g->n_items > 0) CK(launch_adjoint(ap, grid, block, st));
+        if (g->n_items > 0) CK(launch_adjoint(ap, h->num_sms, block, st));
         if (g->n_mci_items > 0) {
             // the MCI cells of the separate grid: further tiles of their CUTs
             AdjParams am = ap;
@@ -1087,13 +1070,14 @@ isrs_status run_forward(isrs_handle h, const isrs_fibre *fb, Geom *g, int precis
         const bool tab = g->profile == ISRS_PROFILE_RAMAN_ODE;
         if (tab && quad_tab_smem_bytes(precision, M, g->G, g->nc_max) > 200 * 1024)
             return fail(h, ISRS_ERR_UNSUPPORTED, "profile tables exceed shared memory at this precision");
-        const int per_sm = tab ? quad_tab_blocks_per_sm(precision, M, g->G, g->nc_max, block)
-                               : quad_blocks_per_sm(precision, M, g->G, block);
-        int grid = h->num_sms * per_sm;
-        if (g->n_items < grid) grid = std::max(1, g->n_items);
         if ((s = mark(h, 0, 0, st)) != ISRS_OK) return s;
-        if (g->n_items > 0) CK(tab ? launch_quad_tab(qp, precision, grid, block, st)
-                                   : launch_quad(qp, precision, grid, block, st));
+        if (tab && g->n_items > 0) {
+            int grid = h->num_sms * quad_tab_blocks_per_sm(precision, M, g->G, g->nc_max, block);
+            if (g->n_items < grid) grid = std::max(1, g->n_items);
+            CK(launch_quad_tab(qp, precision, grid, block, st));
+        } else if (g->n_items > 0) {
+            CK(launch_quad(qp, precision, h->num_sms, block, st));
+        }
         if (g->n_mci_items > 0) {
             QuadParams qm = qp;
             qm.items = (const DevItem *)g->mci_items.p;
@@ -1560,7 +1544,7 @@ isrs_status isrs_destroy(isrs_handle h)
                       &h->counter, &h->o_sigma, &h->o_pnli, &h->o_eta, &h->o_snr, &h->o_pase, &h->o_T,
                       &h->gA, &h->gK, &h->gPd, &h->ybar, &h->dTdP, &h->ab, &h->ode_y, &h->gAB, &h->gV,
                       &h->gAt, &h->partial_mci, &h->eta_all, &h->tab_rows, &h->tab_rowsV, &h->gVs,
-                      &h->gY, &h->dbg, &h->ab_f};
+                      &h->dbg, &h->ab_f};
     for (DevBuf *b : bufs) release(*b);
     release(h->paths);
     release(h->kapL);
@@ -2049,16 +2033,24 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     std::vector<int2> slot_items;
     std::vector<int> slot_cut, item_slot;
     const int64_t G2 = (int64_t)quad->G * quad->G;
-    const int chunk = (int)std::max<int64_t>(1, (int64_t)(1 << 20) / G2);
+    std::vector<int> cut_end;
     for (int i = 0; i < n; ++i) {
-        const int p0 = (int)pieces.size();
         if ((s = cut_pieces(nullptr, ch, 0, i, quad->cell_set, pieces)) != ISRS_OK) return s;
-        const int p1 = (int)pieces.size();
+        cut_end.push_back((int)pieces.size());
+    }
+    // tiles as in the handle calls; where the scratch is nearly full of pieces,
+    // larger ones, so that the tile tables never make a plan too large
+    const TileSplit ts = sizeof(DevPiece) * pieces.size() < kNoAllocBytes / 4
+                             ? tile_split(nullptr, n, quad->cell_set, quad->G)
+                             : TileSplit{(int)std::max<int64_t>(1, (int64_t)(1 << 20) / G2), 1};
+    for (int i = 0; i < n; ++i) {
+        const int p0 = i > 0 ? cut_end[i - 1] : 0, p1 = cut_end[i];
         const int it0 = (int)items.size();
-        for (int a = p0; a < p1; a += chunk) {
-            items.push_back(DevItem{0, a, std::min(a + chunk, p1), i});
-            item_slot.push_back(i);
-        }
+        for (int a = p0; a < p1; a += ts.chunk)
+            for (int t = 0; t < ts.parts; ++t) {
+                items.push_back(DevItem{0, a, std::min(a + ts.chunk, p1), i, t | ts.parts << 16});
+                item_slot.push_back(i);
+            }
         slot_items.push_back(make_int2(it0, (int)items.size()));
         slot_cut.push_back(i);
     }
@@ -2069,11 +2061,10 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
         av[k] = ch->alpha_per_km[k];
         gv[k] = ch->gamma_per_W_km[k];
     }
-    std::vector<float4> za, zb, zg, zgs;
-    std::vector<int4> segv;
+    std::vector<float4> za, zb, zg;
     std::vector<double2> zd;
-    float dz_max = 0.f, phi_seg[3] = {0.f, 0.f, 0.f};
-    zgrid_tables(fibre->L_km, fibre->alpha_R_per_km, quad->n_edges, za, zb, zd, dz_max, &zg, &zgs, &segv, phi_seg);
+    float dz_max = 0.f;
+    zgrid_tables(fibre->L_km, fibre->alpha_R_per_km, quad->n_edges, za, zb, zd, dz_max, &zg);
     const int M = quad->n_edges - 1;
     if (quad->precision == ISRS_PREC_FP32) {
         const double pi = 3.14159265358979323846;
@@ -2102,8 +2093,6 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     const size_t o_za = L.take(sizeof(float4) * M), o_zb = L.take(sizeof(float4) * M);
     const size_t o_zd = L.take(sizeof(double2) * M);
     const size_t o_zg = L.take(sizeof(float4) * zg.size());   // centred step moments (contracted small phase)
-    const size_t o_zgs = L.take(sizeof(float4) * zgs.size());  // the same about segment centres
-    const size_t o_seg = L.take(sizeof(int4) * segv.size());
     const size_t o_kapL = L.take(sizeof(double));
     const size_t o_P = L.take(sizeof(double) * n);
     const size_t o_pdd = L.take(sizeof(double) * n), o_pdf = L.take(sizeof(float) * n);
@@ -2116,6 +2105,8 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
 
     unsigned char *base = nullptr;
     if ((s = noalloc_scratch(dev, (void **)&base)) != ISRS_OK) return s;
+    const float2 *gauss = nullptr;
+    if (gauss_rules(dev, st, &gauss) != cudaSuccess) return ISRS_ERR_CUDA;
     struct Up { size_t off; const void *src; size_t bytes; } ups[] = {
         {o_pieces, pieces.data(), sizeof(DevPiece) * pieces.size()},
         {o_items, items.data(), sizeof(DevItem) * items.size()},
@@ -2125,8 +2116,7 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
         {o_B, Bv.data(), sizeof(double) * n}, {o_alpha, av.data(), sizeof(double) * n},
         {o_gamma, gv.data(), sizeof(double) * n}, {o_za, za.data(), sizeof(float4) * M},
         {o_zb, zb.data(), sizeof(float4) * M}, {o_zd, zd.data(), sizeof(double2) * M},
-        {o_zg, zg.data(), sizeof(float4) * zg.size()}, {o_zgs, zgs.data(), sizeof(float4) * zgs.size()},
-        {o_seg, segv.data(), sizeof(int4) * segv.size()}};
+        {o_zg, zg.data(), sizeof(float4) * zg.size()}};
     for (const Up &u : ups)
         if (u.bytes && cudaMemcpyAsync(base + u.off, u.src, u.bytes, cudaMemcpyHostToDevice, st) != cudaSuccess)
             return ISRS_ERR_CUDA;
@@ -2156,6 +2146,7 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     pp.lnrho_L = (double *)(base + o_lnL);
     pp.ptot = (double *)(base + o_ptot);
     pp.kap_L = (double *)(base + o_kapL);
+    if (launch_piece_logs((DevPiece *)(base + o_pieces), (int)pieces.size(), st) != cudaSuccess) return ISRS_ERR_CUDA;
     if (launch_prep(pp, 1, st) != cudaSuccess) return ISRS_ERR_CUDA;
 
     QuadParams qp;
@@ -2167,6 +2158,7 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     qp.G = quad->G;
     qp.n_steps = M;
     qp.eps_v1 = quad->eps_v1;
+    qp.ln_eps = -std::log(quad->eps_v1);
     qp.beta2 = fibre->beta2;
     qp.beta3 = fibre->beta3;
     qp.beta4 = fibre->beta4;
@@ -2182,9 +2174,7 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     qp.zs_b = (const float4 *)(base + o_zb);
     qp.zs_d = pp.zs_d;
     qp.zs_g = (const float4 *)(base + o_zg);
-    qp.zs_gseg = (const float4 *)(base + o_zgs);
-    qp.seg = (const int4 *)(base + o_seg);
-    for (int v = 0; v < 3; ++v) qp.phi_seg[v] = phi_seg[v];
+    qp.gauss = gauss;
     qp.kap_L = pp.kap_L;
     qp.n_spans = 1;
     qp.dz_max = dz_max;
@@ -2194,9 +2184,7 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     qp.path_count = (unsigned long long *)(base + o_paths);
     int n_sms = 1;
     cudaDeviceGetAttribute(&n_sms, cudaDevAttrMultiProcessorCount, dev);
-    int grid = n_sms * quad_blocks_per_sm(quad->precision, M, quad->G, 256);
-    if ((int)items.size() < grid) grid = std::max(1, (int)items.size());
-    if (!items.empty() && launch_quad(qp, quad->precision, grid, 256, st) != cudaSuccess) return ISRS_ERR_CUDA;
+    if (!items.empty() && launch_quad(qp, quad->precision, n_sms, 256, st) != cudaSuccess) return ISRS_ERR_CUDA;
 
     FinishParams fp;
     std::memset(&fp, 0, sizeof(fp));

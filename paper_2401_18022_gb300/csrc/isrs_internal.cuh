@@ -21,10 +21,6 @@ constexpr int kMaxSteps = 2048;     // max z-steps (n_edges - 1)
 constexpr int kMaxG = 4096;         // max grid points per dimension
 constexpr int kMaxRamanCh = 2048;   // max channels of a plan with the Raman-ODE profile
 constexpr int kMaxRamanGradCh = 1536;   // ... and of its gradient (shared memory of the ODE adjoint)
-constexpr int kSegLevels = 3;       // segmented small phase: 2, 4 and 8 segments ...
-constexpr int kSegSlots = 14;       // ... 14 segments in all
-constexpr int kSegMinG = 160;       // ... used from G = 160: their tables cost a fixed time per piece,
-                                    // which the few points they serve repay only on large pieces
 constexpr double kPi = 3.14159265358979323846;
 constexpr double kLog2e = 1.44269504088896340736;
 
@@ -35,18 +31,22 @@ constexpr double kLog2e = 1.44269504088896340736;
 // piece (f1 <-> f2) is folded in.  Channel indices are plan-local.
 struct DevPiece {
     double xlo, xhi, ylo, yhi;
+    double lnx, lny;              // ln(xhi / xlo), ln(yhi / ylo), 1e30 for a zero limit (k_piece_logs)
     int cut, a, b, c_lo;
-    int c_hi, flags, plan, pad;   // flags bit0: s1 < 0, bit1: s2 < 0
-    float mult, pad2, pad3, pad4;
+    int c_hi, flags, plan;        // flags bit0: s1 < 0, bit1: s2 < 0
+    float mult;
 };
 static_assert(sizeof(DevPiece) == 80, "DevPiece layout");
 
-// One work tile: pieces [piece0, piece1) of one CUT for one profile.
+// One work tile: pieces [piece0, piece1) of one CUT for one profile; where a
+// plan has too few pieces to fill the chip, the `part`-th of `parts` shares of
+// their nodes (FP64: grid points).
 struct DevItem {
     int prof;
     int piece0;
     int piece1;
-    int cut;        // plan-local CUT index (for bookkeeping)
+    int cut;        // plan-local CUT index
+    int part;       // share | shares << 16
 };
 
 // Per-launch constants of the quadrature kernels.
@@ -59,6 +59,7 @@ struct QuadParams {
     int G;
     int n_steps;
     double eps_v1;
+    double ln_eps;              // -ln(eps_v1)
     // fibre
     double beta2, beta3, beta4;
     // per plan channel tables (concatenated, index plan_ch_off[plan] + c)
@@ -79,13 +80,7 @@ struct QuadParams {
     const float4 *zs_b;         // {z_{m+1}/2pi hi, lo (float-float), z_m/2pi, 0}
     const double2 *zs_d;        // {z_m, dz_m}
     const float4 *zs_g;         // [5 per step] g_0..g_19: mean of (zeta - L/2)^n over step m (g_19 = 0)
-    // segmented small-phase series (forward FP32): the span cut at step edges
-    // into 2, 4 and 8 segments (kSegLevels levels, kSegSlots segments in all);
-    // per level and step the moments about the step's segment centre, and per
-    // segment its steps and centre in revolutions (float-float).  Null: off.
-    const float4 *zs_gseg;      // [kSegLevels][M][5]
-    const int4 *seg;            // [kSegSlots] {m0, m1, bits of centre/2pi hi, lo}
-    float phi_seg[3];           // per level: |phi| limit [rad/km] (6 / longest segment)
+    const float2 *gauss;        // Gauss rules of the row sums (quad_nodes.cuh): {t, weight}
     const double *kap_L;        // per profile: kappa(L) [1/THz]
     float dz_max;
     float L;                    // span length [km]

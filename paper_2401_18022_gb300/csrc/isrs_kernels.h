@@ -52,7 +52,6 @@ struct AdjParams {
     double *V;                  // [n_items x n_ch]
     const int *item_slot;       // output slot of each item
     int n_ch;
-    double *Yg;                 // per block and warp: FP64 contracted bucket sums (adjoint_scratch_bytes)
 };
 
 // Chain rule from the buckets to dT/dP_j (FP64, single profile).  The
@@ -166,10 +165,13 @@ size_t raman_smem_bytes(int n_ch);
 size_t raman_adj_smem_bytes(int n_ch);
 cudaError_t launch_raman_adj(const RamanAdjParams &ap, cudaStream_t st);
 cudaError_t launch_raman(const RamanParams &rp, int n_prof, int max_n, cudaStream_t st);
-size_t quad_smem_bytes(int precision, int n_steps, int G);
-int quad_blocks_per_sm(int precision, int n_steps, int G, int block);
+// Gauss rules of the row sums: the module's array on the current device, and its fill
+cudaError_t gauss_array(void **out);
+cudaError_t launch_gauss(float2 *out, cudaStream_t st);
+// fills DevPiece::lnx, lny
+cudaError_t launch_piece_logs(DevPiece *pieces, int n, cudaStream_t st);
 cudaError_t launch_prep(const PrepParams &pp, int n_prof, cudaStream_t st);
-cudaError_t launch_quad(const QuadParams &qp, int precision, int grid, int block, cudaStream_t st);
+cudaError_t launch_quad(const QuadParams &qp, int precision, int num_sms, int block, cudaStream_t st);
 // the same quadratures with the tabulated profile (qp.ab set)
 size_t quad_tab_smem_bytes(int precision, int n_steps, int G, int nc_max);
 int quad_tab_blocks_per_sm(int precision, int n_steps, int G, int nc_max, int block);
@@ -187,14 +189,11 @@ size_t quad_mci_tab_smem_bytes(int precision, int n_steps, int n_max, int cpc);
 int quad_mci_tab_blocks_per_sm(int precision, int n_steps, int n_max, int cpc, int block);
 cudaError_t launch_tab_half_log2(const double2 *ab, float2 *abf, int n, int n_sms, cudaStream_t st);
 cudaError_t launch_quad_mci_tab(const QuadParams &qp, int precision, int grid, int block, cudaStream_t st);
-size_t adjoint_smem_bytes(int n_steps, int G, int block);
-size_t adjoint_scratch_bytes(int grid);   // AdjParams.Yg of a launch of `grid` blocks
 // adjoint over the MCI cells of a separate grid (closed-form profile)
 size_t adjoint_mci_smem_bytes(int n_steps, int n_max, int block);
 int adjoint_mci_blocks_per_sm(int n_steps, int n_max, int block);
 cudaError_t launch_adjoint_mci(const AdjParams &ap, int grid, int block, cudaStream_t st);
-int adjoint_blocks_per_sm(int n_steps, int G, int block);
-cudaError_t launch_adjoint(const AdjParams &ap, int grid, int block, cudaStream_t st);
+cudaError_t launch_adjoint(const AdjParams &ap, int num_sms, int block, cudaStream_t st);
 cudaError_t launch_chain(const ChainParams &cp, cudaStream_t st);
 
 }  // namespace isrs

@@ -13,25 +13,21 @@
 //   V_ij  = sum_points w W |S|^2 (number of j among the point's a, b, c).
 //
 // k_quad_adj evaluates the forward sum and these buckets in one pass over the
-// grid, and every step term of Eq. slow_vary is evaluated once.  A warp first
-// takes 32 grid points, one per lane, for their geometry, phase and z-sum
-// form.  Small-phase points (|phi| L <= 6, the forward's range) whose moments
-// come from the contracted centred series (6, 11 or 19 moments by phase) are
-// finished there: their bucket terms sum_n 2 (A|B) phi^n f_n w_m g_n(m) are
-// expanded in the same Chebyshev series in the point's in-channel coordinate,
-// so per F_c candidate at most 95 point sums are kept (one to three 32-value
-// warp butterflies per batch, as many orders as the batch's largest phase
-// needs) and turned into per-step terms once per piece.  The other points join one list per z-sum form and
-// are walked two at a time on half-warps: each of the 16 lanes of a half owns
-// K = ceil(M/16) consecutive steps (112 = 16 x 7), computes their terms t_m
-// into registers, the half sums them with shuffles into S, and the same
-// registers give d|S|^2/d ln p_m = 2 Re(conj(S) t_m) for the lane's own step
-// buckets, which stay in registers between FP64 folds.
+// nodes of the row sums (quad_nodes.cuh; the bucket terms have the band limit of
+// |S|^2, so the nodes that sum a row sum its derivatives too), and every step
+// term of Eq. slow_vary is evaluated once: a node is walked by a half-warp, each
+// of the 16 lanes owning K = ceil(M/16) consecutive steps (112 = 16 x 7),
+// computes their terms t_m into registers, the half sums them with shuffles into
+// S, and the same registers give d|S|^2/d ln p_m = 2 Re(conj(S) t_m) for the
+// lane's own step buckets, which stay in registers between FP64 folds.
 #include <cuda_runtime.h>
 
 #include "isrs_internal.cuh"
 #include "isrs_kernels.h"
+#include <algorithm>
+
 #include "quad_common.cuh"
+#include "quad_nodes.cuh"
 #include "quad_walk.cuh"
 
 namespace isrs {
@@ -39,95 +35,34 @@ namespace isrs {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kClsSmall = 0, kClsDirect = 1, kClsTele = 2;
-constexpr int kListCap = 34;    // a form's list: one carried point + 32 new (+1 pad)
-constexpr int kCtr = 3;         // F_c candidates whose small-phase points are contracted
-constexpr int kCtrN = kChebMom * 5;   // per candidate: moments nu_0..nu_18 x T_0..T_4
-constexpr int kCtrS = 96;       // slots per candidate (three 32-value butterflies)
-// The bucket sums of a batch keep at least the orders its largest contracted
-// |phi| L needs: n <= 5 up to 0.2 (one butterfly, values 0..31; omitted
-// orders below (0.1)^6/6! = 1.4e-9 of the derivative), n <= 10 up to 2 (two,
-// values 0..63; below 2 (1)^11/11! = 5e-8), n <= 18 up to 6 (three, values
-// 0..94; below 2 (3)^19/19! = 1.9e-8).  Rows of the grid have nearly constant
-// phi, so most batches take one form throughout.
-constexpr float kShortPhiL = 0.2f;
-constexpr float kMidPhiL = 2.0f;
-constexpr int kFoldBatches = 256; // batches between FP64 folds of the FP32 accumulators (one per piece at G = 256)
-constexpr int kTeleCand = 4;      // F_c candidates with their own telescoped-walk rows (attenuation folded in)
-constexpr int kAdjWarps = 8;      // warps per block at most (launch bound 256 threads)
+constexpr int kAdjSlots = 256;   // node slots of a chunk
+constexpr int kAdjCand = 3;      // F_c candidates swept together (most pieces have two)
 constexpr float kPadLog2 = -1000.0f;   // log2 weight of the padding steps (ex2 -> 0)
+using AdjNodes = WarpNodes<kAdjSlots>;
 
-// Forward-sum bookkeeping of one grid point: the point's owner (every lane
-// for a contracted point, lane 0 of each half for a walked one) adds its value
-// to the compensated sum and to its F_c candidate's PSD bucket: registers for
-// the first four candidates, beyond them this half-warp's own row of sVc.  Only
-// that half's owner lane ever adds to the row, so its adds run in program
-// order (deterministic); they are issued as shared-memory reductions, which
-// hold no register across the add (a plain load-add-store here doubled the
-// kernel's spills).
-struct FwdAcc {
-    float sum, comp, v0, v1, v2, v3;
+// One warp's shared memory: nodes, the points to walk, step rows per
+// candidate, FP64 step buckets.
+template <int K>
+struct __align__(16) AdjWarp {
+    AdjNodes ns;
+    float4 L[32];                // {w W af, phi, phi_lo, u}
+    int Lc[32];                  // candidate, from the sweep's first
+    float2 ek[kAdjCand][K * 16]; // {log2 p at f_c, K2}, [k][lane of the half]
+    double2 B[K * 16];
 };
-
-__device__ __forceinline__ void fwd_add(FwdAcc &a, float val, int ci, bool owner, float *sVc)
-{
-    const float vv = owner ? val : 0.0f;
-    const float y = vv - a.comp;
-    const float t = a.sum + y;
-    a.comp = (t - a.sum) - y;
-    a.sum = t;
-    a.v0 += ci == 0 ? vv : 0.0f;
-    a.v1 += ci == 1 ? vv : 0.0f;
-    a.v2 += ci == 2 ? vv : 0.0f;
-    a.v3 += ci == 3 ? vv : 0.0f;
-    if (owner && ci >= 4) atomicAdd(&sVc[(threadIdx.x >> 4) * kMaxCand + ci], val);
-}
-
-// Warp sums of the contracted bucket values of group G0 (values 32 G0 ..
-// 32 G0 + 31): value v = al_n T_k(x) with n = v / 5, k = v mod 5, al_n = ae
-// phi^n (n even) or ao phi^(n-1) (n odd; ao carries one phi).  Only the
-// orders the group spans are formed.  A batch that needs fewer orders than
-// the group holds still sums all 32: the extra ones are further terms of the
-// same series, so they can only be kept (slots up to 94) or dropped.
-template <int G0>
-__device__ __forceinline__ float ctr_group(float ae, float ao, float p2, const float (&Tk)[5], int lane)
-{
-    constexpr int N0 = (32 * G0) / 5;          // 0, 6, 12: even
-    float pw = 1.0f;
-#pragma unroll
-    for (int i = 0; i < N0 / 2; ++i) pw *= p2;
-    float a[8];
-    a[0] = ae * pw;
-    a[1] = ao * pw;
-#pragma unroll
-    for (int j = 2; j < 8; ++j) a[j] = a[j - 2] * p2;
-    return butterfly32(
-        [&](int v) {
-            const int va = 32 * G0 + v;
-            return a[va / 5 - N0] * Tk[va % 5];
-        },
-        lane);
-}
 
 }  // namespace
 
 // ---------------------------------------------------------------------------
 // k_quad_adj<K>: fused forward + adjoint, persistent over work tiles of one
-// profile.  Per batch of 32 grid points a warp
-//  1. classifies its points (one per lane); contracted small-phase points are
-//     finished here, the others are appended to the warp's list of their
-//     z-sum form (non-contracted small phase, direct, telescoped);
-//  2. walks every list two points at a time, one per half-warp, so both
-//     halves always run the same form; an odd point waits for the next batch
-//     (or, at the end of the piece, is walked beside a zero-weight copy).
-// The owned step tables are lane-contiguous float4 copies in shared memory
-// (conflict-free, both halves broadcast).  Lane buckets accumulate in
-// registers and are folded into per-warp FP64 shared buckets every 256 batches
-// (once per piece at G = 256: FP32 sums of at most ~512 terms, and the FP64
-// pipe, ~1/64 of the FP32 rate on this GPU, stays nearly idle).
-// Every reduction has a fixed order (the PSD buckets go to the tile's own row,
-// summed per CUT in tile order by k_v_reduce), so results are bit for bit
-// reproducible.
+// profile; every warp takes its own tiles.  Per batch of 32 slots a warp sets up
+// one node per lane, lists the direct ones from the front and the telescoped
+// ones from the back, and walks them two at a time, one per half-warp (an odd
+// one beside a zero-weight copy of itself).  Lane buckets accumulate in
+// registers over a piece and are folded into the warp's FP64 buckets, which go
+// to the tile's own row; PSD buckets are added to the tile's own row by one
+// lane.  Every sum has a fixed order (k_v_reduce sums a CUT's rows in tile
+// order), so results are bit for bit reproducible.
 // ---------------------------------------------------------------------------
 #ifndef ISRS_ADJ_MIN_BLOCKS
 #define ISRS_ADJ_MIN_BLOCKS 3   // resident blocks per SM the register budget is sized for
@@ -139,417 +74,180 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
     const QuadParams &qp = ap.q;
     extern __shared__ float4 smem_f4[];
     const int M = qp.n_steps, G = qp.G;
-    const int nw = blockDim.x >> 5;
-    float4 *sT = smem_f4;                                     // [M] {A2 + log2 dz, K2, z, z^2 + dz^2/12}
-    float4 *sO0 = sT + M;                                     // [K][16] owned {A2 + log2 dz, K2, z, dz}
-    float4 *sO1 = sO0 + K * 16;                               // [K][16] owned {edge/2pi hi, lo, A2, c}
-    float4 *sOc = sO1 + K * 16;                               // [kTeleCand][K][16] {hi, lo, A2 - at_c z, K2}
-    float4 *sL = sOc + kTeleCand * K * 16;                    // [nw][3][kListCap] {w W af, phi, F_c, ci}
-    double2 *sB = reinterpret_cast<double2 *>(sL + nw * 3 * kListCap);   // [nw][K][16] FP64 step buckets
-    RowF *rows = reinterpret_cast<RowF *>(sB + nw * K * 16);             // [G]
-    __shared__ PieceConst<float> kc;
-    __shared__ ChebTabN<kCtr> ct;
-    __shared__ float sVc[16 * kMaxCand];    // PSD buckets of candidates past the fourth, per half-warp
-    __shared__ double scratch[32];
-    __shared__ int s_item;
-    // small-phase points of contracted candidates: per-warp moment sums (FP32
-    // between folds in shared memory, FP64 after in this block's global
-    // scratch, touched once per fold), their block totals, and the per-step
-    // bucket terms they give for the tile
-    __shared__ float sYf[kAdjWarps][kCtr][kCtrS];
-    double *gY = ap.Yg + (size_t)blockIdx.x * kAdjWarps * kCtr * kCtrN;   // [warp][c][v]
-    __shared__ double sYt[kCtr][kCtrN];
-    __shared__ double2 sC[128];
-
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int t = threadIdx.x; t < kAdjWarps * kCtr * kCtrN; t += blockDim.x) gY[t] = 0.0;
-    for (int t = threadIdx.x; t < kAdjWarps * kCtr * kCtrS; t += blockDim.x) (&sYf[0][0][0])[t] = 0.0f;
-    for (int t = threadIdx.x; t < 128; t += blockDim.x) sC[t] = make_double2(0.0, 0.0);
-    for (int t = threadIdx.x; t < nw * K * 16; t += blockDim.x) sB[t] = make_double2(0.0, 0.0);
-    for (int t = threadIdx.x; t < 16 * kMaxCand; t += blockDim.x) sVc[t] = 0.0f;
+    const int l16 = lane & 15, half = lane >> 4;       // lane l owns steps [K (l mod 16), K (l mod 16) + K)
+    float4 *zt = smem_f4;                              // [K][16] {edge/2pi hi, lo, z, dz}
+    AdjWarp<K> &w = reinterpret_cast<AdjWarp<K> *>(zt + K * 16)[warp];
+    AdjNodes &ns = w.ns;
 
-    const float c3 = (float)(kPi * qp.beta3);
-    const float c4 = (float)(2.0 * kPi * kPi / 3.0 * qp.beta4);
-    const float b2 = (float)qp.beta2;
-    const float m4pi2 = (float)(-4.0 * kPi * kPi);
+    // padding steps past M repeat the last edge
+    for (int t = threadIdx.x; t < K * 16; t += blockDim.x) {
+        const int m = min((t & 15) * K + (t >> 4), M - 1);
+        const float4 za = qp.zs_a[m], zb = qp.zs_b[m];
+        zt[t] = make_float4(zb.x, zb.y, za.x, za.w);
+    }
+    __syncthreads();
     const float phi_direct = 3.14159265f / qp.dz_max;
-    const float phi_small = 0.02f / qp.L;
-    const float phi_cheb = kChebPhiL / qp.L;
-    const float phi_c6 = kChebPhiL6 / qp.L, phi_c11 = kChebPhiL11 / qp.L;
+    const float phi_small = kBlkPhiL / qp.L;
     const float log2e = (float)kLog2e;
-    const float invG = 1.0f / (float)G;
-    // the walks run on half-warps: lane l owns steps [K (l mod 16), K (l mod 16) + K)
-    const int l16 = lane & 15, half = lane >> 4;
-    const float4 *o0s = sO0 + l16;
-    const float4 *o1s = sO1 + l16;
-    float4 *Ls = sL + warp * 3 * kListCap;
-    float4 *Ld = Ls + kListCap;
-    float4 *Lt = Ld + kListCap;
-    double2 *myB = sB + warp * K * 16;
     const unsigned lt_mask = (1u << lane) - 1u;
-    unsigned n_small = 0, n_direct = 0, n_tele = 0;    // points per z-sum form (lane 0 counts)
-    int cur_prof = -1;
+    unsigned long long n_small = 0;
+    unsigned n_direct = 0, n_tele = 0;
 
     for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_item = atomicAdd(qp.counter, 1);
-        __syncthreads();
-        const int it = s_item;
+        int it = 0;
+        if (lane == 0) it = atomicAdd(qp.counter, 1);
+        it = __shfl_sync(kFull, it, 0);
         if (it >= qp.n_items) break;
         const DevItem item = qp.items[it];
+        const float2 *st = qp.step_f + (size_t)item.prof * M;
+        const float tilt = (float)qp.kap_L[item.prof];
+        const int part = item.part & 0xffff, parts = item.part >> 16;
         double *Vrow = ap.V + (size_t)it * ap.n_ch;     // this tile's PSD buckets
-        for (int c = threadIdx.x; c < ap.n_ch; c += blockDim.x) Vrow[c] = 0.0;
-        if (item.prof != cur_prof) {
-            const float2 *st = qp.step_f + (size_t)item.prof * M;
-            for (int m = threadIdx.x; m < M; m += blockDim.x) {
-                const float2 v = st[m];
-                const float4 za = qp.zs_a[m];
-                sT[m] = make_float4(v.x + za.z, v.y, za.x, za.y);
-            }
-            // lane-contiguous copies of every lane's owned step tables; the
-            // padding steps past M have zero weight and repeat the last edge
-            const float4 zl = qp.zs_b[M - 1];
-            for (int t = threadIdx.x; t < K * 16; t += blockDim.x) {
-                const int k = t >> 4, l = t & 15, m = l * K + k;
-                float4 o0 = make_float4(kPadLog2, 0.f, 0.f, 0.f);
-                float4 o1 = make_float4(zl.x, zl.y, kPadLog2, 0.f);
-                if (m < M) {
-                    const float2 v = st[m];
-                    const float4 za = qp.zs_a[m];
-                    const float4 zb = qp.zs_b[m];
-                    o0 = make_float4(v.x + za.z, v.y, za.x, za.w);
-                    o1 = make_float4(zb.x, zb.y, v.x, za.y);
-                }
-                sO0[k * 16 + l] = o0;
-                sO1[k * 16 + l] = o1;
-            }
-            cur_prof = item.prof;
-        }
-        double acc = 0.0;
+        for (int c = lane; c < ap.n_ch; c += 32) Vrow[c] = 0.0;
+        for (int t = lane; t < K * 16; t += 32) w.B[t] = make_double2(0.0, 0.0);
+        double acc = 0.0;                               // lane 0
         for (int kp = item.piece0; kp < item.piece1; ++kp) {
-            const DevPiece pc = qp.pieces[dbg_clamp(kp, qp.n_pieces, kDbgPiece, qp.dbg)];
-            piece_rows<RowF>(pc, G, qp.eps_v1, rows);
-            piece_consts<float>(qp, pc, item.prof, log2e, qp.pd_f, kc);
-            __syncthreads();
-            // telescoped-walk rows of the first candidates (read after the setup's sync)
-            for (int t = threadIdx.x; t < kTeleCand * K * 16; t += blockDim.x) {
-                const int c = t / (K * 16), r = t - c * (K * 16);
-                if (c < kc.nc) {
-                    const float4 a = sO0[r], b = sO1[r];
-                    sOc[t] = make_float4(b.x, b.y, fmaf(-(kc.at_ab + kc.hat[c]), a.z, b.z), a.y);
-                }
-            }
-            // step weights of the contracted candidates, once per piece, in the
-            // (empty until the points start) list space
-            int nW = 0;
-            if (cheb_applies(qp, pc, item.prof, kc) && min(kc.nc, kCtr) * M <= nw * 3 * kListCap) {
-                nW = min(kc.nc, kCtr);
-                cheb_weights(qp, pc, sT, M, kc, nW, sL);
-                __syncthreads();
-            }
-            cheb_setup<kChebMom>(qp, pc, item.prof, sT, M, kc, ct, sL, nW);
-            __syncthreads();
-            const bool cheb = ct.ok != 0;
-            const float fi = kc.fi, s1g = kc.s1, s2g = kc.s2, mult = kc.mult;
-            const float three_fi2 = 3.0f * fi * fi;
-            FwdAcc fa = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+            const DevPiece &pc = qp.pieces[dbg_clamp(kp, qp.n_pieces, kDbgPiece, qp.dbg)];
+            __syncwarp();
+            node_geo(qp, pc, item.prof, log2e, qp.pd_f, tilt, ns.geo);
+            __syncwarp();
+            const PieceGeo &g = ns.geo;
+            const float mult = g.mult;
             float R[K], Rp[K];
 #pragma unroll
             for (int k = 0; k < K; ++k) {
                 R[k] = 0.0f;
                 Rp[k] = 0.0f;
             }
-            int ns = 0, nd = 0, nt = 0;      // list lengths (warp-uniform)
-            const int npts = G * G;
-            int batches = 0;
-            for (int qb = warp * 32; qb < npts; qb += blockDim.x) {
-                // ---- 1. this lane's grid point
-                const int q = qb + lane;
-                float phi = 0.0f, Fc = 0.0f, wwa = 0.0f, cpt = 0.0f;
-                int cls = -1, ci = -1;
-                bool ctr = false;            // contracted small-phase point
-                float cx = 0.0f, cA = 0.0f, cB = 0.0f;
-                if (q < npts) {
-                    const int r = (int)(((float)q + 0.5f) * invG);
-                    const int j = q - r * G;
-                    const RowF rw = rows[dbg_clamp(r, G, kDbgRow, qp.dbg)];
-                    if (rw.w != 0.0f) {
-                        const float d = ((float)j + 0.5f - 0.5f * (float)G) * rw.du2;
-                        const float e = expf(d);
-                        const float f1 = s1g * (rw.xc * e);
-                        const float f2 = s2g * (rw.yc * __frcp_rn(e));
-                        const float u = f1 + f2;
-                        for (int c = 0; c < kc.nc; ++c) {
-                            if (u >= kc.lo[c] && u < kc.hi[c]) { ci = c; break; }
+            double ptot = 0.0;
+            for (int ca = 0; ca < g.nc; ca += kAdjCand) {
+                const int cb = min(g.nc, ca + kAdjCand);
+                for (int c = ca; c < cb; ++c) {
+                    const float at = g.at_ab + g.hat[c], F = g.Fc0 + 0.5f * (g.lo[c] + g.hi[c]);
+                    for (int t = lane; t < K * 16; t += 32) {
+                        const int m = (t & 15) * K + (t >> 4);
+                        float2 e = make_float2(kPadLog2, 0.0f);
+                        if (m < M) {
+                            const float2 v = st[m];
+                            e = make_float2(fmaf(v.y, F, fmaf(-at, zt[t].z, v.x)), v.y);
                         }
-                        if (ci >= 0) {
-                            const float W = kc.wab * kc.pd[ci];
-                            Fc = fi + u;
-                            const float br = b2 + c3 * (u + 2.0f * fi) +
-                                             c4 * (f1 * f1 + 1.5f * f1 * f2 + 3.0f * fi * u + f2 * f2 + three_fi2);
-                            phi = m4pi2 * f1 * f2 * br;
-                            const float aphi = fabsf(phi);
-                            wwa = rw.w * W * array_factor_f(phi, qp);
-                            if (cheb && ci < kCtr && aphi <= phi_cheb) {
-                                cheb_point(ct, ci, u, phi, aphi, phi_c6, phi_c11, cx, cA, cB);
-                                ctr = true;
-                                cls = kClsSmall;
-                                fwd_add(fa, wwa * fmaf(cA, cA, cB * cB), ci, true, sVc);
-                                cpt = mult * wwa;
-                            } else if (aphi <= phi_small) {
-                                cls = kClsSmall;
-                            } else {
-                                cls = aphi <= phi_direct ? kClsDirect : kClsTele;
-                            }
-                        }
+                        w.ek[c - ca][t] = e;
                     }
                 }
-                // Contracted small-phase points: |S|^2 = A^2 + B^2 with A (B) the sum of
-                // phi^n nu'_n over even (odd) n, so d|S|^2/d ln p_m = sum_n 2 (A|B)
-                // phi^n f_n w_m g_n(m) with w_m = base_m sum_k b_k(a_m) T_k(x).  Their
-                // bucket terms need only, per candidate, the sums of cp 2 (A|B) phi^n
-                // T_k(x) (k <= 4 for the F_c-weighted bucket, x T_k = (T_{k+1} +
-                // T_{|k-1|})/2): 95 values, of which a batch reduces the first 32, 64
-                // or 96 over the warp (one to three butterflies) by its largest
-                // phase; they become per-step terms once per piece.
-                unsigned cmask = __ballot_sync(kFull, ctr);
-                const unsigned cmask0 = cmask;
-                if (cmask) {
-                    // positive floats order as their bit patterns
-                    const unsigned phl = __reduce_max_sync(kFull, __float_as_uint(ctr ? fabsf(phi) * qp.L : 0.0f));
-                    const float phLmax = __uint_as_float(phl);
-                    const int form = phLmax <= kShortPhiL ? 0 : (phLmax <= kMidPhiL ? 1 : 2);
-                    const float T2 = fmaf(2.0f * cx, cx, -1.0f);
-                    const float T3 = fmaf(2.0f * cx, T2, -cx);
-                    const float T4 = fmaf(2.0f * cx, T3, -T2);
-                    const float Tk[5] = {1.0f, cx, T2, T3, T4};
-                    while (cmask) {
-                        const int cl = __shfl_sync(kFull, ci, __ffs(cmask) - 1);
-                        const bool mine = ctr && ci == cl;
-                        const float ae = mine ? 2.0f * cpt * cA : 0.0f;
-                        const float ao = mine ? 2.0f * cpt * cB * phi : 0.0f;
-                        const float p2 = phi * phi;
-                        float *Yw = sYf[warp][cl];
-                        const float y0 = ctr_group<0>(ae, ao, p2, Tk, lane);
-                        Yw[lane] += y0;
-                        if (form >= 1) {
-                            const float y1 = ctr_group<1>(ae, ao, p2, Tk, lane);
-                            Yw[lane + 32] += y1;
-                        }
-                        if (form == 2) {
-                            const float y2 = ctr_group<2>(ae, ao, p2, Tk, lane);
-                            Yw[lane + 64] += y2;
-                        }
-                        cmask &= ~__ballot_sync(kFull, mine);
-                    }
-                }
-                // append the other points to their form's list
-                const bool stage = cls >= 0 && !ctr;
-                const unsigned bs = __ballot_sync(kFull, stage && cls == kClsSmall);
-                const unsigned bd = __ballot_sync(kFull, stage && cls == kClsDirect);
-                const unsigned bt = __ballot_sync(kFull, stage && cls == kClsTele);
-                if (stage) {
-                    const float4 v = make_float4(wwa, phi, Fc, __int_as_float(ci));
-                    if (cls == kClsSmall) Ls[dbg_clamp(ns + __popc(bs & lt_mask), kListCap, kDbgList, qp.dbg)] = v;
-                    else if (cls == kClsDirect) Ld[dbg_clamp(nd + __popc(bd & lt_mask), kListCap, kDbgList, qp.dbg)] = v;
-                    else Lt[dbg_clamp(nt + __popc(bt & lt_mask), kListCap, kDbgList, qp.dbg)] = v;
-                }
-                if (lane == 0) {
-                    n_small += __popc(bs) + __popc(cmask0);
-                    n_direct += __popc(bd);
-                    n_tele += __popc(bt);
-                }
-                ns += __popc(bs);
-                nd += __popc(bd);
-                nt += __popc(bt);
                 __syncwarp();
-                // ---- 2. walk the lists in pairs, one point per half-warp
-                for (int p = half; p + 1 - half < nd; p += 2) {
-                    const float4 st = Ld[p];
-                    const int pci = __float_as_int(st.w);
-                    const float at = kc.at_ab + kc.hat[pci];
-                    const float val = walk_direct<K>(o0s, st.x, st.y, st.z, at, mult, R, Rp);
-                    fwd_add(fa, val, pci, l16 == 0, sVc);
-                }
-                for (int p = half; p + 1 - half < nt; p += 2) {
-                    const float4 st = Lt[p];
-                    const int pci = __float_as_int(st.w);
-                    const float at = kc.at_ab + kc.hat[pci];
-                    // both halves on folded rows, or both on the shared tables
-                    const float val = __all_sync(kFull, pci < kTeleCand)
-                                          ? walk_tele<K, false, true>(o0s, sOc + pci * K * 16 + l16, l16, st.x, st.y,
-                                                                      st.z, at, mult, R, Rp)
-                                          : walk_tele<K>(o0s, o1s, l16, st.x, st.y, st.z, at, mult, R, Rp);
-                    fwd_add(fa, val, pci, l16 == 0, sVc);
-                }
-                for (int p = half; p + 1 - half < ns; p += 2) {
-                    const float4 st = Ls[p];
-                    const int pci = __float_as_int(st.w);
-                    const float at = kc.at_ab + kc.hat[pci];
-                    const float val = walk_small<K>(o0s, o1s, st.x, st.y, st.z, at, mult, R, Rp);
-                    fwd_add(fa, val, pci, l16 == 0, sVc);
-                }
-                // an odd point waits at the head of its list for the next batch
-                __syncwarp();
-                if (lane == 0) {
-                    if (nd & 1) Ld[0] = Ld[nd - 1];
-                    if (nt & 1) Lt[0] = Lt[nt - 1];
-                    if (ns & 1) Ls[0] = Ls[ns - 1];
-                }
-                nd &= 1;
-                nt &= 1;
-                ns &= 1;
-                if (++batches == kFoldBatches) {
-                    batches = 0;
-                    // step buckets: the two halves' registers meet, then FP64
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        const float rx = R[k] + __shfl_xor_sync(kFull, R[k], 16);
-                        const float ry = Rp[k] + __shfl_xor_sync(kFull, Rp[k], 16);
-                        if (half == 0) {
-                            double2 &d = myB[k * 16 + l16];
-                            d.x += (double)rx;
-                            d.y += (double)ry;
+                // forward sum (compensated) and PSD buckets of the candidates, on
+                // lane 0 of each half
+                float sum = 0.0f, comp = 0.0f, v0 = 0.0f, v1 = 0.0f, v2 = 0.0f;
+                const auto add = [&](float val, int c) {
+                    const float y = val - comp;
+                    const float t = sum + y;
+                    comp = (t - sum) - y;
+                    sum = t;
+                    v0 += c == 0 ? val : 0.0f;
+                    v1 += c == 1 ? val : 0.0f;
+                    v2 += c == 2 ? val : 0.0f;
+                };
+                int small;
+                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int nq) {
+                    for (int q0 = 32 * part; q0 < nq; q0 += 32 * parts) {
+                        Node nd;
+                        int cls = -1;
+                        if (q0 + lane < nq && node_get(ns, qp.gauss, q0 + lane, nd)) {
+                            const float aphi = fabsf(nd.phi);
+                            cls = aphi <= phi_direct ? 0 : 1;
+                            n_small += aphi <= phi_small ? nd.N : 0;
+                            n_direct += aphi > phi_small && cls == 0 ? nd.N : 0;
+                            n_tele += cls == 0 ? 0 : nd.N;
                         }
-                        R[k] = 0.0f;
-                        Rp[k] = 0.0f;
+                        const unsigned bd = __ballot_sync(kFull, cls == 0), bt = __ballot_sync(kFull, cls == 1);
+                        if (cls >= 0) {
+                            const int ci = dbg_clamp(nd.ci, g.nc, kDbgCand, qp.dbg);
+                            const int at = cls == 0 ? __popc(bd & lt_mask) : 31 - __popc(bt & lt_mask);
+                            w.L[at] = make_float4(nd.wq * g.wab * g.pd[ci] * array_factor_f(nd.phi, qp, nd.phi_lo),
+                                                  nd.phi, nd.phi_lo, nd.x + nd.y);
+                            w.Lc[at] = ci - ca;
+                        }
+                        __syncwarp();
+                        const int nd0 = __popc(bd), nt0 = __popc(bt);
+                        for (int p = 0; p < nd0; p += 2) {
+                            const int at = min(p + half, nd0 - 1);
+                            const float4 v = w.L[at];
+                            const int c = w.Lc[at];
+                            const float wq = p + half < nd0 ? v.x : 0.0f;
+                            const float dF = v.w - 0.5f * (g.lo[ca + c] + g.hi[ca + c]);
+                            const float val = walk_direct_n<K>(zt + l16, w.ek[c] + l16, wq, v.y, dF, g.Fc0 + v.w,
+                                                               mult, R, Rp);
+                            add(l16 == 0 ? val : 0.0f, c);
+                        }
+                        for (int p = 0; p < nt0; p += 2) {
+                            const int at = 31 - min(p + half, nt0 - 1);
+                            const float4 v = w.L[at];
+                            const int c = w.Lc[at];
+                            const float wq = p + half < nt0 ? v.x : 0.0f;
+                            const float dF = v.w - 0.5f * (g.lo[ca + c] + g.hi[ca + c]);
+                            const float val = walk_tele_n<K>(zt + l16, w.ek[c] + l16, l16, wq, v.y, v.z, dF,
+                                                             g.Fc0 + v.w, mult, R, Rp);
+                            add(l16 == 0 ? val : 0.0f, c);
+                        }
+                        __syncwarp();
                     }
-                    for (int t = lane; t < kCtr * kCtrS; t += 32) {
-                        const int c = t / kCtrS, v = t - c * kCtrS;
-                        if (v < kCtrN) gY[(warp * kCtr + c) * kCtrN + v] += (double)sYf[warp][c][v];
-                        sYf[warp][c][v] = 0.0f;
+                });
+                n_small += lane == 0 && part == 0 ? small : 0;
+                // sweep totals: the two halves' lane 0 meet on lane 0
+                const double s = (double)sum - (double)comp;
+                const double sw = (double)mult * (s + __shfl_down_sync(kFull, s, 16));
+                const float w0 = __shfl_down_sync(kFull, v0, 16), w1 = __shfl_down_sync(kFull, v1, 16),
+                            w2 = __shfl_down_sync(kFull, v2, 16);
+                if (lane == 0) {
+                    ptot += sw;
+                    // one lane, in order; the row is this tile's
+                    for (int c = ca; c < cb; ++c) {
+                        const double vc = c == ca ? (double)v0 + (double)w0
+                                        : c == ca + 1 ? (double)v1 + (double)w1 : (double)v2 + (double)w2;
+                        atomicAdd(&Vrow[dbg_clamp(pc.c_lo + c, ap.n_ch, kDbgVrow, qp.dbg)], (double)mult * vc);
                     }
                 }
-                __syncwarp();          // the next batch appends to the lists
+                __syncwarp();
             }
-            // the last odd point of each form, beside a zero-weight copy of itself
-            if (nd) {
-                float4 st = Ld[0];
-                const int pci = __float_as_int(st.w);
-                if (half) st.x = 0.0f;
-                const float val = walk_direct<K>(o0s, st.x, st.y, st.z, kc.at_ab + kc.hat[pci], mult, R, Rp);
-                fwd_add(fa, val, pci, l16 == 0, sVc);
-            }
-            if (nt) {
-                float4 st = Lt[0];
-                const int pci = __float_as_int(st.w);
-                if (half) st.x = 0.0f;
-                const float val = pci < kTeleCand
-                                      ? walk_tele<K, false, true>(o0s, sOc + pci * K * 16 + l16, l16, st.x, st.y,
-                                                                  st.z, 0.0f, mult, R, Rp)
-                                      : walk_tele<K>(o0s, o1s, l16, st.x, st.y, st.z, kc.at_ab + kc.hat[pci], mult,
-                                                     R, Rp);
-                fwd_add(fa, val, pci, l16 == 0, sVc);
-            }
-            if (ns) {
-                float4 st = Ls[0];
-                const int pci = __float_as_int(st.w);
-                if (half) st.x = 0.0f;
-                const float val = walk_small<K>(o0s, o1s, st.x, st.y, st.z, kc.at_ab + kc.hat[pci], mult, R, Rp);
-                fwd_add(fa, val, pci, l16 == 0, sVc);
+            if (lane == 0) {
+                acc += ptot;
+                atomicAdd(&Vrow[dbg_clamp(pc.a, ap.n_ch, kDbgVrow, qp.dbg)], ptot);
+                atomicAdd(&Vrow[dbg_clamp(pc.b, ap.n_ch, kDbgVrow, qp.dbg)], ptot);
             }
 #pragma unroll
             for (int k = 0; k < K; ++k) {
                 const float rx = R[k] + __shfl_xor_sync(kFull, R[k], 16);
                 const float ry = Rp[k] + __shfl_xor_sync(kFull, Rp[k], 16);
                 if (half == 0) {
-                    double2 &d = myB[k * 16 + l16];
+                    double2 &d = w.B[k * 16 + l16];
                     d.x += (double)rx;
                     d.y += (double)ry;
                 }
             }
-            __syncwarp();
-            for (int t = lane; t < kCtr * kCtrS; t += 32) {
-                const int c = t / kCtrS, v = t - c * kCtrS;
-                if (v < kCtrN) gY[(warp * kCtr + c) * kCtrN + v] += (double)sYf[warp][c][v];
-                sYf[warp][c][v] = 0.0f;
-            }
-            // piece totals: the forward sum and the PSD buckets V_ij
-            const double ptot = block_sum_d((double)fa.sum - (double)fa.comp, scratch);
-            if (cheb) {
-                // contracted small-phase terms of this piece -> per-step tile buckets
-                const int ncc = min(kc.nc, kCtr);
-                for (int t = threadIdx.x; t < ncc * kCtrN; t += blockDim.x) {
-                    const int c = t / kCtrN, e = t - c * kCtrN;
-                    double y = 0.0;
-                    for (int w = 0; w < nw; ++w) {
-                        double &g = gY[(w * kCtr + c) * kCtrN + e];
-                        y += g;
-                        g = 0.0;
-                    }
-                    sYt[c][e] = y;
-                }
-                __syncthreads();
-                const int coff = qp.plan_ch_off[pc.plan];
-                for (int m = threadIdx.x; m < M; m += blockDim.x) {
-                    const float4 a = sT[m];           // {A2 + log2 dz, K2, z, z^2 + dz^2/12}
-                    const float *gm = reinterpret_cast<const float *>(qp.zs_g + kZsG * m);   // g_0..g_18
-                    double rx = 0.0, ry = 0.0;
-                    for (int c = 0; c < ncc; ++c) {
-                        const double *Y = sYt[c];
-                        const double F0 = qp.ch_frel[coff + pc.c_lo + c];
-                        const double h = 0.5 * qp.ch_B[coff + pc.c_lo + c];
-                        const double atc = (double)(kc.at_ab + kc.hat[c]);
-                        const double base = exp2((double)a.x - atc * (double)a.z + (double)a.y * F0);
-                        const float t = (float)(0.5 * (double)a.y * h * 0.69314718055994530942), t2 = t * t;
-                        const float b0 = 1.0f + t2 * (1.0f + t2 * (0.25f + t2 / 36.0f));                 // I0
-                        const float b1 = 2.0f * t * (1.0f + t2 * (0.5f + t2 / 12.0f));                    // 2 I1
-                        const float b2 = 2.0f * t2 * (0.5f + t2 * (1.0f / 6.0f + t2 / 48.0f));            // 2 I2
-                        const float b3 = 2.0f * t2 * t * (1.0f / 6.0f + t2 * (1.0f / 24.0f + t2 / 240.0f)); // 2 I3
-                        float rs = 0.0f, xs = 0.0f;
-#pragma unroll
-                        for (int n = 0; n < kChebMom; ++n) {
-                            const double *Yn = Y + 5 * n;
-                            const float y0 = (float)Yn[0], y1 = (float)Yn[1], y2 = (float)Yn[2], y3 = (float)Yn[3],
-                                        y4 = (float)Yn[4];
-                            const float gf = (float)cheb_fold(n) * gm[n];
-                            rs = fmaf(gf, b0 * y0 + b1 * y1 + b2 * y2 + b3 * y3, rs);
-                            xs = fmaf(gf, b0 * y1 + 0.5f * (b1 * (y2 + y0) + b2 * (y3 + y1) + b3 * (y4 + y2)), xs);
-                        }
-                        rx += base * (double)rs;
-                        ry += base * (F0 * (double)rs + h * (double)xs);
-                    }
-                    sC[m].x += rx;
-                    sC[m].y += ry;
-                }
-            }
-            const double t0 = block_sum_d((double)fa.v0, scratch);
-            const double t1 = block_sum_d((double)fa.v1, scratch);
-            const double t2 = block_sum_d((double)fa.v2, scratch);
-            const double t3 = block_sum_d((double)fa.v3, scratch);   // syncs: sVc complete
-            acc += (double)mult * ptot;
-            if (threadIdx.x == 0) {                 // one thread, in order (the row is this tile's)
-                Vrow[dbg_clamp(pc.a, ap.n_ch, kDbgVrow, qp.dbg)] += (double)mult * ptot;
-                Vrow[dbg_clamp(pc.b, ap.n_ch, kDbgVrow, qp.dbg)] += (double)mult * ptot;
-                for (int c = 0; c < kc.nc; ++c) {
-                    double vc = c == 0 ? t0 : c == 1 ? t1 : c == 2 ? t2 : c == 3 ? t3 : 0.0;
-                    for (int hw = 0; hw < 2 * nw; ++hw) vc += (double)sVc[hw * kMaxCand + c];
-                    Vrow[dbg_clamp(pc.c_lo + c, ap.n_ch, kDbgVrow, qp.dbg)] += (double)mult * vc;
-                }
-            }
-            __syncthreads();
-            for (int t = threadIdx.x; t < 16 * kMaxCand; t += blockDim.x) sVc[t] = 0.0f;
         }
         // tile outputs: the forward partial and the step buckets
-        if (threadIdx.x == 0) qp.partial[it] = acc;
-        __syncthreads();
-        for (int m = threadIdx.x; m < M; m += blockDim.x) {
+        if (lane == 0) qp.partial[it] = acc;
+        __syncwarp();
+        for (int m = lane; m < M; m += 32) {
             const int ln = m / K, kk = m - ln * K;
-            double rx = 0.0, ry = 0.0;
-            for (int w = 0; w < nw; ++w) {
-                double2 &b = sB[(w * K + kk) * 16 + ln];
-                rx += b.x;
-                ry += b.y;
-                b = make_double2(0.0, 0.0);
-            }
-            ap.item_R[(size_t)it * M + m] = make_double2(rx + sC[m].x, ry + sC[m].y);
-            sC[m] = make_double2(0.0, 0.0);
+            ap.item_R[(size_t)it * M + m] = w.B[kk * 16 + ln];
         }
+        __syncwarp();
     }
-    if (qp.path_count && lane == 0) {
-        atomicAdd(&qp.path_count[0], (unsigned long long)n_small);
-        atomicAdd(&qp.path_count[1], (unsigned long long)n_direct);
-        atomicAdd(&qp.path_count[2], (unsigned long long)n_tele);
+    if (qp.path_count) {
+        unsigned long long c0 = n_small, c1 = n_direct, c2 = n_tele;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            c0 += __shfl_xor_sync(kFull, c0, o);
+            c1 += __shfl_xor_sync(kFull, c1, o);
+            c2 += __shfl_xor_sync(kFull, c2, o);
+        }
+        if (lane == 0) {
+            atomicAdd(&qp.path_count[0], c0);
+            atomicAdd(&qp.path_count[1], c1);
+            atomicAdd(&qp.path_count[2], c2);
+        }
     }
 }
 
@@ -738,60 +436,39 @@ __global__ void __launch_bounds__(256) k_chain_ch(ChainParams cp)
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-size_t adjoint_smem_bytes(int n_steps, int G, int block)
-{
-    const int K = (n_steps + 15) / 16, nw = block / 32;
-    return (size_t)(n_steps + (2 + kTeleCand) * K * 16 + nw * 3 * kListCap) * sizeof(float4) +
-           (size_t)nw * K * 16 * sizeof(double2) + (size_t)G * sizeof(RowF);
-}
-
-size_t adjoint_scratch_bytes(int grid)
-{
-    return (size_t)grid * kAdjWarps * kCtr * kCtrN * sizeof(double);
-}
+namespace {
 
 template <int K>
-static void *adj_fn()
+cudaError_t launch_adj_k(const AdjParams &ap, int num_sms, int block, cudaStream_t st)
 {
-    return (void *)k_quad_adj<K>;
-}
-
-static void *adj_kernel_for(int n_steps)
-{
-    const int K = (n_steps + 15) / 16;
-    switch (K) {
-    case 1: return adj_fn<1>();
-    case 2: return adj_fn<2>();
-    case 3: return adj_fn<3>();
-    case 4: return adj_fn<4>();
-    case 5: return adj_fn<5>();
-    case 6: return adj_fn<6>();
-    case 7: return adj_fn<7>();
-    case 8: return adj_fn<8>();
-    }
-    return nullptr;
-}
-
-int adjoint_blocks_per_sm(int n_steps, int G, int block)
-{
-    void *fn = adj_kernel_for(n_steps);
-    if (!fn) return 0;
-    const size_t smem = adjoint_smem_bytes(n_steps, G, block);
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (ap.q.n_items < num_sms * (block / 32)) block = 32;      // too few tiles for full blocks on every SM
+    const int nw = block / 32;
+    const size_t smem = sizeof(float4) * K * 16 + sizeof(AdjWarp<K>) * nw;
+    cudaError_t e = cudaFuncSetAttribute(k_quad_adj<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
     int nb = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, block, smem);
-    return nb > 0 ? nb : 1;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_quad_adj<K>, block, smem);
+    if (e != cudaSuccess) return e;
+    const int grid = std::max(1, std::min((ap.q.n_items + nw - 1) / nw, num_sms * std::max(1, nb)));
+    k_quad_adj<K><<<grid, block, smem, st>>>(ap);
+    return cudaGetLastError();
 }
 
-cudaError_t launch_adjoint(const AdjParams &ap, int grid, int block, cudaStream_t st)
+}  // namespace
+
+cudaError_t launch_adjoint(const AdjParams &ap, int num_sms, int block, cudaStream_t st)
 {
-    void *fn = adj_kernel_for(ap.q.n_steps);
-    if (!fn) return cudaErrorInvalidValue;
-    const size_t smem = adjoint_smem_bytes(ap.q.n_steps, ap.q.G, block);
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    AdjParams a = ap;
-    void *args[] = {&a};
-    return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, smem, st);
+    switch ((ap.q.n_steps + 15) / 16) {
+    case 1: return launch_adj_k<1>(ap, num_sms, block, st);
+    case 2: return launch_adj_k<2>(ap, num_sms, block, st);
+    case 3: return launch_adj_k<3>(ap, num_sms, block, st);
+    case 4: return launch_adj_k<4>(ap, num_sms, block, st);
+    case 5: return launch_adj_k<5>(ap, num_sms, block, st);
+    case 6: return launch_adj_k<6>(ap, num_sms, block, st);
+    case 7: return launch_adj_k<7>(ap, num_sms, block, st);
+    case 8: return launch_adj_k<8>(ap, num_sms, block, st);
+    }
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_ybar(const ChainParams &cp, cudaStream_t st)

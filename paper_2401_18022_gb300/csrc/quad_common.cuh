@@ -169,13 +169,16 @@ __device__ __forceinline__ void sincos_rev(float t, float &sn, float &cs)
 }
 
 // e^{j phi z}: the phase phi (hi + lo) in revolutions as an error-free
-// float-float product, reduced to [-1/2, 1/2] (Xu: round with FRND)
+// float-float product, reduced to [-1/2, 1/2] (Xu: round with FRND); phi_lo
+// is the low part of a float-float phi
 template <bool Xu = false>
-__device__ __forceinline__ void phasor_rev_ff(float phi, float hi, float lo, float &sn, float &cs)
+__device__ __forceinline__ void phasor_rev_ff(float phi, float hi, float lo, float &sn, float &cs,
+                                              float phi_lo = 0.0f)
 {
     const float th = phi * hi;
     float tl = fmaf(phi, hi, -th);
     tl = fmaf(phi, lo, tl);
+    tl = fmaf(phi_lo, hi, tl);
     const float fr = __fadd_rn(th, -(Xu ? round_nearest(th) : round_magic(th))) + tl;
     __sincosf(fr * 6.283185307179586f, &sn, &cs);
 }
@@ -189,11 +192,11 @@ __device__ __forceinline__ double sinc_d(double x)
 // Phased-array factor of n identical spans (Eq. new_gn_model with
 // L-tilde_k = (k-1) L): |sum_{k<n} e^{j k phi L}|^2, by rotation from the
 // float-float phase phi L / 2pi.
-__device__ __forceinline__ float array_factor_f(float phi, const QuadParams &qp)
+__device__ __forceinline__ float array_factor_f(float phi, const QuadParams &qp, float phi_lo = 0.0f)
 {
     if (qp.n_spans <= 1) return 1.0f;
     float sn, cs;
-    phasor_rev_ff(phi, qp.Lrev_hi, qp.Lrev_lo, sn, cs);
+    phasor_rev_ff(phi, qp.Lrev_hi, qp.Lrev_lo, sn, cs, phi_lo);
     float sr = 0.0f, si = 0.0f, zr = 1.0f, zi = 0.0f;
     for (int k = 0; k < qp.n_spans; ++k) {
         sr += zr;
@@ -490,80 +493,6 @@ __device__ __forceinline__ void cheb_point(const ChebTabN<NC> &ct, int ci, float
         cheb_moments<kChebMom>(ct, ci, u, nu, x);
         cheb_AB<kChebMom>(nu, phi, A, B);
     }
-}
-
-// ---------------------------------------------------------------------------
-// Segmented small-phase series (forward FP32).  Cut the span at step edges
-// into segments s with centres c_s; each segment's part of Eq. slow_vary is,
-// exactly as for the whole span,
-//   S_s = e^{j phi c_s} sum_n (j phi)^n / n! nu_n^s,  nu_n^s = sum_{m in s} w_m g_n^s(m),
-// g_n^s(m) the mean of (zeta - c_s)^n over step m, and S = sum_s S_s.  With
-// |phi| (segment length) <= 6 the 19-moment truncation stays below 2e-8 of
-// each part, so a point that is too fast for the whole-span series but slow
-// enough for 2, 4 or 8 segments costs 2, 4 or 8 series evaluations (and as
-// many phasors) instead of a walk over all steps.  The moments are contracted
-// in F_c as in cheb_setup, per piece, candidate and segment.
-// ---------------------------------------------------------------------------
-constexpr int kSegCand = 3;          // F_c candidates with segment tables
-
-struct SegTab {
-    float4 c[kSegCand][kSegSlots][kChebMom];   // as ChebTab.c, per segment
-    float hi[kSegSlots], lo[kSegSlots];        // segment centre / 2pi (float-float)
-};
-
-// Called by every thread after cheb_setup (ct.ok block-uniform); the caller
-// syncs.  One warp per (candidate, segment); the step weights of the first nW
-// candidates come from sW as in cheb_setup.
-__device__ __forceinline__ void seg_setup(const QuadParams &qp, const DevPiece &pc, const float4 *sT, int M,
-                                          const PieceConst<float> &k, SegTab &sg, const float4 *sW = nullptr,
-                                          int nW = 0)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int coff = qp.plan_ch_off[pc.plan];
-    const int ncs = k.nc < kSegCand ? k.nc : kSegCand;
-    if (threadIdx.x < kSegSlots) {
-        const int4 si = qp.seg[threadIdx.x];
-        sg.hi[threadIdx.x] = __int_as_float(si.z);
-        sg.lo[threadIdx.x] = __int_as_float(si.w);
-    }
-    for (int t = warp; t < ncs * kSegSlots; t += nw) {
-        const int c = t / kSegSlots, sl = t - c * kSegSlots;
-        const int lv = sl < 2 ? 0 : (sl < 6 ? 1 : 2);
-        const int4 si = qp.seg[sl];
-        const float4 *gtab = qp.zs_gseg + (size_t)lv * M * kZsG;
-        const double F0 = qp.ch_frel[coff + pc.c_lo + c];
-        const double h = 0.5 * qp.ch_B[coff + pc.c_lo + c];
-        const double at = (double)(k.at_ab + k.hat[c]);
-        float4 *out = sg.c[c][sl];
-        const float4 *sWc = c < nW ? sW + (size_t)c * M : nullptr;
-        cheb_sums<0, 6>(gtab, sT, sWc, si.x, si.y, F0, (float)h, at, lane, out);
-        cheb_sums<6, 6>(gtab, sT, sWc, si.x, si.y, F0, (float)h, at, lane, out + 6);
-        cheb_sums<12, kChebMom - 12>(gtab, sT, sWc, si.x, si.y, F0, (float)h, at, lane, out + 12);
-    }
-}
-
-// |S|^2 of a point of candidate ci at in-channel coordinate x (T2, T3 its
-// Chebyshev values) from the segments [s0, s1).
-__device__ __forceinline__ float seg_s2(const SegTab &sg, int ci, int s0, int s1, float x, float T2, float T3,
-                                        float phi)
-{
-    float Sr = 0.0f, Si = 0.0f;
-    for (int s = s0; s < s1; ++s) {
-        float nu[kChebMom];
-        const float4 *C = sg.c[ci][s];
-#pragma unroll
-        for (int n = 0; n < kChebMom; ++n) {
-            const float4 c = C[n];
-            nu[n] = fmaf(c.w, T3, fmaf(c.z, T2, fmaf(c.y, x, c.x)));
-        }
-        float A, B;
-        cheb_AB<kChebMom>(nu, phi, A, B);
-        float sn, cs;
-        phasor_rev_ff(phi, sg.hi[s], sg.lo[s], sn, cs);
-        Sr = fmaf(cs, A, fmaf(-sn, B, Sr));
-        Si = fmaf(sn, A, fmaf(cs, B, Si));
-    }
-    return fmaf(Sr, Sr, Si * Si);
 }
 
 }  // namespace isrs

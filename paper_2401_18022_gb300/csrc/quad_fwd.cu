@@ -4,23 +4,27 @@
 //                normalisation ln N(z_m) by log-sum-exp over channels, and the
 //                per-step power tables of Eq. pk for the linear-slope
 //                closed-form profile.
+//  k_gauss       the Gauss rules of the discrete uniform measures (quad_nodes.cuh).
 //  k_quad_f32    persistent quadrature: one block per work tile (a range of
 //                pieces of one CUT); G x G hyperbolic grid per piece
-//                (Eqs. q1..q4), z-sum of Eq. slow_vary per grid point in FP32:
-//                the moment series about the span centre (|phi| L <= 6) or
-//                about the centres of 2, 4 or 8 segments (|phi| L up to ~42),
-//                else the direct or telescoped step sums with a float-float
-//                phase and mod-2pi reduction; compensated accumulation; one
-//                FP64 partial per tile.
+//                (Eqs. q1..q4), each row's sum taken from a few nodes
+//                (quad_nodes.cuh), the z-sum of Eq. slow_vary per node in FP32:
+//                the moment series about the span centre (|phi| L <= 6), else
+//                the direct or telescoped step sums with a float-float phase
+//                and mod-2pi reduction; compensated accumulation; one FP64
+//                partial per tile.
 //  k_quad_f64    the same quadrature in plain FP64 (direct form of
 //                Eq. slow_vary with sinc), used as the reference GPU path.
 //  k_finish      per profile: deterministic FP64 sum of tile partials per CUT,
 //                eta (Eq. gain_fin), P_NLI, SNR and throughput (Eq. loss).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "isrs_internal.cuh"
 #include "isrs_kernels.h"
 #include "quad_common.cuh"
+#include "quad_nodes.cuh"
 #include "quad_zsum.cuh"
 
 namespace isrs {
@@ -103,23 +107,104 @@ __global__ void __launch_bounds__(256) k_prep(PrepParams pp)
 }
 
 // ---------------------------------------------------------------------------
-// k_quad_f32: persistent FP32 quadrature.
+// k_gauss: nodes and weights of the n-node Gauss rules of the uniform measure
+// on t_j = (2 j + 1 - N)/N, j < N, for every N <= kGaussMaxN.  The monic
+// orthogonal polynomials (discrete Chebyshev, Gautschi 2004) satisfy
+// p_{i+1} = t p_i - b_i p_{i-1} with b_i = i^2 (N^2 - i^2) / (N^2 (4 i^2 - 1)).
+// One thread per node: the k-th smallest zero by bisection on the sign changes
+// of the sequence p_0..p_n (Sturm), then Newton; weight N / sum of the squared
+// orthonormal polynomials.  FP64, run once per device (about 1 ms).
 // ---------------------------------------------------------------------------
-constexpr int kFwdCand = 4;          // F_c candidates with their own step rows (attenuation folded in) ...
-constexpr int kFwdCandSteps = 256;   // ... when the z-grid has at most this many steps (shared memory)
-
-__host__ __device__ constexpr int fwd_cand_rows(int n_steps)
+__global__ void __launch_bounds__(128) k_gauss(float2 *out)
 {
-    return n_steps <= kFwdCandSteps ? kFwdCand : 0;
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= kGaussEntries) return;
+    const int N = e / kGaussPerN + 1, o = e - (N - 1) * kGaussPerN;
+    int m = 0;
+    while (m + 1 < kGaussMenu && gauss_offset(m + 1) <= o) ++m;
+    const int n = gauss_nodes(m), k = o - gauss_offset(m);
+    if (n >= N) {                      // never used: a run takes its columns then
+        out[e] = make_float2(0.0f, 0.0f);
+        return;
+    }
+    const double N2 = (double)N * N;
+    const auto b = [&](int i) { return (double)i * i * (N2 - (double)i * i) / (N2 * (4.0 * i * i - 1.0)); };
+    // zeros below t, from the signs of the Sturm quotients p_{i+1}/p_i
+    const auto below = [&](double t) {
+        int cnt = 0;
+        double q = -t;
+        for (int i = 0;; ++i) {
+            if (q < 0.0) ++cnt;
+            if (i + 1 == n) break;
+            if (q == 0.0) q = 1e-300;
+            q = -t - b(i + 1) / q;
+        }
+        return cnt;
+    };
+    double lo = -1.0, hi = 1.0;
+    for (int s = 0; s < 26; ++s) {
+        const double mid = 0.5 * (lo + hi);
+        if (below(mid) > k) hi = mid;
+        else lo = mid;
+    }
+    double t = 0.5 * (lo + hi), sum = 0.0;
+    for (int s = 0; s < 3; ++s) {
+        double p0 = 1.0, p1 = t, d0 = 0.0, d1 = 1.0, h = 1.0;
+        sum = 1.0;
+        for (int i = 1; i < n; ++i) {
+            const double bi = b(i);
+            h *= bi;
+            sum += p1 * p1 / h;
+            const double p2 = t * p1 - bi * p0, d2 = p1 + t * d1 - bi * d0;
+            p0 = p1;
+            p1 = p2;
+            d0 = d1;
+            d1 = d2;
+        }
+        if (s < 2) t -= p1 / d1;
+    }
+    out[e] = make_float2((float)t, (float)(N / sum));
 }
 
-// Dynamic shared memory of k_quad_f32 in float4 units: the step tables, the
-// per-candidate rows, the G row descriptors, then (G >= kSegMinG) the
-// segment tables.
-__host__ __device__ constexpr size_t fwd_seg_offset_f4(int n_steps, int G)
+cudaError_t launch_gauss(float2 *out, cudaStream_t st)
 {
-    return (size_t)n_steps * (3 + 2 * fwd_cand_rows(n_steps)) +
-           ((size_t)G * sizeof(RowF) + sizeof(float4) - 1) / sizeof(float4);
+    k_gauss<<<(kGaussEntries + 127) / 128, 128, 0, st>>>(out);
+    return cudaGetLastError();
+}
+
+__device__ float2 g_isrs_gauss[kGaussEntries];
+
+// ln(xhi / xlo) and ln(yhi / ylo) of every piece, once per plan (the quadrature
+// would otherwise take two FP64 logarithms per piece and launch).
+__global__ void __launch_bounds__(256) k_piece_logs(DevPiece *pieces, int n)
+{
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+        DevPiece &p = pieces[k];
+        p.lnx = p.xlo > 0.0 ? log(p.xhi / p.xlo) : 1e30;
+        p.lny = p.ylo > 0.0 ? log(p.yhi / p.ylo) : 1e30;
+    }
+}
+
+cudaError_t launch_piece_logs(DevPiece *pieces, int n, cudaStream_t st)
+{
+    if (n > 0) k_piece_logs<<<std::min(2048, (n + 255) / 256), 256, 0, st>>>(pieces, n);
+    return cudaGetLastError();
+}
+
+cudaError_t gauss_array(void **out) { return cudaGetSymbolAddress(out, g_isrs_gauss); }
+
+// ---------------------------------------------------------------------------
+// k_quad_f32: persistent FP32 quadrature.
+// ---------------------------------------------------------------------------
+constexpr int kFwdSlots = 320;       // node slots of a chunk
+constexpr int kFwdCand = 3;          // F_c candidates swept together (most pieces have two)
+using FwdNodes = WarpNodes<kFwdSlots>;
+
+// Dynamic shared memory of k_quad_f32: zt [M], then per warp the nodes and the
+// candidates' step rows.
+__host__ __device__ constexpr size_t fwd_warp_bytes(int n_steps)
+{
+    return sizeof(FwdNodes) + (sizeof(float2) * kFwdCand * (size_t)n_steps + 15) / 16 * 16;
 }
 #ifndef ISRS_FWD_MIN_BLOCKS
 #define ISRS_FWD_MIN_BLOCKS 4   // resident blocks per SM the register budget is sized for
@@ -129,158 +214,80 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
 {
     extern __shared__ float4 smem_f4[];
     const int M = qp.n_steps, G = qp.G;
-    float4 *sT = smem_f4;                              // [M] {A2 + log2 dz, K2, z, z^2 + dz^2/12}
-    float4 *sE = sT + M;                               // [M] {edge/2pi hi, lo, A2, K2}
-    float4 *sR = sE + M;                               // [M] {A2 + log2 dz, K2, z, dz}
-    const int ncr = fwd_cand_rows(M);
-    float4 *sRc = sR + M;                              // [ncr][M] sR rows with - at_c z folded in
-    float4 *sEc = sRc + ncr * M;                       // [ncr][M] sE rows with - at_c z folded in
-    RowF *rows = reinterpret_cast<RowF *>(sEc + ncr * M);   // [G]
-    // segment tables (G >= kSegMinG only; the launch sizes the space for them)
-    SegTab *sg = reinterpret_cast<SegTab *>(smem_f4 + fwd_seg_offset_f4(M, G));
-    __shared__ PieceConst<float> kc;
-    __shared__ ChebTab ct;
-    __shared__ double scratch[32];
-    __shared__ int s_item;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float4 *zt = smem_f4;                              // [M] {edge(m+1)/2pi hi, lo, z, dz}
+    unsigned char *mine = reinterpret_cast<unsigned char *>(zt + M) + fwd_warp_bytes(M) * warp;
+    FwdNodes &ns = *reinterpret_cast<FwdNodes *>(mine);
+    float2 *ek = reinterpret_cast<float2 *>(mine + sizeof(FwdNodes));   // [kFwdCand][M] {log2 p at f_c, K2}
 
     for (int m = threadIdx.x; m < M; m += blockDim.x) {
         const float4 za = qp.zs_a[m];   // {z_m, c_m, log2 dz_m, dz_m}
         const float4 zb = qp.zs_b[m];   // {edge(m+1)/2pi hi, lo, z_m/2pi, 0}
-        sT[m] = make_float4(0.0f, 0.0f, za.x, za.y);
-        sE[m] = make_float4(zb.x, zb.y, 0.0f, 0.0f);
-        sR[m] = make_float4(0.0f, 0.0f, za.x, za.w);
+        zt[m] = make_float4(zb.x, zb.y, za.x, za.w);
     }
-    const float c3 = (float)(kPi * qp.beta3);
-    const float c4 = (float)(2.0 * kPi * kPi / 3.0 * qp.beta4);
-    const float b2 = (float)qp.beta2;
-    const float m4pi2 = (float)(-4.0 * kPi * kPi);
+    __syncthreads();
     const float phi_direct = 3.14159265f / qp.dz_max;
-    const float phi_small = 0.02f / qp.L;
-    const float phi_cheb = kChebPhiL / qp.L;
-    const float phi_c6 = kChebPhiL6 / qp.L, phi_c11 = kChebPhiL11 / qp.L;
-    const float phi_s0 = qp.phi_seg[0], phi_s1 = qp.phi_seg[1], phi_s2 = qp.phi_seg[2];
+    const float phi_small = kBlkPhiL / qp.L;
     const float log2e = (float)kLog2e;
-    const float invG = 1.0f / (float)G;
-    unsigned n_small = 0, n_direct = 0, n_tele = 0;
-    int cur_prof = -1;
+    unsigned long long n_small = 0;
+    unsigned n_direct = 0, n_tele = 0;
 
     for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_item = atomicAdd(qp.counter, 1);
-        __syncthreads();
-        const int it = s_item;
+        int it = 0;
+        if (lane == 0) it = atomicAdd(qp.counter, 1);
+        it = __shfl_sync(0xffffffffu, it, 0);
         if (it >= qp.n_items) break;
         const DevItem item = qp.items[it];
-        if (item.prof != cur_prof) {
-            const float2 *st = qp.step_f + (size_t)item.prof * M;
-            for (int m = threadIdx.x; m < M; m += blockDim.x) {
-                const float2 v = st[m];
-                const float a2d = v.x + qp.zs_a[m].z;
-                sT[m].x = a2d;
-                sT[m].y = v.y;
-                sE[m].z = v.x;
-                sE[m].w = v.y;
-                sR[m].x = a2d;
-                sR[m].y = v.y;
-            }
-            cur_prof = item.prof;
-        }
+        const float2 *st = qp.step_f + (size_t)item.prof * M;
+        const float tilt = (float)qp.kap_L[item.prof];
+        const int part = item.part & 0xffff, parts = item.part >> 16;
         double acc = 0.0;
         for (int k = item.piece0; k < item.piece1; ++k) {
-            const DevPiece pc = qp.pieces[dbg_clamp(k, qp.n_pieces, kDbgPiece, qp.dbg)];
-            piece_rows<RowF>(pc, G, qp.eps_v1, rows);
-            piece_consts<float>(qp, pc, item.prof, log2e, qp.pd_f, kc);
-            __syncthreads();
-            // step weights of the contracted candidates, once per piece, in the
-            // space of the per-candidate rows (filled after the tables)
-            int nW = 0;
-            if (ncr > 0 && cheb_applies(qp, pc, item.prof, kc)) {
-                nW = min(kc.nc, 2 * ncr);
-                cheb_weights(qp, pc, sT, M, kc, nW, sRc);
-                __syncthreads();
-            }
-            const bool segs = cheb_setup<kChebMom>(qp, pc, item.prof, sT, M, kc, ct, sRc, nW) &&
-                              qp.zs_gseg != nullptr && G >= kSegMinG;
-            if (segs) seg_setup(qp, pc, sT, M, kc, *sg, sRc, nW);
-            if (nW > 0) __syncthreads();
-            // per-candidate step rows with the candidate's attenuation folded in
-            const int ncf = min(kc.nc, ncr);
-            for (int t = threadIdx.x; t < ncf * M; t += blockDim.x) {
-                const int c = t / M, m = t - c * M;
-                const float at = kc.at_ab + kc.hat[c];
-                const float4 r = sR[m], e = sE[m];
-                sRc[t] = make_float4(fmaf(-at, r.z, r.x), r.y, r.z, r.w);
-                sEc[t] = make_float4(e.x, e.y, fmaf(-at, r.z, e.z), e.w);
-            }
-            __syncthreads();
-            const float fi = kc.fi, s1g = kc.s1, s2g = kc.s2;
-            const float three_fi2 = 3.0f * fi * fi;
-            const bool cheb = ct.ok != 0;
-            const float phi_lim = cheb ? phi_cheb : phi_small;   // upper |phi| of the small-phase forms
+            const DevPiece &pc = qp.pieces[dbg_clamp(k, qp.n_pieces, kDbgPiece, qp.dbg)];
+            __syncwarp();
+            node_geo(qp, pc, item.prof, log2e, qp.pd_f, tilt, ns.geo);
+            __syncwarp();
+            const PieceGeo &g = ns.geo;
             float sum = 0.0f, comp = 0.0f;
-            const int npts = G * G;
-            for (int q = threadIdx.x; q < npts; q += blockDim.x) {
-                // row r = floor(q / G): (q + 1/2)/G is at least 1/(2G) from an integer
-                const int r = (int)(((float)q + 0.5f) * invG);
-                const int j = q - r * G;
-                const RowF rw = rows[dbg_clamp(r, G, kDbgRow, qp.dbg)];
-                if (rw.w == 0.0f) continue;
-                const float d = ((float)j + 0.5f - 0.5f * (float)G) * rw.du2;
-                const float e = expf(d);
-                const float f1 = s1g * (rw.xc * e);
-                const float f2 = s2g * (rw.yc * __frcp_rn(e));
-                const float u = f1 + f2;                    // F_c - f_i
-                int ci = -1;
-                for (int c = 0; c < kc.nc; ++c) {
-                    if (u >= kc.lo[c] && u < kc.hi[c]) { ci = c; break; }
-                }
-                if (ci < 0) continue;                       // F_c in a gap
-                ci = dbg_clamp(ci, kc.nc, kDbgCand, qp.dbg);
-                const float W = kc.wab * kc.pd[ci];
-                const float at = kc.at_ab + kc.hat[ci];
-                const float Fc = fi + u;                    // F_c - f_ref
-                // Eq. phi
-                const float br = b2 + c3 * (u + 2.0f * fi) +
-                                 c4 * (f1 * f1 + 1.5f * f1 * f2 + 3.0f * fi * u + f2 * f2 + three_fi2);
-                const float phi = m4pi2 * f1 * f2 * br;
-                const float aphi = fabsf(phi);
-                float S2;
-                if (aphi <= phi_lim) {
-                    if (cheb) {
-                        float x, A, B;
-                        cheb_point(ct, ci, u, phi, aphi, phi_c6, phi_c11, x, A, B);
-                        S2 = fmaf(A, A, B * B);
-                    } else {
-                        S2 = zsum_small_f(phi, Fc, at, sT, M);
+            for (int ca = 0; ca < g.nc; ca += kFwdCand) {
+                const int cb = min(g.nc, ca + kFwdCand);
+                // step rows of the candidates: ln p at the channel's centre
+                for (int c = ca; c < cb; ++c) {
+                    const float at = g.at_ab + g.hat[c], F = g.Fc0 + 0.5f * (g.lo[c] + g.hi[c]);
+                    for (int m = lane; m < M; m += 32) {
+                        const float2 v = st[m];
+                        ek[(c - ca) * M + m] = make_float2(fmaf(v.y, F, fmaf(-at, zt[m].z, v.x)), v.y);
                     }
-                    ++n_small;
-                } else if (segs && ci < kSegCand && aphi <= phi_s2) {
-                    // the series per segment: 2, 4 or 8 segments by |phi|
-                    const int s0 = aphi <= phi_s0 ? 0 : (aphi <= phi_s1 ? 2 : 6);
-                    const int s1 = aphi <= phi_s0 ? 2 : (aphi <= phi_s1 ? 6 : kSegSlots);
-                    const float x = (u - ct.mid[ci]) * ct.invh[ci];
-                    const float T2 = fmaf(2.0f * x, x, -1.0f);
-                    const float T3 = fmaf(2.0f * x, T2, -x);
-                    S2 = seg_s2(*sg, ci, s0, s1, x, T2, T3, phi);
-                    ++n_small;
-                } else if (aphi <= phi_direct) {
-                    S2 = ci < ncr ? zsum_direct_fc(phi, Fc, sRc + ci * M, M) : zsum_direct_f(phi, Fc, at, sR, M);
-                    ++n_direct;
-                } else {
-                    S2 = ci < ncr ? zsum_tele_fc(phi, Fc, sEc + ci * M, M) : zsum_tele_f(phi, Fc, at, sT, sE, M);
-                    ++n_tele;
                 }
-                // compensated accumulation over this thread's points
-                const float y = rw.w * W * S2 * array_factor_f(phi, qp) - comp;
-                const float t = sum + y;
-                comp = (t - sum) - y;
-                sum = t;
+                __syncwarp();
+                int small;
+                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int nq) {
+                    for (int q = lane + 32 * part; q < nq; q += 32 * parts) {
+                        Node nd;
+                        if (!node_get(ns, qp.gauss, q, nd)) continue;
+                        const int ci = dbg_clamp(nd.ci, g.nc, kDbgCand, qp.dbg);
+                        const float aphi = fabsf(nd.phi);
+                        const float dF = (nd.x + nd.y) - 0.5f * (g.lo[ci] + g.hi[ci]);
+                        const float2 *e = ek + (ci - ca) * M;
+                        const bool direct = aphi <= phi_direct;
+                        const float S2 = direct ? zsum_direct_n(nd.phi, dF, zt, e, M)
+                                                : zsum_tele_n(nd.phi, nd.phi_lo, dF, zt, e, M);
+                        n_small += aphi <= phi_small ? nd.N : 0;
+                        n_direct += aphi > phi_small && direct ? nd.N : 0;
+                        n_tele += direct ? 0 : nd.N;
+                        // compensated accumulation over this lane's nodes
+                        const float y = nd.wq * g.pd[ci] * S2 * array_factor_f(nd.phi, qp, nd.phi_lo) - comp;
+                        const float t = sum + y;
+                        comp = (t - sum) - y;
+                        sum = t;
+                    }
+                });
+                n_small += lane == 0 && part == 0 ? small : 0;
             }
-            acc += (double)kc.mult * ((double)sum - (double)comp);
-            __syncthreads();
+            acc += (double)(g.mult * g.wab) * ((double)sum - (double)comp);
         }
-        const double tot = block_sum_d(acc, scratch);
-        if (threadIdx.x == 0) qp.partial[it] = tot;
+        const double tot = warp_sum_d(acc);
+        if (lane == 0) qp.partial[it] = tot;
     }
     if (qp.path_count) {
         unsigned long long c0 = n_small, c1 = n_direct, c2 = n_tele;
@@ -290,7 +297,7 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
             c1 += __shfl_xor_sync(0xffffffffu, c1, o);
             c2 += __shfl_xor_sync(0xffffffffu, c2, o);
         }
-        if ((threadIdx.x & 31) == 0) {
+        if (lane == 0) {
             atomicAdd(&qp.path_count[0], c0);
             atomicAdd(&qp.path_count[1], c1);
             atomicAdd(&qp.path_count[2], c2);
@@ -337,7 +344,8 @@ __global__ void __launch_bounds__(256) k_quad_f64(QuadParams qp)
             const double fi = kc.fi;
             double sum = 0.0;
             const int npts = G * G;
-            for (int q = threadIdx.x; q < npts; q += blockDim.x) {
+            for (int q = threadIdx.x + (item.part & 0xffff) * blockDim.x; q < npts;
+                 q += (item.part >> 16) * blockDim.x) {
                 const int r = q / G;
                 const int j = q - r * G;
                 const RowD rw = rows[dbg_clamp(r, G, kDbgRow, qp.dbg)];
@@ -470,50 +478,50 @@ cudaError_t launch_snr_from_eta(const SnrFromEtaParams &sp, cudaStream_t st)
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-size_t quad_smem_bytes(int precision, int n_steps, int G)
-{
-    if (precision == 0)
-        return fwd_seg_offset_f4(n_steps, G) * sizeof(float4) + (G >= kSegMinG ? sizeof(SegTab) : 0);
-    return (size_t)n_steps * 2 * sizeof(double2) + (size_t)G * sizeof(RowD);
-}
-
 cudaError_t launch_prep(const PrepParams &pp, int n_prof, cudaStream_t st)
 {
     k_prep<<<dim3(n_prof, pp.n_steps + 1), 256, 0, st>>>(pp);
     return cudaGetLastError();
 }
 
-cudaError_t launch_quad(const QuadParams &qp, int precision, int grid, int block, cudaStream_t st)
+namespace {
+
+size_t fwd_smem(int n_steps, int block)
 {
-    const size_t smem = quad_smem_bytes(precision, qp.n_steps, qp.G);
+    return sizeof(float4) * (size_t)n_steps + fwd_warp_bytes(n_steps) * (size_t)(block / 32);
+}
+
+}  // namespace
+
+// Persistent launch of the quadrature.  FP32: the warps of a block work alone,
+// so a block is any number of them: as many as fit in shared memory (fewer than
+// asked only past ~900 z-steps), one where there are too few tiles to give every
+// SM a full block (a 5-channel plan's ~90 tiles then run on as many SMs).
+cudaError_t launch_quad(const QuadParams &qp, int precision, int num_sms, int block, cudaStream_t st)
+{
+    int nb = 0, tiles = qp.n_items;
+    size_t smem = (size_t)qp.n_steps * 2 * sizeof(double2) + (size_t)qp.G * sizeof(RowD);
+    const void *fn = (const void *)k_quad_f64;
     if (precision == 0) {
-        cudaFuncSetAttribute(k_quad_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_quad_f32<<<grid, block, smem, st>>>(qp);
-    } else {
-        cudaFuncSetAttribute(k_quad_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_quad_f64<<<grid, block, smem, st>>>(qp);
+        fn = (const void *)k_quad_f32;
+        if (qp.n_items < num_sms * (block / 32)) block = 32;
+        while (block > 32 && fwd_smem(qp.n_steps, block) > 200 * 1024) block -= 32;
+        smem = fwd_smem(qp.n_steps, block);
+        tiles = (qp.n_items + block / 32 - 1) / (block / 32);
     }
-    return cudaGetLastError();
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, block, smem);
+    if (e != cudaSuccess) return e;
+    const int grid = std::max(1, std::min(tiles, num_sms * std::max(1, nb)));
+    void *args[] = {(void *)&qp};
+    return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, smem, st);
 }
 
 cudaError_t launch_finish(const FinishParams &fp, int n_prof, cudaStream_t st)
 {
     k_finish<<<n_prof, 256, 0, st>>>(fp);
     return cudaGetLastError();
-}
-
-int quad_blocks_per_sm(int precision, int n_steps, int G, int block)
-{
-    int nb = 0;
-    const size_t smem = quad_smem_bytes(precision, n_steps, G);
-    if (precision == 0) {
-        cudaFuncSetAttribute(k_quad_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_quad_f32, block, smem);
-    } else {
-        cudaFuncSetAttribute(k_quad_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_quad_f64, block, smem);
-    }
-    return nb > 0 ? nb : 1;
 }
 
 }  // namespace isrs

@@ -1,0 +1,579 @@
+// Row sums of the hyperbolic grid from a few nodes (App. A, Eqs. q1..q4).
+//
+// Along one grid row upsilon1 = |f1||f2| is constant, so the phase of Eq. phi,
+// F_c and the power profile of Eq. pk depend on the point only through
+// u = F_c - f_i, a smooth function of the column index j.  Inside one F_c
+// channel the row's points are a run of N consecutive columns, and their sum
+//   sum_{j = j0}^{j0 + N - 1} f(j)
+// is the integral of f against the discrete uniform measure on N points.  The
+// Gauss rule of that measure (its orthogonal polynomials are the discrete
+// Chebyshev polynomials, Gautschi, "Orthogonal Polynomials: Computation and
+// Approximation", 2004, Sec. 1.5) with n nodes reproduces the sum exactly for
+// every polynomial of degree 2 n - 1.  |S|^2 is band limited along the row
+// (|d phi| L per half run, A below), so its Chebyshev coefficients vanish
+// faster than exponentially past degree ~A and n a little above A / 2 gives
+// the same Riemann sum to < 1e-8: it is a regrouping of the sum over the G
+// points, not another grid.  The rule holds for the adjoint's bucket terms
+// too, which have the same band limit.
+//
+// The rows are uniform in ln upsilon1, so the row sums of a block of low rows
+// (one F_c channel, |phi| L small) are smooth in the row index as well, and the
+// same rules take the block's sum from a few rows at real-valued indices.
+//
+// Why: the quadratures are bound by the z-sums (112 steps per point).  A piece
+// of the 589-channel plan has 65,536 points at G = 256 (4,096 at G = 64) and
+// takes about 1,000 (250) nodes.
+//
+// Coordinates are carried relative to a corner of the piece, U = s1 xhi +
+// s2 yhi, so that an FP32 point is located to ~1e-8 THz also where F_c - f_i
+// is tens of THz, and phi is split per row into its value at the row's centre
+// (FP64, kept as a float-float pair) and an increment quadratic in u.
+//
+// One warp works on one piece: lane = row while rows are set up and their runs
+// listed, lane = node (or half-warp = node) afterwards.  Blocks working on one
+// piece together spent a third of their issue slots at barriers, because the
+// set-up is a chain of short FP64 steps.
+#pragma once
+#include <cuda_runtime.h>
+
+#include "quad_common.cuh"
+
+namespace isrs {
+
+// Node counts of the rules: 4..8, 10, 12 .. 20, 24, 28, 32, 40, 48.  One table
+// of {t, weight} per run length N <= kGaussMaxN and node count; node k lies at
+// column centre + t N / 2.
+constexpr int kGaussMaxN = 256;
+constexpr int kGaussMaxNodes = 48;
+constexpr int kGaussMenu = 16;
+constexpr int kGaussPerN = 292;                        // nodes of all rules of one N
+constexpr int kGaussEntries = kGaussMaxN * kGaussPerN;
+constexpr int kNodeMin = 4;                            // slots a run takes at least
+
+__host__ __device__ constexpr int gauss_nodes(int k)
+{
+    return k <= 4 ? 4 + k : k <= 10 ? 2 * k : k <= 13 ? 20 + 4 * (k - 10) : 32 + 8 * (k - 13);
+}
+
+__host__ __device__ constexpr int gauss_offset(int k)
+{
+    return k <= 4 ? 4 * k + k * (k - 1) / 2 : k <= 10 ? k * (k - 1) + 10
+         : k <= 13 ? 120 + 24 * (k - 11) + 2 * (k - 11) * (k - 12) : 204 + 40 * (k - 14);
+}
+
+// smallest rule with at least `need` nodes (need <= kGaussMaxNodes)
+__host__ __device__ inline int gauss_pick(int need)
+{
+    return need <= 4 ? 0 : need <= 8 ? need - 4 : need <= 20 ? 4 + (need - 7) / 2
+         : need <= 32 ? 10 + (need - 17) / 4 : 13 + (need - 25) / 8;
+}
+
+// Nodes that give a run's sum to < 1e-8 of itself: A bounds the phase swing of
+// |S|^2 over half the run, D its half-length in upsilon2 (the map from column
+// to u is exp-like).  2 n = A + 7.2 + 2.6 sqrt(A) + 1.4 D covers what the runs
+// of the 589-ch, O-band and multi-span plans need (A up to 670, D up to 11.5).
+__host__ __device__ inline int gauss_need(float A, float D)
+{
+    const float two_n = A + 7.2f + 2.6f * sqrtf(A) + 1.4f * D;
+    return two_n < 8192.0f ? (int)ceilf(0.5f * two_n) : 4096;
+}
+
+constexpr int kBlkMax = 18;              // row blocks of a piece at most (kMaxG / 256 + 2)
+constexpr float kBlkPhiL = 6.0f;         // |phi| n_spans L up to which rows join a block ...
+constexpr float kBlkPhiLow = 0.15f;      // ... and up to which they join the low ones
+
+// One piece's geometry, |f1| the longer axis (f1 and f2 enter symmetrically,
+// so swapping them only reverses the columns).
+struct PieceGeo {
+    double u1hi;                // xhi yhi
+    double br0;                 // bracket of Eq. phi: br0 + br1 u + c4 u^2 - c4/2 f1 f2, u from the corner
+    double ds2;                 // row pitch in log2 upsilon1
+    float br1, c4;
+    float ds;                   // row pitch in ln upsilon1
+    float xhi, yhi;             // corner of the piece
+    float s1, s2;               // signs of f1, f2
+    float R, Rb;                // ln(xhi / xlo), ln(yhi / ylo) (1e30 where the lower limit is 0)
+    float band;                 // n_spans L: phase swing per |d phi|
+    float tilt;                 // bound of |d ln p / dF|
+    float Fc0;                  // F_c - f_ref at the corner
+    float wab, at_ab, mult;     // P_a P_b / (B_a B_b), attenuation part of ln p, mirror weight
+    int nc;                     // F_c candidates: edges from the corner, P/B, half attenuation
+    float lo[kMaxCand], hi[kMaxCand], pd[kMaxCand], hat[kMaxCand];
+};
+
+// One grid row: centre, column pitch, weight; f1 - s1 xhi and f2 - s2 yhi at
+// the centre, and phi there as a float-float pair: |S|^2 turns through hundreds
+// of radians of phi L that the rows sample far apart, so an FP32 relative error
+// of a whole row's phase would show in the sum (errors of single points
+// average out along the row).
+struct __align__(16) NodeRow {
+    float xc, yc, du2, w;
+    float x0, y0, phi0, phi0_lo;
+};
+
+// A run of N columns of one row inside one F_c candidate, with its rule.
+struct __align__(16) NodeRun {
+    float jc;                   // centre column, from the row's centre
+    float half;                 // N / 2
+    int toff;                   // first entry of the rule; -1: the N columns themselves
+    unsigned id;                // first slot | candidate << 12 | row << 17 | row of a block << 31
+};
+
+struct RowBlock {
+    int unit0, r0, N, toff;     // first unit, first row, rows, rule (-1: every row)
+};
+
+template <int Cap>
+struct WarpNodes {
+    static constexpr int kSpan = Cap - kGaussMaxNodes;    // slots a chunk starts runs in
+    NodeRow row[32];
+    NodeRun run[Cap / kNodeMin];
+    unsigned short of[Cap];     // run of each slot (0xffff: none)
+    RowBlock blk[kBlkMax];
+    PieceGeo geo;
+};
+
+// The piece's geometry (whole warp; the caller syncs the warp).  sw: the
+// longer axis belongs to F_b.
+__device__ __forceinline__ bool node_geo(const QuadParams &qp, const DevPiece &pc, int prof, float at_scale,
+                                         const float *pdv, float tilt, PieceGeo &g)
+{
+    const int lane = threadIdx.x & 31;
+    const bool sw = pc.yhi > pc.xhi;
+    const double xhi = sw ? pc.yhi : pc.xhi, yhi = sw ? pc.xhi : pc.yhi;
+    const double R = sw ? pc.lny : pc.lnx, Rb = sw ? pc.lnx : pc.lny;
+    const bool n1 = pc.flags & (sw ? 2 : 1), n2 = pc.flags & (sw ? 1 : 2);
+    const double s1 = n1 ? -1.0 : 1.0, s2 = n2 ? -1.0 : 1.0;
+    const int coff = qp.plan_ch_off[pc.plan], poff = qp.prof_ch_off[prof];
+    const double fi = qp.ch_frel[coff + pc.cut];
+    const double U = s1 * xhi + s2 * yhi;
+    const int nc = min(pc.c_hi - pc.c_lo + 1, kMaxCand);
+    if (lane < nc) {
+        const double fc = qp.ch_frel[coff + pc.c_lo + lane], hb = 0.5 * qp.ch_B[coff + pc.c_lo + lane];
+        g.lo[lane] = (float)(((fc - hb) - fi) - U);
+        g.hi[lane] = (float)(((fc + hb) - fi) - U);
+        g.pd[lane] = pdv[poff + pc.c_lo + lane];
+        g.hat[lane] = (float)(0.5 * qp.ch_alpha[coff + pc.c_lo + lane]) * at_scale;
+    }
+    if (lane == 0) {
+        const double c3 = kPi * qp.beta3, c4 = 2.0 * kPi * kPi / 3.0 * qp.beta4;
+        const double ds = fmin(R + Rb, qp.ln_eps) / qp.G;     // upsilon1 from max(xlo ylo, eps xhi yhi)
+        g.u1hi = xhi * yhi;
+        g.br0 = qp.beta2 + c3 * (U + 2.0 * fi) + c4 * (U * U + 3.0 * fi * U + 3.0 * fi * fi);
+        g.br1 = (float)(c3 + c4 * (2.0 * U + 3.0 * fi));
+        g.c4 = (float)c4;
+        g.ds = (float)ds;
+        g.ds2 = ds * kLog2e;
+        g.xhi = (float)xhi;
+        g.yhi = (float)yhi;
+        g.s1 = (float)s1;
+        g.s2 = (float)s2;
+        g.R = (float)R;
+        g.Rb = (float)Rb;
+        g.band = qp.L * (float)qp.n_spans;
+        g.tilt = tilt;
+        g.Fc0 = (float)(fi + U);
+        g.wab = pdv[poff + pc.a] * pdv[poff + pc.b];
+        g.at_ab = (float)(0.5 * (qp.ch_alpha[coff + pc.a] + qp.ch_alpha[coff + pc.b] -
+                                 qp.ch_alpha[coff + pc.cut])) * at_scale;
+        g.mult = pc.mult;
+        g.nc = nc;
+    }
+    return sw;
+}
+
+// 2^-t for t >= 0 in FP64 to ~1e-11 relative: the Taylor series of e^x on |x|
+// <= ln 2 / 2 to x^9 (remainder (0.347)^10 / 10! = 7e-12), exponent by its bits.
+__device__ __forceinline__ double exp2_neg(double t)
+{
+    const double n = rint(t);
+    const double x = (n - t) * 0.69314718055994530942;
+    double p = 1.0 / 362880.0;
+    p = fma(p, x, 1.0 / 40320.0);
+    p = fma(p, x, 1.0 / 5040.0);
+    p = fma(p, x, 1.0 / 720.0);
+    p = fma(p, x, 1.0 / 120.0);
+    p = fma(p, x, 1.0 / 24.0);
+    p = fma(p, x, 1.0 / 6.0);
+    p = fma(p, x, 0.5);
+    p = fma(p, x, 1.0);
+    p = fma(p, x, 1.0);
+    if (n > 1000.0) return 0.0;
+    return __hiloint2double(__double2hiint(p) - ((int)n << 20), __double2loint(p));
+}
+
+// The row k = G - 1/2 - r pitches below the corner (r real-valued in a block).
+// In logarithms relative to the corner, l = ln(upsilon1 / (xhi yhi)), |f2| runs
+// over [max(-Rb, l), min(0, l + R)] and the row's centre lies at ln(xc / xhi) =
+// gx, ln(yc / yhi) = gy.  Returns which limits hold: bit 0 the one set by xhi,
+// bit 1 by xlo (else by ylo, yhi); -1 for an empty row.
+__device__ __forceinline__ int node_row(const PieceGeo &g, int G, double k, NodeRow &o)
+{
+    const double u1d = g.u1hi * exp2_neg(k * g.ds2);
+    const float u1 = (float)u1d;
+    const float l = -(float)k * g.ds;
+    const bool a = l > -g.Rb, b = l + g.R < 0.0f;
+    const float D = a ? (b ? g.R : -l) : (b ? l + g.R + g.Rb : g.Rb);
+    const float gx = a ? (b ? -0.5f * g.R : 0.5f * l) : (b ? 0.5f * (l + g.Rb - g.R) : l + 0.5f * g.Rb);
+    const float gy = a ? (b ? l + 0.5f * g.R : 0.5f * l) : (b ? 0.5f * (l + g.R - g.Rb) : -0.5f * g.Rb);
+    if (!(D > 0.0f) || u1 < 1e-37f) {
+        o.xc = o.yc = o.du2 = o.w = o.x0 = o.y0 = o.phi0 = o.phi0_lo = 0.0f;
+        return -1;
+    }
+    o.xc = g.xhi * expf(gx);
+    o.yc = __fdividef(u1, o.xc);
+    o.du2 = __fdividef(D, (float)G);
+    o.w = u1 * g.ds * o.du2;
+    o.x0 = g.s1 * g.xhi * expm1f(gx);
+    o.y0 = g.s2 * g.yhi * expm1f(gy);
+    const float u0 = o.x0 + o.y0;
+    const double v = (double)(g.s1 * g.s2) * u1d;
+    const double br = g.br0 + (double)(u0 * fmaf(g.c4, u0, g.br1)) - (double)(0.5f * g.c4) * v;
+    const double phi = (-4.0 * kPi * kPi) * v * br;
+    o.phi0 = (float)phi;
+    o.phi0_lo = (float)(phi - (double)o.phi0);
+    return (a ? 1 : 0) | (b ? 2 : 0);
+}
+
+// phi = phi0 + du (p1 + p2 du) along a row, du = u - u0
+__device__ __forceinline__ void row_slopes(const PieceGeo &g, const NodeRow &o, float &p1, float &p2)
+{
+    const float cv = -39.47841760435743f * g.s1 * g.s2 * (o.xc * o.yc);      // -4 pi^2 f1 f2
+    p1 = cv * fmaf(2.0f * g.c4, o.x0 + o.y0, g.br1);
+    p2 = cv * g.c4;
+}
+
+// e^d - 1 and e^{-d} - 1, both to FP32 relative accuracy
+__device__ __forceinline__ void expm1_pair(float d, float &ep, float &em)
+{
+    const float E = expm1f(fabsf(d));
+    const float En = __fdividef(-E, 1.0f + E);
+    ep = d >= 0.0f ? E : En;
+    em = d >= 0.0f ? En : E;
+}
+
+// u from the corner at d = upsilon2 - (row centre)
+__device__ __forceinline__ float row_u(const PieceGeo &g, const NodeRow &o, float d)
+{
+    float ep, em;
+    expm1_pair(d, ep, em);
+    return (o.x0 + o.y0) + fmaf(g.s1 * o.xc, ep, g.s2 * o.yc * em);
+}
+
+// first column of the row past |f1| = |f2|, where u turns if both have one sign
+__device__ __forceinline__ int row_turn(const PieceGeo &g, const NodeRow &o, int G)
+{
+    if (g.s1 != g.s2) return 0;
+    const float x = __fdividef(0.5f * __logf(__fdividef(o.yc, o.xc)), o.du2) + 0.5f * (float)G - 0.5f;
+    return x > 0.0f ? (x < (float)G ? (int)ceilf(x) : G) : 0;
+}
+
+// The runs of one row in column order: f(candidate, j0, N).  On one half-open
+// interval of columns u is monotone, so a candidate's columns are a run found
+// by bisection.
+template <typename F>
+__device__ __forceinline__ void row_runs(const PieceGeo &g, const NodeRow &o, int G, int ca, int cb, const F &f)
+{
+    const float c0 = 0.5f - 0.5f * (float)G;
+    const auto u_at = [&](int j) { return row_u(g, o, ((float)j + c0) * o.du2); };
+    const int jm = row_turn(g, o, G);
+    for (int part = 0; part < 2; ++part) {
+        const int ja = part == 0 ? 0 : jm, jb = part == 0 ? jm : G;
+        if (jb <= ja) continue;
+        const bool up = (g.s1 > 0.0f) == (part == 1 || g.s1 != g.s2);
+        const float ua = u_at(ja), ub = u_at(jb - 1);
+        // first column of [ja, jb) at or past edge e in the direction of travel
+        const auto first = [&](float e) {
+            int lo = ja, hi = jb;
+            while (lo < hi) {
+                const int m = (lo + hi) >> 1;
+                const float u = m == ja ? ua : m == jb - 1 ? ub : u_at(m);
+                if (up ? u >= e : u < e) hi = m;
+                else lo = m + 1;
+            }
+            return lo;
+        };
+        for (int q = ca; q < cb; ++q) {
+            const int c = up ? q : ca + cb - 1 - q;
+            const float lo = g.lo[c], hi = g.hi[c];
+            if ((up ? ub : ua) < lo || (up ? ua : ub) >= hi) continue;
+            // entering edge, leaving edge
+            const int j0 = (up ? ua >= lo : ua < hi) ? ja : first(up ? lo : hi);
+            const int j1 = (up ? ub < hi : ub >= lo) ? jb : first(up ? hi : lo);
+            if (j1 > j0) f(c, j0, j1 - j0);
+        }
+    }
+}
+
+// Bound of |du/dt| per column of a run's half-length, t in [-1, 1], from the
+// row's largest |f1|, |f2|, and the phase swing it brings.
+__device__ __forceinline__ float row_swing(const PieceGeo &g, const NodeRow &o, int G)
+{
+    float p1, p2;
+    row_slopes(g, o, p1, p2);
+    const float e = expf(0.5f * (float)G * o.du2) * (o.xc + o.yc) * 0.5f * o.du2;
+    return e * (g.band * (fabsf(p1) + 2.0f * fabsf(p2) * e * (float)G) + 2.0f * g.tilt);
+}
+
+// A run cut into the parts one rule each covers: f(j0, N, n), n = N where the
+// columns themselves are no more than the rule needs.  n <= kGaussMaxNodes: a
+// part of a run that needs n > 48 nodes has (A + 1.4 D) / parts <= 48 and so
+// needs at most 37, and a part of <= 48 columns takes at most its columns.
+template <typename F>
+__device__ __forceinline__ void run_parts(const PieceGeo &g, const NodeRow &o, int G, int j0, int N, const F &f)
+{
+    const float per = row_swing(g, o, G), hd = 0.5f * o.du2;
+    int n = gauss_need(per * (float)N, hd * (float)N);
+    int parts = 1;
+    if (N > kGaussMaxNodes && (n > kGaussMaxNodes || N > kGaussMaxN)) {
+        parts = max((N + kGaussMaxN - 1) / kGaussMaxN, (n + 23) / 24);
+        parts = min(parts, (N + kGaussMaxNodes - 1) / kGaussMaxNodes);
+    }
+    for (int s = 0; s < parts; ++s) {
+        const int a = (int)((long long)N * s / parts), b = (int)((long long)N * (s + 1) / parts);
+        const int Ns = b - a;
+        if (parts > 1) n = gauss_need(per * (float)Ns, hd * (float)Ns);
+        const int nn = n <= kGaussMaxNodes ? gauss_nodes(gauss_pick(n)) : Ns;
+        f(j0 + a, Ns, nn < Ns ? nn : Ns);
+    }
+}
+
+// The F_c candidate that holds every column of the row, or -1; ph: bound of
+// |phi| band over the row's columns.
+__device__ __forceinline__ int row_whole(const PieceGeo &g, const NodeRow &o, int G, float &ph)
+{
+    const float c0 = 0.5f - 0.5f * (float)G;
+    const float ua = row_u(g, o, c0 * o.du2), ub = row_u(g, o, -c0 * o.du2);
+    float mn = fminf(ua, ub), mx = fmaxf(ua, ub);
+    const int jm = row_turn(g, o, G);
+    if (jm > 0 && jm < G) {
+        const float um = row_u(g, o, ((float)jm + c0) * o.du2), un = row_u(g, o, ((float)jm - 1.0f + c0) * o.du2);
+        mn = fminf(mn, fminf(um, un));
+        mx = fmaxf(mx, fmaxf(um, un));
+    }
+    float p1, p2;
+    row_slopes(g, o, p1, p2);
+    const float r = mx - mn;
+    ph = g.band * (fabsf(o.phi0) + r * (fabsf(p1) + fabsf(p2) * r));
+    int c = -1;
+    for (int q = 0; q < g.nc; ++q)
+        if (mn >= g.lo[q] && mx < g.hi[q]) c = q;
+    return c;
+}
+
+// The blocks of low rows: the rows [0, R1) whose columns all lie in one
+// candidate, with one set of limits and |phi| band <= kBlkPhiL, cut at |phi|
+// band = kBlkPhiLow and into parts of kGaussMaxN rows.  Along t in [-1, 1] over
+// N rows upsilon1 (so the weight and phi) is exp-like with D = N ds / 2, and the
+// phase swings by at most |phi| band D.  Whole warp; writes ns.blk, returns the
+// units (rows of the rules) of all blocks, R1 and the candidate.
+template <int Cap>
+__device__ __forceinline__ int row_blocks(WarpNodes<Cap> &ns, int G, int &R1, int &nblk, int &cand)
+{
+    const PieceGeo &g = ns.geo;
+    const int lane = threadIdx.x & 31;
+    float ph_last = 0.0f;
+    R1 = 0;
+    cand = -1;
+    // candidate and limits of row r (-1: not in one candidate), |phi| band
+    const auto test = [&](int r, float &ph) {
+        NodeRow o;
+        const int lim = node_row(g, G, (double)(G - r) - 0.5, o);
+        ph = 0.0f;
+        const int c = lim >= 0 ? row_whole(g, o, G, ph) : -1;
+        return c >= 0 ? (c << 2 | lim) : -1;
+    };
+    // lanes take rows step apart; the first that fails bounds the next, finer
+    // sweep.  A row between two that pass passes too: with both limits of |f2|
+    // following upsilon1, or f1 and f2 of one sign, the ends of the row's u are
+    // monotone in upsilon1; otherwise every row is tested.
+    const int step = (G + 31) / 32;
+    int key0;
+    {
+        float ph;
+        const int key = test(min(lane * step, G - 1), ph);
+        key0 = __shfl_sync(0xffffffffu, key, 0);
+        if (key0 < 0 || !(__shfl_sync(0xffffffffu, ph, 0) <= kBlkPhiL)) return 0;
+        if ((key0 & 3) == 3 || g.s1 == g.s2) {
+            const bool ok = lane * step < G && key == key0 && ph <= kBlkPhiL;
+            const int bad = __ffs(~__ballot_sync(0xffffffffu, ok)) - 1;      // -1: none
+            R1 = bad < 0 ? min(G, 31 * step + 1) : (bad - 1) * step + 1;
+            ph_last = __shfl_sync(0xffffffffu, ph, bad < 0 ? 31 : bad - 1);
+        }
+    }
+    for (int r0 = R1; r0 < G; r0 += 32) {
+        float ph;
+        const int r = min(r0 + lane, G - 1);
+        const int key = test(r, ph);
+        const bool ok = r0 + lane < G && key == key0 && ph <= kBlkPhiL;
+        const int bad = __ffs(~__ballot_sync(0xffffffffu, ok)) - 1;
+        const int n = bad < 0 ? 32 : bad;
+        if (n > 0) ph_last = __shfl_sync(0xffffffffu, ph, n - 1);
+        R1 += n;
+        if (n < 32) break;
+    }
+    cand = key0 >> 2;
+    // rows from the block's top down to |phi| band = kBlkPhiLow
+    int top = ph_last > kBlkPhiLow ? (int)ceilf(__fdividef(__logf(ph_last / kBlkPhiLow), g.ds)) : 0;
+    top = min(top, R1);
+    int units = 0;
+    nblk = 0;
+    for (int low = 1; low >= 0; --low) {
+        const int n_rows = low ? R1 - top : top, parts = (n_rows + kGaussMaxN - 1) / kGaussMaxN;
+        for (int s = 0; s < parts; ++s) {
+            const int a = n_rows * s / parts, b = n_rows * (s + 1) / parts, N = b - a;
+            const float D = 0.5f * (float)N * g.ds;
+            const int need = gauss_need(fminf(ph_last, low ? kBlkPhiLow : kBlkPhiL) * D, D);
+            const int n = need <= kGaussMaxNodes ? gauss_nodes(gauss_pick(need)) : N;
+            if (lane == 0)
+                ns.blk[nblk] = RowBlock{units, (low ? 0 : R1 - top) + a, N,
+                                        n < N ? (N - 1) * kGaussPerN + gauss_offset(gauss_pick(need)) : -1};
+            ++nblk;
+            units += min(n, N);
+        }
+    }
+    __syncwarp();
+    return units;
+}
+
+// Unit q of the piece: a row of a block's rule (q < nv) or a row of its own.
+template <int Cap>
+__device__ __forceinline__ void unit_row(const WarpNodes<Cap> &ns, const float2 *gauss, int G, int q, int nv, int R1,
+                                         int nblk, NodeRow &o)
+{
+    double k = (double)(G - (R1 + q - nv)) - 0.5;
+    float wt = 1.0f;
+    if (q < nv) {
+        int b = 0;
+        while (b + 1 < nblk && ns.blk[b + 1].unit0 <= q) ++b;
+        const RowBlock bl = ns.blk[b];
+        if (bl.toff >= 0) {
+            const float2 e = __ldg(gauss + bl.toff + (q - bl.unit0));
+            k = (double)(G - bl.r0) - 0.5 * (double)bl.N - 0.5 * (double)bl.N * (double)e.x;
+            wt = e.y;
+        } else {
+            k = (double)(G - (bl.r0 + q - bl.unit0)) - 0.5;
+        }
+    }
+    node_row(ns.geo, G, k, o);
+    o.w *= wt;
+}
+
+// The runs of unit `row` of the warp's 32 (candidates [ca, cb); whole >= 0:
+// the one candidate that holds every column): returns the slots they take.
+// With c0 >= 0 also writes those whose first slot (counted from `off`) falls in
+// [c0, c0 + kSpan), and marks the rest of the window [c0, c0 + Cap) that the
+// row covers as empty.  One function for both, never inlined, so that the
+// counting and the writing pass evaluate every edge with the same instructions.
+template <int Cap>
+__device__ __noinline__ int node_emit(WarpNodes<Cap> &ns, int G, int row, int ca, int cb, int whole, int off, int c0)
+{
+    constexpr int span = WarpNodes<Cap>::kSpan;
+    const NodeRow o = ns.row[row];
+    if (o.w == 0.0f) return 0;
+    const int off0 = off;
+    const auto take_run = [&](int c, int j0, int N) {
+        run_parts(ns.geo, o, G, j0, N, [&](int j, int Ns, int n) {
+            const int take = max(n, kNodeMin);
+            if (c0 >= 0) {
+                const bool here = off >= c0 && off < c0 + span;
+                const int s = off - c0, id = s >> 2;      // runs start >= kNodeMin slots apart
+                if (here) {
+                    NodeRun r;
+                    r.jc = (float)j + 0.5f * (float)(Ns - G);
+                    r.half = 0.5f * (float)Ns;
+                    r.toff = n == Ns ? -1 : (Ns - 1) * kGaussPerN + gauss_offset(gauss_pick(n));
+                    r.id = (unsigned)s | (unsigned)c << 12 | (unsigned)row << 17 | (whole >= 0 ? 1u << 31 : 0u);
+                    ns.run[id] = r;
+                }
+                for (int q = max(s, 0); q < min(s + take, Cap); ++q)
+                    ns.of[q] = here && q - s < n ? (unsigned short)id : 0xffff;
+            }
+            off += take;
+        });
+    };
+    if (whole >= 0) take_run(whole, 0, G);
+    else row_runs(ns.geo, o, G, ca, cb, take_run);
+    return off - off0;
+}
+
+// One node: its row, candidate, f1 and f2 from the corner, phi and weight.
+struct Node {
+    int ci, N;                  // N: columns of a row's run at its first node, else 0
+    float x, y, phi, phi_lo, wq;
+};
+
+template <int Cap>
+__device__ __forceinline__ bool node_get(const WarpNodes<Cap> &ns, const float2 *gauss, int q, Node &nd)
+{
+    const unsigned id = ns.of[q];
+    if (id == 0xffffu) return false;
+    const NodeRun r = ns.run[id];
+    const int k = q - (int)(r.id & 0xfffu);
+    nd.ci = (int)(r.id >> 12 & 31u);
+    nd.N = k == 0 && !(r.id >> 31) ? (int)(2.0f * r.half) : 0;
+    float pos, wt = 1.0f;
+    if (r.toff >= 0) {
+        const float2 e = __ldg(gauss + r.toff + k);
+        pos = fmaf(e.x, r.half, r.jc);
+        wt = e.y;
+    } else {
+        pos = r.jc - r.half + 0.5f + (float)k;
+    }
+    const PieceGeo &g = ns.geo;
+    const NodeRow o = ns.row[r.id >> 17 & 31u];
+    float ep, em, p1, p2;
+    expm1_pair(pos * o.du2, ep, em);
+    row_slopes(g, o, p1, p2);
+    const float dx = g.s1 * o.xc * ep, dy = g.s2 * o.yc * em, du = dx + dy;
+    nd.x = o.x0 + dx;
+    nd.y = o.y0 + dy;
+    const float dphi = du * fmaf(p2, du, p1);
+    nd.phi = __fadd_rn(o.phi0, dphi);                 // two-sum
+    const float t = __fadd_rn(nd.phi, -o.phi0);
+    nd.phi_lo = __fadd_rn(__fadd_rn(o.phi0, -__fadd_rn(nd.phi, -t)), __fadd_rn(dphi, -t)) + o.phi0_lo;
+    nd.wq = o.w * wt;
+    return true;
+}
+
+// The nodes of a piece in chunks: f(number of slots) is called by the whole
+// warp for each chunk, with ns filled for node_get.  small gets the columns of
+// the rows taken in blocks.
+template <int Cap, typename F>
+__device__ __forceinline__ void piece_nodes(WarpNodes<Cap> &ns, const float2 *gauss, int G, int ca, int cb,
+                                            int &small, const F &f)
+{
+    const int lane = threadIdx.x & 31;
+    int R1, nblk = 0, cand;
+    const int nv = row_blocks(ns, G, R1, nblk, cand);
+    const bool mine = cand >= ca && cand < cb;        // the blocks' candidate belongs to this sweep
+    small = mine ? R1 * G : 0;
+    const int first = mine ? 0 : nv;
+    const int units = nv + (G - R1);
+    for (int u0 = first; u0 < units; u0 += 32) {
+        const int q = u0 + lane;
+        int slots = 0, whole = -1;
+        if (q < units) {
+            NodeRow o;
+            unit_row(ns, gauss, G, q, nv, R1, nblk, o);
+            ns.row[lane] = o;
+            whole = q < nv ? cand : -1;
+            slots = node_emit(ns, G, lane, ca, cb, whole, 0, -1);
+        }
+        int incl = slots;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += v;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, 31), base = incl - slots;
+        for (int c0 = 0; c0 < total; c0 += WarpNodes<Cap>::kSpan) {
+            if (slots > 0 && base < c0 + Cap && incl > c0) node_emit(ns, G, lane, ca, cb, whole, base, c0);
+            __syncwarp();
+            f(min(total - c0, Cap));
+            __syncwarp();
+        }
+    }
+}
+
+}  // namespace isrs

@@ -174,4 +174,95 @@ __device__ __forceinline__ float walk_small(const float4 *o0s, const float4 *o1s
     return wq * fmaf(-ph2, fmaf(s0, s2, -s1 * s1), s0 * s0);
 }
 
+// ---------------------------------------------------------------------------
+// Walks of a node of the row sums: zt[k][16] = {z_{m+1}/2pi hi, lo, z_m, dz_m}
+// and, for the node's F_c candidate, ek[k][16] = {log2 p_m at the channel's
+// centre, K2_m} of lane l16's steps (both already offset by l16; padding steps
+// carry log2 weight -1000); dF = F_c - f_c, Fc = F_c - f_ref, phi float-float.
+// ---------------------------------------------------------------------------
+template <int K>
+__device__ __forceinline__ float walk_direct_n(const float4 *zt, const float2 *ek, float wq, float ph, float dF,
+                                               float Fc, float mult, float (&R)[K], float (&Rp)[K])
+{
+    const float hph = 0.5f * ph;
+    const float phr = ph * 0.15915494309189535f;
+    float tr[K], ti[K];
+    float sr = 0.0f, si = 0.0f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const float4 o = zt[k * 16];
+        const float2 e = ek[k * 16];
+        float sn, cs;
+        sincos_rev<true>(phr * o.z, sn, cs);
+        const float amp = ex2_approx(fmaf(e.y, dF, e.x)) * (sinc_poly(hph * o.w) * o.w);
+        tr[k] = amp * cs;
+        ti[k] = amp * sn;
+        sr += tr[k];
+        si += ti[k];
+    }
+    sr = half_sum(sr);
+    si = half_sum(si);
+    const float c2 = 2.0f * mult * wq, c2F = c2 * Fc;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const float rr = fmaf(sr, tr[k], si * ti[k]);
+        R[k] = fmaf(c2, rr, R[k]);
+        Rp[k] = fmaf(c2F, rr, Rp[k]);
+    }
+    return wq * fmaf(sr, sr, si * si);
+}
+
+template <int K>
+__device__ __forceinline__ float walk_tele_n(const float4 *zt, const float2 *ek, int l16, float wq, float ph,
+                                             float ph_lo, float dF, float Fc, float mult, float (&R)[K],
+                                             float (&Rp)[K])
+{
+    float tr[K], ti[K];
+    float Er = 1.0f, Ei = 0.0f, p0 = 0.0f, e1r = 1.0f, e1i = 0.0f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const float4 b = zt[k * 16];
+        const float2 e = ek[k * 16];
+        float sn, cs;
+        phasor_rev_ff<true>(ph, b.x, b.y, sn, cs, ph_lo);
+        const float pm = ex2_approx(fmaf(e.y, dF, e.x));
+        if (k == 0) {
+            p0 = pm;
+            e1r = cs;
+            e1i = sn;
+            tr[0] = 0.0f;
+            ti[0] = 0.0f;
+        } else {
+            tr[k] = pm * (cs - Er);
+            ti[k] = pm * (sn - Ei);
+        }
+        Er = cs;
+        Ei = sn;
+    }
+    // the lower edge of this lane's first step is the previous lane's last edge
+    float elr = __shfl_up_sync(kWarpAll, Er, 1, 16);
+    float eli = __shfl_up_sync(kWarpAll, Ei, 1, 16);
+    elr = l16 == 0 ? 1.0f : elr;
+    eli = l16 == 0 ? 0.0f : eli;
+    tr[0] = p0 * (e1r - elr);
+    ti[0] = p0 * (e1i - eli);
+    float ur = 0.0f, ui = 0.0f;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        ur += tr[k];
+        ui += ti[k];
+    }
+    ur = half_sum(ur);
+    ui = half_sum(ui);
+    const float iph2 = __fdividef(1.0f, ph * ph);
+    const float c2 = 2.0f * mult * wq * iph2, c2F = c2 * Fc;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const float rr = fmaf(ur, tr[k], ui * ti[k]);
+        R[k] = fmaf(c2, rr, R[k]);
+        Rp[k] = fmaf(c2F, rr, Rp[k]);
+    }
+    return wq * fmaf(ur, ur, ui * ui) * iph2;
+}
+
 }  // namespace isrs

@@ -98,19 +98,19 @@ __device__ __forceinline__ float zsum_tele_f(float phi, float Fc, float at, cons
     return __fdividef(Sr * Sr + Si * Si, phi * phi);
 }
 
-// The same two forms with the candidate's attenuation folded into the step
-// tables (rows of a per-candidate copy):
-//   sRc[m] = {A2_m + log2 dz_m - at z_m, K2_m, z_m, dz_m},
-//   sEc[m] = {z_{m+1}/2pi hi, lo, A2_m - at z_m, K2_m},
-// so log2 p_m = row + K2_m Fc in one FMA and the telescoped form needs no z.
-__device__ __forceinline__ float zsum_direct_fc(float phi, float Fc, const float4 *sRc, int M)
+// The same two forms for a node of the row sums: zt[m] = {z_{m+1}/2pi hi, lo,
+// z_m, dz_m} and, for the node's F_c candidate, ek[m] = {log2 p_m at the
+// channel's centre, K2_m}, so log2 p_m = ek.x + K2_m dF with dF = F_c - f_c; phi
+// is a float-float value (the direct form's phases need only its head).
+__device__ __forceinline__ float zsum_direct_n(float phi, float dF, const float4 *zt, const float2 *ek, int M)
 {
     float Sr = 0.0f, Si = 0.0f;
     const float hphi = 0.5f * phi;
     const float phir = phi * 0.15915494309189535f;
 #pragma unroll 4
     for (int m = 0; m < M; ++m) {
-        const float4 a = sRc[m];
+        const float4 a = zt[m];
+        const float2 e = ek[m];
         float sn, cs;
         sincos_rev(phir * a.z, sn, cs);
         const float x = hphi * a.w;
@@ -120,22 +120,24 @@ __device__ __forceinline__ float zsum_direct_fc(float phi, float Fc, const float
         sc = fmaf(x2, sc, 8.3333333e-3f);                      // 1/5!
         sc = fmaf(x2, sc, -1.6666667e-1f);                     // -1/3!
         sc = fmaf(x2, sc, 1.0f);
-        const float amp = ex2_approx(fmaf(a.y, Fc, a.x)) * sc;
+        const float amp = ex2_approx(fmaf(e.y, dF, e.x)) * (sc * a.w);
         Sr = fmaf(amp, cs, Sr);
         Si = fmaf(amp, sn, Si);
     }
     return Sr * Sr + Si * Si;
 }
 
-__device__ __forceinline__ float zsum_tele_fc(float phi, float Fc, const float4 *sEc, int M)
+__device__ __forceinline__ float zsum_tele_n(float phi, float phi_lo, float dF, const float4 *zt, const float2 *ek,
+                                             int M)
 {
     float Er = 1.0f, Ei = 0.0f, Sr = 0.0f, Si = 0.0f;
 #pragma unroll 4
     for (int m = 0; m < M; ++m) {
-        const float4 e = sEc[m];
+        const float4 a = zt[m];
+        const float2 e = ek[m];
         float sn, cs;
-        phasor_rev_ff(phi, e.x, e.y, sn, cs);
-        const float p = ex2_approx(fmaf(e.w, Fc, e.z));
+        phasor_rev_ff(phi, a.x, a.y, sn, cs, phi_lo);
+        const float p = ex2_approx(fmaf(e.y, dF, e.x));
         Sr = fmaf(p, cs - Er, Sr);
         Si = fmaf(p, sn - Ei, Si);
         Er = cs;

@@ -702,7 +702,7 @@ __global__ void __launch_bounds__(256, 4) k_quad_f32_tab(QuadParams qp)
             const float three_fi2 = 3.0f * fi * fi;
             float sum = 0.0f, comp = 0.0f;
             const int npts = G * G;
-            for (int q = threadIdx.x; q < npts; q += blockDim.x) {
+            for (int q = threadIdx.x + (item.part & 0xffff) * blockDim.x; q < npts; q += (item.part >> 16) * blockDim.x) {
                 const int r = (int)(((float)q + 0.5f) * invG);
                 const int j = q - r * G;
                 const RowF rw = rows[dbg_clamp(r, G, kDbgRow, qp.dbg)];
@@ -817,7 +817,7 @@ __global__ void __launch_bounds__(256) k_quad_f64_tab(QuadParams qp)
             const double da0 = s_d0[0], db0 = s_d0[1];
             double sum = 0.0;
             const int npts = G * G;
-            for (int q = threadIdx.x; q < npts; q += blockDim.x) {
+            for (int q = threadIdx.x + (item.part & 0xffff) * blockDim.x; q < npts; q += (item.part >> 16) * blockDim.x) {
                 const int r = q / G;
                 const int j = q - r * G;
                 const RowD rw = rows[dbg_clamp(r, G, kDbgRow, qp.dbg)];

@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
                 float vsum = 0.0f;
                 int ns = 0, nd = 0, nt = 0;
                 int batches = 0;
-                for (int qb = warp * 32; qb < npts; qb += blockDim.x) {
+                for (int qb = warp * 32 + (item.part & 0xffff) * blockDim.x; qb < npts; qb += (item.part >> 16) * blockDim.x) {
                     // ---- 1. this lane's grid point, if its F_c is in candidate cc
                     const int q = qb + lane;
                     float cp = 0.0f, phi = 0.0f, da = 0.0f, db = 0.0f;
