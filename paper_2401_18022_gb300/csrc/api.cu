@@ -723,7 +723,7 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
         int ncm = 1;
         for (const DevPiece &pc : pieces) ncm = std::max(ncm, std::min(pc.c_hi - pc.c_lo + 1, kMaxCand));
         g->nc_max = ncm;
-        if (quad_tab_smem_bytes(0, g->n_steps, q->G, ncm) > 200 * 1024)
+        if (quad_tab_limit_bytes(0, g->n_steps, q->G, ncm) > 200 * 1024)
             return fail(h, ISRS_ERR_UNSUPPORTED, "Raman-ODE tables of %d candidates x %d steps exceed shared memory",
                         ncm, g->n_steps);
     }
@@ -1068,16 +1068,11 @@ isrs_status run_forward(isrs_handle h, const isrs_fibre *fb, Geom *g, int precis
         if ((s = mark(h, 1, 1, st)) != ISRS_OK) return s;
     } else {
         const bool tab = g->profile == ISRS_PROFILE_RAMAN_ODE;
-        if (tab && quad_tab_smem_bytes(precision, M, g->G, g->nc_max) > 200 * 1024)
+        if (tab && quad_tab_limit_bytes(precision, M, g->G, g->nc_max) > 200 * 1024)
             return fail(h, ISRS_ERR_UNSUPPORTED, "profile tables exceed shared memory at this precision");
         if ((s = mark(h, 0, 0, st)) != ISRS_OK) return s;
-        if (tab && g->n_items > 0) {
-            int grid = h->num_sms * quad_tab_blocks_per_sm(precision, M, g->G, g->nc_max, block);
-            if (g->n_items < grid) grid = std::max(1, g->n_items);
-            CK(launch_quad_tab(qp, precision, grid, block, st));
-        } else if (g->n_items > 0) {
-            CK(launch_quad(qp, precision, h->num_sms, block, st));
-        }
+        if (g->n_items > 0) CK(tab ? launch_quad_tab(qp, precision, h->num_sms, block, st)
+                                   : launch_quad(qp, precision, h->num_sms, block, st));
         if (g->n_mci_items > 0) {
             QuadParams qm = qp;
             qm.items = (const DevItem *)g->mci_items.p;
@@ -1334,12 +1329,10 @@ isrs_status run_grad_tab_fwd(isrs_handle h, const isrs_fibre *fb, Geom *g, cudaS
     ap.rows = (double2 *)h->tab_rows.p;
     ap.rowsV = (double *)h->tab_rowsV.p;
     const int block = h->tile_threads > 0 ? h->tile_threads : 256;
-    int grid = h->num_sms * adjoint_tab_blocks_per_sm(M, g->G, g->nc_max, block);
-    if (g->n_items < grid) grid = std::max(1, g->n_items);
     {
         Range r_adj("isrs quadrature + adjoint (tabulated profile)");
         if ((s = mark(h, 1, 0, st)) != ISRS_OK) return s;
-        if (g->n_items > 0) CK(launch_adjoint_tab(ap, grid, block, st));
+        if (g->n_items > 0) CK(launch_adjoint_tab(ap, h->num_sms, block, st));
         if ((s = mark(h, 1, 1, st)) != ISRS_OK) return s;
     }
     h->last_points = g->n_points;

@@ -156,9 +156,7 @@ struct TabGatherParams {
 };
 cudaError_t launch_tab_gather(const TabGatherParams &gp, cudaStream_t st);
 
-size_t adjoint_tab_smem_bytes(int n_steps, int G, int nc_max, int block);
-int adjoint_tab_blocks_per_sm(int n_steps, int G, int nc_max, int block);
-cudaError_t launch_adjoint_tab(const AdjTabParams &ap, int grid, int block, cudaStream_t st);
+cudaError_t launch_adjoint_tab(const AdjTabParams &ap, int num_sms, int block, cudaStream_t st);
 cudaError_t launch_ybar(const ChainParams &cp, cudaStream_t st);
 
 size_t raman_smem_bytes(int n_ch);
@@ -173,9 +171,10 @@ cudaError_t launch_piece_logs(DevPiece *pieces, int n, cudaStream_t st);
 cudaError_t launch_prep(const PrepParams &pp, int n_prof, cudaStream_t st);
 cudaError_t launch_quad(const QuadParams &qp, int precision, int num_sms, int block, cudaStream_t st);
 // the same quadratures with the tabulated profile (qp.ab set)
-size_t quad_tab_smem_bytes(int precision, int n_steps, int G, int nc_max);
-int quad_tab_blocks_per_sm(int precision, int n_steps, int G, int nc_max, int block);
-cudaError_t launch_quad_tab(const QuadParams &qp, int precision, int grid, int block, cudaStream_t st);
+// (calls with quad_tab_limit_bytes over 200 KB are UNSUPPORTED: the FP64 kernel's
+// tables, and for FP32 the same order of size)
+size_t quad_tab_limit_bytes(int precision, int n_steps, int G, int nc_max);
+cudaError_t launch_quad_tab(const QuadParams &qp, int precision, int num_sms, int block, cudaStream_t st);
 cudaError_t launch_finish(const FinishParams &fp, int n_prof, cudaStream_t st);
 // MCI cells with their own grid (closed-form profile)
 size_t quad_mci_smem_bytes(int precision, int n_steps, int n_max);

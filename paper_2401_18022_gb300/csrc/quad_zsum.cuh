@@ -146,6 +146,54 @@ __device__ __forceinline__ float zsum_tele_n(float phi, float phi_lo, float dF, 
     return __fdividef(Sr * Sr + Si * Si, phi * phi);
 }
 
+// ... with the tabulated profile: q[m] = {log2 p_m, slope along the node's
+// longer axis, along the shorter}, dl and dd the offsets of F_a, F_b inside
+// their channels (in that order of axes).
+__device__ __forceinline__ float zsum_direct_nt(float phi, float dl, float dd, const float4 *zt, const float4 *q,
+                                                int M)
+{
+    float Sr = 0.0f, Si = 0.0f;
+    const float hphi = 0.5f * phi;
+    const float phir = phi * 0.15915494309189535f;
+#pragma unroll 4
+    for (int m = 0; m < M; ++m) {
+        const float4 a = zt[m];
+        const float4 e = q[m];
+        float sn, cs;
+        sincos_rev(phir * a.z, sn, cs);
+        const float x = hphi * a.w;
+        const float x2 = x * x;
+        float sc = fmaf(x2, -2.5052108e-8f, 2.7557319e-6f);   // -1/11!, 1/9!
+        sc = fmaf(x2, sc, -1.9841270e-4f);                     // -1/7!
+        sc = fmaf(x2, sc, 8.3333333e-3f);                      // 1/5!
+        sc = fmaf(x2, sc, -1.6666667e-1f);                     // -1/3!
+        sc = fmaf(x2, sc, 1.0f);
+        const float amp = ex2_approx(fmaf(e.z, dd, fmaf(e.y, dl, e.x))) * (sc * a.w);
+        Sr = fmaf(amp, cs, Sr);
+        Si = fmaf(amp, sn, Si);
+    }
+    return Sr * Sr + Si * Si;
+}
+
+__device__ __forceinline__ float zsum_tele_nt(float phi, float phi_lo, float dl, float dd, const float4 *zt,
+                                              const float4 *q, int M)
+{
+    float Er = 1.0f, Ei = 0.0f, Sr = 0.0f, Si = 0.0f;
+#pragma unroll 4
+    for (int m = 0; m < M; ++m) {
+        const float4 a = zt[m];
+        const float4 e = q[m];
+        float sn, cs;
+        phasor_rev_ff(phi, a.x, a.y, sn, cs, phi_lo);
+        const float p = ex2_approx(fmaf(e.z, dd, fmaf(e.y, dl, e.x)));
+        Sr = fmaf(p, cs - Er, Sr);
+        Si = fmaf(p, sn - Ei, Si);
+        Er = cs;
+        Ei = sn;
+    }
+    return __fdividef(Sr * Sr + Si * Si, phi * phi);
+}
+
 // As phasor_rev_ff, for phases far beyond 2^22 revolutions (the MCI cells):
 // once |phi z / 2pi| >= 2^22 the first magic-number rounding leaves an
 // integer (or half-integer) on top of the fraction, and FRND's exact

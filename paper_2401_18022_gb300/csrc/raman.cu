@@ -36,9 +36,14 @@
 //               grid point costs the same two FMAs per step as the closed form.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "isrs_internal.cuh"
 #include "isrs_kernels.h"
 #include "quad_common.cuh"
+#include "quad_nodes.cuh"
+#include "quad_tab.cuh"
+#include "quad_zsum.cuh"
 
 namespace isrs {
 
@@ -454,298 +459,100 @@ cudaError_t launch_raman_adj(const RamanAdjParams &ap, cudaStream_t st)
 // ---------------------------------------------------------------------------
 // Quadratures with the tabulated profile.
 // ---------------------------------------------------------------------------
-namespace {
+constexpr int kTabSlots = 224;       // node slots of a chunk
+constexpr int kTabCand = 2;          // F_c candidates swept together (most pieces have two)
+using TabNodes = WarpNodes<kTabSlots>;
 
-// Per-piece table: for every candidate channel ci of F_c and step m (log2
-// units, FP32) {A + log2 dz, Sa, Sb, A}, built in FP64 from the profile
-// tables.  Every thread calls; the caller syncs before use.
-__device__ void tab_setup_f(const QuadParams &qp, const DevPiece &pc, int prof, int nc, float4 *sQ)
+// Dynamic shared memory of k_quad_f32_tab: zt [M], then per warp the nodes and
+// the candidates' step rows.
+__host__ __device__ constexpr size_t tab_warp_bytes(int n_steps)
 {
-    const int M = qp.n_steps;
-    const int coff = qp.plan_ch_off[pc.plan];
-    const double2 *T = qp.ab + (size_t)qp.prof_ch_off[prof] * M;
-    const double fa = qp.ch_frel[coff + pc.a], fb = qp.ch_frel[coff + pc.b], fi = qp.ch_frel[coff + pc.cut];
-    for (int t = threadIdx.x; t < nc * M; t += blockDim.x) {
-        const int ci = t / M, m = t - ci * M;
-        const int c = pc.c_lo + ci;
-        const double2 ta = T[(size_t)pc.a * M + m], tb = T[(size_t)pc.b * M + m];
-        const double2 ti = T[(size_t)pc.cut * M + m], tc = T[(size_t)c * M + m];
-        const double D = (fa + fb) - (fi + qp.ch_frel[coff + c]);
-        const double A = 0.5 * (ta.x + tb.x + tc.x - ti.x + tc.y * D) * kLog2e;
-        sQ[t] = make_float4((float)A + qp.zs_a[m].z, (float)(0.5 * (ta.y + tc.y) * kLog2e),
-                            (float)(0.5 * (tb.y + tc.y) * kLog2e), (float)A);
-    }
+    return sizeof(TabNodes) + sizeof(float4) * kTabCand * (size_t)n_steps;
 }
 
-// FP32 z-sums of Eq. slow_vary with log2 p_m = Q.w + Q.y da + Q.z db (the
-// three forms of the closed-form kernel: small-phase expansion, direct,
-// telescoped).  sZ[m] = {z_m, z_m^2 + dz_m^2/12, dz_m, -}, sE[m] = {z_{m+1}/2pi
-// hi, lo, -, -}.
-__device__ __forceinline__ float zsum_small_t(float phi, float da, float db, const float4 *Q, const float4 *sZ,
-                                              int M)
-{
-    float M0 = 0.0f, M1 = 0.0f, M2 = 0.0f;
-#pragma unroll 4
-    for (int m = 0; m < M; ++m) {
-        const float4 q = Q[m];
-        const float4 z = sZ[m];
-        float lp = fmaf(q.y, da, q.x);
-        lp = fmaf(q.z, db, lp);
-        const float w = ex2_approx(lp);          // p_m dz_m
-        M0 += w;
-        M1 = fmaf(w, z.x, M1);
-        M2 = fmaf(w, z.y, M2);
-    }
-    return fmaf(-phi * phi, fmaf(M0, M2, -M1 * M1), M0 * M0);
-}
-
-__device__ __forceinline__ float zsum_direct_t(float phi, float da, float db, const float4 *Q, const float4 *sZ,
-                                               int M)
-{
-    float Sr = 0.0f, Si = 0.0f;
-    const float hphi = 0.5f * phi;
-    const float phir = phi * 0.15915494309189535f;
-#pragma unroll 4
-    for (int m = 0; m < M; ++m) {
-        const float4 q = Q[m];
-        const float4 z = sZ[m];
-        float sn, cs;
-        sincos_rev(phir * z.x, sn, cs);
-        const float x = hphi * z.z;
-        const float x2 = x * x;
-        float sc = fmaf(x2, -2.5052108e-8f, 2.7557319e-6f);   // -1/11!, 1/9!
-        sc = fmaf(x2, sc, -1.9841270e-4f);                     // -1/7!
-        sc = fmaf(x2, sc, 8.3333333e-3f);                      // 1/5!
-        sc = fmaf(x2, sc, -1.6666667e-1f);                     // -1/3!
-        sc = fmaf(x2, sc, 1.0f);
-        float lp = fmaf(q.y, da, q.x);
-        lp = fmaf(q.z, db, lp);
-        const float amp = ex2_approx(lp) * sc;
-        Sr = fmaf(amp, cs, Sr);
-        Si = fmaf(amp, sn, Si);
-    }
-    return Sr * Sr + Si * Si;
-}
-
-__device__ __forceinline__ float zsum_tele_t(float phi, float da, float db, const float4 *Q, const float4 *sE,
-                                             int M)
-{
-    float Er = 1.0f, Ei = 0.0f, Sr = 0.0f, Si = 0.0f;
-#pragma unroll 4
-    for (int m = 0; m < M; ++m) {
-        const float4 q = Q[m];
-        const float4 e = sE[m];
-        float sn, cs;
-        phasor_rev_ff(phi, e.x, e.y, sn, cs);
-        float lp = fmaf(q.y, da, q.w);
-        lp = fmaf(q.z, db, lp);
-        const float p = ex2_approx(lp);
-        Sr = fmaf(p, cs - Er, Sr);
-        Si = fmaf(p, sn - Ei, Si);
-        Er = cs;
-        Ei = sn;
-    }
-    return __fdividef(Sr * Sr + Si * Si, phi * phi);
-}
-
-// ---------------------------------------------------------------------------
-// Contracted small-phase series for the tabulated profile (the moment series
-// of the closed-form kernels, App. A Eq. slow_vary, at 11 moments for
-// |phi| L <= 2: the 2-D expansion costs 16 coefficients per moment).  Inside
-// the piece, log2 w_m = Ad_m + Sa_m da + Sb_m db with da = h_a x, db = h_b y the offsets
-// of F_a and F_b inside their channels, so
-//   w_m = 2^{Ad_m} e^{alpha_m x} e^{beta_m y},  alpha = Sa h_a ln 2, beta = Sb h_b ln 2,
-// and with e^{a x} = I0(a) + 2 sum Ik(a) Tk(x) in each offset
-//   nu_n(x, y) = sum_{k,l <= 3} C_nkl Tk(x) Tl(y),
-//   C_nkl = sum_m 2^{Ad_m} b_k(alpha_m) b_l(beta_m) g_n(m)
-// (truncation ~ (a/2)^4/12 per offset for |alpha|, |beta| <= 0.05).  The
-// coefficients are stored times (-1)^{floor(n/2)}/n!, as row k = float4 over l.
-// ---------------------------------------------------------------------------
-constexpr int kTabMom = kChebMomA;
-
-// Every thread calls after tab_setup_f (synced); returns whether the piece's
-// small-phase points use the contraction.  sW: [M][4] float4 scratch,
-// sG: [M][4 kZsG] moments, sC: [nc][kTabMom][4] float4, s_flag: shared int.
-__device__ bool tab_cheb_setup(const QuadParams &qp, const DevPiece &pc, int nc, const float4 *sQ, float4 *sW,
-                               float *sG, float4 *sC, float *s_amax)
-{
-    const int M = qp.n_steps;
-    if (qp.zs_g == nullptr) return false;
-    const int coff = qp.plan_ch_off[pc.plan];
-    const float ha = (float)(0.5 * qp.ch_B[coff + pc.a]), hb = (float)(0.5 * qp.ch_B[coff + pc.b]);
-    const float ln2 = 0.69314718f;
-    if (threadIdx.x == 0) *s_amax = 0.0f;
-    __syncthreads();
-    float amax = 0.0f;
-    for (int t = threadIdx.x; t < nc * M; t += blockDim.x) {
-        const float4 q = sQ[t];
-        amax = fmaxf(amax, fmaxf(fabsf(q.y * ha), fabsf(q.z * hb)) * ln2);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<unsigned *>(s_amax), __float_as_uint(amax));
-    for (int t = threadIdx.x; t < M * 4 * kZsG; t += blockDim.x) sG[t] = reinterpret_cast<const float *>(qp.zs_g)[t];
-    __syncthreads();
-    if (!(*s_amax <= kChebMaxA)) return false;
-    for (int c = 0; c < nc; ++c) {
-        const float4 *Q = sQ + c * M;
-        for (int m = threadIdx.x; m < M; m += blockDim.x) {
-            const float4 q = Q[m];
-            const float base = ex2_approx(q.x);
-            const float4 bk = bessel_b4(q.y * ha * ln2), bl = bessel_b4(q.z * hb * ln2);
-            const float bkv[4] = {bk.x, bk.y, bk.z, bk.w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const float wk = base * bkv[k];
-                sW[m * 4 + k] = make_float4(wk * bl.x, wk * bl.y, wk * bl.z, wk * bl.w);
-            }
-        }
-        __syncthreads();
-        // one coefficient (n, k, l) per thread: compensated sum over the steps
-        for (int t = threadIdx.x; t < kTabMom * 16; t += blockDim.x) {
-            const int n = t >> 4, k = (t >> 2) & 3, l = t & 3;
-            float sum = 0.0f, comp = 0.0f;
-            for (int m = 0; m < M; ++m) {
-                const float4 w = sW[m * 4 + k];
-                const float wl = l == 0 ? w.x : (l == 1 ? w.y : (l == 2 ? w.z : w.w));
-                const float y = wl * sG[m * 4 * kZsG + n] - comp;
-                const float tt = sum + y;
-                comp = (tt - sum) - y;
-                sum = tt;
-            }
-            reinterpret_cast<float *>(sC + (c * kTabMom + n) * 4 + k)[l] = sum * (float)cheb_fold(n);
-        }
-        __syncthreads();
-    }
-    return true;
-}
-
-// |S|^2 of a small-phase point of candidate ci from the contracted series
-// (6 moments serve |phi| L <= 0.2, as in cheb_point).
-__device__ __forceinline__ float tab_cheb_s2(const float4 *sC, int ci, float x, float y, float phi, float aphi,
-                                             float phi6)
-{
-    const float4 *C = sC + ci * kTabMom * 4;
-    float A, B;
-    if (aphi <= phi6) cheb2_AB<6>(C, x, y, phi, A, B);
-    else cheb2_AB<kTabMom>(C, x, y, phi, A, B);
-    return fmaf(A, A, B * B);
-}
-
-}  // namespace
-
+// As k_quad_f32 (quad_fwd.cu: one warp per tile, row sums from nodes), with the
+// step rows of the tabulated profile.  The low rows' blocks replace the 2-D
+// contraction of the small-phase moments (176 coefficients per candidate and
+// piece) that this kernel used to build.
 __global__ void __launch_bounds__(256, 4) k_quad_f32_tab(QuadParams qp)
 {
     extern __shared__ float4 smem_f4[];
     const int M = qp.n_steps, G = qp.G;
-    float4 *sZ = smem_f4;                              // [M] {z, z^2 + dz^2/12, dz, 0}
-    float4 *sE = sZ + M;                               // [M] {edge/2pi hi, lo, 0, 0}
-    float4 *sQ = sE + M;                               // [nc_max][M] {A + log2 dz, Sa, Sb, A}
-    float4 *sW = sQ + (size_t)qp.nc_max * M;           // [M][4] contraction weights of one candidate
-    float4 *sC = sW + (size_t)M * 4;                   // [nc_max][kTabMom][4] contracted coefficients
-    float *sG = reinterpret_cast<float *>(sC + (size_t)qp.nc_max * kTabMom * 4);   // [M][4 kZsG] step moments
-    RowF *rows = reinterpret_cast<RowF *>(sG + (size_t)M * 4 * kZsG);   // [G]
-    __shared__ PieceConst<float> kc;
-    __shared__ float s_d0[2];
-    __shared__ float s_amax;
-    __shared__ double scratch[32];
-    __shared__ int s_item;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float4 *zt = smem_f4;                              // [M] {edge(m+1)/2pi hi, lo, z, dz}
+    unsigned char *mine = reinterpret_cast<unsigned char *>(zt + M) + tab_warp_bytes(M) * warp;
+    TabNodes &ns = *reinterpret_cast<TabNodes *>(mine);
+    float4 *Q = reinterpret_cast<float4 *>(mine + sizeof(TabNodes));   // [kTabCand][M]
 
     for (int m = threadIdx.x; m < M; m += blockDim.x) {
-        const float4 za = qp.zs_a[m];   // {z_m, c_m, log2 dz_m, dz_m}
-        const float4 zb = qp.zs_b[m];   // {edge(m+1)/2pi hi, lo, z_m/2pi, 0}
-        sZ[m] = make_float4(za.x, za.y, za.w, 0.0f);
-        sE[m] = make_float4(zb.x, zb.y, 0.0f, 0.0f);
+        const float4 za = qp.zs_a[m], zb = qp.zs_b[m];
+        zt[m] = make_float4(zb.x, zb.y, za.x, za.w);
     }
-    const float c3 = (float)(kPi * qp.beta3);
-    const float c4 = (float)(2.0 * kPi * kPi / 3.0 * qp.beta4);
-    const float b2 = (float)qp.beta2;
-    const float m4pi2 = (float)(-4.0 * kPi * kPi);
+    __syncthreads();
     const float phi_direct = 3.14159265f / qp.dz_max;
-    const float phi_small = 0.02f / qp.L;
-    const float phi_cheb = kChebPhiLA / qp.L;
-    const float phi_c6 = kChebPhiL6 / qp.L;
-    const float invG = 1.0f / (float)G;
-    unsigned n_small = 0, n_direct = 0, n_tele = 0;
+    const float phi_small = kBlkPhiL / qp.L;
+    unsigned long long n_small = 0;
+    unsigned n_direct = 0, n_tele = 0;
 
     for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) s_item = atomicAdd(qp.counter, 1);
-        __syncthreads();
-        const int it = s_item;
+        int it = 0;
+        if (lane == 0) it = atomicAdd(qp.counter, 1);
+        it = __shfl_sync(0xffffffffu, it, 0);
         if (it >= qp.n_items) break;
         const DevItem item = qp.items[it];
+        const int part = item.part & 0xffff, parts = item.part >> 16;
         double acc = 0.0;
         for (int k = item.piece0; k < item.piece1; ++k) {
-            const DevPiece pc = qp.pieces[dbg_clamp(k, qp.n_pieces, kDbgPiece, qp.dbg)];
-            piece_rows<RowF>(pc, G, qp.eps_v1, rows);
-            piece_consts<float>(qp, pc, item.prof, 0.0f, qp.pd_f, kc);
-            if (threadIdx.x == 0) {
-                const int coff = qp.plan_ch_off[pc.plan];
-                const double fi = qp.ch_frel[coff + pc.cut];
-                s_d0[0] = (float)(qp.ch_frel[coff + pc.a] - fi);
-                s_d0[1] = (float)(qp.ch_frel[coff + pc.b] - fi);
-            }
-            __syncthreads();
-            tab_setup_f(qp, pc, item.prof, kc.nc, sQ);
-            __syncthreads();
-            const bool cheb = tab_cheb_setup(qp, pc, kc.nc, sQ, sW, sG, sC, &s_amax);
-            const float phi_lim = cheb ? phi_cheb : phi_small;   // upper |phi| of the small-phase forms
-            float inv_ha = 0.0f, inv_hb = 0.0f;
-            {
-                const int coff = qp.plan_ch_off[pc.plan];
-                inv_ha = (float)(2.0 / qp.ch_B[coff + pc.a]);
-                inv_hb = (float)(2.0 / qp.ch_B[coff + pc.b]);
-            }
-            const float fi = kc.fi, s1g = kc.s1, s2g = kc.s2;
-            const float da0 = s_d0[0], db0 = s_d0[1];
-            const float three_fi2 = 3.0f * fi * fi;
+            const DevPiece &pc = qp.pieces[dbg_clamp(k, qp.n_pieces, kDbgPiece, qp.dbg)];
+            __syncwarp();
+            const bool sw = node_geo(qp, pc, item.prof, 0.0f, qp.pd_f, 0.0f, ns.geo);
+            const TabPiece tp = tab_piece(qp, pc, item.prof, sw);
+            const int coff = qp.plan_ch_off[pc.plan];
+            __syncwarp();
+            PieceGeo &g = ns.geo;
             float sum = 0.0f, comp = 0.0f;
-            const int npts = G * G;
-            for (int q = threadIdx.x + (item.part & 0xffff) * blockDim.x; q < npts; q += (item.part >> 16) * blockDim.x) {
-                const int r = (int)(((float)q + 0.5f) * invG);
-                const int j = q - r * G;
-                const RowF rw = rows[dbg_clamp(r, G, kDbgRow, qp.dbg)];
-                if (rw.w == 0.0f) continue;
-                const float d = ((float)j + 0.5f - 0.5f * (float)G) * rw.du2;
-                const float e = expf(d);
-                const float f1 = s1g * (rw.xc * e);
-                const float f2 = s2g * (rw.yc * __frcp_rn(e));
-                const float u = f1 + f2;                    // F_c - f_i
-                int ci = -1;
-                for (int c = 0; c < kc.nc; ++c) {
-                    if (u >= kc.lo[c] && u < kc.hi[c]) { ci = c; break; }
+            for (int ca = 0; ca < g.nc; ca += kTabCand) {
+                const int cb = min(g.nc, ca + kTabCand);
+                float tilt = 0.0f;
+                for (int c = ca; c < cb; ++c) {
+                    const double fc = qp.ch_frel[coff + pc.c_lo + c];
+                    for (int m = lane; m < M; m += 32) {
+                        const float4 r = tab_row(tp, pc.c_lo + c, fc, m, M);
+                        Q[(c - ca) * M + m] = r;
+                        tilt = fmaxf(tilt, fmaxf(fabsf(r.y), fabsf(r.z)));
+                    }
                 }
-                if (ci < 0) continue;                       // F_c in a gap
-                const float W = kc.wab * kc.pd[ci];
-                const float da = f1 - da0, db = f2 - db0;   // F_a - f_a, F_b - f_b
-                const float4 *Q = sQ + ci * M;
-                // Eq. phi
-                const float br = b2 + c3 * (u + 2.0f * fi) +
-                                 c4 * (f1 * f1 + 1.5f * f1 * f2 + 3.0f * fi * u + f2 * f2 + three_fi2);
-                const float phi = m4pi2 * f1 * f2 * br;
-                const float aphi = fabsf(phi);
-                float S2;
-                if (aphi <= phi_lim) {
-                    S2 = cheb ? tab_cheb_s2(sC, ci, da * inv_ha, db * inv_hb, phi, aphi, phi_c6) : zsum_small_t(phi, da, db, Q, sZ, M);
-                    ++n_small;
-                } else if (aphi <= phi_direct) {
-                    S2 = zsum_direct_t(phi, da, db, Q, sZ, M);
-                    ++n_direct;
-                } else {
-                    S2 = zsum_tele_t(phi, da, db, Q, sE, M);
-                    ++n_tele;
-                }
-                const float y = rw.w * W * S2 * array_factor_f(phi, qp) - comp;
-                const float t = sum + y;
-                comp = (t - sum) - y;
-                sum = t;
+                // the largest slope of ln p bounds its swing along a row
+                tilt = 0.69314718f * __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(tilt)));
+                if (lane == 0) g.tilt = tilt;
+                __syncwarp();
+                int small;
+                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int nq) {
+                    for (int q = lane + 32 * part; q < nq; q += 32 * parts) {
+                        Node nd;
+                        if (!node_get(ns, qp.gauss, q, nd)) continue;
+                        const int ci = dbg_clamp(nd.ci, g.nc, kDbgCand, qp.dbg);
+                        const float aphi = fabsf(nd.phi);
+                        const float dl = tp.ol + nd.x, dd = tp.od + nd.y;
+                        const float4 *e = Q + (ci - ca) * M;
+                        const bool direct = aphi <= phi_direct;
+                        const float S2 = direct ? zsum_direct_nt(nd.phi, dl, dd, zt, e, M)
+                                                : zsum_tele_nt(nd.phi, nd.phi_lo, dl, dd, zt, e, M);
+                        n_small += aphi <= phi_small ? nd.N : 0;
+                        n_direct += aphi > phi_small && direct ? nd.N : 0;
+                        n_tele += direct ? 0 : nd.N;
+                        const float y = nd.wq * g.pd[ci] * S2 * array_factor_f(nd.phi, qp, nd.phi_lo) - comp;
+                        const float t = sum + y;
+                        comp = (t - sum) - y;
+                        sum = t;
+                    }
+                });
+                n_small += lane == 0 && part == 0 ? small : 0;
             }
-            acc += (double)kc.mult * ((double)sum - (double)comp);
-            __syncthreads();
+            acc += (double)(g.mult * g.wab) * ((double)sum - (double)comp);
         }
-        const double tot = block_sum_d(acc, scratch);
-        if (threadIdx.x == 0) qp.partial[it] = tot;
+        const double tot = warp_sum_d(acc);
+        if (lane == 0) qp.partial[it] = tot;
     }
     if (qp.path_count) {
         unsigned long long c0 = n_small, c1 = n_direct, c2 = n_tele;
@@ -755,7 +562,7 @@ __global__ void __launch_bounds__(256, 4) k_quad_f32_tab(QuadParams qp)
             c1 += __shfl_xor_sync(0xffffffffu, c1, o);
             c2 += __shfl_xor_sync(0xffffffffu, c2, o);
         }
-        if ((threadIdx.x & 31) == 0) {
+        if (lane == 0) {
             atomicAdd(&qp.path_count[0], c0);
             atomicAdd(&qp.path_count[1], c1);
             atomicAdd(&qp.path_count[2], c2);
@@ -858,32 +665,33 @@ __global__ void __launch_bounds__(256) k_quad_f64_tab(QuadParams qp)
     }
 }
 
-size_t quad_tab_smem_bytes(int precision, int n_steps, int G, int nc_max)
+size_t quad_tab_limit_bytes(int precision, int n_steps, int G, int nc_max)
 {
     if (precision == 0)
-        return (size_t)n_steps * (2 + nc_max + 4) * sizeof(float4) + (size_t)nc_max * kTabMom * 4 * sizeof(float4) +
-               (size_t)n_steps * 4 * kZsG * sizeof(float) + (size_t)G * sizeof(RowF);
+        return (size_t)n_steps * (6 + nc_max) * 16 + (size_t)nc_max * 704 + (size_t)n_steps * 80 + (size_t)G * 16;
     return (size_t)n_steps * (1 + 2 * nc_max) * sizeof(double2) + (size_t)G * sizeof(RowD);
 }
 
-int quad_tab_blocks_per_sm(int precision, int n_steps, int G, int nc_max, int block)
+cudaError_t launch_quad_tab(const QuadParams &qp, int precision, int num_sms, int block, cudaStream_t st)
 {
-    int nb = 0;
-    const size_t smem = quad_tab_smem_bytes(precision, n_steps, G, nc_max);
-    void *fn = precision == 0 ? (void *)k_quad_f32_tab : (void *)k_quad_f64_tab;
-    cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, block, smem);
-    return nb > 0 ? nb : 1;
-}
-
-cudaError_t launch_quad_tab(const QuadParams &qp, int precision, int grid, int block, cudaStream_t st)
-{
-    const size_t smem = quad_tab_smem_bytes(precision, qp.n_steps, qp.G, qp.nc_max);
-    void *fn = precision == 0 ? (void *)k_quad_f32_tab : (void *)k_quad_f64_tab;
+    int nb = 0, tiles = qp.n_items;
+    size_t smem = quad_tab_limit_bytes(1, qp.n_steps, qp.G, qp.nc_max);
+    const void *fn = (const void *)k_quad_f64_tab;
+    if (precision == 0) {
+        // as launch_quad: any number of warps to a block
+        const auto bytes = [&](int b) { return sizeof(float4) * (size_t)qp.n_steps + tab_warp_bytes(qp.n_steps) * (b / 32); };
+        fn = (const void *)k_quad_f32_tab;
+        if (qp.n_items < num_sms * (block / 32)) block = 32;
+        while (block > 32 && bytes(block) > 200 * 1024) block -= 32;
+        smem = bytes(block);
+        tiles = (qp.n_items + block / 32 - 1) / (block / 32);
+    }
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    QuadParams q = qp;
-    void *args[] = {&q};
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, block, smem);
+    if (e != cudaSuccess) return e;
+    const int grid = std::max(1, std::min(tiles, num_sms * std::max(1, nb)));
+    void *args[] = {(void *)&qp};
     return cudaLaunchKernel(fn, dim3(grid), dim3(block), args, smem, st);
 }
 
