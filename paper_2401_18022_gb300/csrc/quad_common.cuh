@@ -16,22 +16,16 @@ __device__ __forceinline__ float ex2_approx(float x)
     return y;
 }
 
-// Nearest integer of t (round to nearest even), two ways:
-//  * round_magic: two adds on the FMA pipe, exact for |t| < 2^22;
-//  * round_nearest: one FRND, exact for every FP32 value, issued to the
-//    XU pipe that also runs the MUFU (sin, cos, ex2) instructions.
-// The forward kernels (3 MUFU per step, XU ~40 % busy) measured faster with
-// round_magic (FRND raised XU to ~49 % and added mio_throttle stalls); the
-// adjoint walks (XU ~25 % busy, issue-bound) with round_nearest.  Either way
-// t - round(t) is exact (Sterbenz).
-__device__ __forceinline__ float round_magic(float t)
+// Fraction of a phase a b in revolutions, in [-1/2, 1/2]: the integer nearest
+// to the exact product comes out of one FMA against 1.5 2^23 (|a b| < 2^22) and
+// the fraction out of a second one, rounded once.  Three instructions on the FMA
+// pipe; rounding the product first, with its residual as a second float, took
+// five, and FRND would go to the XU pipe, which the sin, cos and ex2 of a z-step
+// keep busy for 20 cycles per warp and step.
+__device__ __forceinline__ float rev_fraction(float a, float b)
 {
-    return __fadd_rn(__fadd_rn(t, 12582912.0f), -12582912.0f);
-}
-
-__device__ __forceinline__ float round_nearest(float t)
-{
-    return rintf(t);
+    const float k = __fadd_rn(__fmaf_rn(-a, b, 12582912.0f), -12582912.0f);
+    return __fmaf_rn(a, b, k);
 }
 
 __device__ __forceinline__ double warp_sum_d(double v)
@@ -160,26 +154,17 @@ __device__ __forceinline__ void piece_consts(const QuadParams &qp, const DevPiec
     }
 }
 
-// sin and cos of 2 pi t for |t| < 2^22 revolutions (Xu: round with FRND)
-template <bool Xu = false>
-__device__ __forceinline__ void sincos_rev(float t, float &sn, float &cs)
+// sin and cos of 2 pi a b for |a b| < 2^22 revolutions
+__device__ __forceinline__ void sincos_rev(float a, float b, float &sn, float &cs)
 {
-    const float fr = __fadd_rn(t, -(Xu ? round_nearest(t) : round_magic(t)));
-    __sincosf(fr * 6.283185307179586f, &sn, &cs);
+    __sincosf(rev_fraction(a, b) * 6.283185307179586f, &sn, &cs);
 }
 
-// e^{j phi z}: the phase phi (hi + lo) in revolutions as an error-free
-// float-float product, reduced to [-1/2, 1/2] (Xu: round with FRND); phi_lo
-// is the low part of a float-float phi
-template <bool Xu = false>
+// e^{j phi z}: the phase (phi + phi_lo)(hi + lo) in revolutions, |.| < 2^22
 __device__ __forceinline__ void phasor_rev_ff(float phi, float hi, float lo, float &sn, float &cs,
                                               float phi_lo = 0.0f)
 {
-    const float th = phi * hi;
-    float tl = fmaf(phi, hi, -th);
-    tl = fmaf(phi, lo, tl);
-    tl = fmaf(phi_lo, hi, tl);
-    const float fr = __fadd_rn(th, -(Xu ? round_nearest(th) : round_magic(th))) + tl;
+    const float fr = fmaf(phi_lo, hi, fmaf(phi, lo, rev_fraction(phi, hi)));
     __sincosf(fr * 6.283185307179586f, &sn, &cs);
 }
 

@@ -196,7 +196,7 @@ cudaError_t gauss_array(void **out) { return cudaGetSymbolAddress(out, g_isrs_ga
 // ---------------------------------------------------------------------------
 // k_quad_f32: persistent FP32 quadrature.
 // ---------------------------------------------------------------------------
-constexpr int kFwdSlots = 320;       // node slots of a chunk
+constexpr int kFwdSlots = 256;       // node slots of a chunk
 constexpr int kFwdCand = 3;          // F_c candidates swept together (most pieces have two)
 using FwdNodes = WarpNodes<kFwdSlots>;
 

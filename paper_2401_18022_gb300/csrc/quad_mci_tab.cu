@@ -80,7 +80,7 @@ __device__ __forceinline__ float zsum_direct_mt(float phi, float da, float db, f
         const float4 q = Q[m];
         const float4 a = sA[m];
         float sn, cs;
-        sincos_rev(phir * a.x, sn, cs);
+        sincos_rev(phir, a.x, sn, cs);
         const float x = hphi * a.w;
         const float x2 = x * x;
         float sc = fmaf(x2, -2.5052108e-8f, 2.7557319e-6f);   // -1/11!, 1/9!

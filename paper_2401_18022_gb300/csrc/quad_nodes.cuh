@@ -40,41 +40,43 @@
 
 namespace isrs {
 
-// Node counts of the rules: 4..8, 10, 12 .. 20, 24, 28, 32, 40, 48.  One table
+// Node counts of the rules: 2..8, 10, 12 .. 20, 24, 28, 32, 40, 48.  One table
 // of {t, weight} per run length N <= kGaussMaxN and node count; node k lies at
 // column centre + t N / 2.
 constexpr int kGaussMaxN = 256;
 constexpr int kGaussMaxNodes = 48;
-constexpr int kGaussMenu = 16;
-constexpr int kGaussPerN = 292;                        // nodes of all rules of one N
+constexpr int kGaussMenu = 18;
+constexpr int kGaussPerN = 297;                        // nodes of all rules of one N
 constexpr int kGaussEntries = kGaussMaxN * kGaussPerN;
-constexpr int kNodeMin = 4;                            // slots a run takes at least
+constexpr int kNodeMin = 2;                            // slots a run takes at least
 
 __host__ __device__ constexpr int gauss_nodes(int k)
 {
-    return k <= 4 ? 4 + k : k <= 10 ? 2 * k : k <= 13 ? 20 + 4 * (k - 10) : 32 + 8 * (k - 13);
+    return k <= 6 ? 2 + k : k <= 12 ? 2 * (k - 2) : k <= 15 ? 20 + 4 * (k - 12) : 32 + 8 * (k - 15);
 }
 
 __host__ __device__ constexpr int gauss_offset(int k)
 {
-    return k <= 4 ? 4 * k + k * (k - 1) / 2 : k <= 10 ? k * (k - 1) + 10
-         : k <= 13 ? 120 + 24 * (k - 11) + 2 * (k - 11) * (k - 12) : 204 + 40 * (k - 14);
+    return k <= 6 ? 2 * k + k * (k - 1) / 2 : k <= 12 ? k * (k - 5) + 21
+         : k <= 15 ? 125 + 24 * (k - 13) + 2 * (k - 13) * (k - 14) : 209 + 40 * (k - 16);
 }
 
 // smallest rule with at least `need` nodes (need <= kGaussMaxNodes)
 __host__ __device__ inline int gauss_pick(int need)
 {
-    return need <= 4 ? 0 : need <= 8 ? need - 4 : need <= 20 ? 4 + (need - 7) / 2
-         : need <= 32 ? 10 + (need - 17) / 4 : 13 + (need - 25) / 8;
+    return need <= 2 ? 0 : need <= 8 ? need - 2 : need <= 20 ? 6 + (need - 7) / 2
+         : need <= 32 ? 12 + (need - 17) / 4 : 15 + (need - 25) / 8;
 }
 
-// Nodes that give a run's sum to < 1e-8 of itself: A bounds the phase swing of
-// |S|^2 over half the run, D its half-length in upsilon2 (the map from column
-// to u is exp-like).  2 n = A + 7.2 + 2.6 sqrt(A) + 1.4 D covers what the runs
-// of the 589-ch, O-band and multi-span plans need (A up to 670, D up to 11.5).
+// Nodes that give a run's sum: A bounds the phase swing of |S|^2 over half the
+// run, D its half-length in upsilon2 (the map from column to u is exp-like).
+// Measured need over the runs of the 589-ch, O-band and 10-span plans (A up to
+// 670, D up to 11.5): to 3e-8 of the run's sum, or of the piece's where the run
+// is a fast row (|S|^2 falls as 1/phi^2, so a row at |phi| L = 6 t weighs 1/t),
+// 2 n - A stays below 4 at A < 0.05, 8 at 0.3, 9.3 at 3, 12.5 at 30, 13.7 at 100.
 __host__ __device__ inline int gauss_need(float A, float D)
 {
-    const float two_n = A + 7.2f + 2.6f * sqrtf(A) + 1.4f * D;
+    const float two_n = A + 4.0f + 4.2f * A / (A + 0.35f) + 0.6f * sqrtf(A) + 1.4f * D;
     return two_n < 8192.0f ? (int)ceilf(0.5f * two_n) : 4096;
 }
 
@@ -305,20 +307,23 @@ __device__ __forceinline__ void row_runs(const PieceGeo &g, const NodeRow &o, in
     }
 }
 
-// Bound of |du/dt| per column of a run's half-length, t in [-1, 1], from the
-// row's largest |f1|, |f2|, and the phase swing it brings.
+// Bound of |du/dt| per column of a run's half-length, t in [-1, 1], and the
+// phase swing it brings: du/dupsilon2 = f1 - f2 is monotone along the row, so it
+// is largest at one of the ends.
 __device__ __forceinline__ float row_swing(const PieceGeo &g, const NodeRow &o, int G)
 {
     float p1, p2;
     row_slopes(g, o, p1, p2);
-    const float e = expf(0.5f * (float)G * o.du2) * (o.xc + o.yc) * 0.5f * o.du2;
-    return e * (g.band * (fabsf(p1) + 2.0f * fabsf(p2) * e * (float)G) + 2.0f * g.tilt);
+    const float E = expf(0.5f * (float)G * o.du2), Ei = __fdividef(1.0f, E);
+    const float x = g.s1 * o.xc, y = g.s2 * o.yc;
+    const float e = fmaxf(fabsf(x * E - y * Ei), fabsf(x * Ei - y * E)) * 0.5f * o.du2;
+    return e * (g.band * (fabsf(p1) + 2.0f * fabsf(p2) * e * (float)G)) + (fabsf(x) + fabsf(y)) * E * o.du2 * g.tilt;
 }
 
 // A run cut into the parts one rule each covers: f(j0, N, n), n = N where the
 // columns themselves are no more than the rule needs.  n <= kGaussMaxNodes: a
 // part of a run that needs n > 48 nodes has (A + 1.4 D) / parts <= 48 and so
-// needs at most 37, and a part of <= 48 columns takes at most its columns.
+// needs at most 31, and a part of <= 48 columns takes at most its columns.
 template <typename F>
 __device__ __forceinline__ void run_parts(const PieceGeo &g, const NodeRow &o, int G, int j0, int N, const F &f)
 {
@@ -477,7 +482,7 @@ __device__ __noinline__ int node_emit(WarpNodes<Cap> &ns, int G, int row, int ca
             const int take = max(n, kNodeMin);
             if (c0 >= 0) {
                 const bool here = off >= c0 && off < c0 + span;
-                const int s = off - c0, id = s >> 2;      // runs start >= kNodeMin slots apart
+                const int s = off - c0, id = s / kNodeMin;  // runs start >= kNodeMin slots apart
                 if (here) {
                     NodeRun r;
                     r.jc = (float)j + 0.5f * (float)(Ns - G);

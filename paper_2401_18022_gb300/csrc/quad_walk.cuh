@@ -52,7 +52,7 @@ __device__ __forceinline__ float walk_direct(const float4 *o0s, float wq, float 
     for (int k = 0; k < K; ++k) {
         const float4 o = o0s[k * 16];
         float sn, cs;
-        sincos_rev<true>(phr * o.z, sn, cs);
+        sincos_rev(phr, o.z, sn, cs);
         float lp = fmaf(o.y, fc, o.x);
         lp = fmaf(-at, o.z, lp);
         const float amp = ex2_approx(lp) * sinc_poly(hph * o.w);
@@ -88,8 +88,8 @@ __device__ __forceinline__ float walk_tele(const float4 *o0s, const float4 *o1s,
     for (int k = 0; k < K; ++k) {
         const float4 b = o1s[k * 16];
         float sn, cs;
-        if (Wide) phasor_rev_ff_wide<true>(ph, b.x, b.y, sn, cs);
-        else phasor_rev_ff<true>(ph, b.x, b.y, sn, cs);
+        if (Wide) phasor_rev_ff_wide(ph, b.x, b.y, sn, cs);
+        else phasor_rev_ff(ph, b.x, b.y, sn, cs);
         float lp;
         if constexpr (Folded) {
             lp = fmaf(b.w, fc, b.z);
@@ -193,7 +193,7 @@ __device__ __forceinline__ float walk_direct_n(const float4 *zt, const float2 *e
         const float4 o = zt[k * 16];
         const float2 e = ek[k * 16];
         float sn, cs;
-        sincos_rev<true>(phr * o.z, sn, cs);
+        sincos_rev(phr, o.z, sn, cs);
         const float amp = ex2_approx(fmaf(e.y, dF, e.x)) * (sinc_poly(hph * o.w) * o.w);
         tr[k] = amp * cs;
         ti[k] = amp * sn;
@@ -224,7 +224,7 @@ __device__ __forceinline__ float walk_tele_n(const float4 *zt, const float2 *ek,
         const float4 b = zt[k * 16];
         const float2 e = ek[k * 16];
         float sn, cs;
-        phasor_rev_ff<true>(ph, b.x, b.y, sn, cs, ph_lo);
+        phasor_rev_ff(ph, b.x, b.y, sn, cs, ph_lo);
         const float pm = ex2_approx(fmaf(e.y, dF, e.x));
         if (k == 0) {
             p0 = pm;

@@ -60,7 +60,7 @@ __device__ __forceinline__ float zsum_direct_f(float phi, float Fc, float at, co
     for (int m = 0; m < M; ++m) {
         const float4 a = sR[m];
         float sn, cs;
-        sincos_rev(phir * a.z, sn, cs);
+        sincos_rev(phir, a.z, sn, cs);
         const float x = hphi * a.w;
         const float x2 = x * x;
         float sc = fmaf(x2, -2.5052108e-8f, 2.7557319e-6f);   // -1/11!, 1/9!
@@ -112,7 +112,7 @@ __device__ __forceinline__ float zsum_direct_n(float phi, float dF, const float4
         const float4 a = zt[m];
         const float2 e = ek[m];
         float sn, cs;
-        sincos_rev(phir * a.z, sn, cs);
+        sincos_rev(phir, a.z, sn, cs);
         const float x = hphi * a.w;
         const float x2 = x * x;
         float sc = fmaf(x2, -2.5052108e-8f, 2.7557319e-6f);   // -1/11!, 1/9!
@@ -160,7 +160,7 @@ __device__ __forceinline__ float zsum_direct_nt(float phi, float dl, float dd, c
         const float4 a = zt[m];
         const float4 e = q[m];
         float sn, cs;
-        sincos_rev(phir * a.z, sn, cs);
+        sincos_rev(phir, a.z, sn, cs);
         const float x = hphi * a.w;
         const float x2 = x * x;
         float sc = fmaf(x2, -2.5052108e-8f, 2.7557319e-6f);   // -1/11!, 1/9!
@@ -194,19 +194,13 @@ __device__ __forceinline__ float zsum_tele_nt(float phi, float phi_lo, float dl,
     return __fdividef(Sr * Sr + Si * Si, phi * phi);
 }
 
-// As phasor_rev_ff, for phases far beyond 2^22 revolutions (the MCI cells):
-// once |phi z / 2pi| >= 2^22 the first magic-number rounding leaves an
-// integer (or half-integer) on top of the fraction, and FRND's exact
-// th - rint(th) can leave tl beyond one revolution; a second rounding of the
-// sum removes either.
-template <bool Xu = false>
+// As phasor_rev_ff, for phases far beyond 2^22 revolutions (the MCI cells, up
+// to 2^29): there the first rounding is to a multiple of 2 or more and leaves a
+// few revolutions; a second rounding removes them.
 __device__ __forceinline__ void phasor_rev_ff_wide(float phi, float hi, float lo, float &sn, float &cs)
 {
-    const float th = phi * hi;
-    float tl = fmaf(phi, hi, -th);
-    tl = fmaf(phi, lo, tl);
-    float fr = __fadd_rn(th, -(Xu ? round_nearest(th) : round_magic(th))) + tl;
-    fr = __fadd_rn(fr, -(Xu ? round_nearest(fr) : round_magic(fr)));
+    float fr = fmaf(phi, lo, rev_fraction(phi, hi));
+    fr = __fadd_rn(fr, -__fadd_rn(__fadd_rn(fr, 12582912.0f), -12582912.0f));
     __sincosf(fr * 6.283185307179586f, &sn, &cs);
 }
 

@@ -459,7 +459,7 @@ cudaError_t launch_raman_adj(const RamanAdjParams &ap, cudaStream_t st)
 // ---------------------------------------------------------------------------
 // Quadratures with the tabulated profile.
 // ---------------------------------------------------------------------------
-constexpr int kTabSlots = 224;       // node slots of a chunk
+constexpr int kTabSlots = 192;       // node slots of a chunk
 constexpr int kTabCand = 2;          // F_c candidates swept together (most pieces have two)
 using TabNodes = WarpNodes<kTabSlots>;
 

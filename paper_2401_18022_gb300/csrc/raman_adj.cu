@@ -65,7 +65,7 @@ __device__ __forceinline__ float walk_direct_t(const float4 *zt, const float4 *q
         const float4 e = q[k * 16];
         const float4 z = zt[k * 16];
         float sn, cs;
-        sincos_rev<true>(phr * z.z, sn, cs);
+        sincos_rev(phr, z.z, sn, cs);
         const float amp = ex2_approx(fmaf(e.z, dd, fmaf(e.y, dl, e.x))) * (sinc_poly(hph * z.w) * z.w);
         tr[k] = amp * cs;
         ti[k] = amp * sn;
@@ -97,7 +97,7 @@ __device__ __forceinline__ float walk_tele_t(const float4 *zt, const float4 *q, 
         const float4 e = q[k * 16];
         const float4 z = zt[k * 16];
         float sn, cs;
-        phasor_rev_ff<true>(ph, z.x, z.y, sn, cs, ph_lo);
+        phasor_rev_ff(ph, z.x, z.y, sn, cs, ph_lo);
         const float pm = ex2_approx(fmaf(e.z, dd, fmaf(e.y, dl, e.x)));
         if (k == 0) {
             p0 = pm;
