@@ -903,7 +903,7 @@ RamanParams raman_params(isrs_handle h, const isrs_fibre *fb, Geom *g, bool keep
     rp.photon = fb->raman_photon;
     rp.ab = (double2 *)h->ab.p;
     rp.lnrho_L = (double *)h->lnrho_L.p;
-    rp.y_nodes = keep_nodes ? (double *)h->ode_y.p : nullptr;
+    rp.stage_P = keep_nodes ? (double *)h->ode_y.p : nullptr;
     return rp;
 }
 
@@ -1018,7 +1018,7 @@ isrs_status run_forward(isrs_handle h, const isrs_fibre *fb, Geom *g, int precis
             // the Raman ODE overwrites ln rho(L) and fills the {a, b} tables
             if ((s = ensure(h, h->ab, sizeof(double2) * (size_t)g->total_prof_ch * M)) != ISRS_OK) return s;
             if (keep_nodes &&
-                (s = ensure(h, h->ode_y, sizeof(double) * (size_t)(g->n_rk + 1) * g->plan_n[0])) != ISRS_OK)
+                (s = ensure(h, h->ode_y, sizeof(double) * 4 * (size_t)g->n_rk * g->plan_n[0])) != ISRS_OK)
                 return s;
             CK(launch_raman(raman_params(h, fb, g, keep_nodes), g->n_prof, g->max_plan_n, st));
         }
@@ -1370,7 +1370,6 @@ isrs_status run_grad_tab_bwd(isrs_handle h, const isrs_fibre *fb, Geom *g, const
     rap.r = raman_params(h, fb, g, true);
     rap.n = n;
     rap.n_rk = g->n_rk;
-    rap.y_nodes = (const double *)h->ode_y.p;
     rap.gAB = (const double2 *)h->gAB.p;
     rap.gAt = (double *)h->gAt.p;
     rap.aase = cp.aase;

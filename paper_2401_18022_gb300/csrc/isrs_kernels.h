@@ -106,18 +106,17 @@ struct RamanParams {
     int photon;
     double2 *ab;                // out: (prof_ch_off[p] + c) * n_steps + m -> {a, b}
     double *lnrho_L;            // out: prof_ch_off[p] + c
-    double *y_nodes;            // out (nullable, profile 0 only): state before every RK4 step and at L
+    double *stage_P;            // out (nullable, profile 0 only): [n_rk x 4 x n] powers e^y of every RK4 stage
 };
 
 // Discrete adjoint of the Raman ODE and of the profile tables (single
 // profile): from dT/d{a, b} (per channel and step) and dT/d ln rho(L) to
-// dT/dP through the RK4 steps (states of k_raman_ode's y_nodes), then the
+// dT/dP through the RK4 steps (r.stage_P of k_raman_ode), then the
 // total gradient with the PSD and SNR-numerator terms.
 struct RamanAdjParams {
     RamanParams r;              // the forward's tables (profile 0)
     int n;                      // channels
     int n_rk;                   // RK4 steps
-    const double *y_nodes;      // [(n_rk + 1) x n]
     const double2 *gAB;         // [n x n_steps] dT/da, dT/db
     double *gAt;                // [n x n_steps] scratch: dT/da with the slope stencil folded in
     const double *aase;         // [n] dT/d ln G_i (G = 1/rho(L))
@@ -159,8 +158,6 @@ cudaError_t launch_tab_gather(const TabGatherParams &gp, cudaStream_t st);
 cudaError_t launch_adjoint_tab(const AdjTabParams &ap, int num_sms, int block, cudaStream_t st);
 cudaError_t launch_ybar(const ChainParams &cp, cudaStream_t st);
 
-size_t raman_smem_bytes(int n_ch);
-size_t raman_adj_smem_bytes(int n_ch);
 cudaError_t launch_raman_adj(const RamanAdjParams &ap, cudaStream_t st);
 cudaError_t launch_raman(const RamanParams &rp, int n_prof, int max_n, cudaStream_t st);
 // Gauss rules of the row sums: the module's array on the current device, and its fill

@@ -12,11 +12,11 @@
 // sorted plan, and the sum splits into prefix sums over the window:
 //   above i:  sum (fr_k - fr_i) P_k = S(fr P) - fr_i S(P)
 //   below i:  sum (fr_k - fr_i) (f_i / f_k) P_k = f_i (S(fr P / f) - fr_i S(P / f))
-// (fr = f - f_ref), i.e. four block-wide scans per right-hand side instead of
-// an n x n sum.  A slot with P = 0 pumps nothing and follows the gain of a
+// (fr = f - f_ref), i.e. four prefix sums per right-hand side instead of an
+// n x n sum.  A slot with P = 0 pumps nothing and follows the gain of a
 // zero-power probe (its y starts at 0).
 //
-// k_raman_ode   one block per profile: classical RK4 through the nodes
+// k_raman_ode   one cluster per profile: classical RK4 through the nodes
 //               e_m -> z_m -> e_{m+1} of every z-step, each half in
 //               half_steps[m] equal steps; tables
 //                 a_c(m) = y_c(z_m) - y_c(0),  ln rho_c(L) = y_c(L) - y_c(0),
@@ -34,6 +34,7 @@
 //               b_c (f_a + f_b - f_i - f_c)) / 2, Sa = (b_a + b_c)/2,
 //               Sb = (b_b + b_c)/2, tabulated per piece and candidate, so a
 //               grid point costs the same two FMAs per step as the closed form.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -47,208 +48,200 @@
 
 namespace isrs {
 
+namespace cg = cooperative_groups;
+
 namespace {
 
-constexpr int kOdeThreads = 1024;
+// The ODE kernels run one thread-block cluster per profile, one lane per
+// channel.  A right-hand side is a chain of short FP64 steps (exp, prefix sums,
+// combination), ~1,800 of them one after another over 80 km.  On one SM the
+// FP64 pipe (2 lanes a clock) and the block barriers of a 1,024-thread scan took
+// 18 us each on the 557-channel plan (12.5 us on 41 channels); two warps to an
+// SM and one cluster barrier a stage bring that down (DESIGN table).
+constexpr int kOdeWarps = 2;             // warps of a block at most 32 warps of channels
+constexpr int kOdeMaxCluster = 16;
+constexpr int kOdeMaxWarps = kMaxRamanCh / 32;
 
-// Exclusive prefix sums of four arrays v0..v3 [0, n) into x0..x3 [0, n]
-// (x[k] = sum_{j<k} v[j]), all in shared memory.  Each thread scans a run of
-// ceil(n / blockDim) consecutive entries; run totals are scanned by warp
-// shuffles.  Called by every thread of the block.
-__device__ void scan4(const double *v0, const double *v1, const double *v2, const double *v3, double *x0,
-                      double *x1, double *x2, double *x3, int n, double *wsum /* [4 * 32] */)
-{
-    const int per = (n + blockDim.x - 1) / blockDim.x;
-    const int b = threadIdx.x * per, e = min(n, b + per);
-    double t0 = 0.0, t1 = 0.0, t2 = 0.0, t3 = 0.0;
-    for (int k = b; k < e; ++k) {
-        t0 += v0[k];
-        t1 += v1[k];
-        t2 += v2[k];
-        t3 += v3[k];
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double i0 = t0, i1 = t1, i2 = t2, i3 = t3;            // inclusive within the warp
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const double u0 = __shfl_up_sync(0xffffffffu, i0, o), u1 = __shfl_up_sync(0xffffffffu, i1, o);
-        const double u2 = __shfl_up_sync(0xffffffffu, i2, o), u3 = __shfl_up_sync(0xffffffffu, i3, o);
-        if (lane >= o) {
-            i0 += u0;
-            i1 += u1;
-            i2 += u2;
-            i3 += u3;
-        }
-    }
-    if (lane == 31) {
-        wsum[wid] = i0;
-        wsum[32 + wid] = i1;
-        wsum[64 + wid] = i2;
-        wsum[96 + wid] = i3;
-    }
-    __syncthreads();
-    if (wid == 0) {
-        double w0 = lane < nw ? wsum[lane] : 0.0, w1 = lane < nw ? wsum[32 + lane] : 0.0;
-        double w2 = lane < nw ? wsum[64 + lane] : 0.0, w3 = lane < nw ? wsum[96 + lane] : 0.0;
-        const double s0 = w0, s1 = w1, s2 = w2, s3 = w3;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const double u0 = __shfl_up_sync(0xffffffffu, w0, o), u1 = __shfl_up_sync(0xffffffffu, w1, o);
-            const double u2 = __shfl_up_sync(0xffffffffu, w2, o), u3 = __shfl_up_sync(0xffffffffu, w3, o);
-            if (lane >= o) {
-                w0 += u0;
-                w1 += u1;
-                w2 += u2;
-                w3 += u3;
-            }
-        }
-        if (lane < nw) {                                  // exclusive warp offsets
-            wsum[lane] = w0 - s0;
-            wsum[32 + lane] = w1 - s1;
-            wsum[64 + lane] = w2 - s2;
-            wsum[96 + lane] = w3 - s3;
-        }
-    }
-    __syncthreads();
-    double r0 = wsum[wid] + i0 - t0, r1 = wsum[32 + wid] + i1 - t1;
-    double r2 = wsum[64 + wid] + i2 - t2, r3 = wsum[96 + wid] + i3 - t3;
-    for (int k = b; k < e; ++k) {
-        x0[k] = r0;
-        x1[k] = r1;
-        x2[k] = r2;
-        x3[k] = r3;
-        r0 += v0[k];
-        r1 += v1[k];
-        r2 += v2[k];
-        r3 += v3[k];
-    }
-    if (threadIdx.x == blockDim.x - 1) {                  // its running sum is the total
-        x0[n] = r0;
-        x1[n] = r1;
-        x2[n] = r2;
-        x3[n] = r3;
-    }
-    __syncthreads();
-}
-
-struct OdeShared {
-    double *y, *yt, *kacc, *ev0, *ev1, *ev2, *ev3, *x0, *x1, *x2, *x3;
+// Window sums over the sorted plan, one channel per lane.  Every warp scans its
+// 32 channels; the in-warp inclusive prefixes stay in their block's shared
+// memory (read remotely at the window's two ends), the warps' totals are pushed
+// to every block.  Double-buffered, so one cluster barrier per call suffices: a
+// buffer is written again two calls later, after the barrier in between.
+struct OdeWindow {
+    double2 x[2][2][32 * kOdeMaxWarps / 8];      // [buffer][pair][channel of the block]
+    double2 tot[2][2][kOdeMaxWarps];             // [buffer][pair][warp of the plan]
 };
 
-// dy/dz at state Y into K (shared arrays; every thread calls).
-__device__ void raman_rhs(const RamanParams &rp, int coff, int poff, int n, const double *Y, double *K,
-                          const OdeShared &s, double *wsum)
+struct OdeLane {
+    int n, i, wpc;                // channels, this lane's, warps per block
+    bool live;
+    int wi, whi, wlo;             // warps of i, of the window's last, of the one before its first
+    bool has_lo;                  // the window does not start at channel 0
+    const double2 *xhi, *xlo;     // remote prefixes at hi and lo - 1 (buffer 0, pair 0)
+    double fr, f, invf, alpha, sc, P0;
+};
+
+__device__ __forceinline__ OdeLane ode_lane(cg::cluster_group &cl, OdeWindow &win, const RamanParams &rp, int coff,
+                                            int poff, int n)
 {
-    const double *fr = rp.ch_frel + coff;
-    const double *P0 = rp.P + poff;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        const double e = P0[k] > 0.0 ? exp(Y[k]) : 0.0;
-        const double invf = 1.0 / (fr[k] + rp.f_ref);
-        s.ev0[k] = e;
-        s.ev1[k] = fr[k] * e;
-        s.ev2[k] = e * invf;
-        s.ev3[k] = fr[k] * e * invf;
-    }
-    __syncthreads();
-    scan4(s.ev0, s.ev1, s.ev2, s.ev3, s.x0, s.x1, s.x2, s.x3, n, wsum);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int lo = rp.win_lo[coff + i], hi = rp.win_hi[coff + i];
-        const double fri = fr[i];
-        // partners above i: k in (i, hi]
-        double g = 0.0;
-        if (hi > i) g += (s.x1[hi + 1] - s.x1[i + 1]) - fri * (s.x0[hi + 1] - s.x0[i + 1]);
-        // partners below i: k in [lo, i)
-        if (lo < i) {
-            if (rp.photon)
-                g += (fri + rp.f_ref) * ((s.x3[i] - s.x3[lo]) - fri * (s.x2[i] - s.x2[lo]));
-            else
-                g += (s.x1[i] - s.x1[lo]) - fri * (s.x0[i] - s.x0[lo]);
+    OdeLane L;
+    L.n = n;
+    L.wpc = blockDim.x >> 5;
+    L.i = (int)cl.block_rank() * blockDim.x + threadIdx.x;
+    L.live = L.i < n;
+    const int i = min(L.i, n - 1);
+    const int lo = rp.win_lo[coff + i], hi = rp.win_hi[coff + i];
+    const auto at = [&](int j) {
+        const int r = j / (32 * L.wpc);
+        return cl.map_shared_rank(&win.x[0][0][0], r) + (j - r * 32 * L.wpc);
+    };
+    L.wi = L.i >> 5;
+    L.has_lo = lo > 0;
+    L.xhi = at(hi);
+    L.xlo = at(max(lo - 1, 0));
+    L.whi = L.live ? hi >> 5 : L.wi;
+    L.wlo = L.live ? max(lo - 1, 0) >> 5 : L.wi;
+    L.fr = rp.ch_frel[coff + i];
+    L.f = L.fr + rp.f_ref;
+    L.invf = 1.0 / L.f;
+    L.alpha = rp.ch_alpha[coff + i];
+    L.sc = rp.ch_scale[coff + i];
+    L.P0 = L.live ? rp.P[poff + i] : 0.0;
+    return L;
+}
+
+// Sums of pair (v0, v1) [or (v2, v3)] over the channels above i in its window
+// (up), and below (dn): up from pair pu, dn from pair pd.
+__device__ __forceinline__ void ode_window(cg::cluster_group &cl, OdeWindow &win, const OdeLane &L, int buf, double v0,
+                                           double v1, double v2, double v3, int pu, int pd, double2 &up, double2 &dn)
+{
+    const int lane = threadIdx.x & 31;
+    double x0 = v0, x1 = v1, x2 = v2, x3 = v3;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const double u0 = __shfl_up_sync(0xffffffffu, x0, o), u1 = __shfl_up_sync(0xffffffffu, x1, o);
+        const double u2 = __shfl_up_sync(0xffffffffu, x2, o), u3 = __shfl_up_sync(0xffffffffu, x3, o);
+        if (lane >= o) {
+            x0 += u0;
+            x1 += u1;
+            x2 += u2;
+            x3 += u3;
         }
-        K[i] = -rp.ch_alpha[coff + i] + rp.ch_scale[coff + i] * rp.Cr * g;
     }
-    __syncthreads();
+    win.x[buf][0][threadIdx.x] = make_double2(x0, x1);
+    win.x[buf][1][threadIdx.x] = make_double2(x2, x3);
+    // totals of this warp to every block: lane r (r + 16) takes pair 0 (1) of block r
+    const double2 t0 = make_double2(__shfl_sync(0xffffffffu, x0, 31), __shfl_sync(0xffffffffu, x1, 31));
+    const double2 t1 = make_double2(__shfl_sync(0xffffffffu, x2, 31), __shfl_sync(0xffffffffu, x3, 31));
+    const int r = lane & 15;
+    if (r < (int)cl.num_blocks()) {
+        double2 *dst = cl.map_shared_rank(&win.tot[buf][lane >> 4][0], r);
+        dst[L.wi] = lane < 16 ? t0 : t1;
+    }
+    cl.sync();
+    const int per = 2 * (int)(sizeof(win.x[0][0]) / sizeof(double2));      // entries of one buffer
+    const int one = per / 2;
+    const double2 h = L.xhi[buf * per + pu * one], l = L.xlo[buf * per + pd * one];
+    const double2 iu = pu ? make_double2(x2, x3) : make_double2(x0, x1);
+    const double2 id = pd ? make_double2(x2, x3) : make_double2(x0, x1);
+    up = make_double2(h.x - iu.x, h.y - iu.y);
+    for (int w = L.wi; w < L.whi; ++w) {
+        const double2 t = win.tot[buf][pu][w];
+        up.x += t.x;
+        up.y += t.y;
+    }
+    dn = make_double2(id.x - (pd ? v2 : v0), id.y - (pd ? v3 : v1));
+    if (L.has_lo) {
+        dn.x -= l.x;
+        dn.y -= l.y;
+    }
+    for (int w = L.has_lo ? L.wlo : 0; w < L.wi; ++w) {
+        const double2 t = win.tot[buf][pd][w];
+        dn.x += t.x;
+        dn.y += t.y;
+    }
+}
+
+// e^x: Taylor to x^11 for |x| <= 1/8 (remainder 3e-20), else the library's
+__device__ __forceinline__ double exp_small(double x)
+{
+    if (fabs(x) > 0.125) return exp(x);
+    double p = 1.0 / 39916800.0;
+    p = fma(p, x, 1.0 / 3628800.0);
+    p = fma(p, x, 1.0 / 362880.0);
+    p = fma(p, x, 1.0 / 40320.0);
+    p = fma(p, x, 1.0 / 5040.0);
+    p = fma(p, x, 1.0 / 720.0);
+    p = fma(p, x, 1.0 / 120.0);
+    p = fma(p, x, 1.0 / 24.0);
+    p = fma(p, x, 1.0 / 6.0);
+    p = fma(p, x, 0.5);
+    p = fma(p, x, 1.0);
+    return fma(p, x, 1.0);
+}
+
+// dy/dz of the lane's channel, P its power e^y (0 for an empty slot)
+__device__ __forceinline__ double ode_rhs(cg::cluster_group &cl, OdeWindow &win, const OdeLane &L,
+                                          const RamanParams &rp, int &buf, double P)
+{
+    double2 up, dn;
+    const double q = P * L.invf;
+    ode_window(cl, win, L, buf, P, L.fr * P, q, L.fr * q, 0, rp.photon ? 1 : 0, up, dn);
+    buf ^= 1;
+    const double below = fma(-L.fr, dn.x, dn.y);
+    const double g = fma(-L.fr, up.x, up.y) + (rp.photon ? L.f * below : below);
+    return fma(L.sc * rp.Cr, g, -L.alpha);
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(kOdeThreads) k_raman_ode(RamanParams rp)
+__global__ void __launch_bounds__(256) k_raman_ode(RamanParams rp)
 {
-    extern __shared__ double smem_d[];
-    __shared__ double wsum[128];
-    const int p = blockIdx.x;
+    __shared__ OdeWindow win;
+    cg::cluster_group cl = cg::this_cluster();
+    const int p = blockIdx.x / cl.num_blocks();
     const int plan = rp.prof_plan[p];
-    const int n = rp.plan_n[plan];
-    const int coff = rp.plan_ch_off[plan];
-    const int poff = rp.prof_ch_off[p];
+    const int n = rp.plan_n[plan], coff = rp.plan_ch_off[plan], poff = rp.prof_ch_off[p];
     const int M = rp.n_steps;
-    OdeShared s;
-    s.y = smem_d;
-    s.yt = s.y + n;
-    s.kacc = s.yt + n;
-    s.ev0 = s.kacc + n;
-    s.ev1 = s.ev0 + n;
-    s.ev2 = s.ev1 + n;
-    s.ev3 = s.ev2 + n;
-    s.x0 = s.ev3 + n;
-    s.x1 = s.x0 + n + 1;
-    s.x2 = s.x1 + n + 1;
-    s.x3 = s.x2 + n + 1;
-    double *K = s.x3 + n + 1;                 // [n] stage slope
-    double *y0 = K + n;                       // [n] initial state
-    const double *P0 = rp.P + poff;
+    const OdeLane L = ode_lane(cl, win, rp, coff, poff, n);
     double2 *ab = rp.ab + (size_t)poff * M;
-    double *yn = (p == 0) ? rp.y_nodes : nullptr;
-
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        const double v = P0[c] > 0.0 ? log(P0[c]) : 0.0;
-        s.y[c] = v;
-        y0[c] = v;
-    }
-    __syncthreads();
-    int node = 0;
+    double *sp = p == 0 ? rp.stage_P : nullptr;
+    const double y0 = L.P0 > 0.0 ? log(L.P0) : 0.0;
+    double y = y0;
+    int buf = 0;
+    size_t node = 0;
+    const auto keep = [&](int s, double P) {
+        if (sp && L.live) sp[(4 * node + s) * n + L.i] = P;
+    };
     for (int m = 0; m < M; ++m) {
         const int ns = rp.half_steps[m];
         const double h = 0.5 * rp.zs_d[m].y / ns;
         for (int half = 0; half < 2; ++half) {
             for (int t = 0; t < ns; ++t) {
-                if (yn)
-                    for (int c = threadIdx.x; c < n; c += blockDim.x) yn[(size_t)node * n + c] = s.y[c];
+                const double P1 = L.P0 > 0.0 ? exp(y) : 0.0;
+                const double k1 = ode_rhs(cl, win, L, rp, buf, P1);
+                const double P2 = P1 * exp_small(0.5 * h * k1);
+                const double k2 = ode_rhs(cl, win, L, rp, buf, P2);
+                const double P3 = P1 * exp_small(0.5 * h * k2);
+                const double k3 = ode_rhs(cl, win, L, rp, buf, P3);
+                const double P4 = P1 * exp_small(h * k3);
+                const double k4 = ode_rhs(cl, win, L, rp, buf, P4);
+                y += h / 6.0 * ((k1 + 2.0 * k2) + 2.0 * k3 + k4);
+                keep(0, P1);
+                keep(1, P2);
+                keep(2, P3);
+                keep(3, P4);
                 ++node;
-                raman_rhs(rp, coff, poff, n, s.y, K, s, wsum);                   // k1
-                for (int c = threadIdx.x; c < n; c += blockDim.x) {
-                    s.kacc[c] = K[c];
-                    s.yt[c] = s.y[c] + 0.5 * h * K[c];
-                }
-                __syncthreads();
-                raman_rhs(rp, coff, poff, n, s.yt, K, s, wsum);                  // k2
-                for (int c = threadIdx.x; c < n; c += blockDim.x) {
-                    s.kacc[c] += 2.0 * K[c];
-                    s.yt[c] = s.y[c] + 0.5 * h * K[c];
-                }
-                __syncthreads();
-                raman_rhs(rp, coff, poff, n, s.yt, K, s, wsum);                  // k3
-                for (int c = threadIdx.x; c < n; c += blockDim.x) {
-                    s.kacc[c] += 2.0 * K[c];
-                    s.yt[c] = s.y[c] + h * K[c];
-                }
-                __syncthreads();
-                raman_rhs(rp, coff, poff, n, s.yt, K, s, wsum);                  // k4
-                for (int c = threadIdx.x; c < n; c += blockDim.x) s.y[c] += h / 6.0 * (s.kacc[c] + K[c]);
-                __syncthreads();
             }
-            if (half == 0)
-                for (int c = threadIdx.x; c < n; c += blockDim.x) ab[(size_t)c * M + m].x = s.y[c] - y0[c];
+            if (half == 0 && L.live) ab[(size_t)L.i * M + m].x = y - y0;
         }
     }
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        rp.lnrho_L[poff + c] = s.y[c] - y0[c];
-        if (yn) yn[(size_t)node * n + c] = s.y[c];
-    }
-    __syncthreads();
+    if (L.live) rp.lnrho_L[poff + L.i] = y - y0;
+    cl.sync();                       // the tables of every block; no block leaves while others read its prefixes
     // in-channel slopes: central differences of a + alpha z_m
     const double *fr = rp.ch_frel + coff;
     const double *al = rp.ch_alpha + coff;
-    for (int t = threadIdx.x; t < n * M; t += blockDim.x) {
+    for (int t = (int)cl.thread_rank(); t < n * M; t += (int)cl.num_threads()) {
         const int c = t / M, m = t - c * M;
         const int lo = c > 0 ? c - 1 : 0, hi = c < n - 1 ? c + 1 : n - 1;
         double b = 0.0;
@@ -262,18 +255,46 @@ __global__ void __launch_bounds__(kOdeThreads) k_raman_ode(RamanParams rp)
     }
 }
 
-size_t raman_smem_bytes(int n_ch)
+namespace {
+
+// One cluster per profile: warps of 32 channels, kOdeWarps to a block where 16
+// blocks (8 if the device cannot place 16) hold them, else more.
+template <typename Params>
+cudaError_t launch_clusters(void (*fn)(Params), const Params &prm, int n_prof, int max_n, cudaStream_t st)
 {
-    return sizeof(double) * (size_t)(13 * n_ch + 4);
+    const int warps = (max_n + 31) / 32;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    for (int most = kOdeMaxCluster; most >= 8; most /= 2) {
+        const int wpc = std::max(kOdeWarps, (warps + most - 1) / most);
+        const int size = (warps + wpc - 1) / wpc;
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute at[1];
+        cfg.gridDim = dim3(n_prof * size);
+        cfg.blockDim = dim3(32 * wpc);
+        cfg.stream = st;
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = size;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        if (size > 8) {
+            int nc = 0;
+            if (cudaOccupancyMaxActiveClusters(&nc, fn, &cfg) != cudaSuccess || nc < 1) {
+                cudaGetLastError();
+                continue;
+            }
+        }
+        return cudaLaunchKernelEx(&cfg, fn, prm);
+    }
+    return cudaErrorInvalidConfiguration;
 }
+
+}  // namespace
 
 cudaError_t launch_raman(const RamanParams &rp, int n_prof, int max_n, cudaStream_t st)
 {
-    const size_t smem = raman_smem_bytes(max_n);
-    cudaError_t e = cudaFuncSetAttribute(k_raman_ode, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_raman_ode<<<n_prof, kOdeThreads, smem, st>>>(rp);
-    return cudaGetLastError();
+    return launch_clusters(k_raman_ode, rp, n_prof, max_n, st);
 }
 
 // ---------------------------------------------------------------------------
@@ -286,8 +307,8 @@ cudaError_t launch_raman(const RamanParams &rp, int n_prof, int max_n, cudaStrea
 //   mu4 = J(Y4)^T (h/6 lambda),            mu3 = J(Y3)^T (h/3 lambda + h mu4),
 //   mu2 = J(Y2)^T (h/3 lambda + h/2 mu3),  mu1 = J(Y1)^T (h/6 lambda + h/2 mu2),
 //   dT/dy = lambda + mu1 + mu2 + mu3 + mu4,
-// with the stage states Y recomputed from the stored step states, the table
-// sensitivities injected at the nodes z_m and L, and
+// with the stage powers e^Y kept by the forward run, the table sensitivities
+// injected at the nodes z_m and L, and
 //   (J^T v)_k = C_r e^{Y_k} sum_i s_i v_i h(f_k, f_i)
 // again by prefix sums over the partner window of k:
 //   i below k:  sum u_i (fr_k - fr_i)              = fr_k S(u) - S(fr u)
@@ -315,132 +336,72 @@ __global__ void __launch_bounds__(256) k_fold_slope(RamanAdjParams ap)
 
 namespace {
 
-// out = J(Y)^T v (shared arrays; every thread calls)
-__device__ void raman_jt(const RamanParams &rp, int n, const double *Y, const double *v, double *out,
-                         const OdeShared &s, double *wsum)
+// (J^T v) of the lane's channel at the stage power P = e^{Y_k}
+__device__ __forceinline__ double ode_jt(cg::cluster_group &cl, OdeWindow &win, const OdeLane &L,
+                                         const RamanParams &rp, int &buf, double P, double v)
 {
-    const double *fr = rp.ch_frel;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const double u = rp.ch_scale[i] * v[i];
-        const double f = fr[i] + rp.f_ref;
-        s.ev0[i] = u;
-        s.ev1[i] = fr[i] * u;
-        s.ev2[i] = f * u;
-        s.ev3[i] = fr[i] * f * u;
-    }
-    __syncthreads();
-    scan4(s.ev0, s.ev1, s.ev2, s.ev3, s.x0, s.x1, s.x2, s.x3, n, wsum);
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        double r = 0.0;
-        if (rp.P[k] > 0.0) {
-            const int lo = rp.win_lo[k], hi = rp.win_hi[k];
-            const double frk = fr[k];
-            double g = 0.0;
-            if (lo < k) g += frk * (s.x0[k] - s.x0[lo]) - (s.x1[k] - s.x1[lo]);
-            if (hi > k) {
-                if (rp.photon)
-                    g += (frk * (s.x2[hi + 1] - s.x2[k + 1]) - (s.x3[hi + 1] - s.x3[k + 1])) / (frk + rp.f_ref);
-                else
-                    g += frk * (s.x0[hi + 1] - s.x0[k + 1]) - (s.x1[hi + 1] - s.x1[k + 1]);
-            }
-            r = rp.Cr * exp(Y[k]) * g;
-        }
-        out[k] = r;
-    }
-    __syncthreads();
+    double2 up, dn;
+    const double u = L.live ? L.sc * v : 0.0, w = L.f * u;
+    ode_window(cl, win, L, buf, u, L.fr * u, w, L.fr * w, rp.photon ? 1 : 0, 0, up, dn);
+    buf ^= 1;
+    const double above = fma(L.fr, up.x, -up.y);
+    const double g = fma(L.fr, dn.x, -dn.y) + (rp.photon ? above * L.invf : above);
+    return rp.Cr * P * g;
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(kOdeThreads) k_raman_adj(RamanAdjParams ap)
+__global__ void __launch_bounds__(256) k_raman_adj(RamanAdjParams ap)
 {
-    extern __shared__ double smem_d[];
-    __shared__ double wsum[128];
+    __shared__ OdeWindow win;
+    cg::cluster_group cl = cg::this_cluster();
     const RamanParams &rp = ap.r;
     const int n = ap.n, M = rp.n_steps;
-    double *lam = smem_d, *acc = lam + n, *w = acc + n, *mu = w + n, *Y2 = mu + n, *Y3 = Y2 + n, *Y4 = Y3 + n;
-    OdeShared s;
-    s.y = s.yt = s.kacc = nullptr;
-    s.ev0 = Y4 + n;
-    s.ev1 = s.ev0 + n;
-    s.ev2 = s.ev1 + n;
-    s.ev3 = s.ev2 + n;
-    s.x0 = s.ev3 + n;
-    s.x1 = s.x0 + n + 1;
-    s.x2 = s.x1 + n + 1;
-    s.x3 = s.x2 + n + 1;
-
-    for (int c = threadIdx.x; c < n; c += blockDim.x)
-        lam[c] = ap.with_direct ? -ap.aase[c] : 0.0;                               // dT/d ln rho(L)
-    __syncthreads();
-    int node = ap.n_rk;
+    const OdeLane L = ode_lane(cl, win, rp, 0, 0, n);
+    const int c = min(L.i, n - 1);
+    double lam = L.live && ap.with_direct ? -ap.aase[c] : 0.0;             // dT/d ln rho(L)
+    int buf = 0;
+    size_t node = (size_t)ap.n_rk;
+    const auto stage = [&](size_t k, int s) { return rp.stage_P[(4 * k + s) * n + c]; };
+    // the stage powers of the next step back are fetched while this one runs
+    double q1 = stage(node - 1, 0), q2 = stage(node - 1, 1), q3 = stage(node - 1, 2), q4 = stage(node - 1, 3);
     for (int m = M - 1; m >= 0; --m) {
         const int ns = rp.half_steps[m];
         const double h = 0.5 * rp.zs_d[m].y / ns;
+        const double inj = L.live ? ap.gAt[(size_t)c * M + m] : 0.0;
         for (int half = 1; half >= 0; --half) {
             for (int t = 0; t < ns; ++t) {
                 --node;
-                const double *Y1 = ap.y_nodes + (size_t)node * n;
-                // stage states of this step
-                raman_rhs(rp, 0, 0, n, Y1, mu, s, wsum);
-                for (int c = threadIdx.x; c < n; c += blockDim.x) Y2[c] = Y1[c] + 0.5 * h * mu[c];
-                __syncthreads();
-                raman_rhs(rp, 0, 0, n, Y2, mu, s, wsum);
-                for (int c = threadIdx.x; c < n; c += blockDim.x) Y3[c] = Y1[c] + 0.5 * h * mu[c];
-                __syncthreads();
-                raman_rhs(rp, 0, 0, n, Y3, mu, s, wsum);
-                for (int c = threadIdx.x; c < n; c += blockDim.x) {
-                    Y4[c] = Y1[c] + h * mu[c];
-                    acc[c] = lam[c];
-                    w[c] = h / 6.0 * lam[c];
-                }
-                __syncthreads();
-                raman_jt(rp, n, Y4, w, mu, s, wsum);                         // mu4
-                for (int c = threadIdx.x; c < n; c += blockDim.x) {
-                    acc[c] += mu[c];
-                    w[c] = h / 3.0 * lam[c] + h * mu[c];
-                }
-                __syncthreads();
-                raman_jt(rp, n, Y3, w, mu, s, wsum);                         // mu3
-                for (int c = threadIdx.x; c < n; c += blockDim.x) {
-                    acc[c] += mu[c];
-                    w[c] = h / 3.0 * lam[c] + 0.5 * h * mu[c];
-                }
-                __syncthreads();
-                raman_jt(rp, n, Y2, w, mu, s, wsum);                         // mu2
-                for (int c = threadIdx.x; c < n; c += blockDim.x) {
-                    acc[c] += mu[c];
-                    w[c] = h / 6.0 * lam[c] + 0.5 * h * mu[c];
-                }
-                __syncthreads();
-                raman_jt(rp, n, Y1, w, mu, s, wsum);                         // mu1
-                for (int c = threadIdx.x; c < n; c += blockDim.x) lam[c] = acc[c] + mu[c];
-                __syncthreads();
+                const double P1 = q1, P2 = q2, P3 = q3, P4 = q4;
+                const size_t nx = node > 0 ? node - 1 : 0;
+                q1 = stage(nx, 0);
+                q2 = stage(nx, 1);
+                q3 = stage(nx, 2);
+                q4 = stage(nx, 3);
+                const double h6 = h / 6.0 * lam, h3 = h / 3.0 * lam;
+                const double m4 = ode_jt(cl, win, L, rp, buf, P4, h6);
+                const double m3 = ode_jt(cl, win, L, rp, buf, P3, fma(h, m4, h3));
+                const double m2 = ode_jt(cl, win, L, rp, buf, P2, fma(0.5 * h, m3, h3));
+                const double m1 = ode_jt(cl, win, L, rp, buf, P1, fma(0.5 * h, m2, h6));
+                lam += ((m4 + m3) + m2) + m1;
             }
-            if (half == 1)
-                for (int c = threadIdx.x; c < n; c += blockDim.x) lam[c] += ap.gAt[(size_t)c * M + m];
-            __syncthreads();
+            if (half == 1) lam += inj;
         }
     }
+    cl.sync();                       // no block leaves while others read its prefixes
+    if (!L.live) return;
     // a = y - y(0): every table entry also depends on y(0) directly
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        double direct = ap.with_direct ? ap.aase[j] : 0.0;             // - dT/d ln rho(L)
-        for (int m = 0; m < M; ++m) direct -= ap.gAt[(size_t)j * M + m];
-        const double P = rp.P[j];
-        double g = (lam[j] + direct + ap.gV[j]) / P;
-        if (ap.with_direct) {                                          // the SNR numerator
-            const double snr = ap.snr[j], B = ap.ch_B[j];
-            const double N = ap.pnli[j] + ap.pase[j];
-            const double dTds = 2.0 * B / (0.69314718055994530942 * (1.0 + snr));
-            g += dTds * snr * snr * N / (P * P);
-        }
-        ap.dT_dP[j] = g;
+    double direct = ap.with_direct ? ap.aase[c] : 0.0;             // - dT/d ln rho(L)
+    for (int m = 0; m < M; ++m) direct -= ap.gAt[(size_t)c * M + m];
+    const double P = rp.P[c];
+    double g = (lam + direct + ap.gV[c]) / P;
+    if (ap.with_direct) {                                          // the SNR numerator
+        const double snr = ap.snr[c], B = ap.ch_B[c];
+        const double N = ap.pnli[c] + ap.pase[c];
+        const double dTds = 2.0 * B / (0.69314718055994530942 * (1.0 + snr));
+        g += dTds * snr * snr * N / (P * P);
     }
-}
-
-size_t raman_adj_smem_bytes(int n_ch)
-{
-    return sizeof(double) * (size_t)(15 * n_ch + 4);
+    ap.dT_dP[c] = g;
 }
 
 cudaError_t launch_raman_adj(const RamanAdjParams &ap, cudaStream_t st)
@@ -449,11 +410,7 @@ cudaError_t launch_raman_adj(const RamanAdjParams &ap, cudaStream_t st)
     k_fold_slope<<<(nm + 255) / 256, 256, 0, st>>>(ap);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const size_t smem = raman_adj_smem_bytes(ap.n);
-    e = cudaFuncSetAttribute(k_raman_adj, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_raman_adj<<<1, kOdeThreads, smem, st>>>(ap);
-    return cudaGetLastError();
+    return launch_clusters(k_raman_adj, ap, 1, ap.n, st);
 }
 
 // ---------------------------------------------------------------------------
