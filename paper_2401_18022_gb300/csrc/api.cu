@@ -630,11 +630,9 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
     }
 
     // work items, output slots
-    const int tile_pts = h->tile_points > 0 ? h->tile_points : (1 << 20);
     std::vector<DevItem> items, mitems;
     std::vector<int2> slot_items, slot_items2;
     std::vector<int> slot_cut, prof_slot_off, item_slot, mitem_slot;
-    const int mchunk = mci ? (int)std::max<int64_t>(1, tile_pts / ((int64_t)q->G_mci * q->G_mci)) : 1;
     g->n_points = 0;
     g->n_points_unfolded = 0;
     for (int p = 0; p < g->n_prof; ++p) {
@@ -667,6 +665,13 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
                 const int n2 = plans[k].n_ch - 1;
                 const int ncell = n2 * (n2 + 1) / 2;
                 const int m0 = (int)mitems.size();
+                // ~16 tiles per resident block of a whole plan (a 295-ch plan with
+                // 16,384 cells to a tile ran 1.9 waves); plan-dependent only, as tile_split
+                const int64_t cells = (int64_t)ncell * plans[k].n_ch;
+                const int mchunk =
+                    h->tile_points > 0
+                        ? (int)std::max<int64_t>(1, h->tile_points / ((int64_t)q->G_mci * q->G_mci))
+                        : (int)std::max<int64_t>(32, std::min<int64_t>(16384, cells / (152 * 3 * 16)));
                 for (int t = 0; t < ncell; t += mchunk) {
                     mitems.push_back(DevItem{p, t, std::min(t + mchunk, ncell), i, 1 << 16});
                     mitem_slot.push_back(slot);
@@ -1092,8 +1097,14 @@ isrs_status run_forward(isrs_handle h, const isrs_fibre *fb, Geom *g, int precis
                         return fail(h, ISRS_ERR_UNSUPPORTED, "profile tables of %zu entries exceed the MCI conversion", nab);
                     if ((s = ensure(h, h->ab_f, sizeof(float2) * nab)) != ISRS_OK) return s;
                     qm.ab_f = (const float2 *)h->ab_f.p;
-                    CK(launch_tab_half_log2((const double2 *)h->ab.p, (float2 *)h->ab_f.p, (int)nab, h->num_sms,
-                                            st));
+                    TabHalfParams hp;
+                    hp.ab = (const double2 *)h->ab.p;
+                    hp.abf = (float2 *)h->ab_f.p;
+                    hp.plan_n = qm.plan_n;
+                    hp.prof_plan = qm.prof_plan;
+                    hp.prof_ch_off = qm.prof_ch_off;
+                    hp.n_steps = M;
+                    CK(launch_tab_half_log2(hp, g->n_prof, qm.mci_n_max, h->num_sms, st));
                 }
                 qm.mci_cpc = cpc;
                 int mgrid = h->num_sms * quad_mci_tab_blocks_per_sm(precision, M, qm.mci_n_max, cpc, block);

@@ -23,6 +23,14 @@ struct PrepParams {
     double *kap_L;              // kappa(L) per profile (the largest ISRS exponent slope)
 };
 
+// FP32 copy of the profile tables for the MCI cells (steps outermost)
+struct TabHalfParams {
+    const double2 *ab;
+    float2 *abf;
+    const int *plan_n, *prof_plan, *prof_ch_off;
+    int n_steps;
+};
+
 struct FinishParams {
     const double *partial;
     const int2 *slot_items;     // per output slot: item range
@@ -183,7 +191,7 @@ cudaError_t launch_quad_mci(const QuadParams &qp, int precision, int grid, int b
 int quad_mci_tab_cells(int n_steps, int n_max, int G, int block);
 size_t quad_mci_tab_smem_bytes(int precision, int n_steps, int n_max, int cpc);
 int quad_mci_tab_blocks_per_sm(int precision, int n_steps, int n_max, int cpc, int block);
-cudaError_t launch_tab_half_log2(const double2 *ab, float2 *abf, int n, int n_sms, cudaStream_t st);
+cudaError_t launch_tab_half_log2(const TabHalfParams &hp, int n_prof, int max_n, int n_sms, cudaStream_t st);
 cudaError_t launch_quad_mci_tab(const QuadParams &qp, int precision, int grid, int block, cudaStream_t st);
 // adjoint over the MCI cells of a separate grid (closed-form profile)
 size_t adjoint_mci_smem_bytes(int n_steps, int n_max, int block);

@@ -32,18 +32,25 @@ namespace {
 
 constexpr int kMciTabCells = 32;   // cells per chunk at most (their step rows share the block's memory)
 
-// {1/2 log2(e) a_c(m), 1/2 log2(e) b_c(m)} in FP32, same index as qp.ab
-__global__ void __launch_bounds__(256) k_tab_half_log2(const double2 *ab, float2 *abf, int n)
+// {1/2 log2(e) a_c(m), 1/2 log2(e) b_c(m)} in FP32, steps outermost: entry
+// prof_ch_off[p] M + m n + c.  Neighbouring points of a chunk have F_c in
+// neighbouring channels, so a warp's 32 rows at one step lie in one or two
+// lines; with the channel outermost (as qp.ab) every lane read its own sector
+// and the loads bound the kernel.  One block row per profile.
+__global__ void __launch_bounds__(256) k_tab_half_log2(TabHalfParams hp)
 {
-    for (int t = threadIdx.x + blockIdx.x * blockDim.x; t < n; t += blockDim.x * gridDim.x) {
-        const double2 v = ab[t];
-        abf[t] = make_float2((float)(0.5 * kLog2e * v.x), (float)(0.5 * kLog2e * v.y));
+    const int p = blockIdx.y, n = hp.plan_n[hp.prof_plan[p]], M = hp.n_steps;
+    const size_t off = (size_t)hp.prof_ch_off[p] * M;
+    for (int t = threadIdx.x + blockIdx.x * blockDim.x; t < n * M; t += blockDim.x * gridDim.x) {
+        const int m = t / n, c = t - m * n;
+        const double2 v = hp.ab[off + (size_t)c * M + m];
+        hp.abf[off + t] = make_float2((float)(0.5 * kLog2e * v.x), (float)(0.5 * kLog2e * v.y));
     }
 }
 
 // FP32 z-sums of Eq. slow_vary with
 //   log2 p_m (dz_m) = Q.x + Q.y da + Q.z db + T.x + T.y dc   (Q.w for the
-// telescoped form, without log2 dz); sA[m] = {z, z^2 + dz^2/12, log2 dz, dz},
+// telescoped form, without log2 dz), T the F_c channel's row at Tc + m n; sA[m] = {z, z^2 + dz^2/12, log2 dz, dz},
 // sB[m] = {z_{m+1}/2pi hi, lo, ., .}.
 __device__ __forceinline__ float lp_tab(const float4 &q, float qx, const float2 &t, float da, float db, float dc)
 {
@@ -54,14 +61,14 @@ __device__ __forceinline__ float lp_tab(const float4 &q, float qx, const float2 
 }
 
 __device__ __forceinline__ float zsum_small_mt(float phi, float da, float db, float dc, const float4 *Q,
-                                               const float2 *Tc, const float4 *sA, int M)
+                                               const float2 *Tc, int n, const float4 *sA, int M)
 {
     float M0 = 0.0f, M1 = 0.0f, M2 = 0.0f;
 #pragma unroll 4
     for (int m = 0; m < M; ++m) {
         const float4 q = Q[m];
         const float4 a = sA[m];
-        const float w = ex2_approx(lp_tab(q, q.x, __ldg(Tc + m), da, db, dc));   // p_m dz_m
+        const float w = ex2_approx(lp_tab(q, q.x, __ldg(Tc + m * n), da, db, dc));   // p_m dz_m
         M0 += w;
         M1 = fmaf(w, a.x, M1);
         M2 = fmaf(w, a.y, M2);
@@ -70,7 +77,7 @@ __device__ __forceinline__ float zsum_small_mt(float phi, float da, float db, fl
 }
 
 __device__ __forceinline__ float zsum_direct_mt(float phi, float da, float db, float dc, const float4 *Q,
-                                                const float2 *Tc, const float4 *sA, int M)
+                                                const float2 *Tc, int n, const float4 *sA, int M)
 {
     float Sr = 0.0f, Si = 0.0f;
     const float hphi = 0.5f * phi;
@@ -88,7 +95,7 @@ __device__ __forceinline__ float zsum_direct_mt(float phi, float da, float db, f
         sc = fmaf(x2, sc, 8.3333333e-3f);                      // 1/5!
         sc = fmaf(x2, sc, -1.6666667e-1f);                     // -1/3!
         sc = fmaf(x2, sc, 1.0f);
-        const float amp = ex2_approx(lp_tab(q, q.x, __ldg(Tc + m), da, db, dc)) * sc;   // p_m dz_m sinc
+        const float amp = ex2_approx(lp_tab(q, q.x, __ldg(Tc + m * n), da, db, dc)) * sc;   // p_m dz_m sinc
         Sr = fmaf(amp, cs, Sr);
         Si = fmaf(amp, sn, Si);
     }
@@ -96,7 +103,7 @@ __device__ __forceinline__ float zsum_direct_mt(float phi, float da, float db, f
 }
 
 __device__ __forceinline__ float zsum_tele_mt(float phi, float da, float db, float dc, const float4 *Q,
-                                              const float2 *Tc, const float4 *sB, int M)
+                                              const float2 *Tc, int n, const float4 *sB, int M)
 {
     float Er = 1.0f, Ei = 0.0f, Sr = 0.0f, Si = 0.0f;
 #pragma unroll 4
@@ -105,7 +112,7 @@ __device__ __forceinline__ float zsum_tele_mt(float phi, float da, float db, flo
         const float4 e = sB[m];
         float sn, cs;
         phasor_rev_ff_wide(phi, e.x, e.y, sn, cs);
-        const float p = ex2_approx(lp_tab(q, q.w, __ldg(Tc + m), da, db, dc));
+        const float p = ex2_approx(lp_tab(q, q.w, __ldg(Tc + m * n), da, db, dc));
         Sr = fmaf(p, cs - Er, Sr);
         Si = fmaf(p, sn - Ei, Si);
         Er = cs;
@@ -128,8 +135,9 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
     const int M = qp.n_steps, G = qp.G, CPC = qp.mci_cpc;
     float4 *sA = smem_f4;                              // [M] {z, z^2 + dz^2/12, log2 dz, dz}
     float4 *sB = sA + M;                               // [M] {edge/2pi hi, lo, ., .}
-    float4 *sQ = sB + M;                               // [CPC][M] {A + log2 dz, Sa, Sb, A}
-    float *rel = reinterpret_cast<float *>(sQ + (size_t)CPC * M);   // [n] channel centre - f_i
+    float4 *sQ = sB + M;                               // [CPC][M | 1] {A + log2 dz, Sa, Sb, A}
+    const int MS = M | 1;                              // row pitch: the cells of a warp in different banks
+    float *rel = reinterpret_cast<float *>(sQ + (size_t)CPC * MS);  // [n] channel centre - f_i
     float *hb = rel + qp.mci_n_max;                    // [n] B/2
     float *pd = hb + qp.mci_n_max;                     // [n] P/B
     __shared__ int2 sCell[kMciTabCells];
@@ -187,11 +195,12 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
             }
             __syncthreads();
             for (int e = threadIdx.x; e < ncc * M; e += blockDim.x) {
-                const int cc = e / M, m = e - cc * M;
+                const int m = e / ncc, cc = e - m * ncc;
                 const int2 ab = sCell[cc];
-                const float2 ta = T[(size_t)ab.x * M + m], tb = T[(size_t)ab.y * M + m];
-                const float A = (ta.x + tb.x) - T[(size_t)i * M + m].x;
-                sQ[e] = make_float4(A + sA[m].z, ta.y, tb.y, A);
+                const float2 *Tm = T + (size_t)m * n;
+                const float2 ta = Tm[ab.x], tb = Tm[ab.y];
+                const float A = (ta.x + tb.x) - Tm[i].x;
+                sQ[cc * MS + m] = make_float4(A + sA[m].z, ta.y, tb.y, A);
             }
             __syncthreads();
             for (int q = threadIdx.x; q < ncc * G; q += blockDim.x) {
@@ -214,7 +223,7 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
                 const float yc = sqrtf(ymin * ymax), xc = u1 / yc;
                 const float w = u1 * ds * du2 * mult;
                 const float Wab = pd[a] * pd[b];
-                const float4 *Q = sQ + (size_t)cc * M;
+                const float4 *Q = sQ + (size_t)cc * MS;
                 for (int j = 0; j < G; ++j) {
                     const float d = ((float)j + 0.5f - 0.5f * (float)G) * du2;
                     const float ex = expf(d);
@@ -229,11 +238,11 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
                                      c4 * (f1 * f1 + 1.5f * f1 * f2 + 3.0f * fi * u + f2 * f2 + three_fi2);
                     const float phi = m4pi2 * f1 * f2 * br;
                     const float aphi = fabsf(phi);
-                    const float2 *Tc = T + (size_t)c * M;
+                    const float2 *Tc = T + c;
                     float S2;
-                    if (aphi <= phi_small) S2 = zsum_small_mt(phi, da, db, dc, Q, Tc, sA, M);
-                    else if (aphi <= phi_direct) S2 = zsum_direct_mt(phi, da, db, dc, Q, Tc, sA, M);
-                    else S2 = zsum_tele_mt(phi, da, db, dc, Q, Tc, sB, M);
+                    if (aphi <= phi_small) S2 = zsum_small_mt(phi, da, db, dc, Q, Tc, n, sA, M);
+                    else if (aphi <= phi_direct) S2 = zsum_direct_mt(phi, da, db, dc, Q, Tc, n, sA, M);
+                    else S2 = zsum_tele_mt(phi, da, db, dc, Q, Tc, n, sB, M);
                     const float y = w * W * S2 * array_factor_f(phi, qp) - comp;
                     const float t = sum + y;
                     comp = (t - sum) - y;
@@ -348,7 +357,7 @@ __global__ void __launch_bounds__(256) k_quad_mci_f64_tab(QuadParams qp)
 size_t quad_mci_tab_smem_bytes(int precision, int n_steps, int n_max, int cpc)
 {
     if (precision == 0)
-        return (size_t)n_steps * (2 + cpc) * sizeof(float4) + (size_t)n_max * 3 * sizeof(float);
+        return ((size_t)n_steps * 2 + (size_t)(n_steps | 1) * cpc) * sizeof(float4) + (size_t)n_max * 3 * sizeof(float);
     return (size_t)n_steps * (sizeof(double2) + sizeof(double));
 }
 
@@ -357,7 +366,7 @@ int quad_mci_tab_cells(int n_steps, int n_max, int G, int block)
     const size_t fixed = (size_t)n_steps * 2 * sizeof(float4) + (size_t)n_max * 3 * sizeof(float);
     const size_t budget = 200 * 1024;
     if (fixed >= budget) return 0;
-    const int by_mem = (int)((budget - fixed) / ((size_t)n_steps * sizeof(float4)));
+    const int by_mem = (int)((budget - fixed) / ((size_t)(n_steps | 1) * sizeof(float4)));
     return std::min(std::min(kMciTabCells, block / std::max(1, G)), by_mem);
 }
 
@@ -376,10 +385,10 @@ int quad_mci_tab_blocks_per_sm(int precision, int n_steps, int n_max, int cpc, i
     return nb > 0 ? nb : 1;
 }
 
-cudaError_t launch_tab_half_log2(const double2 *ab, float2 *abf, int n, int n_sms, cudaStream_t st)
+cudaError_t launch_tab_half_log2(const TabHalfParams &hp, int n_prof, int max_n, int n_sms, cudaStream_t st)
 {
-    const int grid = std::max(1, std::min((n + 255) / 256, 4 * n_sms));
-    k_tab_half_log2<<<grid, 256, 0, st>>>(ab, abf, n);
+    const int grid = std::max(1, std::min((max_n * hp.n_steps + 255) / 256, 4 * n_sms));
+    k_tab_half_log2<<<dim3(grid, n_prof), 256, 0, st>>>(hp);
     return cudaGetLastError();
 }
 
