@@ -13,8 +13,8 @@
 //                the direct or telescoped step sums with a float-float phase
 //                and mod-2pi reduction; compensated accumulation; one FP64
 //                partial per tile.
-//  k_quad_f64    the same quadrature in plain FP64 (direct form of
-//                Eq. slow_vary with sinc), used as the reference GPU path.
+//  k_quad_f64    the same quadrature in plain FP64 at every grid point, used as
+//                the reference GPU path.
 //  k_finish      per profile: deterministic FP64 sum of tile partials per CUT,
 //                eta (Eq. gain_fin), P_NLI, SNR and throughput (Eq. loss).
 #include <cuda_runtime.h>
@@ -306,8 +306,15 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
 }
 
 // ---------------------------------------------------------------------------
-// k_quad_f64: the same quadrature in plain FP64 (direct form, libm functions).
+// k_quad_f64: the same quadrature in plain FP64, every grid point.
 // ---------------------------------------------------------------------------
+// F_c candidates with their powers at the channel centre in shared memory (0
+// where a huge grid and z-grid leave no room)
+__host__ __device__ constexpr int f64_cand(int n_steps, int G)
+{
+    return 64 * (size_t)n_steps + sizeof(RowD) * (size_t)G <= 200 * 1024 ? 4 : 0;
+}
+
 __global__ void __launch_bounds__(256) k_quad_f64(QuadParams qp)
 {
     extern __shared__ double2 smem_d2[];
@@ -315,6 +322,9 @@ __global__ void __launch_bounds__(256) k_quad_f64(QuadParams qp)
     double2 *sz = smem_d2;                 // [M] {z_m, dz_m}
     double2 *st = sz + M;                  // [M] {lnPtot - lnN, kappa}
     RowD *rows = reinterpret_cast<RowD *>(st + M);
+    double *sP = reinterpret_cast<double *>(rows + G);   // [f64_cand][M] p_m at the candidate's centre
+    const int ncp = f64_cand(M, G);
+    const double phi_direct = kF64Direct / qp.dz_max;
     __shared__ PieceConst<double> kc;
     __shared__ double scratch[32];
     __shared__ int s_item;
@@ -342,6 +352,12 @@ __global__ void __launch_bounds__(256) k_quad_f64(QuadParams qp)
             piece_consts<double>(qp, pc, item.prof, 1.0, qp.pd_d, kc);
             __syncthreads();
             const double fi = kc.fi;
+            // powers at the channel centres of the first candidates
+            for (int t = threadIdx.x; t < min(kc.nc, ncp) * M; t += blockDim.x) {
+                const int c = t / M, m = t - c * M;
+                sP[t] = exp(st[m].x - st[m].y * (fi + 0.5 * (kc.lo[c] + kc.hi[c])) - (kc.at_ab + kc.hat[c]) * sz[m].x);
+            }
+            __syncthreads();
             double sum = 0.0;
             const int npts = G * G;
             for (int q = threadIdx.x + (item.part & 0xffff) * blockDim.x; q < npts;
@@ -365,18 +381,13 @@ __global__ void __launch_bounds__(256) k_quad_f64(QuadParams qp)
                 const double br = qp.beta2 + c3 * (u + 2.0 * fi) +
                                   c4 * (f1 * f1 + 1.5 * f1 * f2 + 3.0 * fi * u + f2 * f2 + 3.0 * fi * fi);
                 const double phi = -4.0 * kPi * kPi * f1 * f2 * br;
-                double Sr = 0.0, Si = 0.0;
-                for (int m = 0; m < M; ++m) {
-                    const double2 zz = sz[m];
+                const double du = u - 0.5 * (kc.lo[ci] + kc.hi[ci]);
+                const double *P = sP + (size_t)ci * M;
+                const double S2 = zsum_f64(phi, phi_direct, sz, M, [&](int m) {
                     const double2 tt = st[m];
-                    const double p = exp(tt.x - tt.y * Fc - at * zz.x);
-                    const double amp = p * zz.y * sinc_d(0.5 * phi * zz.y);
-                    double sn, cs;
-                    sincos(phi * zz.x, &sn, &cs);
-                    Sr += amp * cs;
-                    Si += amp * sn;
-                }
-                sum += rw.w * W * (Sr * Sr + Si * Si) * array_factor_d(phi, qp);
+                    return ci < ncp ? P[m] * exp_small(-tt.y * du) : exp(tt.x - tt.y * Fc - at * sz[m].x);
+                });
+                sum += rw.w * W * S2 * array_factor_d(phi, qp);
             }
             acc += kc.mult * sum;
             __syncthreads();
@@ -500,7 +511,8 @@ size_t fwd_smem(int n_steps, int block)
 cudaError_t launch_quad(const QuadParams &qp, int precision, int num_sms, int block, cudaStream_t st)
 {
     int nb = 0, tiles = qp.n_items;
-    size_t smem = (size_t)qp.n_steps * 2 * sizeof(double2) + (size_t)qp.G * sizeof(RowD);
+    size_t smem = (size_t)qp.n_steps * (2 * sizeof(double2) + f64_cand(qp.n_steps, qp.G) * sizeof(double)) +
+                  (size_t)qp.G * sizeof(RowD);
     const void *fn = (const void *)k_quad_f64;
     if (precision == 0) {
         fn = (const void *)k_quad_f32;

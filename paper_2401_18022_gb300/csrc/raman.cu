@@ -162,24 +162,6 @@ __device__ __forceinline__ void ode_window(cg::cluster_group &cl, OdeWindow &win
     }
 }
 
-// e^x: Taylor to x^11 for |x| <= 1/8 (remainder 3e-20), else the library's
-__device__ __forceinline__ double exp_small(double x)
-{
-    if (fabs(x) > 0.125) return exp(x);
-    double p = 1.0 / 39916800.0;
-    p = fma(p, x, 1.0 / 3628800.0);
-    p = fma(p, x, 1.0 / 362880.0);
-    p = fma(p, x, 1.0 / 40320.0);
-    p = fma(p, x, 1.0 / 5040.0);
-    p = fma(p, x, 1.0 / 720.0);
-    p = fma(p, x, 1.0 / 120.0);
-    p = fma(p, x, 1.0 / 24.0);
-    p = fma(p, x, 1.0 / 6.0);
-    p = fma(p, x, 0.5);
-    p = fma(p, x, 1.0);
-    return fma(p, x, 1.0);
-}
-
 // dy/dz of the lane's channel, P its power e^y (0 for an empty slot)
 __device__ __forceinline__ double ode_rhs(cg::cluster_group &cl, OdeWindow &win, const OdeLane &L,
                                           const RamanParams &rp, int &buf, double P)
@@ -533,7 +515,7 @@ __global__ void __launch_bounds__(256) k_quad_f64_tab(QuadParams qp)
     extern __shared__ double2 smem_d2[];
     const int M = qp.n_steps, G = qp.G;
     double2 *sz = smem_d2;                              // [M] {z_m, dz_m}
-    double2 *sQ = sz + M;                               // [nc_max][M][2] {A, Sa}, {Sb, 0}
+    double2 *sQ = sz + M;                               // [nc_max][M][2] {A, Sa}, {Sb, e^A}
     RowD *rows = reinterpret_cast<RowD *>(sQ + (size_t)2 * qp.nc_max * M);
     __shared__ PieceConst<double> kc;
     __shared__ double s_d0[2];
@@ -541,6 +523,7 @@ __global__ void __launch_bounds__(256) k_quad_f64_tab(QuadParams qp)
     __shared__ int s_item;
 
     for (int m = threadIdx.x; m < M; m += blockDim.x) sz[m] = qp.zs_d[m];
+    const double phi_direct = kF64Direct / qp.dz_max;
     const double c3 = kPi * qp.beta3;
     const double c4 = 2.0 * kPi * kPi / 3.0 * qp.beta4;
 
@@ -572,8 +555,9 @@ __global__ void __launch_bounds__(256) k_quad_f64_tab(QuadParams qp)
                     const double2 ta = T[(size_t)pc.a * M + m], tb = T[(size_t)pc.b * M + m];
                     const double2 ti = T[(size_t)pc.cut * M + m], tc = T[(size_t)c * M + m];
                     const double D = (fa + fb) - (fic + qp.ch_frel[coff + c]);
-                    sQ[2 * t] = make_double2(0.5 * (ta.x + tb.x + tc.x - ti.x + tc.y * D), 0.5 * (ta.y + tc.y));
-                    sQ[2 * t + 1] = make_double2(0.5 * (tb.y + tc.y), 0.0);
+                    const double A = 0.5 * (ta.x + tb.x + tc.x - ti.x + tc.y * D);
+                    sQ[2 * t] = make_double2(A, 0.5 * (ta.y + tc.y));
+                    sQ[2 * t + 1] = make_double2(0.5 * (tb.y + tc.y), exp(A));
                 }
             }
             __syncthreads();
@@ -601,18 +585,11 @@ __global__ void __launch_bounds__(256) k_quad_f64_tab(QuadParams qp)
                                   c4 * (f1 * f1 + 1.5 * f1 * f2 + 3.0 * fi * u + f2 * f2 + 3.0 * fi * fi);
                 const double phi = -4.0 * kPi * kPi * f1 * f2 * br;
                 const double2 *Q = sQ + (size_t)2 * ci * M;
-                double Sr = 0.0, Si = 0.0;
-                for (int m = 0; m < M; ++m) {
-                    const double2 zz = sz[m];
+                const double S2 = zsum_f64(phi, phi_direct, sz, M, [&](int m) {
                     const double2 q0 = Q[2 * m], q1 = Q[2 * m + 1];
-                    const double p = exp(q0.x + q0.y * da + q1.x * db);
-                    const double amp = p * zz.y * sinc_d(0.5 * phi * zz.y);
-                    double sn, cs;
-                    sincos(phi * zz.x, &sn, &cs);
-                    Sr += amp * cs;
-                    Si += amp * sn;
-                }
-                sum += rw.w * W * (Sr * Sr + Si * Si) * array_factor_d(phi, qp);
+                    return q1.y * exp_small(q0.y * da + q1.x * db);
+                });
+                sum += rw.w * W * S2 * array_factor_d(phi, qp);
             }
             acc += kc.mult * sum;
             __syncthreads();
