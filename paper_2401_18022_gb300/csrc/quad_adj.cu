@@ -35,7 +35,7 @@ namespace isrs {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kAdjSlots = 256;   // node slots of a chunk
+constexpr int kAdjSlots = 512;   // node slots of a chunk
 constexpr int kAdjCand = 3;      // F_c candidates swept together (most pieces have two)
 constexpr float kPadLog2 = -1000.0f;   // log2 weight of the padding steps (ex2 -> 0)
 using AdjNodes = WarpNodes<kAdjSlots>;
@@ -149,11 +149,12 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
                     v2 += c == 2 ? val : 0.0f;
                 };
                 int small;
-                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int nq) {
+                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int c0, int nq) {
                     for (int q0 = 32 * part; q0 < nq; q0 += 32 * parts) {
                         Node nd;
                         int cls = -1;
-                        if (q0 + lane < nq && node_get(ns, qp.gauss, q0 + lane, nd)) {
+                        if (q0 + lane < nq) {
+                            node_get(ns, qp.gauss, c0, q0 + lane, nd);
                             const float aphi = fabsf(nd.phi);
                             cls = aphi <= phi_direct ? 0 : 1;
                             n_small += aphi <= phi_small ? nd.N : 0;

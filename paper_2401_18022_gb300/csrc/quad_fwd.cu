@@ -196,7 +196,7 @@ cudaError_t gauss_array(void **out) { return cudaGetSymbolAddress(out, g_isrs_ga
 // ---------------------------------------------------------------------------
 // k_quad_f32: persistent FP32 quadrature.
 // ---------------------------------------------------------------------------
-constexpr int kFwdSlots = 256;       // node slots of a chunk
+constexpr int kFwdSlots = 512;       // node slots of a chunk
 constexpr int kFwdCand = 3;          // F_c candidates swept together (most pieces have two)
 using FwdNodes = WarpNodes<kFwdSlots>;
 
@@ -261,10 +261,10 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
                 }
                 __syncwarp();
                 int small;
-                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int nq) {
+                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int c0, int nq) {
                     for (int q = lane + 32 * part; q < nq; q += 32 * parts) {
                         Node nd;
-                        if (!node_get(ns, qp.gauss, q, nd)) continue;
+                        node_get(ns, qp.gauss, c0, q, nd);
                         const int ci = dbg_clamp(nd.ci, g.nc, kDbgCand, qp.dbg);
                         const float aphi = fabsf(nd.phi);
                         const float dF = (nd.x + nd.y) - 0.5f * (g.lo[ci] + g.hi[ci]);

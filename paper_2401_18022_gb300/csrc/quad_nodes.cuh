@@ -48,7 +48,7 @@ constexpr int kGaussMaxNodes = 48;
 constexpr int kGaussMenu = 18;
 constexpr int kGaussPerN = 297;                        // nodes of all rules of one N
 constexpr int kGaussEntries = kGaussMaxN * kGaussPerN;
-constexpr int kNodeMin = 2;                            // slots a run takes at least
+constexpr int kRowRuns = 4;                            // runs of a row listed at a time
 
 __host__ __device__ constexpr int gauss_nodes(int k)
 {
@@ -118,7 +118,7 @@ struct __align__(16) NodeRun {
     float jc;                   // centre column, from the row's centre
     float half;                 // N / 2
     int toff;                   // first entry of the rule; -1: the N columns themselves
-    unsigned id;                // first slot | candidate << 12 | row << 17 | row of a block << 31
+    unsigned id;                // first slot of the warp's rows | candidate << 16 | nodes << 24
 };
 
 struct RowBlock {
@@ -127,10 +127,9 @@ struct RowBlock {
 
 template <int Cap>
 struct WarpNodes {
-    static constexpr int kSpan = Cap - kGaussMaxNodes;    // slots a chunk starts runs in
     NodeRow row[32];
-    NodeRun run[Cap / kNodeMin];
-    unsigned short of[Cap];     // run of each slot (0xffff: none)
+    NodeRun run[32 * kRowRuns];         // [row][run]
+    unsigned char of[Cap];              // run of each slot of the chunk
     RowBlock blk[kBlkMax];
     PieceGeo geo;
 };
@@ -245,9 +244,21 @@ __device__ __forceinline__ void row_slopes(const PieceGeo &g, const NodeRow &o, 
     p2 = cv * g.c4;
 }
 
-// e^d - 1 and e^{-d} - 1, both to FP32 relative accuracy
+// e^d - 1 and e^{-d} - 1, both to FP32 relative accuracy: cosh d - 1 +- sinh d
+// by their Taylor series for |d| <= 0.6 (remainders below 2e-11), which covers all
+// rows but those of the CUT's own cell.
 __device__ __forceinline__ void expm1_pair(float d, float &ep, float &em)
 {
+    if (fabsf(d) <= 0.6f) {
+        const float x = d * d;
+        const float sh = d * fmaf(x, fmaf(x, fmaf(x, fmaf(x, 1.0f / 362880.0f, 1.0f / 5040.0f), 1.0f / 120.0f),
+                                          1.0f / 6.0f), 1.0f);
+        const float ch = x * fmaf(x, fmaf(x, fmaf(x, fmaf(x, 1.0f / 3628800.0f, 1.0f / 40320.0f), 1.0f / 720.0f),
+                                          1.0f / 24.0f), 0.5f);
+        ep = ch + sh;
+        em = ch - sh;
+        return;
+    }
     const float E = expm1f(fabsf(d));
     const float En = __fdividef(-E, 1.0f + E);
     ep = d >= 0.0f ? E : En;
@@ -284,14 +295,21 @@ __device__ __forceinline__ void row_runs(const PieceGeo &g, const NodeRow &o, in
         if (jb <= ja) continue;
         const bool up = (g.s1 > 0.0f) == (part == 1 || g.s1 != g.s2);
         const float ua = u_at(ja), ub = u_at(jb - 1);
-        // first column of [ja, jb) at or past edge e in the direction of travel
+        // first column of [ja, jb) at or past edge e in the direction of travel (ja
+        // is before it, jb - 1 at or past it or nothing is): the column a straight
+        // line between the ends gives and a neighbour of it usually bracket it (u
+        // is nearly linear on most rows), bisection does the rest
+        const float slope = __fdividef((float)(jb - 1 - ja), ub - ua);
         const auto first = [&](float e) {
-            int lo = ja, hi = jb;
-            while (lo < hi) {
-                const int m = (lo + hi) >> 1;
-                const float u = m == ja ? ua : m == jb - 1 ? ub : u_at(m);
-                if (up ? u >= e : u < e) hi = m;
+            int lo = ja + 1, hi = jb;
+            int m = (int)fminf(fmaxf(ceilf((e - ua) * slope), 1.0f), (float)(jb - 1 - ja)) + ja;
+            for (int it = 0; lo < hi; ++it) {
+                const float u = m == jb - 1 ? ub : u_at(m);
+                const bool past = up ? u >= e : u < e;
+                if (past) hi = m;
                 else lo = m + 1;
+                m = it > 0 ? (lo + hi) >> 1 : past ? m - 1 : m + 1;
+                m = max(lo, min(m, hi - 1));
             }
             return lo;
         };
@@ -464,42 +482,34 @@ __device__ __forceinline__ void unit_row(const WarpNodes<Cap> &ns, const float2 
     o.w *= wt;
 }
 
-// The runs of unit `row` of the warp's 32 (candidates [ca, cb); whole >= 0:
-// the one candidate that holds every column): returns the slots they take.
-// With c0 >= 0 also writes those whose first slot (counted from `off`) falls in
-// [c0, c0 + kSpan), and marks the rest of the window [c0, c0 + Cap) that the
-// row covers as empty.  One function for both, never inlined, so that the
-// counting and the writing pass evaluate every edge with the same instructions.
+// Lists runs [first, first + kRowRuns) of unit `row` of the warp's 32 (candidates
+// [ca, cb); whole >= 0: the one candidate that holds every column), their slots
+// counted from 0; returns the slots, `more` whether further runs follow.
 template <int Cap>
-__device__ __noinline__ int node_emit(WarpNodes<Cap> &ns, int G, int row, int ca, int cb, int whole, int off, int c0)
+__device__ __forceinline__ int node_emit(WarpNodes<Cap> &ns, const NodeRow &o, int G, int row, int ca, int cb,
+                                         int whole, int first, bool &more)
 {
-    constexpr int span = WarpNodes<Cap>::kSpan;
-    const NodeRow o = ns.row[row];
-    if (o.w == 0.0f) return 0;
-    const int off0 = off;
+    int slots = 0, k = 0;
     const auto take_run = [&](int c, int j0, int N) {
         run_parts(ns.geo, o, G, j0, N, [&](int j, int Ns, int n) {
-            const int take = max(n, kNodeMin);
-            if (c0 >= 0) {
-                const bool here = off >= c0 && off < c0 + span;
-                const int s = off - c0, id = s / kNodeMin;  // runs start >= kNodeMin slots apart
-                if (here) {
-                    NodeRun r;
-                    r.jc = (float)j + 0.5f * (float)(Ns - G);
-                    r.half = 0.5f * (float)Ns;
-                    r.toff = n == Ns ? -1 : (Ns - 1) * kGaussPerN + gauss_offset(gauss_pick(n));
-                    r.id = (unsigned)s | (unsigned)c << 12 | (unsigned)row << 17 | (whole >= 0 ? 1u << 31 : 0u);
-                    ns.run[id] = r;
-                }
-                for (int q = max(s, 0); q < min(s + take, Cap); ++q)
-                    ns.of[q] = here && q - s < n ? (unsigned short)id : 0xffff;
+            if (k >= first && k < first + kRowRuns) {
+                NodeRun r;
+                r.jc = (float)j + 0.5f * (float)(Ns - G);
+                r.half = 0.5f * (float)Ns;
+                r.toff = n == Ns ? -1 : (Ns - 1) * kGaussPerN + gauss_offset(gauss_pick(n));
+                r.id = (unsigned)slots | (unsigned)c << 16 | (unsigned)n << 24;
+                ns.run[row * kRowRuns + (k - first)] = r;
+                slots += n;
             }
-            off += take;
+            ++k;
         });
     };
-    if (whole >= 0) take_run(whole, 0, G);
-    else row_runs(ns.geo, o, G, ca, cb, take_run);
-    return off - off0;
+    if (o.w != 0.0f) {
+        if (whole >= 0) take_run(whole, 0, G);
+        else row_runs(ns.geo, o, G, ca, cb, take_run);
+    }
+    more = k > first + kRowRuns;
+    return slots | min(max(k - first, 0), kRowRuns) << 16;
 }
 
 // One node: its row, candidate, f1 and f2 from the corner, phi and weight.
@@ -509,14 +519,13 @@ struct Node {
 };
 
 template <int Cap>
-__device__ __forceinline__ bool node_get(const WarpNodes<Cap> &ns, const float2 *gauss, int q, Node &nd)
+__device__ __forceinline__ void node_get(const WarpNodes<Cap> &ns, const float2 *gauss, int c0, int q, Node &nd)
 {
-    const unsigned id = ns.of[q];
-    if (id == 0xffffu) return false;
+    const int id = ns.of[q];
     const NodeRun r = ns.run[id];
-    const int k = q - (int)(r.id & 0xfffu);
-    nd.ci = (int)(r.id >> 12 & 31u);
-    nd.N = k == 0 && !(r.id >> 31) ? (int)(2.0f * r.half) : 0;
+    const int k = c0 + q - (int)(r.id & 0xffffu);
+    nd.ci = (int)(r.id >> 16 & 31u);
+    nd.N = k == 0 && !(r.id >> 21 & 1u) ? (int)(2.0f * r.half) : 0;
     float pos, wt = 1.0f;
     if (r.toff >= 0) {
         const float2 e = __ldg(gauss + r.toff + k);
@@ -526,7 +535,7 @@ __device__ __forceinline__ bool node_get(const WarpNodes<Cap> &ns, const float2 
         pos = r.jc - r.half + 0.5f + (float)k;
     }
     const PieceGeo &g = ns.geo;
-    const NodeRow o = ns.row[r.id >> 17 & 31u];
+    const NodeRow o = ns.row[id / kRowRuns];
     float ep, em, p1, p2;
     expm1_pair(pos * o.du2, ep, em);
     row_slopes(g, o, p1, p2);
@@ -538,10 +547,9 @@ __device__ __forceinline__ bool node_get(const WarpNodes<Cap> &ns, const float2 
     const float t = __fadd_rn(nd.phi, -o.phi0);
     nd.phi_lo = __fadd_rn(__fadd_rn(o.phi0, -__fadd_rn(nd.phi, -t)), __fadd_rn(dphi, -t)) + o.phi0_lo;
     nd.wq = o.w * wt;
-    return true;
 }
 
-// The nodes of a piece in chunks: f(number of slots) is called by the whole
+// The nodes of a piece in chunks: f(c0, number of slots) is called by the whole
 // warp for each chunk, with ns filled for node_get.  small gets the columns of
 // the rows taken in blocks.
 template <int Cap, typename F>
@@ -553,31 +561,46 @@ __device__ __forceinline__ void piece_nodes(WarpNodes<Cap> &ns, const float2 *ga
     const int nv = row_blocks(ns, G, R1, nblk, cand);
     const bool mine = cand >= ca && cand < cb;        // the blocks' candidate belongs to this sweep
     small = mine ? R1 * G : 0;
-    const int first = mine ? 0 : nv;
     const int units = nv + (G - R1);
-    for (int u0 = first; u0 < units; u0 += 32) {
+    for (int u0 = mine ? 0 : nv; u0 < units; u0 += 32) {
         const int q = u0 + lane;
-        int slots = 0, whole = -1;
+        const int whole = q < nv ? cand : -1;
+        NodeRow o;
+        o.w = 0.0f;
         if (q < units) {
-            NodeRow o;
             unit_row(ns, gauss, G, q, nv, R1, nblk, o);
             ns.row[lane] = o;
-            whole = q < nv ? cand : -1;
-            slots = node_emit(ns, G, lane, ca, cb, whole, 0, -1);
         }
-        int incl = slots;
+        bool more = false;
+        int first = 0;
+        do {
+            const int got = node_emit(ns, o, G, lane, ca, cb, whole, first, more);
+            const int slots = got & 0xffff, runs = got >> 16;
+            int incl = slots;
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int v = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += v;
-        }
-        const int total = __shfl_sync(0xffffffffu, incl, 31), base = incl - slots;
-        for (int c0 = 0; c0 < total; c0 += WarpNodes<Cap>::kSpan) {
-            if (slots > 0 && base < c0 + Cap && incl > c0) node_emit(ns, G, lane, ca, cb, whole, base, c0);
-            __syncwarp();
-            f(min(total - c0, Cap));
-            __syncwarp();
-        }
+            for (int d = 1; d < 32; d <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, d);
+                if (lane >= d) incl += v;
+            }
+            const int total = __shfl_sync(0xffffffffu, incl, 31), base = incl - slots;
+            for (int k = 0; k < runs; ++k) {          // slots of the warp's rows; bit 21: a block's row
+                unsigned &id = ns.run[lane * kRowRuns + k].id;
+                id = id + (unsigned)base + (whole >= 0 ? 1u << 21 : 0u);
+            }
+            for (int c0 = 0; c0 < total; c0 += Cap) {
+                if (base < c0 + Cap && incl > c0)
+                    for (int k = 0; k < runs; ++k) {
+                        const unsigned id = ns.run[lane * kRowRuns + k].id;
+                        const int s0 = (int)(id & 0xffffu) - c0, s1 = s0 + (int)(id >> 24);
+                        for (int s = max(s0, 0); s < min(s1, Cap); ++s)
+                            ns.of[s] = (unsigned char)(lane * kRowRuns + k);
+                    }
+                __syncwarp();
+                f(c0, min(total - c0, Cap));
+                __syncwarp();
+            }
+            first += kRowRuns;
+        } while (__any_sync(0xffffffffu, more));
     }
 }
 

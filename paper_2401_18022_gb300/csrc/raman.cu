@@ -398,7 +398,7 @@ cudaError_t launch_raman_adj(const RamanAdjParams &ap, cudaStream_t st)
 // ---------------------------------------------------------------------------
 // Quadratures with the tabulated profile.
 // ---------------------------------------------------------------------------
-constexpr int kTabSlots = 192;       // node slots of a chunk
+constexpr int kTabSlots = 512;       // node slots of a chunk
 constexpr int kTabCand = 2;          // F_c candidates swept together (most pieces have two)
 using TabNodes = WarpNodes<kTabSlots>;
 
@@ -466,10 +466,10 @@ __global__ void __launch_bounds__(256, 4) k_quad_f32_tab(QuadParams qp)
                 if (lane == 0) g.tilt = tilt;
                 __syncwarp();
                 int small;
-                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int nq) {
+                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int c0, int nq) {
                     for (int q = lane + 32 * part; q < nq; q += 32 * parts) {
                         Node nd;
-                        if (!node_get(ns, qp.gauss, q, nd)) continue;
+                        node_get(ns, qp.gauss, c0, q, nd);
                         const int ci = dbg_clamp(nd.ci, g.nc, kDbgCand, qp.dbg);
                         const float aphi = fabsf(nd.phi);
                         const float dl = tp.ol + nd.x, dd = tp.od + nd.y;

@@ -43,7 +43,7 @@ namespace isrs {
 namespace {
 
 constexpr unsigned kFullT = 0xffffffffu;
-constexpr int kTabAdjSlots = 256;   // node slots of a chunk
+constexpr int kTabAdjSlots = 512;   // node slots of a chunk
 constexpr float kPadLog2T = -1000.0f;
 
 // Half-warp walks of a node (weight cp = mult w W af, phi float-float, in-channel
@@ -223,12 +223,14 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
                     sum = t;
                 };
                 int small;
-                piece_nodes(ns, qp.gauss, G, cc, cc + 1, small, [&](int nq) {
+                piece_nodes(ns, qp.gauss, G, cc, cc + 1, small, [&](int c0, int nq) {
                     for (int q0 = 32 * part; q0 < nq; q0 += 32 * parts) {
                         Node nd;
                         int cls = -1;
-                        if (q0 + lane < nq && node_get(ns, qp.gauss, q0 + lane, nd))
+                        if (q0 + lane < nq) {
+                            node_get(ns, qp.gauss, c0, q0 + lane, nd);
                             cls = fabsf(nd.phi) <= phi_direct ? 0 : 1;
+                        }
                         const unsigned bd = __ballot_sync(kFullT, cls == 0), bt = __ballot_sync(kFullT, cls == 1);
                         if (cls >= 0) {
                             const int at = cls == 0 ? __popc(bd & lt_mask) : 31 - __popc(bt & lt_mask);
