@@ -1086,30 +1086,30 @@ isrs_status run_forward(isrs_handle h, const isrs_fibre *fb, Geom *g, int precis
             qm.partial = (double *)h->partial_mci.p;
             qm.counter = (int *)h->counter.p + 1;
             if (tab) {
-                // the MCI cells with the tabulated profile: FP32 rows of {a, b}, cells in chunks
-                int cpc = 0;
+                // the MCI cells with the tabulated profile: FP32 rows of {a, b}
+                int mblock = block;
                 if (precision == ISRS_PREC_FP32) {
-                    cpc = quad_mci_tab_cells(M, qm.mci_n_max, qm.G, block);
-                    if (cpc < 1)
+                    mblock = quad_mci_tab_block(M, qm.mci_n_max, qm.G, block);
+                    if (mblock < 32)
                         return fail(h, ISRS_ERR_UNSUPPORTED, "MCI step rows of %d steps exceed shared memory", M);
                     const size_t nab = (size_t)g->total_prof_ch * M;
                     if (nab > (size_t)INT32_MAX)
                         return fail(h, ISRS_ERR_UNSUPPORTED, "profile tables of %zu entries exceed the MCI conversion", nab);
-                    if ((s = ensure(h, h->ab_f, sizeof(float2) * nab)) != ISRS_OK) return s;
-                    qm.ab_f = (const float2 *)h->ab_f.p;
+                    if ((s = ensure(h, h->ab_f, sizeof(float4) * (size_t)g->total_prof_ch * ((M + 1) / 2))) != ISRS_OK)
+                        return s;
+                    qm.ab_f = (const float4 *)h->ab_f.p;
                     TabHalfParams hp;
                     hp.ab = (const double2 *)h->ab.p;
-                    hp.abf = (float2 *)h->ab_f.p;
+                    hp.abf = (float4 *)h->ab_f.p;
                     hp.plan_n = qm.plan_n;
                     hp.prof_plan = qm.prof_plan;
                     hp.prof_ch_off = qm.prof_ch_off;
                     hp.n_steps = M;
                     CK(launch_tab_half_log2(hp, g->n_prof, qm.mci_n_max, h->num_sms, st));
                 }
-                qm.mci_cpc = cpc;
-                int mgrid = h->num_sms * quad_mci_tab_blocks_per_sm(precision, M, qm.mci_n_max, cpc, block);
+                int mgrid = h->num_sms * quad_mci_tab_blocks_per_sm(precision, M, qm.mci_n_max, qm.G, mblock);
                 if (g->n_mci_items < mgrid) mgrid = g->n_mci_items;
-                CK(launch_quad_mci_tab(qm, precision, mgrid, block, st));
+                CK(launch_quad_mci_tab(qm, precision, mgrid, mblock, st));
             } else {
                 int mgrid = h->num_sms * quad_mci_blocks_per_sm(precision, M, qm.mci_n_max, block);
                 if (g->n_mci_items < mgrid) mgrid = g->n_mci_items;

@@ -23,10 +23,10 @@ struct PrepParams {
     double *kap_L;              // kappa(L) per profile (the largest ISRS exponent slope)
 };
 
-// FP32 copy of the profile tables for the MCI cells (steps outermost)
+// FP32 copy of the profile tables for the MCI cells (pairs of steps outermost)
 struct TabHalfParams {
     const double2 *ab;
-    float2 *abf;
+    float4 *abf;
     const int *plan_n, *prof_plan, *prof_ch_off;
     int n_steps;
 };
@@ -186,11 +186,11 @@ size_t quad_mci_smem_bytes(int precision, int n_steps, int n_max);
 int quad_mci_blocks_per_sm(int precision, int n_steps, int n_max, int block);
 cudaError_t launch_quad_mci(const QuadParams &qp, int precision, int grid, int block, cudaStream_t st);
 // ... with the tabulated (Raman-ODE) profile: qp.ab (FP64 kernel) or qp.ab_f
-// (FP32 kernel, filled by launch_tab_half_log2) and qp.mci_cpc cells per chunk
-// (quad_mci_tab_cells; 0: the step rows do not fit shared memory)
-int quad_mci_tab_cells(int n_steps, int n_max, int G, int block);
-size_t quad_mci_tab_smem_bytes(int precision, int n_steps, int n_max, int cpc);
-int quad_mci_tab_blocks_per_sm(int precision, int n_steps, int n_max, int cpc, int block);
+// (FP32 kernel, filled by launch_tab_half_log2); quad_mci_tab_block: the block
+// the FP32 kernel runs with (0: its step rows do not fit shared memory)
+int quad_mci_tab_block(int n_steps, int n_max, int G, int block);
+size_t quad_mci_tab_smem_bytes(int precision, int n_steps, int n_max, int G, int block);
+int quad_mci_tab_blocks_per_sm(int precision, int n_steps, int n_max, int G, int block);
 cudaError_t launch_tab_half_log2(const TabHalfParams &hp, int n_prof, int max_n, int n_sms, cudaStream_t st);
 cudaError_t launch_quad_mci_tab(const QuadParams &qp, int precision, int grid, int block, cudaStream_t st);
 // adjoint over the MCI cells of a separate grid (closed-form profile)

@@ -20,6 +20,7 @@
 
 #include <algorithm>
 
+#include "f32x2.cuh"
 #include "isrs_internal.cuh"
 #include "isrs_kernels.h"
 #include "quad_cells.cuh"
@@ -30,131 +31,155 @@ namespace isrs {
 
 namespace {
 
-constexpr int kMciTabCells = 32;   // cells per chunk at most (their step rows share the block's memory)
+constexpr int kMciCells = 6;       // cells of a group at most
+constexpr int kMciList = 96;       // points waiting: telescoped from the front, direct from the back (31 + 31 + 32)
+constexpr int kMciRows = 32;       // rows of a group
 
-// {1/2 log2(e) a_c(m), 1/2 log2(e) b_c(m)} in FP32, steps outermost: entry
-// prof_ch_off[p] M + m n + c.  Neighbouring points of a chunk have F_c in
-// neighbouring channels, so a warp's 32 rows at one step lie in one or two
-// lines; with the channel outermost (as qp.ab) every lane read its own sector
-// and the loads bound the kernel.  One block row per profile.
+// Cells a warp takes together: about 32 grid rows.
+__host__ __device__ constexpr int mci_group(int G) { return G >= 32 ? 1 : (32 / G < kMciCells ? 32 / G : kMciCells); }
+
+// Steps go in pairs: pair k holds steps 2k, 2k + 1 (an odd last one beside a step
+// of weight 2^-1000 and the same edge).
+__host__ __device__ constexpr int step_pairs(int n_steps) { return (n_steps + 1) / 2; }
+
+// {1/2 log2(e) a_c, 1/2 log2(e) b_c} in FP32, steps outermost: float4 {a, a', b,
+// b'} of pair k and channel c at prof_ch_off[p] pairs + k n + c.  Neighbouring
+// points of a group have F_c in neighbouring channels, so a warp's 32 rows of one
+// pair lie in a few lines; with the channel outermost (as qp.ab) every lane read
+// its own sector and the loads bound the kernel.  One block row per profile.
 __global__ void __launch_bounds__(256) k_tab_half_log2(TabHalfParams hp)
 {
-    const int p = blockIdx.y, n = hp.plan_n[hp.prof_plan[p]], M = hp.n_steps;
-    const size_t off = (size_t)hp.prof_ch_off[p] * M;
-    for (int t = threadIdx.x + blockIdx.x * blockDim.x; t < n * M; t += blockDim.x * gridDim.x) {
-        const int m = t / n, c = t - m * n;
-        const double2 v = hp.ab[off + (size_t)c * M + m];
-        hp.abf[off + t] = make_float2((float)(0.5 * kLog2e * v.x), (float)(0.5 * kLog2e * v.y));
+    const int p = blockIdx.y, n = hp.plan_n[hp.prof_plan[p]], M = hp.n_steps, M2 = step_pairs(M);
+    const double2 *ab = hp.ab + (size_t)hp.prof_ch_off[p] * M;
+    float4 *out = hp.abf + (size_t)hp.prof_ch_off[p] * M2;
+    for (int t = threadIdx.x + blockIdx.x * blockDim.x; t < n * M2; t += blockDim.x * gridDim.x) {
+        const int k = t / n, c = t - k * n;
+        const double2 v = ab[(size_t)c * M + 2 * k], w = ab[(size_t)c * M + min(2 * k + 1, M - 1)];
+        const double h = 0.5 * kLog2e;
+        out[t] = make_float4((float)(h * v.x), (float)(h * w.x), (float)(h * v.y), (float)(h * w.y));
     }
 }
 
-// FP32 z-sums of Eq. slow_vary with
-//   log2 p_m (dz_m) = Q.x + Q.y da + Q.z db + T.x + T.y dc   (Q.w for the
-// telescoped form, without log2 dz), T the F_c channel's row at Tc + m n; sA[m] = {z, z^2 + dz^2/12, log2 dz, dz},
-// sB[m] = {z_{m+1}/2pi hi, lo, ., .}.
-__device__ __forceinline__ float lp_tab(const float4 &q, float qx, const float2 &t, float da, float db, float dc)
+// One warp's shared memory; the step rows of the group's cells follow it.
+struct __align__(16) MciWarp {
+    float4 row[kMciRows];            // {xc, yc, du2, w P_a P_b / (B_a B_b)}
+    float4 Lp[kMciList];             // {phi, da, db, dc}
+    float2 Lw[kMciList];             // {w W, cell << 16 | channel}
+    int4 cell[kMciCells];            // {a, b, first and last channel F_c can fall in}
+};
+
+__host__ __device__ constexpr size_t mci_warp_bytes(int n_steps, int G)
 {
-    float lp = fmaf(q.y, da, qx);
-    lp = fmaf(q.z, db, lp);
-    lp = fmaf(t.y, dc, lp);
-    return lp + t.x;
+    // per cell float4 {A, A', Sa, Sa'} and float2 {Sb, Sb'} of every pair, the
+    // pitches odd so that the cells of a warp sit in different banks
+    return sizeof(MciWarp) + ((size_t)mci_group(G) * (step_pairs(n_steps) | 1) * 24 + 15) / 16 * 16;
 }
 
-__device__ __forceinline__ float zsum_small_mt(float phi, float da, float db, float dc, const float4 *Q,
-                                               const float2 *Tc, int n, const float4 *sA, int M)
+// |S|^2 of Eq. slow_vary, telescoped, two steps at a time: log2 p = A + Sa da +
+// Sb db + T.a + T.b dc, eB[k] = {edge/2pi hi, hi', lo, lo'}, T the F_c channel's
+// row at Tc + k n.
+__device__ __forceinline__ float zsum_tele_mt(float phi, float da, float db, float dc, const float4 *Qa,
+                                              const float2 *Qb, const float4 *Tc, int n, const float4 *eB, int M2)
 {
-    float M0 = 0.0f, M1 = 0.0f, M2 = 0.0f;
+    const f32x2 ph = dup2(phi), nph = dup2(-phi), a2 = dup2(da), b2 = dup2(db), c2 = dup2(dc);
+    float Er = 1.0f, Ei = 0.0f;
+    f32x2 Sr = dup2(0.0f), Si = dup2(0.0f);
 #pragma unroll 4
-    for (int m = 0; m < M; ++m) {
-        const float4 q = Q[m];
-        const float4 a = sA[m];
-        const float w = ex2_approx(lp_tab(q, q.x, __ldg(Tc + m * n), da, db, dc));   // p_m dz_m
-        M0 += w;
-        M1 = fmaf(w, a.x, M1);
-        M2 = fmaf(w, a.y, M2);
+    for (int k = 0; k < M2; ++k) {
+        const float4 e = eB[k], q = Qa[k], t = __ldg(Tc + k * n);
+        const float2 qb = Qb[k];
+        float s0, c0, s1, c1, l0, l1;
+        sincos_turn2(rev_fraction2<true>(ph, nph, ph, pack2(e.x, e.y), pack2(e.z, e.w)), s0, c0, s1, c1);
+        f32x2 lp = fma2(pack2(q.z, q.w), a2, pack2(q.x, q.y));
+        lp = fma2(pack2(qb.x, qb.y), b2, lp);
+        lp = fma2(pack2(t.z, t.w), c2, lp);
+        unpack2(add2(lp, pack2(t.x, t.y)), l0, l1);
+        const f32x2 p = pack2(ex2_approx(l0), ex2_approx(l1));
+        Sr = fma2(p, pack2(c0 - Er, c1 - c0), Sr);
+        Si = fma2(p, pack2(s0 - Ei, s1 - s0), Si);
+        Er = c1;
+        Ei = s1;
     }
-    return fmaf(-phi * phi, fmaf(M0, M2, -M1 * M1), M0 * M0);
+    float r0, r1, i0, i1;
+    unpack2(Sr, r0, r1);
+    unpack2(Si, i0, i1);
+    const float sr = r0 + r1, si = i0 + i1;
+    return __fdividef(sr * sr + si * si, phi * phi);
 }
 
-__device__ __forceinline__ float zsum_direct_mt(float phi, float da, float db, float dc, const float4 *Q,
-                                                const float2 *Tc, int n, const float4 *sA, int M)
+// ... in the direct form (few points): zA[m] = {z, dz}
+__device__ __forceinline__ float zsum_direct_mt(float phi, float da, float db, float dc, const float4 *Qa,
+                                                const float2 *Qb, const float4 *Tc, int n, const float2 *zA, int M)
 {
     float Sr = 0.0f, Si = 0.0f;
     const float hphi = 0.5f * phi;
     const float phir = phi * 0.15915494309189535f;
-#pragma unroll 4
     for (int m = 0; m < M; ++m) {
-        const float4 q = Q[m];
-        const float4 a = sA[m];
+        const int k = m >> 1, o = m & 1;
+        const float4 q = Qa[k], t = __ldg(Tc + k * n);
+        const float2 a = zA[m];
         float sn, cs;
         sincos_rev(phir, a.x, sn, cs);
-        const float x = hphi * a.w;
+        const float x = hphi * a.y;
         const float x2 = x * x;
         float sc = fmaf(x2, -2.5052108e-8f, 2.7557319e-6f);   // -1/11!, 1/9!
         sc = fmaf(x2, sc, -1.9841270e-4f);                     // -1/7!
         sc = fmaf(x2, sc, 8.3333333e-3f);                      // 1/5!
         sc = fmaf(x2, sc, -1.6666667e-1f);                     // -1/3!
         sc = fmaf(x2, sc, 1.0f);
-        const float amp = ex2_approx(lp_tab(q, q.x, __ldg(Tc + m * n), da, db, dc)) * sc;   // p_m dz_m sinc
+        float lp = fmaf(o ? q.w : q.z, da, o ? q.y : q.x);
+        lp = fmaf(o ? Qb[k].y : Qb[k].x, db, lp);
+        lp = fmaf(o ? t.w : t.z, dc, lp) + (o ? t.y : t.x);
+        const float amp = ex2_approx(lp) * (sc * a.y);        // p_m dz_m sinc
         Sr = fmaf(amp, cs, Sr);
         Si = fmaf(amp, sn, Si);
     }
     return Sr * Sr + Si * Si;
 }
 
-__device__ __forceinline__ float zsum_tele_mt(float phi, float da, float db, float dc, const float4 *Q,
-                                              const float2 *Tc, int n, const float4 *sB, int M)
-{
-    float Er = 1.0f, Ei = 0.0f, Sr = 0.0f, Si = 0.0f;
-#pragma unroll 4
-    for (int m = 0; m < M; ++m) {
-        const float4 q = Q[m];
-        const float4 e = sB[m];
-        float sn, cs;
-        phasor_rev_ff_wide(phi, e.x, e.y, sn, cs);
-        const float p = ex2_approx(lp_tab(q, q.w, __ldg(Tc + m * n), da, db, dc));
-        Sr = fmaf(p, cs - Er, Sr);
-        Si = fmaf(p, sn - Ei, Si);
-        Er = cs;
-        Ei = sn;
-    }
-    return __fdividef(Sr * Sr + Si * Si, phi * phi);
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// k_quad_mci_f32_tab: persistent over MCI work items (cell ranges of one
-// CUT).  The item's cells are taken in chunks of qp.mci_cpc: the chunk's
-// cells are decoded once, their step rows built (FP32, from the FP32 profile
-// tables), then one thread per (cell, grid row) walks the row's G_mci points.
+// k_quad_mci_f32_tab: persistent over MCI work items (cell ranges of one CUT),
+// one block per item, its cells shared by the warps in turns of 32.  Per turn a
+// lane tests one cell (F_c may fall outside every channel: 42 % of the cells of
+// the 557-ch plan), and the warp takes the rest in groups of about 32 grid rows:
+// step rows of the cells, then grid rows, then points, which go to a list per
+// z-sum form and are summed 32 at a time, one per lane.  No barrier inside an
+// item.  Bound by the XU pipe (20 cycles per warp and step) and the issue of the
+// other ~16 instructions.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
 {
     extern __shared__ float4 smem_f4[];
-    const int M = qp.n_steps, G = qp.G, CPC = qp.mci_cpc;
-    float4 *sA = smem_f4;                              // [M] {z, z^2 + dz^2/12, log2 dz, dz}
-    float4 *sB = sA + M;                               // [M] {edge/2pi hi, lo, ., .}
-    float4 *sQ = sB + M;                               // [CPC][M | 1] {A + log2 dz, Sa, Sb, A}
-    const int MS = M | 1;                              // row pitch: the cells of a warp in different banks
-    float *rel = reinterpret_cast<float *>(sQ + (size_t)CPC * MS);  // [n] channel centre - f_i
+    const int M = qp.n_steps, G = qp.G, M2 = step_pairs(M), MS = M2 | 1, GC = mci_group(G);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    float4 *eB = smem_f4;                              // [M2] {edge/2pi hi, hi', lo, lo'}
+    float2 *zA = reinterpret_cast<float2 *>(eB + M2);  // [2 M2] {z, dz}
+    unsigned char *mine = reinterpret_cast<unsigned char *>(zA + 2 * M2) + mci_warp_bytes(M, G) * warp;
+    MciWarp &w = *reinterpret_cast<MciWarp *>(mine);
+    float4 *Qa = reinterpret_cast<float4 *>(mine + sizeof(MciWarp));       // [GC][MS]
+    float2 *Qb = reinterpret_cast<float2 *>(Qa + (size_t)GC * MS);         // [GC][MS]
+    float *rel = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(zA + 2 * M2) +
+                                           mci_warp_bytes(M, G) * nw);     // [n] channel centre - f_i
     float *hb = rel + qp.mci_n_max;                    // [n] B/2
-    float *pd = hb + qp.mci_n_max;                     // [n] P/B
-    __shared__ int2 sCell[kMciTabCells];
     __shared__ double scratch[32];
     __shared__ int s_item;
 
-    for (int m = threadIdx.x; m < M; m += blockDim.x) {
-        sA[m] = qp.zs_a[m];
-        sB[m] = qp.zs_b[m];
+    for (int k = threadIdx.x; k < M2; k += blockDim.x) {
+        const int m0 = 2 * k, m1 = min(2 * k + 1, M - 1);
+        const float4 b0 = qp.zs_b[m0], b1 = qp.zs_b[m1];
+        eB[k] = make_float4(b0.x, b1.x, b0.y, b1.y);
+        zA[m0] = make_float2(qp.zs_a[m0].x, qp.zs_a[m0].w);
+        zA[2 * k + 1] = make_float2(qp.zs_a[m1].x, qp.zs_a[m1].w);
     }
     const float c3 = (float)(kPi * qp.beta3);
     const float c4 = (float)(2.0 * kPi * kPi / 3.0 * qp.beta4);
     const float b2 = (float)qp.beta2;
     const float m4pi2 = (float)(-4.0 * kPi * kPi);
     const float phi_direct = 3.14159265f / qp.dz_max;
-    const float phi_small = 0.02f / qp.L;
     const float eps = (float)qp.eps_v1;
+    const unsigned lt_mask = (1u << lane) - 1u;
     int cur_prof = -1, cur_cut = -1;
 
     for (;;) {
@@ -174,80 +199,152 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
             for (int c = threadIdx.x; c < n; c += blockDim.x) {
                 rel[c] = (float)(qp.ch_frel[coff + c] - fi);
                 hb[c] = (float)(0.5 * qp.ch_B[coff + c]);
-                pd[c] = qp.pd_f[poff + c];
             }
             cur_prof = item.prof;
             cur_cut = i;
         }
-        const float2 *T = qp.ab_f + (size_t)poff * M;   // this profile's channel rows
+        __syncthreads();
+        const float4 *T = qp.ab_f + (size_t)poff * M2;   // this profile's channel rows
+        const float *pd = qp.pd_f + poff;                // [n] P/B
         const float fi = (float)qp.ch_frel[coff + i];
         const float three_fi2 = 3.0f * fi * fi;
         const int n2 = n - 1;
         float sum = 0.0f, comp = 0.0f;
-        for (int t0 = item.piece0; t0 < item.piece1; t0 += CPC) {
-            const int ncc = min(CPC, item.piece1 - t0);
-            __syncthreads();                          // the previous chunk's rows are no longer read
-            if (threadIdx.x < ncc) {
+        int nl[2] = {0, 0};                              // list lengths (direct, telescoped)
+        // one list's first 32 points (or what is left), one per lane
+        const auto flush = [&](int f) {
+            const int cnt = min(nl[f], 32);
+            __syncwarp();
+            const int at = f ? lane : kMciList - 1 - lane, step = f ? cnt : -cnt;
+            if (lane < cnt) {
+                const float4 v = w.Lp[at];
+                const float2 u = w.Lw[at];
+                const int cc = __float_as_int(u.y) >> 16, c = __float_as_int(u.y) & 0xffff;
+                const float S2 = f ? zsum_tele_mt(v.x, v.y, v.z, v.w, Qa + cc * MS, Qb + cc * MS, T + c, n, eB, M2)
+                                   : zsum_direct_mt(v.x, v.y, v.z, v.w, Qa + cc * MS, Qb + cc * MS, T + c, n, zA, M);
+                const float y = u.x * S2 * array_factor_f(v.x, qp) - comp;
+                const float t = sum + y;
+                comp = (t - sum) - y;
+                sum = t;
+            }
+            __syncwarp();
+            nl[f] -= cnt;
+            if (lane < nl[f]) {                          // at most 31 stay
+                w.Lp[at] = w.Lp[at + step];
+                w.Lw[at] = w.Lw[at + step];
+            }
+            __syncwarp();
+        };
+        for (int t0 = item.piece0 + 32 * warp; t0 < item.piece1; t0 += 32 * nw) {
+            // one cell per lane: can F_c fall in a channel?
+            int a = 0, b = 0, c0 = 0, c1 = -1;
+            if (t0 + lane < item.piece1) {
                 int ap, bp;
-                tri_decode(t0 + threadIdx.x, n2, ap, bp);
-                sCell[threadIdx.x] = make_int2(dbg_clamp(ap + (ap >= i), n, kDbgCell, qp.dbg),
-                                               dbg_clamp(bp + (bp >= i), n, kDbgCell, qp.dbg));
-            }
-            __syncthreads();
-            for (int e = threadIdx.x; e < ncc * M; e += blockDim.x) {
-                const int m = e / ncc, cc = e - m * ncc;
-                const int2 ab = sCell[cc];
-                const float2 *Tm = T + (size_t)m * n;
-                const float2 ta = Tm[ab.x], tb = Tm[ab.y];
-                const float A = (ta.x + tb.x) - Tm[i].x;
-                sQ[cc * MS + m] = make_float4(A + sA[m].z, ta.y, tb.y, A);
-            }
-            __syncthreads();
-            for (int q = threadIdx.x; q < ncc * G; q += blockDim.x) {
-                const int cc = q / G, r = q - cc * G;
-                const int2 ab = sCell[cc];
-                const int a = ab.x, b = ab.y;
-                const float mult = a == b ? 1.0f : 2.0f;
-                const float ra = rel[a], rb = rel[b];
-                const float s1 = ra > 0.0f ? 1.0f : -1.0f, s2 = rb > 0.0f ? 1.0f : -1.0f;
-                const float xlo = fabsf(ra) - hb[a], xhi = fabsf(ra) + hb[a];
-                const float ylo = fabsf(rb) - hb[b], yhi = fabsf(rb) + hb[b];
-                // row r of the cell's hyperbolic grid
-                const float u1hi = xhi * yhi;
-                const float llo = logf(fmaxf(xlo * ylo, eps * u1hi));
-                const float ds = (logf(u1hi) - llo) / (float)G;
-                const float u1 = expf(fmaf((float)r + 0.5f, ds, llo));
-                const float ymin = fmaxf(ylo, u1 / xhi), ymax = fminf(yhi, u1 / xlo);
-                if (!(ymax > ymin)) continue;
-                const float du2 = log1pf((ymax - ymin) / ymin) / (float)G;
-                const float yc = sqrtf(ymin * ymax), xc = u1 / yc;
-                const float w = u1 * ds * du2 * mult;
-                const float Wab = pd[a] * pd[b];
-                const float4 *Q = sQ + (size_t)cc * MS;
-                for (int j = 0; j < G; ++j) {
-                    const float d = ((float)j + 0.5f - 0.5f * (float)G) * du2;
-                    const float ex = expf(d);
-                    const float f1 = s1 * (xc * ex), f2 = s2 * (yc * __frcp_rn(ex));
-                    const float u = f1 + f2;
-                    const int c = channel_of(rel, hb, n, u);
-                    if (c < 0) continue;
-                    const float W = Wab * pd[c];
-                    if (W == 0.0f) continue;
-                    const float da = f1 - ra, db = f2 - rb, dc = u - rel[c];
-                    const float br = b2 + c3 * (u + 2.0f * fi) +
-                                     c4 * (f1 * f1 + 1.5f * f1 * f2 + 3.0f * fi * u + f2 * f2 + three_fi2);
-                    const float phi = m4pi2 * f1 * f2 * br;
-                    const float aphi = fabsf(phi);
-                    const float2 *Tc = T + c;
-                    float S2;
-                    if (aphi <= phi_small) S2 = zsum_small_mt(phi, da, db, dc, Q, Tc, n, sA, M);
-                    else if (aphi <= phi_direct) S2 = zsum_direct_mt(phi, da, db, dc, Q, Tc, n, sA, M);
-                    else S2 = zsum_tele_mt(phi, da, db, dc, Q, Tc, n, sB, M);
-                    const float y = w * W * S2 * array_factor_f(phi, qp) - comp;
-                    const float t = sum + y;
-                    comp = (t - sum) - y;
-                    sum = t;
+                tri_decode(t0 + lane, n2, ap, bp);
+                a = dbg_clamp(ap + (ap >= i), n, kDbgCell, qp.dbg);
+                b = dbg_clamp(bp + (bp >= i), n, kDbgCell, qp.dbg);
+                if (pd[a] * pd[b] != 0.0f) {
+                    // a little wider than the cell, the points decide
+                    const float uc = rel[a] + rel[b], r = 1.0001f * (hb[a] + hb[b]) + 1e-5f * fabsf(uc) + 1e-6f;
+                    int lo = 0, hi = n;                  // first channel ending above uc - r
+                    while (lo < hi) {
+                        const int m = (lo + hi) >> 1;
+                        if (rel[m] + hb[m] > uc - r) hi = m;
+                        else lo = m + 1;
+                    }
+                    c0 = lo;
+                    c1 = lo - 1;
+                    while (c1 + 1 < n && rel[c1 + 1] - hb[c1 + 1] <= uc + r) ++c1;
                 }
+            }
+            unsigned todo = __ballot_sync(0xffffffffu, c1 >= c0);
+            while (todo) {
+                int ncc = 0;
+                for (; ncc < GC && todo; ++ncc) {        // the next cells, in order
+                    const int src = __ffs(todo) - 1;
+                    if (lane == src) w.cell[ncc] = make_int4(a, b, c0, c1);
+                    todo &= todo - 1;
+                }
+                __syncwarp();
+                // step rows of the cells
+                for (int e = lane; e < ncc * M2; e += 32) {
+                    const int k = e / ncc, cc = e - k * ncc;
+                    const int4 cl = w.cell[cc];
+                    const float4 *Tk = T + (size_t)k * n;
+                    const float4 ta = Tk[cl.x], tb = Tk[cl.y], ti = Tk[i];
+                    float4 q = make_float4((ta.x + tb.x) - ti.x, (ta.y + tb.y) - ti.y, ta.z, ta.w);
+                    if (2 * k + 1 >= M) q.y = -1000.0f;
+                    Qa[cc * MS + k] = q;
+                    Qb[cc * MS + k] = make_float2(tb.z, tb.w);
+                }
+                // grid rows
+                for (int e = lane; e < ncc * G; e += 32) {
+                    const int cc = e / G, r = e - cc * G;
+                    const int4 cl = w.cell[cc];
+                    const float mult = cl.x == cl.y ? 1.0f : 2.0f;
+                    const float ra = fabsf(rel[cl.x]), rb = fabsf(rel[cl.y]);
+                    const float xlo = ra - hb[cl.x], xhi = ra + hb[cl.x];
+                    const float ylo = rb - hb[cl.y], yhi = rb + hb[cl.y];
+                    const float u1hi = xhi * yhi;
+                    const float llo = logf(fmaxf(xlo * ylo, eps * u1hi));
+                    const float ds = (logf(u1hi) - llo) / (float)G;
+                    const float u1 = expf(fmaf((float)r + 0.5f, ds, llo));
+                    const float ymin = fmaxf(ylo, u1 / xhi), ymax = fminf(yhi, u1 / xlo);
+                    float4 o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    if (ymax > ymin) {
+                        o.z = log1pf((ymax - ymin) / ymin) / (float)G;
+                        o.y = sqrtf(ymin * ymax);
+                        o.x = u1 / o.y;
+                        o.w = u1 * ds * o.z * mult * (pd[cl.x] * pd[cl.y]);
+                    }
+                    w.row[e] = o;
+                }
+                __syncwarp();
+                for (int q0 = 0; q0 < ncc * G * G; q0 += 32) {
+                    const int q = q0 + lane;
+                    int cls = -1, ci = -1, cc = 0;
+                    float phi = 0.0f, da = 0.0f, db = 0.0f, dc = 0.0f, W = 0.0f;
+                    if (q < ncc * G * G) {
+                        const int rr = q / G, j = q - rr * G;
+                        cc = rr / G;
+                        const float4 o = w.row[rr];
+                        if (o.w != 0.0f) {
+                            const int4 cl = w.cell[cc];
+                            const float ra = rel[cl.x], rb = rel[cl.y];
+                            const float s1 = ra > 0.0f ? 1.0f : -1.0f, s2 = rb > 0.0f ? 1.0f : -1.0f;
+                            const float d = ((float)j + 0.5f - 0.5f * (float)G) * o.z;
+                            const float ex = expf(d);
+                            const float f1 = s1 * (o.x * ex), f2 = s2 * (o.y * __frcp_rn(ex));
+                            const float u = f1 + f2;
+                            for (int c = cl.z; c <= cl.w; ++c)
+                                if (rel[c] - hb[c] <= u && u < rel[c] + hb[c]) ci = c;
+                            if (ci >= 0) {
+                                W = o.w * pd[ci];
+                                da = f1 - ra;
+                                db = f2 - rb;
+                                dc = u - rel[ci];
+                                const float br = b2 + c3 * (u + 2.0f * fi) +
+                                                 c4 * (f1 * f1 + 1.5f * f1 * f2 + 3.0f * fi * u + f2 * f2 + three_fi2);
+                                phi = m4pi2 * f1 * f2 * br;
+                                if (W != 0.0f) cls = fabsf(phi) <= phi_direct ? 0 : 1;
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int f = 0; f < 2; ++f) {
+                        const unsigned m = __ballot_sync(0xffffffffu, cls == f);
+                        if (cls == f) {
+                            const int e = nl[f] + __popc(m & lt_mask), at = f ? e : kMciList - 1 - e;
+                            w.Lp[at] = make_float4(phi, da, db, dc);
+                            w.Lw[at] = make_float2(W, __int_as_float(cc << 16 | ci));
+                        }
+                        nl[f] += __popc(m);
+                        if (nl[f] >= 32) flush(f);
+                    }
+                }
+                // the next group replaces the step rows
+                for (int f = 0; f < 2; ++f)
+                    if (nl[f] > 0) flush(f);
             }
         }
         const double tot = block_sum_d((double)sum - (double)comp, scratch);
@@ -354,20 +451,19 @@ __global__ void __launch_bounds__(256) k_quad_mci_f64_tab(QuadParams qp)
     }
 }
 
-size_t quad_mci_tab_smem_bytes(int precision, int n_steps, int n_max, int cpc)
+size_t quad_mci_tab_smem_bytes(int precision, int n_steps, int n_max, int G, int block)
 {
     if (precision == 0)
-        return ((size_t)n_steps * 2 + (size_t)(n_steps | 1) * cpc) * sizeof(float4) + (size_t)n_max * 3 * sizeof(float);
+        return (size_t)step_pairs(n_steps) * 32 + mci_warp_bytes(n_steps, G) * (block / 32) +
+               (size_t)n_max * 2 * sizeof(float);
     return (size_t)n_steps * (sizeof(double2) + sizeof(double));
 }
 
-int quad_mci_tab_cells(int n_steps, int n_max, int G, int block)
+// Warps of a block: as many of the asked ones as shared memory holds (0: none)
+int quad_mci_tab_block(int n_steps, int n_max, int G, int block)
 {
-    const size_t fixed = (size_t)n_steps * 2 * sizeof(float4) + (size_t)n_max * 3 * sizeof(float);
-    const size_t budget = 200 * 1024;
-    if (fixed >= budget) return 0;
-    const int by_mem = (int)((budget - fixed) / ((size_t)(n_steps | 1) * sizeof(float4)));
-    return std::min(std::min(kMciTabCells, block / std::max(1, G)), by_mem);
+    while (block > 0 && quad_mci_tab_smem_bytes(0, n_steps, n_max, G, block) > 200 * 1024) block -= 32;
+    return block;
 }
 
 static void *mci_tab_fn(int precision)
@@ -375,10 +471,10 @@ static void *mci_tab_fn(int precision)
     return precision == 0 ? (void *)k_quad_mci_f32_tab : (void *)k_quad_mci_f64_tab;
 }
 
-int quad_mci_tab_blocks_per_sm(int precision, int n_steps, int n_max, int cpc, int block)
+int quad_mci_tab_blocks_per_sm(int precision, int n_steps, int n_max, int G, int block)
 {
     int nb = 0;
-    const size_t smem = quad_mci_tab_smem_bytes(precision, n_steps, n_max, cpc);
+    const size_t smem = quad_mci_tab_smem_bytes(precision, n_steps, n_max, G, block);
     void *fn = mci_tab_fn(precision);
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, fn, block, smem);
@@ -387,14 +483,14 @@ int quad_mci_tab_blocks_per_sm(int precision, int n_steps, int n_max, int cpc, i
 
 cudaError_t launch_tab_half_log2(const TabHalfParams &hp, int n_prof, int max_n, int n_sms, cudaStream_t st)
 {
-    const int grid = std::max(1, std::min((max_n * hp.n_steps + 255) / 256, 4 * n_sms));
+    const int grid = std::max(1, std::min((max_n * step_pairs(hp.n_steps) + 255) / 256, 4 * n_sms));
     k_tab_half_log2<<<dim3(grid, n_prof), 256, 0, st>>>(hp);
     return cudaGetLastError();
 }
 
 cudaError_t launch_quad_mci_tab(const QuadParams &qp, int precision, int grid, int block, cudaStream_t st)
 {
-    const size_t smem = quad_mci_tab_smem_bytes(precision, qp.n_steps, qp.mci_n_max, qp.mci_cpc);
+    const size_t smem = quad_mci_tab_smem_bytes(precision, qp.n_steps, qp.mci_n_max, qp.G, block);
     void *fn = mci_tab_fn(precision);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
