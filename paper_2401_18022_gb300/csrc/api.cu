@@ -1066,9 +1066,7 @@ isrs_status run_forward(isrs_handle h, const isrs_fibre *fb, Geom *g, int precis
             am.item_R = (double2 *)h->gA.p + (size_t)g->n_items * M;
             am.V = (double *)h->gPd.p + (size_t)g->n_items * n_ch;
             am.item_slot = (const int *)g->item_slot_all.p + g->n_items;
-            int mgrid = h->num_sms * adjoint_mci_blocks_per_sm(M, am.q.mci_n_max, block);
-            if (g->n_mci_items < mgrid) mgrid = g->n_mci_items;
-            CK(launch_adjoint_mci(am, mgrid, block, st));
+            CK(launch_adjoint_mci(am, h->num_sms, block, st));
         }
         if ((s = mark(h, 1, 1, st)) != ISRS_OK) return s;
     } else {

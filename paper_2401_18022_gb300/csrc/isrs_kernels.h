@@ -194,9 +194,7 @@ int quad_mci_tab_blocks_per_sm(int precision, int n_steps, int n_max, int G, int
 cudaError_t launch_tab_half_log2(const TabHalfParams &hp, int n_prof, int max_n, int n_sms, cudaStream_t st);
 cudaError_t launch_quad_mci_tab(const QuadParams &qp, int precision, int grid, int block, cudaStream_t st);
 // adjoint over the MCI cells of a separate grid (closed-form profile)
-size_t adjoint_mci_smem_bytes(int n_steps, int n_max, int block);
-int adjoint_mci_blocks_per_sm(int n_steps, int n_max, int block);
-cudaError_t launch_adjoint_mci(const AdjParams &ap, int grid, int block, cudaStream_t st);
+cudaError_t launch_adjoint_mci(const AdjParams &ap, int num_sms, int block, cudaStream_t st);
 cudaError_t launch_adjoint(const AdjParams &ap, int num_sms, int block, cudaStream_t st);
 cudaError_t launch_chain(const ChainParams &cp, cudaStream_t st);
 

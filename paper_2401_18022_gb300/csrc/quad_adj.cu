@@ -15,9 +15,9 @@
 // k_quad_adj evaluates the forward sum and these buckets in one pass over the
 // nodes of the row sums (quad_nodes.cuh; the bucket terms have the band limit of
 // |S|^2, so the nodes that sum a row sum its derivatives too), and every step
-// term of Eq. slow_vary is evaluated once: a node is walked by a half-warp, each
-// of the 16 lanes owning K = ceil(M/16) consecutive steps (112 = 16 x 7),
-// computes their terms t_m into registers, the half sums them with shuffles into
+// term of Eq. slow_vary is evaluated once: a node is walked by a half-warp (quad_walk.cuh), each
+// of the 16 lanes owning 2 K2 consecutive steps computes their terms t_m into
+// registers, the half sums them with shuffles into
 // S, and the same registers give d|S|^2/d ln p_m = 2 Re(conj(S) t_m) for the
 // lane's own step buckets, which stay in registers between FP64 folds.
 #include <cuda_runtime.h>
@@ -37,24 +37,23 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kAdjSlots = 512;   // node slots of a chunk
 constexpr int kAdjCand = 3;      // F_c candidates swept together (most pieces have two)
-constexpr float kPadLog2 = -1000.0f;   // log2 weight of the padding steps (ex2 -> 0)
 using AdjNodes = WarpNodes<kAdjSlots>;
 
 // One warp's shared memory: nodes, the points to walk, step rows per
 // candidate, FP64 step buckets.
-template <int K>
+template <int K2>
 struct __align__(16) AdjWarp {
     AdjNodes ns;
     float4 L[32];                // {w W af, phi, phi_lo, u}
     int Lc[32];                  // candidate, from the sweep's first
-    float2 ek[kAdjCand][K * 16]; // {log2 p at f_c, K2}, [k][lane of the half]
-    double2 B[K * 16];
+    float4 ek[kAdjCand][K2 * 16];   // {log2 p at f_c (2), slope K2 (2)} of a pair, [k][lane of the half]
+    double2 B[2 * K2 * 16];         // [step of the lane][lane]
 };
 
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// k_quad_adj<K>: fused forward + adjoint, persistent over work tiles of one
+// k_quad_adj<K2>: fused forward + adjoint, persistent over work tiles of one
 // profile; every warp takes its own tiles.  Per batch of 32 slots a warp sets up
 // one node per lane, lists the direct ones from the front and the telescoped
 // ones from the back, and walks them two at a time, one per half-warp (an odd
@@ -65,27 +64,22 @@ struct __align__(16) AdjWarp {
 // order), so results are bit for bit reproducible.
 // ---------------------------------------------------------------------------
 #ifndef ISRS_ADJ_MIN_BLOCKS
-#define ISRS_ADJ_MIN_BLOCKS 3   // resident blocks per SM the register budget is sized for
+#define ISRS_ADJ_MIN_BLOCKS 2   // resident blocks per SM the register budget is sized for (3 spill, 4 more so)
 #endif
 
-template <int K>
+template <int K2>
 __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams ap)
 {
     const QuadParams &qp = ap.q;
     extern __shared__ float4 smem_f4[];
     const int M = qp.n_steps, G = qp.G;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int l16 = lane & 15, half = lane >> 4;       // lane l owns steps [K (l mod 16), K (l mod 16) + K)
-    float4 *zt = smem_f4;                              // [K][16] {edge/2pi hi, lo, z, dz}
-    AdjWarp<K> &w = reinterpret_cast<AdjWarp<K> *>(zt + K * 16)[warp];
+    const int l16 = lane & 15, half = lane >> 4;
+    float4 *ze = smem_f4, *zd = ze + K2 * 16;          // walk_tables
+    AdjWarp<K2> &w = reinterpret_cast<AdjWarp<K2> *>(zd + K2 * 16)[warp];
     AdjNodes &ns = w.ns;
 
-    // padding steps past M repeat the last edge
-    for (int t = threadIdx.x; t < K * 16; t += blockDim.x) {
-        const int m = min((t & 15) * K + (t >> 4), M - 1);
-        const float4 za = qp.zs_a[m], zb = qp.zs_b[m];
-        zt[t] = make_float4(zb.x, zb.y, za.x, za.w);
-    }
+    walk_tables<K2>(qp, ze, zd);
     __syncthreads();
     const float phi_direct = 3.14159265f / qp.dz_max;
     const float phi_small = kBlkPhiL / qp.L;
@@ -105,7 +99,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
         const int part = item.part & 0xffff, parts = item.part >> 16;
         double *Vrow = ap.V + (size_t)it * ap.n_ch;     // this tile's PSD buckets
         for (int c = lane; c < ap.n_ch; c += 32) Vrow[c] = 0.0;
-        for (int t = lane; t < K * 16; t += 32) w.B[t] = make_double2(0.0, 0.0);
+        for (int t = lane; t < 2 * K2 * 16; t += 32) w.B[t] = make_double2(0.0, 0.0);
         double acc = 0.0;                               // lane 0
         for (int kp = item.piece0; kp < item.piece1; ++kp) {
             const DevPiece &pc = qp.pieces[dbg_clamp(kp, qp.n_pieces, kDbgPiece, qp.dbg)];
@@ -114,23 +108,26 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
             __syncwarp();
             const PieceGeo &g = ns.geo;
             const float mult = g.mult;
-            float R[K], Rp[K];
+            f32x2 R[K2], Rp[K2];
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                R[k] = 0.0f;
-                Rp[k] = 0.0f;
-            }
+            for (int k = 0; k < K2; ++k) R[k] = Rp[k] = dup2(0.0f);
             double ptot = 0.0;
             for (int ca = 0; ca < g.nc; ca += kAdjCand) {
                 const int cb = min(g.nc, ca + kAdjCand);
                 for (int c = ca; c < cb; ++c) {
                     const float at = g.at_ab + g.hat[c], F = g.Fc0 + 0.5f * (g.lo[c] + g.hi[c]);
-                    for (int t = lane; t < K * 16; t += 32) {
-                        const int m = (t & 15) * K + (t >> 4);
-                        float2 e = make_float2(kPadLog2, 0.0f);
+                    for (int t = lane; t < K2 * 16; t += 32) {
+                        const int m = walk_step<K2>(t >> 4, t & 15, 0);
+                        float4 e = make_float4(kPadLog2, kPadLog2, 0.0f, 0.0f);
                         if (m < M) {
                             const float2 v = st[m];
-                            e = make_float2(fmaf(v.y, F, fmaf(-at, zt[t].z, v.x)), v.y);
+                            e.x = fmaf(v.y, F, fmaf(-at, zd[t].x, v.x));
+                            e.z = v.y;
+                        }
+                        if (m + 1 < M) {
+                            const float2 v = st[m + 1];
+                            e.y = fmaf(v.y, F, fmaf(-at, zd[t].y, v.x));
+                            e.w = v.y;
                         }
                         w.ek[c - ca][t] = e;
                     }
@@ -171,25 +168,37 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
                         }
                         __syncwarp();
                         const int nd0 = __popc(bd), nt0 = __popc(bt);
-                        for (int p = 0; p < nd0; p += 2) {
-                            const int at = min(p + half, nd0 - 1);
-                            const float4 v = w.L[at];
-                            const int c = w.Lc[at];
-                            const float wq = p + half < nd0 ? v.x : 0.0f;
-                            const float dF = v.w - 0.5f * (g.lo[ca + c] + g.hi[ca + c]);
-                            const float val = walk_direct_n<K>(zt + l16, w.ek[c] + l16, wq, v.y, dF, g.Fc0 + v.w,
-                                                               mult, R, Rp);
-                            add(l16 == 0 ? val : 0.0f, c);
-                        }
-                        for (int p = 0; p < nt0; p += 2) {
-                            const int at = 31 - min(p + half, nt0 - 1);
-                            const float4 v = w.L[at];
-                            const int c = w.Lc[at];
-                            const float wq = p + half < nt0 ? v.x : 0.0f;
-                            const float dF = v.w - 0.5f * (g.lo[ca + c] + g.hi[ca + c]);
-                            const float val = walk_tele_n<K>(zt + l16, w.ek[c] + l16, l16, wq, v.y, v.z, dF,
-                                                             g.Fc0 + v.w, mult, R, Rp);
-                            add(l16 == 0 ? val : 0.0f, c);
+                        for (int f = 0; f < 2; ++f) {
+                            const int cnt = f ? nt0 : nd0;
+                            for (int p = 0; p < cnt; p += 2) {
+                                const int e = min(p + half, cnt - 1), at = f ? 31 - e : e;
+                                const float4 v = w.L[at];
+                                const int c = w.Lc[at];
+                                const float wq = p + half < cnt ? v.x : 0.0f;
+                                const f32x2 dF = dup2(v.w - 0.5f * (g.lo[ca + c] + g.hi[ca + c]));
+                                const float4 *ek = w.ek[c] + l16;
+                                const auto lp = [&](int k) {
+                                    const float4 x = ek[k * 16];
+                                    return fma2(pack2(x.z, x.w), dF, pack2(x.x, x.y));
+                                };
+                                f32x2 tr[K2], ti[K2];
+                                float sr, si, sq = wq;
+                                if (f) {
+                                    walk_tele<K2, false>(ze + l16, l16, v.y, v.z, lp, tr, ti, sr, si);
+                                    sq *= __fdividef(1.0f, v.y * v.y);
+                                } else {
+                                    walk_direct<K2>(zd + l16, v.y, lp, tr, ti, sr, si);
+                                }
+                                const f32x2 c2 = dup2(2.0f * mult * sq), cF = dup2(2.0f * mult * sq * (g.Fc0 + v.w));
+                                const f32x2 sr2 = dup2(sr), si2 = dup2(si);
+#pragma unroll
+                                for (int k = 0; k < K2; ++k) {
+                                    const f32x2 rr = walk_term<K2>(tr, ti, k, sr2, si2);
+                                    R[k] = fma2(c2, rr, R[k]);
+                                    Rp[k] = fma2(cF, rr, Rp[k]);
+                                }
+                                add(l16 == 0 ? sq * fmaf(sr, sr, si * si) : 0.0f, c);
+                            }
                         }
                         __syncwarp();
                     }
@@ -217,21 +226,25 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
                 atomicAdd(&Vrow[dbg_clamp(pc.b, ap.n_ch, kDbgVrow, qp.dbg)], ptot);
             }
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                const float rx = R[k] + __shfl_xor_sync(kFull, R[k], 16);
-                const float ry = Rp[k] + __shfl_xor_sync(kFull, Rp[k], 16);
-                if (half == 0) {
-                    double2 &d = w.B[k * 16 + l16];
-                    d.x += (double)rx;
-                    d.y += (double)ry;
-                }
+            for (int k = 0; k < K2; ++k) {
+                float x0, x1, y0, y1;
+                unpack2(R[k], x0, x1);
+                unpack2(Rp[k], y0, y1);
+                x0 += __shfl_xor_sync(kFull, x0, 16);
+                x1 += __shfl_xor_sync(kFull, x1, 16);
+                y0 += __shfl_xor_sync(kFull, y0, 16);
+                y1 += __shfl_xor_sync(kFull, y1, 16);
+                // each half folds one place of the pair
+                double2 &d = w.B[(2 * k + half) * 16 + l16];
+                d.x += (double)(half ? x1 : x0);
+                d.y += (double)(half ? y1 : y0);
             }
         }
         // tile outputs: the forward partial and the step buckets
         if (lane == 0) qp.partial[it] = acc;
         __syncwarp();
         for (int m = lane; m < M; m += 32) {
-            const int ln = m / K, kk = m - ln * K;
+            const int ln = m / (2 * K2), kk = m - ln * 2 * K2;
             ap.item_R[(size_t)it * M + m] = w.B[kk * 16 + ln];
         }
         __syncwarp();
@@ -439,19 +452,19 @@ __global__ void __launch_bounds__(256) k_chain_ch(ChainParams cp)
 // ---------------------------------------------------------------------------
 namespace {
 
-template <int K>
+template <int K2>
 cudaError_t launch_adj_k(const AdjParams &ap, int num_sms, int block, cudaStream_t st)
 {
     if (ap.q.n_items < num_sms * (block / 32)) block = 32;      // too few tiles for full blocks on every SM
     const int nw = block / 32;
-    const size_t smem = sizeof(float4) * K * 16 + sizeof(AdjWarp<K>) * nw;
-    cudaError_t e = cudaFuncSetAttribute(k_quad_adj<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = sizeof(float4) * 2 * K2 * 16 + sizeof(AdjWarp<K2>) * nw;
+    cudaError_t e = cudaFuncSetAttribute(k_quad_adj<K2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_quad_adj<K>, block, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_quad_adj<K2>, block, smem);
     if (e != cudaSuccess) return e;
     const int grid = std::max(1, std::min((ap.q.n_items + nw - 1) / nw, num_sms * std::max(1, nb)));
-    k_quad_adj<K><<<grid, block, smem, st>>>(ap);
+    k_quad_adj<K2><<<grid, block, smem, st>>>(ap);
     return cudaGetLastError();
 }
 
@@ -459,15 +472,11 @@ cudaError_t launch_adj_k(const AdjParams &ap, int num_sms, int block, cudaStream
 
 cudaError_t launch_adjoint(const AdjParams &ap, int num_sms, int block, cudaStream_t st)
 {
-    switch ((ap.q.n_steps + 15) / 16) {
+    switch ((ap.q.n_steps + 31) / 32) {
     case 1: return launch_adj_k<1>(ap, num_sms, block, st);
     case 2: return launch_adj_k<2>(ap, num_sms, block, st);
     case 3: return launch_adj_k<3>(ap, num_sms, block, st);
     case 4: return launch_adj_k<4>(ap, num_sms, block, st);
-    case 5: return launch_adj_k<5>(ap, num_sms, block, st);
-    case 6: return launch_adj_k<6>(ap, num_sms, block, st);
-    case 7: return launch_adj_k<7>(ap, num_sms, block, st);
-    case 8: return launch_adj_k<8>(ap, num_sms, block, st);
     }
     return cudaErrorInvalidValue;
 }

@@ -32,10 +32,11 @@ namespace isrs {
 namespace {
 
 constexpr int kMciCells = 6;       // cells of a group at most
+constexpr int kMciUnits = 6;       // step rows of a group: one per cell and F_c channel
 constexpr int kMciList = 96;       // points waiting: telescoped from the front, direct from the back (31 + 31 + 32)
 constexpr int kMciRows = 32;       // rows of a group
 
-// Cells a warp takes together: about 32 grid rows.
+// Cells a warp takes together: at most 32 grid rows (and kMciUnits step rows).
 __host__ __device__ constexpr int mci_group(int G) { return G >= 32 ? 1 : (32 / G < kMciCells ? 32 / G : kMciCells); }
 
 // Steps go in pairs: pair k holds steps 2k, 2k + 1 (an odd last one beside a step
@@ -63,37 +64,35 @@ __global__ void __launch_bounds__(256) k_tab_half_log2(TabHalfParams hp)
 // One warp's shared memory; the step rows of the group's cells follow it.
 struct __align__(16) MciWarp {
     float4 row[kMciRows];            // {xc, yc, du2, w P_a P_b / (B_a B_b)}
-    float4 Lp[kMciList];             // {phi, da, db, dc}
-    float2 Lw[kMciList];             // {w W, cell << 16 | channel}
-    int4 cell[kMciCells];            // {a, b, first and last channel F_c can fall in}
+    float4 Lp[kMciList];             // {phi, da, db, w W}
+    int Lu[kMciList];                // step row
+    int4 cell[kMciCells];            // {a | b << 16, first F_c channel, last, step row of the first}
+    int2 unit[kMciUnits];            // {cell, F_c channel} of each step row
 };
 
-__host__ __device__ constexpr size_t mci_warp_bytes(int n_steps, int G)
+__host__ __device__ constexpr size_t mci_warp_bytes(int n_steps)
 {
-    // per cell float4 {A, A', Sa, Sa'} and float2 {Sb, Sb'} of every pair, the
-    // pitches odd so that the cells of a warp sit in different banks
-    return sizeof(MciWarp) + ((size_t)mci_group(G) * (step_pairs(n_steps) | 1) * 24 + 15) / 16 * 16;
+    // per step row float4 {A, A', Sa, Sa'} and float2 {Sb, Sb'} of every pair, the
+    // pitches odd so that the rows of a warp's points sit in different banks
+    return sizeof(MciWarp) + ((size_t)kMciUnits * (step_pairs(n_steps) | 1) * 24 + 15) / 16 * 16;
 }
 
 // |S|^2 of Eq. slow_vary, telescoped, two steps at a time: log2 p = A + Sa da +
-// Sb db + T.a + T.b dc, eB[k] = {edge/2pi hi, hi', lo, lo'}, T the F_c channel's
-// row at Tc + k n.
-__device__ __forceinline__ float zsum_tele_mt(float phi, float da, float db, float dc, const float4 *Qa,
-                                              const float2 *Qb, const float4 *Tc, int n, const float4 *eB, int M2)
+// Sb db from the step row of the point's cell and F_c channel, eB[k] = {edge/2pi
+// hi, hi', lo, lo'}.
+__device__ __forceinline__ float zsum_tele_mt(float phi, float da, float db, const float4 *Qa, const float2 *Qb,
+                                              const float4 *eB, int M2)
 {
-    const f32x2 ph = dup2(phi), nph = dup2(-phi), a2 = dup2(da), b2 = dup2(db), c2 = dup2(dc);
+    const f32x2 ph = dup2(phi), nph = dup2(-phi), a2 = dup2(da), b2 = dup2(db);
     float Er = 1.0f, Ei = 0.0f;
     f32x2 Sr = dup2(0.0f), Si = dup2(0.0f);
 #pragma unroll 4
     for (int k = 0; k < M2; ++k) {
-        const float4 e = eB[k], q = Qa[k], t = __ldg(Tc + k * n);
+        const float4 e = eB[k], q = Qa[k];
         const float2 qb = Qb[k];
         float s0, c0, s1, c1, l0, l1;
         sincos_turn2(rev_fraction2<true>(ph, nph, ph, pack2(e.x, e.y), pack2(e.z, e.w)), s0, c0, s1, c1);
-        f32x2 lp = fma2(pack2(q.z, q.w), a2, pack2(q.x, q.y));
-        lp = fma2(pack2(qb.x, qb.y), b2, lp);
-        lp = fma2(pack2(t.z, t.w), c2, lp);
-        unpack2(add2(lp, pack2(t.x, t.y)), l0, l1);
+        unpack2(fma2(pack2(qb.x, qb.y), b2, fma2(pack2(q.z, q.w), a2, pack2(q.x, q.y))), l0, l1);
         const f32x2 p = pack2(ex2_approx(l0), ex2_approx(l1));
         Sr = fma2(p, pack2(c0 - Er, c1 - c0), Sr);
         Si = fma2(p, pack2(s0 - Ei, s1 - s0), Si);
@@ -108,16 +107,16 @@ __device__ __forceinline__ float zsum_tele_mt(float phi, float da, float db, flo
 }
 
 // ... in the direct form (few points): zA[m] = {z, dz}
-__device__ __forceinline__ float zsum_direct_mt(float phi, float da, float db, float dc, const float4 *Qa,
-                                                const float2 *Qb, const float4 *Tc, int n, const float2 *zA, int M)
+__device__ __forceinline__ float zsum_direct_mt(float phi, float da, float db, const float4 *Qa, const float2 *Qb,
+                                                const float2 *zA, int M)
 {
     float Sr = 0.0f, Si = 0.0f;
     const float hphi = 0.5f * phi;
     const float phir = phi * 0.15915494309189535f;
     for (int m = 0; m < M; ++m) {
         const int k = m >> 1, o = m & 1;
-        const float4 q = Qa[k], t = __ldg(Tc + k * n);
-        const float2 a = zA[m];
+        const float4 q = Qa[k];
+        const float2 qb = Qb[k], a = zA[m];
         float sn, cs;
         sincos_rev(phir, a.x, sn, cs);
         const float x = hphi * a.y;
@@ -127,9 +126,7 @@ __device__ __forceinline__ float zsum_direct_mt(float phi, float da, float db, f
         sc = fmaf(x2, sc, 8.3333333e-3f);                      // 1/5!
         sc = fmaf(x2, sc, -1.6666667e-1f);                     // -1/3!
         sc = fmaf(x2, sc, 1.0f);
-        float lp = fmaf(o ? q.w : q.z, da, o ? q.y : q.x);
-        lp = fmaf(o ? Qb[k].y : Qb[k].x, db, lp);
-        lp = fmaf(o ? t.w : t.z, dc, lp) + (o ? t.y : t.x);
+        const float lp = fmaf(o ? qb.y : qb.x, db, fmaf(o ? q.w : q.z, da, o ? q.y : q.x));
         const float amp = ex2_approx(lp) * (sc * a.y);        // p_m dz_m sinc
         Sr = fmaf(amp, cs, Sr);
         Si = fmaf(amp, sn, Si);
@@ -141,28 +138,29 @@ __device__ __forceinline__ float zsum_direct_mt(float phi, float da, float db, f
 
 // ---------------------------------------------------------------------------
 // k_quad_mci_f32_tab: persistent over MCI work items (cell ranges of one CUT),
-// one block per item, its cells shared by the warps in turns of 32.  Per turn a
-// lane tests one cell (F_c may fall outside every channel: 42 % of the cells of
-// the 557-ch plan), and the warp takes the rest in groups of about 32 grid rows:
-// step rows of the cells, then grid rows, then points, which go to a list per
-// z-sum form and are summed 32 at a time, one per lane.  No barrier inside an
-// item.  Bound by the XU pipe (20 cycles per warp and step) and the issue of the
-// other ~16 instructions.
+// one block per item.  A round compacts the next cells whose F_c can fall in a
+// channel and deals them to the warps, which take them in groups of about 32
+// grid rows: a step row for every cell and F_c channel (reading the F_c rows at
+// every step instead left the loop waiting on L2: the block's shared memory leaves
+// the L1 28 KB), then grid rows, then points, which go to a list per z-sum form and
+// are summed 32 at a time, one per lane.  Bound by the XU pipe (20 cycles per warp
+// and step) and the issue of the other ~14 instructions.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
+__global__ void __launch_bounds__(256, 2) k_quad_mci_f32_tab(QuadParams qp)
 {
     extern __shared__ float4 smem_f4[];
     const int M = qp.n_steps, G = qp.G, M2 = step_pairs(M), MS = M2 | 1, GC = mci_group(G);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     float4 *eB = smem_f4;                              // [M2] {edge/2pi hi, hi', lo, lo'}
     float2 *zA = reinterpret_cast<float2 *>(eB + M2);  // [2 M2] {z, dz}
-    unsigned char *mine = reinterpret_cast<unsigned char *>(zA + 2 * M2) + mci_warp_bytes(M, G) * warp;
+    unsigned char *mine = reinterpret_cast<unsigned char *>(zA + 2 * M2) + mci_warp_bytes(M) * warp;
     MciWarp &w = *reinterpret_cast<MciWarp *>(mine);
-    float4 *Qa = reinterpret_cast<float4 *>(mine + sizeof(MciWarp));       // [GC][MS]
-    float2 *Qb = reinterpret_cast<float2 *>(Qa + (size_t)GC * MS);         // [GC][MS]
+    float4 *Qa = reinterpret_cast<float4 *>(mine + sizeof(MciWarp));       // [kMciUnits][MS]
+    float2 *Qb = reinterpret_cast<float2 *>(Qa + (size_t)kMciUnits * MS);  // [kMciUnits][MS]
     float *rel = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(zA + 2 * M2) +
-                                           mci_warp_bytes(M, G) * nw);     // [n] channel centre - f_i
+                                           mci_warp_bytes(M) * nw);     // [n] channel centre - f_i
     float *hb = rel + qp.mci_n_max;                    // [n] B/2
+    __shared__ CellRound cr;
     __shared__ double scratch[32];
     __shared__ int s_item;
 
@@ -208,7 +206,6 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
         const float *pd = qp.pd_f + poff;                // [n] P/B
         const float fi = (float)qp.ch_frel[coff + i];
         const float three_fi2 = 3.0f * fi * fi;
-        const int n2 = n - 1;
         float sum = 0.0f, comp = 0.0f;
         int nl[2] = {0, 0};                              // list lengths (direct, telescoped)
         // one list's first 32 points (or what is left), one per lane
@@ -218,11 +215,10 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
             const int at = f ? lane : kMciList - 1 - lane, step = f ? cnt : -cnt;
             if (lane < cnt) {
                 const float4 v = w.Lp[at];
-                const float2 u = w.Lw[at];
-                const int cc = __float_as_int(u.y) >> 16, c = __float_as_int(u.y) & 0xffff;
-                const float S2 = f ? zsum_tele_mt(v.x, v.y, v.z, v.w, Qa + cc * MS, Qb + cc * MS, T + c, n, eB, M2)
-                                   : zsum_direct_mt(v.x, v.y, v.z, v.w, Qa + cc * MS, Qb + cc * MS, T + c, n, zA, M);
-                const float y = u.x * S2 * array_factor_f(v.x, qp) - comp;
+                const int u = w.Lu[at] * MS;
+                const float S2 = f ? zsum_tele_mt(v.x, v.y, v.z, Qa + u, Qb + u, eB, M2)
+                                   : zsum_direct_mt(v.x, v.y, v.z, Qa + u, Qb + u, zA, M);
+                const float y = v.w * S2 * array_factor_f(v.x, qp) - comp;
                 const float t = sum + y;
                 comp = (t - sum) - y;
                 sum = t;
@@ -231,60 +227,53 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
             nl[f] -= cnt;
             if (lane < nl[f]) {                          // at most 31 stay
                 w.Lp[at] = w.Lp[at + step];
-                w.Lw[at] = w.Lw[at + step];
+                w.Lu[at] = w.Lu[at + step];
             }
             __syncwarp();
         };
-        for (int t0 = item.piece0 + 32 * warp; t0 < item.piece1; t0 += 32 * nw) {
-            // one cell per lane: can F_c fall in a channel?
-            int a = 0, b = 0, c0 = 0, c1 = -1;
-            if (t0 + lane < item.piece1) {
-                int ap, bp;
-                tri_decode(t0 + lane, n2, ap, bp);
-                a = dbg_clamp(ap + (ap >= i), n, kDbgCell, qp.dbg);
-                b = dbg_clamp(bp + (bp >= i), n, kDbgCell, qp.dbg);
-                if (pd[a] * pd[b] != 0.0f) {
-                    // a little wider than the cell, the points decide
-                    const float uc = rel[a] + rel[b], r = 1.0001f * (hb[a] + hb[b]) + 1e-5f * fabsf(uc) + 1e-6f;
-                    int lo = 0, hi = n;                  // first channel ending above uc - r
-                    while (lo < hi) {
-                        const int m = (lo + hi) >> 1;
-                        if (rel[m] + hb[m] > uc - r) hi = m;
-                        else lo = m + 1;
-                    }
-                    c0 = lo;
-                    c1 = lo - 1;
-                    while (c1 + 1 < n && rel[c1 + 1] - hb[c1 + 1] <= uc + r) ++c1;
-                }
-            }
-            unsigned todo = __ballot_sync(0xffffffffu, c1 >= c0);
-            while (todo) {
-                int ncc = 0;
-                for (; ncc < GC && todo; ++ncc) {        // the next cells, in order
-                    const int src = __ffs(todo) - 1;
-                    if (lane == src) w.cell[ncc] = make_int4(a, b, c0, c1);
-                    todo &= todo - 1;
+        for (int t0 = item.piece0; t0 < item.piece1; t0 += blockDim.x) {
+            const int nv = cell_round(cr, t0, item.piece1, n, i, rel, hb, pd, qp.dbg);
+            int v = nv * warp / nw, cs = -1;                     // this warp's cells; next F_c channel of v
+            const int v1 = nv * (warp + 1) / nw;
+            while (v < v1) {
+                // the next cells and F_c channels, in order
+                int ncc = 0, nu = 0;
+                while (v < v1 && ncc < GC && nu < kMciUnits) {
+                    const int4 cl = cr.cell[v];
+                    const int c0 = cs < 0 ? cl.z : cs, c1 = min(cl.w, c0 + kMciUnits - nu - 1);
+                    if (nu > 0 && c1 < cl.w) break;              // whole cells while they fit
+                    if (lane == 0) w.cell[ncc] = make_int4(cl.x | cl.y << 16, c0, c1, nu);
+                    if (lane <= c1 - c0) w.unit[nu + lane] = make_int2(ncc, c0 + lane);
+                    nu += c1 - c0 + 1;
+                    ++ncc;
+                    cs = c1 < cl.w ? c1 + 1 : -1;
+                    v += c1 < cl.w ? 0 : 1;
                 }
                 __syncwarp();
-                // step rows of the cells
-                for (int e = lane; e < ncc * M2; e += 32) {
-                    const int k = e / ncc, cc = e - k * ncc;
-                    const int4 cl = w.cell[cc];
+                // step rows: ln p at da = db = 0 of the cell with F_c in channel c, dc
+                // = da + db + D
+                for (int e = lane; e < nu * M2; e += 32) {
+                    const int k = e / nu, u = e - k * nu;
+                    const int2 un = w.unit[u];
+                    const int ab = w.cell[un.x].x, a = ab & 0xffff, b = ab >> 16;
+                    const float D = (rel[a] + rel[b]) - rel[un.y];
                     const float4 *Tk = T + (size_t)k * n;
-                    const float4 ta = Tk[cl.x], tb = Tk[cl.y], ti = Tk[i];
-                    float4 q = make_float4((ta.x + tb.x) - ti.x, (ta.y + tb.y) - ti.y, ta.z, ta.w);
+                    const float4 ta = Tk[a], tb = Tk[b], ti = Tk[i], tc = Tk[un.y];
+                    float4 q = make_float4(fmaf(tc.z, D, (ta.x + tb.x) + (tc.x - ti.x)),
+                                           fmaf(tc.w, D, (ta.y + tb.y) + (tc.y - ti.y)), ta.z + tc.z, ta.w + tc.w);
                     if (2 * k + 1 >= M) q.y = -1000.0f;
-                    Qa[cc * MS + k] = q;
-                    Qb[cc * MS + k] = make_float2(tb.z, tb.w);
+                    Qa[u * MS + k] = q;
+                    Qb[u * MS + k] = make_float2(tb.z + tc.z, tb.w + tc.w);
                 }
                 // grid rows
                 for (int e = lane; e < ncc * G; e += 32) {
                     const int cc = e / G, r = e - cc * G;
                     const int4 cl = w.cell[cc];
-                    const float mult = cl.x == cl.y ? 1.0f : 2.0f;
-                    const float ra = fabsf(rel[cl.x]), rb = fabsf(rel[cl.y]);
-                    const float xlo = ra - hb[cl.x], xhi = ra + hb[cl.x];
-                    const float ylo = rb - hb[cl.y], yhi = rb + hb[cl.y];
+                    const int a = cl.x & 0xffff, b = cl.x >> 16;
+                    const float mult = a == b ? 1.0f : 2.0f;
+                    const float ra = fabsf(rel[a]), rb = fabsf(rel[b]);
+                    const float xlo = ra - hb[a], xhi = ra + hb[a];
+                    const float ylo = rb - hb[b], yhi = rb + hb[b];
                     const float u1hi = xhi * yhi;
                     const float llo = logf(fmaxf(xlo * ylo, eps * u1hi));
                     const float ds = (logf(u1hi) - llo) / (float)G;
@@ -295,34 +284,33 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
                         o.z = log1pf((ymax - ymin) / ymin) / (float)G;
                         o.y = sqrtf(ymin * ymax);
                         o.x = u1 / o.y;
-                        o.w = u1 * ds * o.z * mult * (pd[cl.x] * pd[cl.y]);
+                        o.w = u1 * ds * o.z * mult * (pd[a] * pd[b]);
                     }
                     w.row[e] = o;
                 }
                 __syncwarp();
                 for (int q0 = 0; q0 < ncc * G * G; q0 += 32) {
                     const int q = q0 + lane;
-                    int cls = -1, ci = -1, cc = 0;
-                    float phi = 0.0f, da = 0.0f, db = 0.0f, dc = 0.0f, W = 0.0f;
+                    int cls = -1, ci = -1, un = 0;
+                    float phi = 0.0f, da = 0.0f, db = 0.0f, W = 0.0f;
                     if (q < ncc * G * G) {
                         const int rr = q / G, j = q - rr * G;
-                        cc = rr / G;
                         const float4 o = w.row[rr];
                         if (o.w != 0.0f) {
-                            const int4 cl = w.cell[cc];
-                            const float ra = rel[cl.x], rb = rel[cl.y];
+                            const int4 cl = w.cell[rr / G];
+                            const float ra = rel[cl.x & 0xffff], rb = rel[cl.x >> 16];
                             const float s1 = ra > 0.0f ? 1.0f : -1.0f, s2 = rb > 0.0f ? 1.0f : -1.0f;
                             const float d = ((float)j + 0.5f - 0.5f * (float)G) * o.z;
                             const float ex = expf(d);
                             const float f1 = s1 * (o.x * ex), f2 = s2 * (o.y * __frcp_rn(ex));
                             const float u = f1 + f2;
-                            for (int c = cl.z; c <= cl.w; ++c)
+                            for (int c = cl.y; c <= cl.z; ++c)
                                 if (rel[c] - hb[c] <= u && u < rel[c] + hb[c]) ci = c;
                             if (ci >= 0) {
                                 W = o.w * pd[ci];
                                 da = f1 - ra;
                                 db = f2 - rb;
-                                dc = u - rel[ci];
+                                un = cl.w + (ci - cl.y);
                                 const float br = b2 + c3 * (u + 2.0f * fi) +
                                                  c4 * (f1 * f1 + 1.5f * f1 * f2 + 3.0f * fi * u + f2 * f2 + three_fi2);
                                 phi = m4pi2 * f1 * f2 * br;
@@ -335,8 +323,8 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32_tab(QuadParams qp)
                         const unsigned m = __ballot_sync(0xffffffffu, cls == f);
                         if (cls == f) {
                             const int e = nl[f] + __popc(m & lt_mask), at = f ? e : kMciList - 1 - e;
-                            w.Lp[at] = make_float4(phi, da, db, dc);
-                            w.Lw[at] = make_float2(W, __int_as_float(cc << 16 | ci));
+                            w.Lp[at] = make_float4(phi, da, db, W);
+                            w.Lu[at] = un;
                         }
                         nl[f] += __popc(m);
                         if (nl[f] >= 32) flush(f);
@@ -454,7 +442,7 @@ __global__ void __launch_bounds__(256) k_quad_mci_f64_tab(QuadParams qp)
 size_t quad_mci_tab_smem_bytes(int precision, int n_steps, int n_max, int G, int block)
 {
     if (precision == 0)
-        return (size_t)step_pairs(n_steps) * 32 + mci_warp_bytes(n_steps, G) * (block / 32) +
+        return (size_t)step_pairs(n_steps) * 32 + mci_warp_bytes(n_steps) * (block / 32) +
                (size_t)n_max * 2 * sizeof(float);
     return (size_t)n_steps * (sizeof(double2) + sizeof(double));
 }

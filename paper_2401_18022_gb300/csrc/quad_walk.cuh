@@ -1,25 +1,44 @@
-// Half-warp walks of the FP32 adjoint kernels (closed-form profile): the
-// z-sum of one grid point (App. A, Eq. slow_vary) spread over the 16 lanes of
-// a half-warp, each lane owning K consecutive steps, with the terms kept in
+// Half-warp walks of the FP32 adjoint kernels: the z-sum of one grid point or
+// node (App. A, Eq. slow_vary) spread over the 16 lanes of a half-warp, each lane
+// owning 2 K2 consecutive steps in K2 pairs (f32x2.cuh), with the terms kept in
 // registers for the bucket terms d|S|^2/d ln p_m = 2 Re(conj(S) t_m).
+//
+// Steps in pairs: the multiply-adds of two steps share an issue slot, and what
+// bounds the walk is the XU pipe (20 cycles per warp and step: sin and cos 8 each,
+// ex2 4) instead of issue.  The span's M steps fill 16 x 2 K2 places (112 steps:
+// 14 lanes of 16); the places past M carry log2 weight -1000 and repeat the last
+// edge.
 #pragma once
 #include <cuda_runtime.h>
 
+#include "f32x2.cuh"
 #include "quad_common.cuh"
 #include "quad_zsum.cuh"
 
 namespace isrs {
 
 constexpr unsigned kWarpAll = 0xffffffffu;
+constexpr float kPadLog2 = -1000.0f;   // log2 weight of the padding steps (ex2 -> 0)
 
-__device__ __forceinline__ float sinc_poly(float x)
+// step of place o of pair k of lane l
+template <int K2>
+__device__ __forceinline__ int walk_step(int k, int l, int o)
 {
-    const float x2 = x * x;
-    float sc = fmaf(x2, -2.5052108e-8f, 2.7557319e-6f);   // -1/11!, 1/9!
-    sc = fmaf(x2, sc, -1.9841270e-4f);                     // -1/7!
-    sc = fmaf(x2, sc, 8.3333333e-3f);                      // 1/5!
-    sc = fmaf(x2, sc, -1.6666667e-1f);                     // -1/3!
-    return fmaf(x2, sc, 1.0f);
+    return l * 2 * K2 + 2 * k + o;
+}
+
+// ze[k][16] = {edge/2pi hi, hi', lo, lo'}, zd[k][16] = {z, z', dz, dz'} of the
+// pairs of all 16 lanes, filled by the whole block.
+template <int K2>
+__device__ __forceinline__ void walk_tables(const QuadParams &qp, float4 *ze, float4 *zd)
+{
+    for (int t = threadIdx.x; t < K2 * 16; t += blockDim.x) {
+        const int m0 = min(walk_step<K2>(t >> 4, t & 15, 0), qp.n_steps - 1);
+        const int m1 = min(walk_step<K2>(t >> 4, t & 15, 1), qp.n_steps - 1);
+        const float4 b0 = qp.zs_b[m0], b1 = qp.zs_b[m1], a0 = qp.zs_a[m0], a1 = qp.zs_a[m1];
+        ze[t] = make_float4(b0.x, b1.x, b0.y, b1.y);
+        zd[t] = make_float4(a0.x, a1.x, a0.w, a1.w);
+    }
 }
 
 // sum over the 16 lanes of each half-warp (both halves in step)
@@ -30,239 +49,100 @@ __device__ __forceinline__ float half_sum(float v)
     return v;
 }
 
-// ---------------------------------------------------------------------------
-// Half-warp walks of one grid point (state: weight w W af, phi, F_c - f_ref,
-// at).  Lane l16 owns steps [K l16, K l16 + K) with tables
-//   o0[k] = {A2 + log2 dz, K2, z, dz},  o1[k] = {edge/2pi hi, lo, A2, c}
-// (padding steps carry log2 weight -1000, so their terms vanish), and for
-// the first F_c candidates of the piece oc[k] = {edge/2pi hi, lo,
-// A2 - at_c z, K2}.  Each walk
-// adds the lane's bucket terms and returns the point's w W af |S|^2.
-// ---------------------------------------------------------------------------
-template <int K>
-__device__ __forceinline__ float walk_direct(const float4 *o0s, float wq, float ph, float fc, float at, float mult,
-                                             float (&R)[K], float (&Rp)[K])
+template <int K2>
+__device__ __forceinline__ void walk_sum(const f32x2 (&tr)[K2], const f32x2 (&ti)[K2], float &sr, float &si)
 {
-    // S = sum_m p_m dz_m sinc(phi dz_m/2) e^{j phi z_m}; d|S|^2/d ln p_m = 2 Re(conj(S) t_m)
-    const float hph = 0.5f * ph;
-    const float phr = ph * 0.15915494309189535f;
-    float tr[K], ti[K];
-    float sr = 0.0f, si = 0.0f;
+    f32x2 a = tr[0], b = ti[0];
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float4 o = o0s[k * 16];
-        float sn, cs;
-        sincos_rev(phr, o.z, sn, cs);
-        float lp = fmaf(o.y, fc, o.x);
-        lp = fmaf(-at, o.z, lp);
-        const float amp = ex2_approx(lp) * sinc_poly(hph * o.w);
-        tr[k] = amp * cs;
-        ti[k] = amp * sn;
-        sr += tr[k];
-        si += ti[k];
+    for (int k = 1; k < K2; ++k) {
+        a = add2(a, tr[k]);
+        b = add2(b, ti[k]);
     }
-    sr = half_sum(sr);
-    si = half_sum(si);
-    const float c2 = 2.0f * mult * wq, c2F = c2 * fc;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float rr = fmaf(sr, tr[k], si * ti[k]);
-        R[k] = fmaf(c2, rr, R[k]);
-        Rp[k] = fmaf(c2F, rr, Rp[k]);
-    }
-    return wq * fmaf(sr, sr, si * si);
+    float x, y;
+    unpack2(a, x, y);
+    sr = half_sum(x + y);
+    unpack2(b, x, y);
+    si = half_sum(x + y);
 }
 
-// Folded: o1s holds the point's candidate rows {edge/2pi hi, lo, A2 - at z, K2}
-// (attenuation folded in), so a step takes one table load and one FMA for
-// ln p; o0s and at are then unused.
-template <int K, bool Wide = false, bool Folded = false>
-__device__ __forceinline__ float walk_tele(const float4 *o0s, const float4 *o1s, int l16, float wq, float ph,
-                                           float fc, float at, float mult, float (&R)[K], float (&Rp)[K])
+__device__ __forceinline__ f32x2 ex2_pair(f32x2 x)
 {
-    // U = sum_m p_m (E_{m+1} - E_m), E_e = e^{j phi z_e}, |S|^2 = |U|^2/phi^2;
-    // d|S|^2/d ln p_m = 2 Re(conj(U) p_m (E_{m+1} - E_m)) / phi^2
-    float tr[K], ti[K];
-    float Er = 1.0f, Ei = 0.0f, p0 = 0.0f, e1r = 1.0f, e1i = 0.0f;
+    float a, b;
+    unpack2(x, a, b);
+    return pack2(ex2_approx(a), ex2_approx(b));
+}
+
+// Terms t_m = p_m dz_m sinc(phi dz_m/2) e^{j phi z_m} and their sum; lp(k) gives
+// log2 p of pair k (zd offset by the lane).
+template <int K2, typename LP>
+__device__ __forceinline__ void walk_direct(const float4 *zd, float ph, const LP &lp, f32x2 (&tr)[K2], f32x2 (&ti)[K2],
+                                            float &sr, float &si)
+{
+    const f32x2 hph = dup2(0.5f * ph), phr = dup2(ph * 0.15915494309189535f), nphr = dup2(-ph * 0.15915494309189535f);
+    const f32x2 mg = dup2(12582912.0f), nm = dup2(-12582912.0f);
 #pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float4 b = o1s[k * 16];
-        float sn, cs;
-        if (Wide) phasor_rev_ff_wide(ph, b.x, b.y, sn, cs);
-        else phasor_rev_ff(ph, b.x, b.y, sn, cs);
-        float lp;
-        if constexpr (Folded) {
-            lp = fmaf(b.w, fc, b.z);
-        } else {
-            const float4 a = o0s[k * 16];
-            lp = fmaf(a.y, fc, b.z);
-            lp = fmaf(-at, a.z, lp);
-        }
-        const float pm = ex2_approx(lp);
+    for (int k = 0; k < K2; ++k) {
+        const float4 z = zd[k * 16];
+        const f32x2 zz = pack2(z.x, z.y), dz = pack2(z.z, z.w);
+        float s0, c0, s1, c1;
+        sincos_turn2(fma2(phr, zz, add2(fma2(nphr, zz, mg), nm)), s0, c0, s1, c1);
+        const f32x2 x = mul2(hph, dz), x2 = mul2(x, x);       // sinc to x^10, |x| <= pi/2
+        f32x2 sc = fma2(x2, dup2(-2.5052108e-8f), dup2(2.7557319e-6f));
+        sc = fma2(x2, sc, dup2(-1.9841270e-4f));
+        sc = fma2(x2, sc, dup2(8.3333333e-3f));
+        sc = fma2(x2, sc, dup2(-1.6666667e-1f));
+        sc = fma2(x2, sc, dup2(1.0f));
+        const f32x2 amp = mul2(ex2_pair(lp(k)), mul2(sc, dz));
+        tr[k] = mul2(amp, pack2(c0, c1));
+        ti[k] = mul2(amp, pack2(s0, s1));
+    }
+    walk_sum<K2>(tr, ti, sr, si);
+}
+
+// Telescoped: terms p_m (E_{m+1} - E_m), E_e = e^{j phi z_e}, and their sum U,
+// |S|^2 = |U|^2 / phi^2 (ze offset by the lane; phi float-float, or Wide: up to
+// 2^29 revolutions).
+template <int K2, bool Wide, typename LP>
+__device__ __forceinline__ void walk_tele(const float4 *ze, int l16, float ph, float ph_lo, const LP &lp,
+                                          f32x2 (&tr)[K2], f32x2 (&ti)[K2], float &ur, float &ui)
+{
+    const f32x2 p2 = dup2(ph), np2 = dup2(-ph), pl2 = dup2(ph_lo);
+    float Er = 0.0f, Ei = 0.0f, f0r = 0.0f, f0i = 0.0f, f1r = 0.0f, f1i = 0.0f;
+    f32x2 p0 = p2;
+#pragma unroll
+    for (int k = 0; k < K2; ++k) {
+        const float4 e = ze[k * 16];
+        float s0, c0, s1, c1;
+        sincos_turn2(rev_fraction2<Wide>(p2, np2, pl2, pack2(e.x, e.y), pack2(e.z, e.w)), s0, c0, s1, c1);
+        const f32x2 p = ex2_pair(lp(k));
         if (k == 0) {
-            p0 = pm;
-            e1r = cs;
-            e1i = sn;
-            tr[0] = 0.0f;
-            ti[0] = 0.0f;
+            p0 = p;
+            f0r = c0;
+            f0i = s0;
+            f1r = c1 - c0;
+            f1i = s1 - s0;
         } else {
-            tr[k] = pm * (cs - Er);
-            ti[k] = pm * (sn - Ei);
+            tr[k] = mul2(p, pack2(c0 - Er, c1 - c0));
+            ti[k] = mul2(p, pack2(s0 - Ei, s1 - s0));
         }
-        Er = cs;
-        Ei = sn;
+        Er = c1;
+        Ei = s1;
     }
     // the lower edge of this lane's first step is the previous lane's last edge
     float elr = __shfl_up_sync(kWarpAll, Er, 1, 16);
     float eli = __shfl_up_sync(kWarpAll, Ei, 1, 16);
     elr = l16 == 0 ? 1.0f : elr;
     eli = l16 == 0 ? 0.0f : eli;
-    tr[0] = p0 * (e1r - elr);
-    ti[0] = p0 * (e1i - eli);
-    float ur = 0.0f, ui = 0.0f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        ur += tr[k];
-        ui += ti[k];
-    }
-    ur = half_sum(ur);
-    ui = half_sum(ui);
-    const float iph2 = __fdividef(1.0f, ph * ph);   // MUFU reciprocal (2 ulp): phi^2 is far from the range limits
-    const float c2 = 2.0f * mult * wq * iph2, c2F = c2 * fc;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float rr = fmaf(ur, tr[k], ui * ti[k]);
-        R[k] = fmaf(c2, rr, R[k]);
-        Rp[k] = fmaf(c2F, rr, Rp[k]);
-    }
-    return wq * fmaf(ur, ur, ui * ui) * iph2;
+    tr[0] = mul2(p0, pack2(f0r - elr, f1r));
+    ti[0] = mul2(p0, pack2(f0i - eli, f1i));
+    walk_sum<K2>(tr, ti, ur, ui);
 }
 
-template <int K>
-__device__ __forceinline__ float walk_small(const float4 *o0s, const float4 *o1s, float wq, float ph, float fc,
-                                            float at, float mult, float (&R)[K], float (&Rp)[K])
+// 2 Re(conj(S) t) / 2 of pair k
+template <int K2>
+__device__ __forceinline__ f32x2 walk_term(const f32x2 (&tr)[K2], const f32x2 (&ti)[K2], int k, f32x2 sr, f32x2 si)
 {
-    // |S|^2 = M0^2 - phi^2 (M0 M2 - M1^2);
-    // d|S|^2/d ln p_m = w_m (2 M0 - phi^2 (M2 + M0 c_m - 2 M1 z_m))
-    float wk[K];
-    float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float4 a = o0s[k * 16];
-        const float cm = o1s[k * 16].w;
-        float lp = fmaf(a.y, fc, a.x);
-        lp = fmaf(-at, a.z, lp);
-        wk[k] = ex2_approx(lp);
-        s0 += wk[k];
-        s1 = fmaf(wk[k], a.z, s1);
-        s2 = fmaf(wk[k], cm, s2);
-    }
-    s0 = half_sum(s0);
-    s1 = half_sum(s1);
-    s2 = half_sum(s2);
-    const float ph2 = ph * ph;
-    const float al0 = 2.0f * s0 - ph2 * s2, al1 = -ph2 * s0, al2 = 2.0f * ph2 * s1;
-    const float cp = mult * wq, cF = cp * fc;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float zm = o0s[k * 16].z;
-        const float cm = o1s[k * 16].w;
-        const float rr = wk[k] * fmaf(al2, zm, fmaf(al1, cm, al0));
-        R[k] = fmaf(cp, rr, R[k]);
-        Rp[k] = fmaf(cF, rr, Rp[k]);
-    }
-    return wq * fmaf(-ph2, fmaf(s0, s2, -s1 * s1), s0 * s0);
-}
-
-// ---------------------------------------------------------------------------
-// Walks of a node of the row sums: zt[k][16] = {z_{m+1}/2pi hi, lo, z_m, dz_m}
-// and, for the node's F_c candidate, ek[k][16] = {log2 p_m at the channel's
-// centre, K2_m} of lane l16's steps (both already offset by l16; padding steps
-// carry log2 weight -1000); dF = F_c - f_c, Fc = F_c - f_ref, phi float-float.
-// ---------------------------------------------------------------------------
-template <int K>
-__device__ __forceinline__ float walk_direct_n(const float4 *zt, const float2 *ek, float wq, float ph, float dF,
-                                               float Fc, float mult, float (&R)[K], float (&Rp)[K])
-{
-    const float hph = 0.5f * ph;
-    const float phr = ph * 0.15915494309189535f;
-    float tr[K], ti[K];
-    float sr = 0.0f, si = 0.0f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float4 o = zt[k * 16];
-        const float2 e = ek[k * 16];
-        float sn, cs;
-        sincos_rev(phr, o.z, sn, cs);
-        const float amp = ex2_approx(fmaf(e.y, dF, e.x)) * (sinc_poly(hph * o.w) * o.w);
-        tr[k] = amp * cs;
-        ti[k] = amp * sn;
-        sr += tr[k];
-        si += ti[k];
-    }
-    sr = half_sum(sr);
-    si = half_sum(si);
-    const float c2 = 2.0f * mult * wq, c2F = c2 * Fc;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float rr = fmaf(sr, tr[k], si * ti[k]);
-        R[k] = fmaf(c2, rr, R[k]);
-        Rp[k] = fmaf(c2F, rr, Rp[k]);
-    }
-    return wq * fmaf(sr, sr, si * si);
-}
-
-template <int K>
-__device__ __forceinline__ float walk_tele_n(const float4 *zt, const float2 *ek, int l16, float wq, float ph,
-                                             float ph_lo, float dF, float Fc, float mult, float (&R)[K],
-                                             float (&Rp)[K])
-{
-    float tr[K], ti[K];
-    float Er = 1.0f, Ei = 0.0f, p0 = 0.0f, e1r = 1.0f, e1i = 0.0f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float4 b = zt[k * 16];
-        const float2 e = ek[k * 16];
-        float sn, cs;
-        phasor_rev_ff(ph, b.x, b.y, sn, cs, ph_lo);
-        const float pm = ex2_approx(fmaf(e.y, dF, e.x));
-        if (k == 0) {
-            p0 = pm;
-            e1r = cs;
-            e1i = sn;
-            tr[0] = 0.0f;
-            ti[0] = 0.0f;
-        } else {
-            tr[k] = pm * (cs - Er);
-            ti[k] = pm * (sn - Ei);
-        }
-        Er = cs;
-        Ei = sn;
-    }
-    // the lower edge of this lane's first step is the previous lane's last edge
-    float elr = __shfl_up_sync(kWarpAll, Er, 1, 16);
-    float eli = __shfl_up_sync(kWarpAll, Ei, 1, 16);
-    elr = l16 == 0 ? 1.0f : elr;
-    eli = l16 == 0 ? 0.0f : eli;
-    tr[0] = p0 * (e1r - elr);
-    ti[0] = p0 * (e1i - eli);
-    float ur = 0.0f, ui = 0.0f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        ur += tr[k];
-        ui += ti[k];
-    }
-    ur = half_sum(ur);
-    ui = half_sum(ui);
-    const float iph2 = __fdividef(1.0f, ph * ph);
-    const float c2 = 2.0f * mult * wq * iph2, c2F = c2 * Fc;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float rr = fmaf(ur, tr[k], ui * ti[k]);
-        R[k] = fmaf(c2, rr, R[k]);
-        Rp[k] = fmaf(c2F, rr, Rp[k]);
-    }
-    return wq * fmaf(ur, ur, ui * ui) * iph2;
+    return fma2(sr, tr[k], mul2(si, ti[k]));
 }
 
 }  // namespace isrs

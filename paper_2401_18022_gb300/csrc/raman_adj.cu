@@ -16,9 +16,8 @@
 //
 // k_quad_adj_tab takes the nodes of every piece's row sums (quad_nodes.cuh) once
 // per candidate channel, so a warp's buckets stay in registers, and evaluates
-// every step term once: a node is walked by a half-warp, each of the 16 lanes
-// owning K = ceil(M/16) consecutive steps, which keeps their terms t_m in
-// registers; the half sums them into S with shuffles, and the same registers
+// every step term once: a node is walked by a half-warp (quad_walk.cuh), whose
+// lanes keep their steps' terms t_m in registers; the half sums them into S with shuffles, and the same registers
 // give d|S|^2/d ln p_m = 2 Re(conj(S) t_m).  The same pass sums the forward
 // value w W |S|^2 (the tile's partial of Sigma_i), so no separate forward runs.
 // The buckets are not yet weighted by dT/dSigma_i (unknown until every tile
@@ -44,117 +43,23 @@ namespace {
 
 constexpr unsigned kFullT = 0xffffffffu;
 constexpr int kTabAdjSlots = 512;   // node slots of a chunk
-constexpr float kPadLog2T = -1000.0f;
-
-// Half-warp walks of a node (weight cp = mult w W af, phi float-float, in-channel
-// offsets dl, dd of the longer and the shorter axis).  Lane l16 owns steps [K
-// l16, K l16 + K) with zt[k][16] = {edge/2pi hi, lo, z, dz} and the candidate's
-// q[k][16] = {A, Sl, Sd} (offset by l16; padding steps carry log2 weight -1000).
-// Each walk adds the lane's bucket terms R += cp d|S|^2/d ln p_m, Rl += dl
-// (same), Rd += dd (same) and returns |S|^2.
-template <int K>
-__device__ __forceinline__ float walk_direct_t(const float4 *zt, const float4 *q, float cp, float ph, float dl,
-                                               float dd, float (&R)[K], float (&Rl)[K], float (&Rd)[K])
-{
-    const float hph = 0.5f * ph;
-    const float phr = ph * 0.15915494309189535f;
-    float tr[K], ti[K];
-    float sr = 0.0f, si = 0.0f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float4 e = q[k * 16];
-        const float4 z = zt[k * 16];
-        float sn, cs;
-        sincos_rev(phr, z.z, sn, cs);
-        const float amp = ex2_approx(fmaf(e.z, dd, fmaf(e.y, dl, e.x))) * (sinc_poly(hph * z.w) * z.w);
-        tr[k] = amp * cs;
-        ti[k] = amp * sn;
-        sr += tr[k];
-        si += ti[k];
-    }
-    sr = half_sum(sr);
-    si = half_sum(si);
-    const float c2 = 2.0f * cp, ca = c2 * dl, cb = c2 * dd;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float rr = fmaf(sr, tr[k], si * ti[k]);
-        R[k] = fmaf(c2, rr, R[k]);
-        Rl[k] = fmaf(ca, rr, Rl[k]);
-        Rd[k] = fmaf(cb, rr, Rd[k]);
-    }
-    return fmaf(sr, sr, si * si);
-}
-
-template <int K>
-__device__ __forceinline__ float walk_tele_t(const float4 *zt, const float4 *q, int l16, float cp, float ph,
-                                             float ph_lo, float dl, float dd, float (&R)[K], float (&Rl)[K],
-                                             float (&Rd)[K])
-{
-    float tr[K], ti[K];
-    float Er = 1.0f, Ei = 0.0f, p0 = 0.0f, e1r = 1.0f, e1i = 0.0f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float4 e = q[k * 16];
-        const float4 z = zt[k * 16];
-        float sn, cs;
-        phasor_rev_ff(ph, z.x, z.y, sn, cs, ph_lo);
-        const float pm = ex2_approx(fmaf(e.z, dd, fmaf(e.y, dl, e.x)));
-        if (k == 0) {
-            p0 = pm;
-            e1r = cs;
-            e1i = sn;
-            tr[0] = 0.0f;
-            ti[0] = 0.0f;
-        } else {
-            tr[k] = pm * (cs - Er);
-            ti[k] = pm * (sn - Ei);
-        }
-        Er = cs;
-        Ei = sn;
-    }
-    // the lower edge of this lane's first step is the previous lane's last edge
-    float elr = __shfl_up_sync(kFullT, Er, 1, 16);
-    float eli = __shfl_up_sync(kFullT, Ei, 1, 16);
-    elr = l16 == 0 ? 1.0f : elr;
-    eli = l16 == 0 ? 0.0f : eli;
-    tr[0] = p0 * (e1r - elr);
-    ti[0] = p0 * (e1i - eli);
-    float ur = 0.0f, ui = 0.0f;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        ur += tr[k];
-        ui += ti[k];
-    }
-    ur = half_sum(ur);
-    ui = half_sum(ui);
-    const float iph2 = __fdividef(1.0f, ph * ph);
-    const float c2 = 2.0f * cp * iph2, ca = c2 * dl, cb = c2 * dd;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const float rr = fmaf(ur, tr[k], ui * ti[k]);
-        R[k] = fmaf(c2, rr, R[k]);
-        Rl[k] = fmaf(ca, rr, Rl[k]);
-        Rd[k] = fmaf(cb, rr, Rd[k]);
-    }
-    return fmaf(ur, ur, ui * ui) * iph2;
-}
-
 // One warp's shared memory: nodes, the points to walk, the candidate's rows.
-template <int K>
+template <int K2>
 struct __align__(16) AdjTabWarp {
     WarpNodes<kTabAdjSlots> ns;
     float4 L[32];                // {mult w W af, phi, phi_lo, dl}
     float Ld[32];                // dd
-    float4 q[K * 16];            // {A, Sl, Sd}, [k][lane of the half]
+    float4 qa[K2 * 16];          // {A, A', Sl, Sl'} of a pair, [k][lane of the half]
+    float2 qb[K2 * 16];          // {Sd, Sd'}
 };
 
 }  // namespace
 
 #ifndef ISRS_ADJ_TAB_MIN_BLOCKS
-#define ISRS_ADJ_TAB_MIN_BLOCKS 3   // resident blocks per SM the register budget is sized for
+#define ISRS_ADJ_TAB_MIN_BLOCKS 2   // resident blocks per SM the register budget is sized for (3 spill, 4 more so)
 #endif
 
-template <int K>
+template <int K2>
 __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(AdjTabParams ap)
 {
     const QuadParams &qp = ap.q;
@@ -162,15 +67,10 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
     const int M = qp.n_steps, G = qp.G;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int l16 = lane & 15, half = lane >> 4;
-    float4 *zt = smem_f4;                              // [K][16] {edge/2pi hi, lo, z, dz}
-    AdjTabWarp<K> &w = reinterpret_cast<AdjTabWarp<K> *>(zt + K * 16)[warp];
+    float4 *ze = smem_f4, *zd = ze + K2 * 16;          // walk_tables
+    AdjTabWarp<K2> &w = reinterpret_cast<AdjTabWarp<K2> *>(zd + K2 * 16)[warp];
     auto &ns = w.ns;
-    // padding steps past M repeat the last edge
-    for (int t = threadIdx.x; t < K * 16; t += blockDim.x) {
-        const int m = min((t & 15) * K + (t >> 4), M - 1);
-        const float4 za = qp.zs_a[m], zb = qp.zs_b[m];
-        zt[t] = make_float4(zb.x, zb.y, za.x, za.w);
-    }
+    walk_tables<K2>(qp, ze, zd);
     __syncthreads();
     const float phi_direct = 3.14159265f / qp.dz_max;
     const unsigned lt_mask = (1u << lane) - 1u;
@@ -202,19 +102,21 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
             for (int cc = 0; cc < g.nc; ++cc) {
                 const double fc = qp.ch_frel[coff + pc.c_lo + cc];
                 float tilt = 0.0f;
-                for (int t = lane; t < K * 16; t += 32) {
-                    const int m = (t & 15) * K + (t >> 4);
-                    float4 r = make_float4(kPadLog2T, 0.0f, 0.0f, 0.0f);
-                    if (m < M) r = tab_row(tp, pc.c_lo + cc, fc, m, M);
-                    w.q[t] = r;
-                    tilt = fmaxf(tilt, fmaxf(fabsf(r.y), fabsf(r.z)));
+                for (int t = lane; t < K2 * 16; t += 32) {
+                    const int m = walk_step<K2>(t >> 4, t & 15, 0);
+                    const float4 none = make_float4(kPadLog2, 0.0f, 0.0f, 0.0f);
+                    const float4 r = m < M ? tab_row(tp, pc.c_lo + cc, fc, m, M) : none;
+                    const float4 u = m + 1 < M ? tab_row(tp, pc.c_lo + cc, fc, m + 1, M) : none;
+                    w.qa[t] = make_float4(r.x, u.x, r.y, u.y);
+                    w.qb[t] = make_float2(r.z, u.z);
+                    tilt = fmaxf(tilt, fmaxf(fmaxf(fabsf(r.y), fabsf(r.z)), fmaxf(fabsf(u.y), fabsf(u.z))));
                 }
                 tilt = 0.69314718f * __uint_as_float(__reduce_max_sync(kFullT, __float_as_uint(tilt)));
                 if (lane == 0) g.tilt = tilt;
                 __syncwarp();
-                float R[K], Rl[K], Rd[K];
+                f32x2 R[K2], Rl[K2], Rd[K2];
 #pragma unroll
-                for (int k = 0; k < K; ++k) R[k] = Rl[k] = Rd[k] = 0.0f;
+                for (int k = 0; k < K2; ++k) R[k] = Rl[k] = Rd[k] = dup2(0.0f);
                 float sum = 0.0f, comp = 0.0f;
                 const auto add = [&](float val) {
                     const float y = val - comp;
@@ -241,20 +143,39 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
                         }
                         __syncwarp();
                         const int nd0 = __popc(bd), nt0 = __popc(bt);
-                        for (int p = 0; p < nd0; p += 2) {
-                            const int at = min(p + half, nd0 - 1);
-                            const float4 v = w.L[at];
-                            const float cp = p + half < nd0 ? v.x : 0.0f;
-                            const float s2 = walk_direct_t<K>(zt + l16, w.q + l16, cp, v.y, v.w, w.Ld[at], R, Rl, Rd);
-                            add(l16 == 0 ? cp * s2 : 0.0f);
-                        }
-                        for (int p = 0; p < nt0; p += 2) {
-                            const int at = 31 - min(p + half, nt0 - 1);
-                            const float4 v = w.L[at];
-                            const float cp = p + half < nt0 ? v.x : 0.0f;
-                            const float s2 = walk_tele_t<K>(zt + l16, w.q + l16, l16, cp, v.y, v.z, v.w, w.Ld[at], R,
-                                                            Rl, Rd);
-                            add(l16 == 0 ? cp * s2 : 0.0f);
+                        for (int f = 0; f < 2; ++f) {
+                            const int cnt = f ? nt0 : nd0;
+                            for (int p = 0; p < cnt; p += 2) {
+                                const int e = min(p + half, cnt - 1), at = f ? 31 - e : e;
+                                const float4 v = w.L[at];
+                                const float dd = w.Ld[at];
+                                const f32x2 dl2 = dup2(v.w), dd2 = dup2(dd);
+                                const float4 *qa = w.qa + l16;
+                                const float2 *qb = w.qb + l16;
+                                const auto lp = [&](int k) {
+                                    const float4 x = qa[k * 16];
+                                    const float2 y = qb[k * 16];
+                                    return fma2(pack2(y.x, y.y), dd2, fma2(pack2(x.z, x.w), dl2, pack2(x.x, x.y)));
+                                };
+                                f32x2 tr[K2], ti[K2];
+                                float sr, si, cp = p + half < cnt ? v.x : 0.0f;
+                                if (f) {
+                                    walk_tele<K2, false>(ze + l16, l16, v.y, v.z, lp, tr, ti, sr, si);
+                                    cp *= __fdividef(1.0f, v.y * v.y);
+                                } else {
+                                    walk_direct<K2>(zd + l16, v.y, lp, tr, ti, sr, si);
+                                }
+                                const f32x2 c2 = dup2(2.0f * cp), cl = dup2(2.0f * cp * v.w), cd = dup2(2.0f * cp * dd);
+                                const f32x2 sr2 = dup2(sr), si2 = dup2(si);
+#pragma unroll
+                                for (int k = 0; k < K2; ++k) {
+                                    const f32x2 rr = walk_term<K2>(tr, ti, k, sr2, si2);
+                                    R[k] = fma2(c2, rr, R[k]);
+                                    Rl[k] = fma2(cl, rr, Rl[k]);
+                                    Rd[k] = fma2(cd, rr, Rd[k]);
+                                }
+                                add(l16 == 0 ? cp * fmaf(sr, sr, si * si) : 0.0f);
+                            }
                         }
                         __syncwarp();
                     }
@@ -269,14 +190,19 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
                 double2 *ra = trows + (size_t)pr.x * M, *rb = trows + (size_t)pr.y * M;
                 double2 *ri = trows + (size_t)pr.z * M, *rc = trows + (size_t)(pr.w + cc) * M;
 #pragma unroll
-                for (int k = 0; k < K; ++k) {
-                    const float f0 = R[k] + __shfl_xor_sync(kFullT, R[k], 16);
-                    const float f1 = Rl[k] + __shfl_xor_sync(kFullT, Rl[k], 16);
-                    const float f2 = Rd[k] + __shfl_xor_sync(kFullT, Rd[k], 16);
-                    const int m = l16 * K + k;
-                    if (half == 0 && m < M) {
-                        const double r0 = 0.5 * (double)f0, r1 = 0.5 * (double)(sw ? f2 : f1),
-                                     r2 = 0.5 * (double)(sw ? f1 : f2);
+                for (int k = 0; k < K2; ++k) {
+                    float v[6];
+                    unpack2(R[k], v[0], v[1]);
+                    unpack2(Rl[k], v[2], v[3]);
+                    unpack2(Rd[k], v[4], v[5]);
+#pragma unroll
+                    for (int t = 0; t < 6; ++t) v[t] += __shfl_xor_sync(kFullT, v[t], 16);
+                    // each half adds one place of the pair
+                    const int m = walk_step<K2>(k, l16, half);
+                    if (m < M) {
+                        const double r0 = 0.5 * (double)(half ? v[1] : v[0]);
+                        const double f1 = 0.5 * (double)(half ? v[3] : v[2]), f2 = 0.5 * (double)(half ? v[5] : v[4]);
+                        const double r1 = sw ? f2 : f1, r2 = sw ? f1 : f2;
                         if (pr.x != pr.z) {              // a = CUT: the two terms cancel
                             atomicAdd(&ra[m].x, r0);
                             atomicAdd(&ri[m].x, -r0);
@@ -337,19 +263,19 @@ cudaError_t launch_tab_gather(const TabGatherParams &gp, cudaStream_t st)
 
 namespace {
 
-template <int K>
+template <int K2>
 cudaError_t launch_adj_tab_k(const AdjTabParams &ap, int num_sms, int block, cudaStream_t st)
 {
     if (ap.q.n_items < num_sms * (block / 32)) block = 32;      // too few tiles for full blocks on every SM
     const int nw = block / 32;
-    const size_t smem = sizeof(float4) * K * 16 + sizeof(AdjTabWarp<K>) * nw;
-    cudaError_t e = cudaFuncSetAttribute(k_quad_adj_tab<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = sizeof(float4) * 2 * K2 * 16 + sizeof(AdjTabWarp<K2>) * nw;
+    cudaError_t e = cudaFuncSetAttribute(k_quad_adj_tab<K2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     int nb = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_quad_adj_tab<K>, block, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_quad_adj_tab<K2>, block, smem);
     if (e != cudaSuccess) return e;
     const int grid = std::max(1, std::min((ap.q.n_items + nw - 1) / nw, num_sms * std::max(1, nb)));
-    k_quad_adj_tab<K><<<grid, block, smem, st>>>(ap);
+    k_quad_adj_tab<K2><<<grid, block, smem, st>>>(ap);
     return cudaGetLastError();
 }
 
@@ -357,15 +283,11 @@ cudaError_t launch_adj_tab_k(const AdjTabParams &ap, int num_sms, int block, cud
 
 cudaError_t launch_adjoint_tab(const AdjTabParams &ap, int num_sms, int block, cudaStream_t st)
 {
-    switch ((ap.q.n_steps + 15) / 16) {
+    switch ((ap.q.n_steps + 31) / 32) {
     case 1: return launch_adj_tab_k<1>(ap, num_sms, block, st);
     case 2: return launch_adj_tab_k<2>(ap, num_sms, block, st);
     case 3: return launch_adj_tab_k<3>(ap, num_sms, block, st);
     case 4: return launch_adj_tab_k<4>(ap, num_sms, block, st);
-    case 5: return launch_adj_tab_k<5>(ap, num_sms, block, st);
-    case 6: return launch_adj_tab_k<6>(ap, num_sms, block, st);
-    case 7: return launch_adj_tab_k<7>(ap, num_sms, block, st);
-    case 8: return launch_adj_tab_k<8>(ap, num_sms, block, st);
     }
     return cudaErrorInvalidValue;
 }
