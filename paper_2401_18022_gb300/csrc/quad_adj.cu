@@ -112,6 +112,8 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
 #pragma unroll
             for (int k = 0; k < K2; ++k) R[k] = Rp[k] = dup2(0.0f);
             double ptot = 0.0;
+            const PieceBlocks pb = row_blocks(ns, G);
+            n_small += lane == 0 && part == 0 ? pb.R1 * G : 0;
             for (int ca = 0; ca < g.nc; ca += kAdjCand) {
                 const int cb = min(g.nc, ca + kAdjCand);
                 for (int c = ca; c < cb; ++c) {
@@ -145,8 +147,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
                     v1 += c == 1 ? val : 0.0f;
                     v2 += c == 2 ? val : 0.0f;
                 };
-                int small;
-                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int c0, int nq) {
+                piece_nodes(ns, pb, qp.gauss, G, ca, cb, [&](int c0, int nq) {
                     for (int q0 = 32 * part; q0 < nq; q0 += 32 * parts) {
                         Node nd;
                         int cls = -1;
@@ -203,7 +204,6 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
                         __syncwarp();
                     }
                 });
-                n_small += lane == 0 && part == 0 ? small : 0;
                 // sweep totals: the two halves' lane 0 meet on lane 0
                 const double s = (double)sum - (double)comp;
                 const double sw = (double)mult * (s + __shfl_down_sync(kFull, s, 16));

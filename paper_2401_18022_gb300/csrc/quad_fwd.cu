@@ -200,14 +200,14 @@ constexpr int kFwdSlots = 512;       // node slots of a chunk
 constexpr int kFwdCand = 3;          // F_c candidates swept together (most pieces have two)
 using FwdNodes = WarpNodes<kFwdSlots>;
 
-// Dynamic shared memory of k_quad_f32: zt [M], then per warp the nodes and the
-// candidates' step rows.
+// Dynamic shared memory of k_quad_f32: eB and zD (pair_tables), then per warp the
+// nodes and the candidates' step rows.
 __host__ __device__ constexpr size_t fwd_warp_bytes(int n_steps)
 {
-    return sizeof(FwdNodes) + (sizeof(float2) * kFwdCand * (size_t)n_steps + 15) / 16 * 16;
+    return sizeof(FwdNodes) + sizeof(float4) * kFwdCand * (size_t)step_pairs(n_steps);
 }
 #ifndef ISRS_FWD_MIN_BLOCKS
-#define ISRS_FWD_MIN_BLOCKS 4   // resident blocks per SM the register budget is sized for
+#define ISRS_FWD_MIN_BLOCKS 3   // resident blocks per SM the register budget is sized for
 #endif
 
 __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParams qp)
@@ -215,16 +215,13 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
     extern __shared__ float4 smem_f4[];
     const int M = qp.n_steps, G = qp.G;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float4 *zt = smem_f4;                              // [M] {edge(m+1)/2pi hi, lo, z, dz}
-    unsigned char *mine = reinterpret_cast<unsigned char *>(zt + M) + fwd_warp_bytes(M) * warp;
+    const int M2 = step_pairs(M);
+    float4 *eB = smem_f4, *zD = eB + M2;
+    unsigned char *mine = reinterpret_cast<unsigned char *>(zD + M2) + fwd_warp_bytes(M) * warp;
     FwdNodes &ns = *reinterpret_cast<FwdNodes *>(mine);
-    float2 *ek = reinterpret_cast<float2 *>(mine + sizeof(FwdNodes));   // [kFwdCand][M] {log2 p at f_c, K2}
+    float4 *ek = reinterpret_cast<float4 *>(mine + sizeof(FwdNodes));   // [kFwdCand][M2] {log2 p at f_c (2), K2 (2)}
 
-    for (int m = threadIdx.x; m < M; m += blockDim.x) {
-        const float4 za = qp.zs_a[m];   // {z_m, c_m, log2 dz_m, dz_m}
-        const float4 zb = qp.zs_b[m];   // {edge(m+1)/2pi hi, lo, z_m/2pi, 0}
-        zt[m] = make_float4(zb.x, zb.y, za.x, za.w);
-    }
+    pair_tables(qp, eB, zD);
     __syncthreads();
     const float phi_direct = 3.14159265f / qp.dz_max;
     const float phi_small = kBlkPhiL / qp.L;
@@ -249,29 +246,38 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
             __syncwarp();
             const PieceGeo &g = ns.geo;
             float sum = 0.0f, comp = 0.0f;
+            const PieceBlocks pb = row_blocks(ns, G);
+            n_small += lane == 0 && part == 0 ? pb.R1 * G : 0;
             for (int ca = 0; ca < g.nc; ca += kFwdCand) {
                 const int cb = min(g.nc, ca + kFwdCand);
                 // step rows of the candidates: ln p at the channel's centre
                 for (int c = ca; c < cb; ++c) {
                     const float at = g.at_ab + g.hat[c], F = g.Fc0 + 0.5f * (g.lo[c] + g.hi[c]);
-                    for (int m = lane; m < M; m += 32) {
-                        const float2 v = st[m];
-                        ek[(c - ca) * M + m] = make_float2(fmaf(v.y, F, fmaf(-at, zt[m].z, v.x)), v.y);
+                    for (int k = lane; k < M2; k += 32) {
+                        const float2 v = st[2 * k], u = st[min(2 * k + 1, M - 1)];
+                        const float4 z = zD[k];
+                        ek[(c - ca) * M2 + k] =
+                            make_float4(fmaf(v.y, F, fmaf(-at, z.x, v.x)),
+                                        2 * k + 1 < M ? fmaf(u.y, F, fmaf(-at, z.y, u.x)) : -1000.0f, v.y, u.y);
                     }
                 }
                 __syncwarp();
-                int small;
-                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int c0, int nq) {
+                piece_nodes(ns, pb, qp.gauss, G, ca, cb, [&](int c0, int nq) {
                     for (int q = lane + 32 * part; q < nq; q += 32 * parts) {
                         Node nd;
                         node_get(ns, qp.gauss, c0, q, nd);
                         const int ci = dbg_clamp(nd.ci, g.nc, kDbgCand, qp.dbg);
                         const float aphi = fabsf(nd.phi);
                         const float dF = (nd.x + nd.y) - 0.5f * (g.lo[ci] + g.hi[ci]);
-                        const float2 *e = ek + (ci - ca) * M;
+                        const float4 *e = ek + (ci - ca) * M2;
+                        const f32x2 dF2 = dup2(dF);
+                        const auto lp = [&](int k) {
+                            const float4 x = e[k];
+                            return fma2(pack2(x.z, x.w), dF2, pack2(x.x, x.y));
+                        };
                         const bool direct = aphi <= phi_direct;
-                        const float S2 = direct ? zsum_direct_n(nd.phi, dF, zt, e, M)
-                                                : zsum_tele_n(nd.phi, nd.phi_lo, dF, zt, e, M);
+                        const float S2 = direct ? zsum_direct_n(nd.phi, lp, zD, M2)
+                                                : zsum_tele_n<false>(nd.phi, nd.phi_lo, lp, eB, M2);
                         n_small += aphi <= phi_small ? nd.N : 0;
                         n_direct += aphi > phi_small && direct ? nd.N : 0;
                         n_tele += direct ? 0 : nd.N;
@@ -282,7 +288,6 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
                         sum = t;
                     }
                 });
-                n_small += lane == 0 && part == 0 ? small : 0;
             }
             acc += (double)(g.mult * g.wab) * ((double)sum - (double)comp);
         }
@@ -499,7 +504,7 @@ namespace {
 
 size_t fwd_smem(int n_steps, int block)
 {
-    return sizeof(float4) * (size_t)n_steps + fwd_warp_bytes(n_steps) * (size_t)(block / 32);
+    return sizeof(float4) * 2 * (size_t)step_pairs(n_steps) + fwd_warp_bytes(n_steps) * (size_t)(block / 32);
 }
 
 }  // namespace

@@ -39,10 +39,6 @@ constexpr int kMciRows = 32;       // rows of a group
 // Cells a warp takes together: at most 32 grid rows (and kMciUnits step rows).
 __host__ __device__ constexpr int mci_group(int G) { return G >= 32 ? 1 : (32 / G < kMciCells ? 32 / G : kMciCells); }
 
-// Steps go in pairs: pair k holds steps 2k, 2k + 1 (an odd last one beside a step
-// of weight 2^-1000 and the same edge).
-__host__ __device__ constexpr int step_pairs(int n_steps) { return (n_steps + 1) / 2; }
-
 // {1/2 log2(e) a_c, 1/2 log2(e) b_c} in FP32, steps outermost: float4 {a, a', b,
 // b'} of pair k and channel c at prof_ch_off[p] pairs + k n + c.  Neighbouring
 // points of a group have F_c in neighbouring channels, so a warp's 32 rows of one
@@ -77,63 +73,6 @@ __host__ __device__ constexpr size_t mci_warp_bytes(int n_steps)
     return sizeof(MciWarp) + ((size_t)kMciUnits * (step_pairs(n_steps) | 1) * 24 + 15) / 16 * 16;
 }
 
-// |S|^2 of Eq. slow_vary, telescoped, two steps at a time: log2 p = A + Sa da +
-// Sb db from the step row of the point's cell and F_c channel, eB[k] = {edge/2pi
-// hi, hi', lo, lo'}.
-__device__ __forceinline__ float zsum_tele_mt(float phi, float da, float db, const float4 *Qa, const float2 *Qb,
-                                              const float4 *eB, int M2)
-{
-    const f32x2 ph = dup2(phi), nph = dup2(-phi), a2 = dup2(da), b2 = dup2(db);
-    float Er = 1.0f, Ei = 0.0f;
-    f32x2 Sr = dup2(0.0f), Si = dup2(0.0f);
-#pragma unroll 4
-    for (int k = 0; k < M2; ++k) {
-        const float4 e = eB[k], q = Qa[k];
-        const float2 qb = Qb[k];
-        float s0, c0, s1, c1, l0, l1;
-        sincos_turn2(rev_fraction2<true>(ph, nph, ph, pack2(e.x, e.y), pack2(e.z, e.w)), s0, c0, s1, c1);
-        unpack2(fma2(pack2(qb.x, qb.y), b2, fma2(pack2(q.z, q.w), a2, pack2(q.x, q.y))), l0, l1);
-        const f32x2 p = pack2(ex2_approx(l0), ex2_approx(l1));
-        Sr = fma2(p, pack2(c0 - Er, c1 - c0), Sr);
-        Si = fma2(p, pack2(s0 - Ei, s1 - s0), Si);
-        Er = c1;
-        Ei = s1;
-    }
-    float r0, r1, i0, i1;
-    unpack2(Sr, r0, r1);
-    unpack2(Si, i0, i1);
-    const float sr = r0 + r1, si = i0 + i1;
-    return __fdividef(sr * sr + si * si, phi * phi);
-}
-
-// ... in the direct form (few points): zA[m] = {z, dz}
-__device__ __forceinline__ float zsum_direct_mt(float phi, float da, float db, const float4 *Qa, const float2 *Qb,
-                                                const float2 *zA, int M)
-{
-    float Sr = 0.0f, Si = 0.0f;
-    const float hphi = 0.5f * phi;
-    const float phir = phi * 0.15915494309189535f;
-    for (int m = 0; m < M; ++m) {
-        const int k = m >> 1, o = m & 1;
-        const float4 q = Qa[k];
-        const float2 qb = Qb[k], a = zA[m];
-        float sn, cs;
-        sincos_rev(phir, a.x, sn, cs);
-        const float x = hphi * a.y;
-        const float x2 = x * x;
-        float sc = fmaf(x2, -2.5052108e-8f, 2.7557319e-6f);   // -1/11!, 1/9!
-        sc = fmaf(x2, sc, -1.9841270e-4f);                     // -1/7!
-        sc = fmaf(x2, sc, 8.3333333e-3f);                      // 1/5!
-        sc = fmaf(x2, sc, -1.6666667e-1f);                     // -1/3!
-        sc = fmaf(x2, sc, 1.0f);
-        const float lp = fmaf(o ? qb.y : qb.x, db, fmaf(o ? q.w : q.z, da, o ? q.y : q.x));
-        const float amp = ex2_approx(lp) * (sc * a.y);        // p_m dz_m sinc
-        Sr = fmaf(amp, cs, Sr);
-        Si = fmaf(amp, sn, Si);
-    }
-    return Sr * Sr + Si * Si;
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -152,25 +91,19 @@ __global__ void __launch_bounds__(256, 2) k_quad_mci_f32_tab(QuadParams qp)
     const int M = qp.n_steps, G = qp.G, M2 = step_pairs(M), MS = M2 | 1, GC = mci_group(G);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     float4 *eB = smem_f4;                              // [M2] {edge/2pi hi, hi', lo, lo'}
-    float2 *zA = reinterpret_cast<float2 *>(eB + M2);  // [2 M2] {z, dz}
-    unsigned char *mine = reinterpret_cast<unsigned char *>(zA + 2 * M2) + mci_warp_bytes(M) * warp;
+    float4 *zD = eB + M2;                              // [M2] {z, z', dz, dz'}
+    unsigned char *mine = reinterpret_cast<unsigned char *>(zD + M2) + mci_warp_bytes(M) * warp;
     MciWarp &w = *reinterpret_cast<MciWarp *>(mine);
     float4 *Qa = reinterpret_cast<float4 *>(mine + sizeof(MciWarp));       // [kMciUnits][MS]
     float2 *Qb = reinterpret_cast<float2 *>(Qa + (size_t)kMciUnits * MS);  // [kMciUnits][MS]
-    float *rel = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(zA + 2 * M2) +
+    float *rel = reinterpret_cast<float *>(reinterpret_cast<unsigned char *>(zD + M2) +
                                            mci_warp_bytes(M) * nw);     // [n] channel centre - f_i
     float *hb = rel + qp.mci_n_max;                    // [n] B/2
     __shared__ CellRound cr;
     __shared__ double scratch[32];
     __shared__ int s_item;
 
-    for (int k = threadIdx.x; k < M2; k += blockDim.x) {
-        const int m0 = 2 * k, m1 = min(2 * k + 1, M - 1);
-        const float4 b0 = qp.zs_b[m0], b1 = qp.zs_b[m1];
-        eB[k] = make_float4(b0.x, b1.x, b0.y, b1.y);
-        zA[m0] = make_float2(qp.zs_a[m0].x, qp.zs_a[m0].w);
-        zA[2 * k + 1] = make_float2(qp.zs_a[m1].x, qp.zs_a[m1].w);
-    }
+    pair_tables(qp, eB, zD);
     const float c3 = (float)(kPi * qp.beta3);
     const float c4 = (float)(2.0 * kPi * kPi / 3.0 * qp.beta4);
     const float b2 = (float)qp.beta2;
@@ -216,8 +149,13 @@ __global__ void __launch_bounds__(256, 2) k_quad_mci_f32_tab(QuadParams qp)
             if (lane < cnt) {
                 const float4 v = w.Lp[at];
                 const int u = w.Lu[at] * MS;
-                const float S2 = f ? zsum_tele_mt(v.x, v.y, v.z, Qa + u, Qb + u, eB, M2)
-                                   : zsum_direct_mt(v.x, v.y, v.z, Qa + u, Qb + u, zA, M);
+                const f32x2 da = dup2(v.y), db = dup2(v.z);
+                const auto lp = [&](int k) {
+                    const float4 x = Qa[u + k];
+                    const float2 y = Qb[u + k];
+                    return fma2(pack2(y.x, y.y), db, fma2(pack2(x.z, x.w), da, pack2(x.x, x.y)));
+                };
+                const float S2 = f ? zsum_tele_n<true>(v.x, 0.0f, lp, eB, M2) : zsum_direct_n(v.x, lp, zD, M2);
                 const float y = v.w * S2 * array_factor_f(v.x, qp) - comp;
                 const float t = sum + y;
                 comp = (t - sum) - y;

@@ -388,16 +388,20 @@ __device__ __forceinline__ int row_whole(const PieceGeo &g, const NodeRow &o, in
 // candidate, with one set of limits and |phi| band <= kBlkPhiL, cut at |phi|
 // band = kBlkPhiLow and into parts of kGaussMaxN rows.  Along t in [-1, 1] over
 // N rows upsilon1 (so the weight and phi) is exp-like with D = N ds / 2, and the
-// phase swings by at most |phi| band D.  Whole warp; writes ns.blk, returns the
-// units (rows of the rules) of all blocks, R1 and the candidate.
+// phase swings by at most |phi| band D.  Whole warp; writes ns.blk.
+struct PieceBlocks {
+    int units;                  // rows of the rules, all blocks
+    int R1, nblk, cand;         // rows covered, blocks, their F_c candidate
+};
+
 template <int Cap>
-__device__ __forceinline__ int row_blocks(WarpNodes<Cap> &ns, int G, int &R1, int &nblk, int &cand)
+__device__ __forceinline__ PieceBlocks row_blocks(WarpNodes<Cap> &ns, int G)
 {
+    PieceBlocks pb = {0, 0, 0, -1};
+    int &R1 = pb.R1, &nblk = pb.nblk, &cand = pb.cand, &units = pb.units;
     const PieceGeo &g = ns.geo;
     const int lane = threadIdx.x & 31;
     float ph_last = 0.0f;
-    R1 = 0;
-    cand = -1;
     // candidate and limits of row r (-1: not in one candidate), |phi| band
     const auto test = [&](int r, float &ph) {
         NodeRow o;
@@ -416,7 +420,7 @@ __device__ __forceinline__ int row_blocks(WarpNodes<Cap> &ns, int G, int &R1, in
         float ph;
         const int key = test(min(lane * step, G - 1), ph);
         key0 = __shfl_sync(0xffffffffu, key, 0);
-        if (key0 < 0 || !(__shfl_sync(0xffffffffu, ph, 0) <= kBlkPhiL)) return 0;
+        if (key0 < 0 || !(__shfl_sync(0xffffffffu, ph, 0) <= kBlkPhiL)) return pb;
         if ((key0 & 3) == 3 || g.s1 == g.s2) {
             const bool ok = lane * step < G && key == key0 && ph <= kBlkPhiL;
             const int bad = __ffs(~__ballot_sync(0xffffffffu, ok)) - 1;      // -1: none
@@ -439,8 +443,6 @@ __device__ __forceinline__ int row_blocks(WarpNodes<Cap> &ns, int G, int &R1, in
     // rows from the block's top down to |phi| band = kBlkPhiLow
     int top = ph_last > kBlkPhiLow ? (int)ceilf(__fdividef(__logf(ph_last / kBlkPhiLow), g.ds)) : 0;
     top = min(top, R1);
-    int units = 0;
-    nblk = 0;
     for (int low = 1; low >= 0; --low) {
         const int n_rows = low ? R1 - top : top, parts = (n_rows + kGaussMaxN - 1) / kGaussMaxN;
         for (int s = 0; s < parts; ++s) {
@@ -456,7 +458,7 @@ __device__ __forceinline__ int row_blocks(WarpNodes<Cap> &ns, int G, int &R1, in
         }
     }
     __syncwarp();
-    return units;
+    return pb;
 }
 
 // Unit q of the piece: a row of a block's rule (q < nv) or a row of its own.
@@ -550,17 +552,14 @@ __device__ __forceinline__ void node_get(const WarpNodes<Cap> &ns, const float2 
 }
 
 // The nodes of a piece in chunks: f(c0, number of slots) is called by the whole
-// warp for each chunk, with ns filled for node_get.  small gets the columns of
-// the rows taken in blocks.
+// warp for each chunk, with ns filled for node_get (candidates [ca, cb)).
 template <int Cap, typename F>
-__device__ __forceinline__ void piece_nodes(WarpNodes<Cap> &ns, const float2 *gauss, int G, int ca, int cb,
-                                            int &small, const F &f)
+__device__ __forceinline__ void piece_nodes(WarpNodes<Cap> &ns, const PieceBlocks &pb, const float2 *gauss, int G,
+                                            int ca, int cb, const F &f)
 {
     const int lane = threadIdx.x & 31;
-    int R1, nblk = 0, cand;
-    const int nv = row_blocks(ns, G, R1, nblk, cand);
+    const int nv = pb.units, R1 = pb.R1, nblk = pb.nblk, cand = pb.cand;
     const bool mine = cand >= ca && cand < cb;        // the blocks' candidate belongs to this sweep
-    small = mine ? R1 * G : 0;
     const int units = nv + (G - R1);
     for (int u0 = mine ? 0 : nv; u0 < units; u0 += 32) {
         const int q = u0 + lane;

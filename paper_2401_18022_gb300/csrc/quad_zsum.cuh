@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "f32x2.cuh"
 #include "quad_common.cuh"
 
 namespace isrs {
@@ -98,100 +99,81 @@ __device__ __forceinline__ float zsum_tele_f(float phi, float Fc, float at, cons
     return __fdividef(Sr * Sr + Si * Si, phi * phi);
 }
 
-// The same two forms for a node of the row sums: zt[m] = {z_{m+1}/2pi hi, lo,
-// z_m, dz_m} and, for the node's F_c candidate, ek[m] = {log2 p_m at the
-// channel's centre, K2_m}, so log2 p_m = ek.x + K2_m dF with dF = F_c - f_c; phi
-// is a float-float value (the direct form's phases need only its head).
-__device__ __forceinline__ float zsum_direct_n(float phi, float dF, const float4 *zt, const float2 *ek, int M)
+// The same two forms for a node of the row sums, two steps at a time (f32x2.cuh):
+// pair k of eB = {z_{m+1}/2pi hi, hi', lo, lo'}, of zD = {z_m, z', dz_m, dz'},
+// and lp(k) gives log2 p of the pair at the node; an odd last step stands beside one
+// of weight 2^-1000 with the same edge.  phi is float-float (the direct form's
+// phases need only its head).  Packed, a step takes ~13 instructions where the
+// scalar form took ~19; bound by the XU pipe (20 cycles per warp and step).
+template <typename LP>
+__device__ __forceinline__ float zsum_direct_n(float phi, const LP &lp, const float4 *zD, int M2)
 {
-    float Sr = 0.0f, Si = 0.0f;
-    const float hphi = 0.5f * phi;
-    const float phir = phi * 0.15915494309189535f;
-#pragma unroll 4
-    for (int m = 0; m < M; ++m) {
-        const float4 a = zt[m];
-        const float2 e = ek[m];
-        float sn, cs;
-        sincos_rev(phir, a.z, sn, cs);
-        const float x = hphi * a.w;
-        const float x2 = x * x;
-        float sc = fmaf(x2, -2.5052108e-8f, 2.7557319e-6f);   // -1/11!, 1/9!
-        sc = fmaf(x2, sc, -1.9841270e-4f);                     // -1/7!
-        sc = fmaf(x2, sc, 8.3333333e-3f);                      // 1/5!
-        sc = fmaf(x2, sc, -1.6666667e-1f);                     // -1/3!
-        sc = fmaf(x2, sc, 1.0f);
-        const float amp = ex2_approx(fmaf(e.y, dF, e.x)) * (sc * a.w);
-        Sr = fmaf(amp, cs, Sr);
-        Si = fmaf(amp, sn, Si);
+    const f32x2 hph = dup2(0.5f * phi), phr = dup2(phi * 0.15915494309189535f),
+                nphr = dup2(-phi * 0.15915494309189535f);
+    const f32x2 mg = dup2(12582912.0f), nm = dup2(-12582912.0f);
+    f32x2 Sr = dup2(0.0f), Si = dup2(0.0f);
+#pragma unroll 2
+    for (int k = 0; k < M2; ++k) {
+        const float4 z = zD[k];
+        const f32x2 zz = pack2(z.x, z.y), dz = pack2(z.z, z.w);
+        float s0, c0, s1, c1, l0, l1;
+        sincos_turn2(fma2(phr, zz, add2(fma2(nphr, zz, mg), nm)), s0, c0, s1, c1);
+        const f32x2 x = mul2(hph, dz), x2 = mul2(x, x);       // sinc to x^10, |x| <= pi/2
+        f32x2 sc = fma2(x2, dup2(-2.5052108e-8f), dup2(2.7557319e-6f));
+        sc = fma2(x2, sc, dup2(-1.9841270e-4f));
+        sc = fma2(x2, sc, dup2(8.3333333e-3f));
+        sc = fma2(x2, sc, dup2(-1.6666667e-1f));
+        sc = fma2(x2, sc, dup2(1.0f));
+        unpack2(lp(k), l0, l1);
+        const f32x2 amp = mul2(pack2(ex2_approx(l0), ex2_approx(l1)), mul2(sc, dz));
+        Sr = fma2(amp, pack2(c0, c1), Sr);
+        Si = fma2(amp, pack2(s0, s1), Si);
     }
-    return Sr * Sr + Si * Si;
+    float r0, r1, i0, i1;
+    unpack2(Sr, r0, r1);
+    unpack2(Si, i0, i1);
+    const float sr = r0 + r1, si = i0 + i1;
+    return sr * sr + si * si;
 }
 
-__device__ __forceinline__ float zsum_tele_n(float phi, float phi_lo, float dF, const float4 *zt, const float2 *ek,
-                                             int M)
+template <bool Wide, typename LP>
+__device__ __forceinline__ float zsum_tele_n(float phi, float phi_lo, const LP &lp, const float4 *eB, int M2)
 {
-    float Er = 1.0f, Ei = 0.0f, Sr = 0.0f, Si = 0.0f;
+    const f32x2 ph = dup2(phi), nph = dup2(-phi), pl = dup2(phi_lo);
+    float Er = 1.0f, Ei = 0.0f;
+    f32x2 Sr = dup2(0.0f), Si = dup2(0.0f);
 #pragma unroll 4
-    for (int m = 0; m < M; ++m) {
-        const float4 a = zt[m];
-        const float2 e = ek[m];
-        float sn, cs;
-        phasor_rev_ff(phi, a.x, a.y, sn, cs, phi_lo);
-        const float p = ex2_approx(fmaf(e.y, dF, e.x));
-        Sr = fmaf(p, cs - Er, Sr);
-        Si = fmaf(p, sn - Ei, Si);
-        Er = cs;
-        Ei = sn;
+    for (int k = 0; k < M2; ++k) {
+        const float4 e = eB[k];
+        float s0, c0, s1, c1, l0, l1;
+        sincos_turn2(rev_fraction2<Wide>(ph, nph, pl, pack2(e.x, e.y), pack2(e.z, e.w)), s0, c0, s1, c1);
+        unpack2(lp(k), l0, l1);
+        const f32x2 p = pack2(ex2_approx(l0), ex2_approx(l1));
+        Sr = fma2(p, pack2(c0 - Er, c1 - c0), Sr);
+        Si = fma2(p, pack2(s0 - Ei, s1 - s0), Si);
+        Er = c1;
+        Ei = s1;
     }
-    return __fdividef(Sr * Sr + Si * Si, phi * phi);
+    float r0, r1, i0, i1;
+    unpack2(Sr, r0, r1);
+    unpack2(Si, i0, i1);
+    const float sr = r0 + r1, si = i0 + i1;
+    return __fdividef(sr * sr + si * si, phi * phi);
 }
 
-// ... with the tabulated profile: q[m] = {log2 p_m, slope along the node's
-// longer axis, along the shorter}, dl and dd the offsets of F_a, F_b inside
-// their channels (in that order of axes).
-__device__ __forceinline__ float zsum_direct_nt(float phi, float dl, float dd, const float4 *zt, const float4 *q,
-                                                int M)
-{
-    float Sr = 0.0f, Si = 0.0f;
-    const float hphi = 0.5f * phi;
-    const float phir = phi * 0.15915494309189535f;
-#pragma unroll 4
-    for (int m = 0; m < M; ++m) {
-        const float4 a = zt[m];
-        const float4 e = q[m];
-        float sn, cs;
-        sincos_rev(phir, a.z, sn, cs);
-        const float x = hphi * a.w;
-        const float x2 = x * x;
-        float sc = fmaf(x2, -2.5052108e-8f, 2.7557319e-6f);   // -1/11!, 1/9!
-        sc = fmaf(x2, sc, -1.9841270e-4f);                     // -1/7!
-        sc = fmaf(x2, sc, 8.3333333e-3f);                      // 1/5!
-        sc = fmaf(x2, sc, -1.6666667e-1f);                     // -1/3!
-        sc = fmaf(x2, sc, 1.0f);
-        const float amp = ex2_approx(fmaf(e.z, dd, fmaf(e.y, dl, e.x))) * (sc * a.w);
-        Sr = fmaf(amp, cs, Sr);
-        Si = fmaf(amp, sn, Si);
-    }
-    return Sr * Sr + Si * Si;
-}
+// Steps in pairs: pair k holds steps 2k, 2k + 1.
+__host__ __device__ constexpr int step_pairs(int n_steps) { return (n_steps + 1) / 2; }
 
-__device__ __forceinline__ float zsum_tele_nt(float phi, float phi_lo, float dl, float dd, const float4 *zt,
-                                              const float4 *q, int M)
+// eB and zD of every pair, filled by the whole block
+__device__ __forceinline__ void pair_tables(const QuadParams &qp, float4 *eB, float4 *zD)
 {
-    float Er = 1.0f, Ei = 0.0f, Sr = 0.0f, Si = 0.0f;
-#pragma unroll 4
-    for (int m = 0; m < M; ++m) {
-        const float4 a = zt[m];
-        const float4 e = q[m];
-        float sn, cs;
-        phasor_rev_ff(phi, a.x, a.y, sn, cs, phi_lo);
-        const float p = ex2_approx(fmaf(e.z, dd, fmaf(e.y, dl, e.x)));
-        Sr = fmaf(p, cs - Er, Sr);
-        Si = fmaf(p, sn - Ei, Si);
-        Er = cs;
-        Ei = sn;
+    const int M = qp.n_steps;
+    for (int k = threadIdx.x; k < step_pairs(M); k += blockDim.x) {
+        const int m0 = 2 * k, m1 = min(2 * k + 1, M - 1);
+        const float4 b0 = qp.zs_b[m0], b1 = qp.zs_b[m1], a0 = qp.zs_a[m0], a1 = qp.zs_a[m1];
+        eB[k] = make_float4(b0.x, b1.x, b0.y, b1.y);
+        zD[k] = make_float4(a0.x, a1.x, a0.w, a1.w);
     }
-    return __fdividef(Sr * Sr + Si * Si, phi * phi);
 }
 
 // As phasor_rev_ff, for phases far beyond 2^22 revolutions (the MCI cells, up

@@ -402,31 +402,34 @@ constexpr int kTabSlots = 512;       // node slots of a chunk
 constexpr int kTabCand = 2;          // F_c candidates swept together (most pieces have two)
 using TabNodes = WarpNodes<kTabSlots>;
 
-// Dynamic shared memory of k_quad_f32_tab: zt [M], then per warp the nodes and
-// the candidates' step rows.
+// Dynamic shared memory of k_quad_f32_tab: eB and zD (pair_tables), then per warp
+// the nodes and the candidates' step rows.
 __host__ __device__ constexpr size_t tab_warp_bytes(int n_steps)
 {
-    return sizeof(TabNodes) + sizeof(float4) * kTabCand * (size_t)n_steps;
+    return sizeof(TabNodes) + ((size_t)24 * kTabCand * step_pairs(n_steps) + 15) / 16 * 16;
 }
 
 // As k_quad_f32 (quad_fwd.cu: one warp per tile, row sums from nodes), with the
 // step rows of the tabulated profile.  The low rows' blocks replace the 2-D
 // contraction of the small-phase moments (176 coefficients per candidate and
 // piece) that this kernel used to build.
-__global__ void __launch_bounds__(256, 4) k_quad_f32_tab(QuadParams qp)
+#ifndef ISRS_TAB_MIN_BLOCKS
+#define ISRS_TAB_MIN_BLOCKS 3   // resident blocks per SM the register budget is sized for
+#endif
+
+__global__ void __launch_bounds__(256, ISRS_TAB_MIN_BLOCKS) k_quad_f32_tab(QuadParams qp)
 {
     extern __shared__ float4 smem_f4[];
     const int M = qp.n_steps, G = qp.G;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float4 *zt = smem_f4;                              // [M] {edge(m+1)/2pi hi, lo, z, dz}
-    unsigned char *mine = reinterpret_cast<unsigned char *>(zt + M) + tab_warp_bytes(M) * warp;
+    const int M2 = step_pairs(M);
+    float4 *eB = smem_f4, *zD = eB + M2;
+    unsigned char *mine = reinterpret_cast<unsigned char *>(zD + M2) + tab_warp_bytes(M) * warp;
     TabNodes &ns = *reinterpret_cast<TabNodes *>(mine);
-    float4 *Q = reinterpret_cast<float4 *>(mine + sizeof(TabNodes));   // [kTabCand][M]
+    float4 *Qa = reinterpret_cast<float4 *>(mine + sizeof(TabNodes));  // [kTabCand][M2] {A, A', Sl, Sl'}
+    float2 *Qb = reinterpret_cast<float2 *>(Qa + kTabCand * M2);       // [kTabCand][M2] {Sd, Sd'}
 
-    for (int m = threadIdx.x; m < M; m += blockDim.x) {
-        const float4 za = qp.zs_a[m], zb = qp.zs_b[m];
-        zt[m] = make_float4(zb.x, zb.y, za.x, za.w);
-    }
+    pair_tables(qp, eB, zD);
     __syncthreads();
     const float phi_direct = 3.14159265f / qp.dz_max;
     const float phi_small = kBlkPhiL / qp.L;
@@ -450,33 +453,43 @@ __global__ void __launch_bounds__(256, 4) k_quad_f32_tab(QuadParams qp)
             __syncwarp();
             PieceGeo &g = ns.geo;
             float sum = 0.0f, comp = 0.0f;
+            const PieceBlocks pb = row_blocks(ns, G);
+            n_small += lane == 0 && part == 0 ? pb.R1 * G : 0;
             for (int ca = 0; ca < g.nc; ca += kTabCand) {
                 const int cb = min(g.nc, ca + kTabCand);
                 float tilt = 0.0f;
                 for (int c = ca; c < cb; ++c) {
                     const double fc = qp.ch_frel[coff + pc.c_lo + c];
-                    for (int m = lane; m < M; m += 32) {
-                        const float4 r = tab_row(tp, pc.c_lo + c, fc, m, M);
-                        Q[(c - ca) * M + m] = r;
-                        tilt = fmaxf(tilt, fmaxf(fabsf(r.y), fabsf(r.z)));
+                    for (int k = lane; k < M2; k += 32) {
+                        const float4 r = tab_row(tp, pc.c_lo + c, fc, 2 * k, M);
+                        float4 u = make_float4(-1000.0f, 0.0f, 0.0f, 0.0f);
+                        if (2 * k + 1 < M) u = tab_row(tp, pc.c_lo + c, fc, 2 * k + 1, M);
+                        Qa[(c - ca) * M2 + k] = make_float4(r.x, u.x, r.y, u.y);
+                        Qb[(c - ca) * M2 + k] = make_float2(r.z, u.z);
+                        tilt = fmaxf(tilt, fmaxf(fmaxf(fabsf(r.y), fabsf(r.z)), fmaxf(fabsf(u.y), fabsf(u.z))));
                     }
                 }
                 // the largest slope of ln p bounds its swing along a row
                 tilt = 0.69314718f * __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(tilt)));
                 if (lane == 0) g.tilt = tilt;
                 __syncwarp();
-                int small;
-                piece_nodes(ns, qp.gauss, G, ca, cb, small, [&](int c0, int nq) {
+                piece_nodes(ns, pb, qp.gauss, G, ca, cb, [&](int c0, int nq) {
                     for (int q = lane + 32 * part; q < nq; q += 32 * parts) {
                         Node nd;
                         node_get(ns, qp.gauss, c0, q, nd);
                         const int ci = dbg_clamp(nd.ci, g.nc, kDbgCand, qp.dbg);
                         const float aphi = fabsf(nd.phi);
-                        const float dl = tp.ol + nd.x, dd = tp.od + nd.y;
-                        const float4 *e = Q + (ci - ca) * M;
+                        const f32x2 dl = dup2(tp.ol + nd.x), dd = dup2(tp.od + nd.y);
+                        const float4 *qa = Qa + (ci - ca) * M2;
+                        const float2 *qb = Qb + (ci - ca) * M2;
+                        const auto lp = [&](int k) {
+                            const float4 x = qa[k];
+                            const float2 y = qb[k];
+                            return fma2(pack2(y.x, y.y), dd, fma2(pack2(x.z, x.w), dl, pack2(x.x, x.y)));
+                        };
                         const bool direct = aphi <= phi_direct;
-                        const float S2 = direct ? zsum_direct_nt(nd.phi, dl, dd, zt, e, M)
-                                                : zsum_tele_nt(nd.phi, nd.phi_lo, dl, dd, zt, e, M);
+                        const float S2 = direct ? zsum_direct_n(nd.phi, lp, zD, M2)
+                                                : zsum_tele_n<false>(nd.phi, nd.phi_lo, lp, eB, M2);
                         n_small += aphi <= phi_small ? nd.N : 0;
                         n_direct += aphi > phi_small && direct ? nd.N : 0;
                         n_tele += direct ? 0 : nd.N;
@@ -486,7 +499,6 @@ __global__ void __launch_bounds__(256, 4) k_quad_f32_tab(QuadParams qp)
                         sum = t;
                     }
                 });
-                n_small += lane == 0 && part == 0 ? small : 0;
             }
             acc += (double)(g.mult * g.wab) * ((double)sum - (double)comp);
         }
@@ -613,7 +625,7 @@ cudaError_t launch_quad_tab(const QuadParams &qp, int precision, int num_sms, in
     const void *fn = (const void *)k_quad_f64_tab;
     if (precision == 0) {
         // as launch_quad: any number of warps to a block
-        const auto bytes = [&](int b) { return sizeof(float4) * (size_t)qp.n_steps + tab_warp_bytes(qp.n_steps) * (b / 32); };
+        const auto bytes = [&](int b) { return sizeof(float4) * 2 * step_pairs(qp.n_steps) + tab_warp_bytes(qp.n_steps) * (b / 32); };
         fn = (const void *)k_quad_f32_tab;
         if (qp.n_items < num_sms * (block / 32)) block = 32;
         while (block > 32 && bytes(block) > 200 * 1024) block -= 32;

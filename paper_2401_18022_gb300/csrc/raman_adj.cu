@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
             const int4 pr = ap.prow[kp];
             __syncwarp();
             PieceGeo &g = ns.geo;
+            const PieceBlocks pb = row_blocks(ns, G);
             for (int cc = 0; cc < g.nc; ++cc) {
                 const double fc = qp.ch_frel[coff + pc.c_lo + cc];
                 float tilt = 0.0f;
@@ -124,8 +125,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
                     comp = (t - sum) - y;
                     sum = t;
                 };
-                int small;
-                piece_nodes(ns, qp.gauss, G, cc, cc + 1, small, [&](int c0, int nq) {
+                piece_nodes(ns, pb, qp.gauss, G, cc, cc + 1, [&](int c0, int nq) {
                     for (int q0 = 32 * part; q0 < nq; q0 += 32 * parts) {
                         Node nd;
                         int cls = -1;
