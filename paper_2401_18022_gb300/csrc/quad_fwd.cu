@@ -239,6 +239,7 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
         const float tilt = (float)qp.kap_L[item.prof];
         const int part = item.part & 0xffff, parts = item.part >> 16;
         double acc = 0.0;
+#pragma unroll 1
         for (int k = item.piece0; k < item.piece1; ++k) {
             const DevPiece &pc = qp.pieces[dbg_clamp(k, qp.n_pieces, kDbgPiece, qp.dbg)];
             __syncwarp();
@@ -248,11 +249,14 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
             float sum = 0.0f, comp = 0.0f;
             const PieceBlocks pb = row_blocks(ns, G);
             n_small += lane == 0 && part == 0 ? pb.R1 * G : 0;
+#pragma unroll 1
             for (int ca = 0; ca < g.nc; ca += kFwdCand) {
                 const int cb = min(g.nc, ca + kFwdCand);
                 // step rows of the candidates: ln p at the channel's centre
+#pragma unroll 1
                 for (int c = ca; c < cb; ++c) {
                     const float at = g.at_ab + g.hat[c], F = g.Fc0 + 0.5f * (g.lo[c] + g.hi[c]);
+#pragma unroll 2
                     for (int k = lane; k < M2; k += 32) {
                         const float2 v = st[2 * k], u = st[min(2 * k + 1, M - 1)];
                         const float4 z = zD[k];
@@ -263,6 +267,7 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
                 }
                 __syncwarp();
                 piece_nodes(ns, pb, qp.gauss, G, ca, cb, [&](int c0, int nq) {
+#pragma unroll 1
                     for (int q = lane + 32 * part; q < nq; q += 32 * parts) {
                         Node nd;
                         node_get(ns, qp.gauss, c0, q, nd);

@@ -283,13 +283,21 @@ __device__ __forceinline__ int row_turn(const PieceGeo &g, const NodeRow &o, int
 
 // The runs of one row in column order: f(candidate, j0, N).  On one half-open
 // interval of columns u is monotone, so a candidate's columns are a run found
-// by bisection.
+// by bisection.  whole: the one candidate that holds every column, or -1.
+// (The loops of the set-up stay rolled: unrolled, a kernel's code is 94 KB and
+// the warps, each at its own place in it, wait for instructions.)
 template <typename F>
-__device__ __forceinline__ void row_runs(const PieceGeo &g, const NodeRow &o, int G, int ca, int cb, const F &f)
+__device__ __forceinline__ void row_runs(const PieceGeo &g, const NodeRow &o, int G, int ca, int cb, int whole,
+                                         const F &f)
 {
     const float c0 = 0.5f - 0.5f * (float)G;
     const auto u_at = [&](int j) { return row_u(g, o, ((float)j + c0) * o.du2); };
-    const int jm = row_turn(g, o, G);
+    const int jm = whole >= 0 ? 0 : row_turn(g, o, G);
+    if (whole >= 0) {
+        ca = whole;
+        cb = whole + 1;
+    }
+#pragma unroll 1
     for (int part = 0; part < 2; ++part) {
         const int ja = part == 0 ? 0 : jm, jb = part == 0 ? jm : G;
         if (jb <= ja) continue;
@@ -303,6 +311,7 @@ __device__ __forceinline__ void row_runs(const PieceGeo &g, const NodeRow &o, in
         const auto first = [&](float e) {
             int lo = ja + 1, hi = jb;
             int m = (int)fminf(fmaxf(ceilf((e - ua) * slope), 1.0f), (float)(jb - 1 - ja)) + ja;
+#pragma unroll 1
             for (int it = 0; lo < hi; ++it) {
                 const float u = m == jb - 1 ? ub : u_at(m);
                 const bool past = up ? u >= e : u < e;
@@ -313,13 +322,22 @@ __device__ __forceinline__ void row_runs(const PieceGeo &g, const NodeRow &o, in
             }
             return lo;
         };
+#pragma unroll 1
         for (int q = ca; q < cb; ++q) {
             const int c = up ? q : ca + cb - 1 - q;
             const float lo = g.lo[c], hi = g.hi[c];
-            if ((up ? ub : ua) < lo || (up ? ua : ub) >= hi) continue;
-            // entering edge, leaving edge
-            const int j0 = (up ? ua >= lo : ua < hi) ? ja : first(up ? lo : hi);
-            const int j1 = (up ? ub < hi : ub >= lo) ? jb : first(up ? hi : lo);
+            int j0 = ja, j1 = jb;
+            if (whole < 0) {
+                if ((up ? ub : ua) < lo || (up ? ua : ub) >= hi) continue;
+#pragma unroll 1
+                for (int side = 0; side < 2; ++side) {            // entering edge, leaving edge
+                    const float e = up == (side == 0) ? lo : hi;
+                    const bool in = side == 0 ? (up ? ua >= e : ua < e) : (up ? ub < e : ub >= e);
+                    const int j = in ? (side == 0 ? ja : jb) : first(e);
+                    if (side == 0) j0 = j;
+                    else j1 = j;
+                }
+            }
             if (j1 > j0) f(c, j0, j1 - j0);
         }
     }
@@ -352,8 +370,11 @@ __device__ __forceinline__ void run_parts(const PieceGeo &g, const NodeRow &o, i
         parts = max((N + kGaussMaxN - 1) / kGaussMaxN, (n + 23) / 24);
         parts = min(parts, (N + kGaussMaxNodes - 1) / kGaussMaxNodes);
     }
+    int b = 0;
+#pragma unroll 1
     for (int s = 0; s < parts; ++s) {
-        const int a = (int)((long long)N * s / parts), b = (int)((long long)N * (s + 1) / parts);
+        const int a = b;
+        b = parts == 1 ? N : N * (s + 1) / parts;
         const int Ns = b - a;
         if (parts > 1) n = gauss_need(per * (float)Ns, hd * (float)Ns);
         const int nn = n <= kGaussMaxNodes ? gauss_nodes(gauss_pick(n)) : Ns;
@@ -379,6 +400,7 @@ __device__ __forceinline__ int row_whole(const PieceGeo &g, const NodeRow &o, in
     const float r = mx - mn;
     ph = g.band * (fabsf(o.phi0) + r * (fabsf(p1) + fabsf(p2) * r));
     int c = -1;
+#pragma unroll 1
     for (int q = 0; q < g.nc; ++q)
         if (mn >= g.lo[q] && mx < g.hi[q]) c = q;
     return c;
@@ -415,36 +437,41 @@ __device__ __forceinline__ PieceBlocks row_blocks(WarpNodes<Cap> &ns, int G)
     // following upsilon1, or f1 and f2 of one sign, the ends of the row's u are
     // monotone in upsilon1; otherwise every row is tested.
     const int step = (G + 31) / 32;
-    int key0;
-    {
+    int key0 = -1;
+#pragma unroll 1
+    for (int r0 = -1; r0 < G;) {
+        const bool coarse = r0 < 0;
+        const int r = coarse ? lane * step : r0 + lane;
         float ph;
-        const int key = test(min(lane * step, G - 1), ph);
-        key0 = __shfl_sync(0xffffffffu, key, 0);
-        if (key0 < 0 || !(__shfl_sync(0xffffffffu, ph, 0) <= kBlkPhiL)) return pb;
-        if ((key0 & 3) == 3 || g.s1 == g.s2) {
-            const bool ok = lane * step < G && key == key0 && ph <= kBlkPhiL;
-            const int bad = __ffs(~__ballot_sync(0xffffffffu, ok)) - 1;      // -1: none
-            R1 = bad < 0 ? min(G, 31 * step + 1) : (bad - 1) * step + 1;
-            ph_last = __shfl_sync(0xffffffffu, ph, bad < 0 ? 31 : bad - 1);
+        const int key = test(min(r, G - 1), ph);
+        if (coarse) {
+            key0 = __shfl_sync(0xffffffffu, key, 0);
+            if (key0 < 0 || !(__shfl_sync(0xffffffffu, ph, 0) <= kBlkPhiL)) return pb;
         }
-    }
-    for (int r0 = R1; r0 < G; r0 += 32) {
-        float ph;
-        const int r = min(r0 + lane, G - 1);
-        const int key = test(r, ph);
-        const bool ok = r0 + lane < G && key == key0 && ph <= kBlkPhiL;
-        const int bad = __ffs(~__ballot_sync(0xffffffffu, ok)) - 1;
+        const bool ok = r < G && key == key0 && ph <= kBlkPhiL;
+        const int bad = __ffs(~__ballot_sync(0xffffffffu, ok)) - 1;          // -1: none
         const int n = bad < 0 ? 32 : bad;
+        if (coarse) {
+            if ((key0 & 3) != 3 && g.s1 != g.s2) {
+                r0 = 0;
+                continue;
+            }
+            R1 = bad < 0 ? min(G, 31 * step + 1) : (bad - 1) * step + 1;
+        } else {
+            R1 += n;
+        }
         if (n > 0) ph_last = __shfl_sync(0xffffffffu, ph, n - 1);
-        R1 += n;
-        if (n < 32) break;
+        if (!coarse && n < 32) break;
+        r0 = R1;
     }
     cand = key0 >> 2;
     // rows from the block's top down to |phi| band = kBlkPhiLow
     int top = ph_last > kBlkPhiLow ? (int)ceilf(__fdividef(__logf(ph_last / kBlkPhiLow), g.ds)) : 0;
     top = min(top, R1);
+#pragma unroll 1
     for (int low = 1; low >= 0; --low) {
         const int n_rows = low ? R1 - top : top, parts = (n_rows + kGaussMaxN - 1) / kGaussMaxN;
+#pragma unroll 1
         for (int s = 0; s < parts; ++s) {
             const int a = n_rows * s / parts, b = n_rows * (s + 1) / parts, N = b - a;
             const float D = 0.5f * (float)N * g.ds;
@@ -470,6 +497,7 @@ __device__ __forceinline__ void unit_row(const WarpNodes<Cap> &ns, const float2 
     float wt = 1.0f;
     if (q < nv) {
         int b = 0;
+#pragma unroll 1
         while (b + 1 < nblk && ns.blk[b + 1].unit0 <= q) ++b;
         const RowBlock bl = ns.blk[b];
         if (bl.toff >= 0) {
@@ -506,10 +534,7 @@ __device__ __forceinline__ int node_emit(WarpNodes<Cap> &ns, const NodeRow &o, i
             ++k;
         });
     };
-    if (o.w != 0.0f) {
-        if (whole >= 0) take_run(whole, 0, G);
-        else row_runs(ns.geo, o, G, ca, cb, take_run);
-    }
+    if (o.w != 0.0f) row_runs(ns.geo, o, G, ca, cb, whole, take_run);
     more = k > first + kRowRuns;
     return slots | min(max(k - first, 0), kRowRuns) << 16;
 }
@@ -561,6 +586,7 @@ __device__ __forceinline__ void piece_nodes(WarpNodes<Cap> &ns, const PieceBlock
     const int nv = pb.units, R1 = pb.R1, nblk = pb.nblk, cand = pb.cand;
     const bool mine = cand >= ca && cand < cb;        // the blocks' candidate belongs to this sweep
     const int units = nv + (G - R1);
+#pragma unroll 1
     for (int u0 = mine ? 0 : nv; u0 < units; u0 += 32) {
         const int q = u0 + lane;
         const int whole = q < nv ? cand : -1;
@@ -582,15 +608,19 @@ __device__ __forceinline__ void piece_nodes(WarpNodes<Cap> &ns, const PieceBlock
                 if (lane >= d) incl += v;
             }
             const int total = __shfl_sync(0xffffffffu, incl, 31), base = incl - slots;
+#pragma unroll 1
             for (int k = 0; k < runs; ++k) {          // slots of the warp's rows; bit 21: a block's row
                 unsigned &id = ns.run[lane * kRowRuns + k].id;
                 id = id + (unsigned)base + (whole >= 0 ? 1u << 21 : 0u);
             }
+#pragma unroll 1
             for (int c0 = 0; c0 < total; c0 += Cap) {
                 if (base < c0 + Cap && incl > c0)
+#pragma unroll 1
                     for (int k = 0; k < runs; ++k) {
                         const unsigned id = ns.run[lane * kRowRuns + k].id;
                         const int s0 = (int)(id & 0xffffu) - c0, s1 = s0 + (int)(id >> 24);
+#pragma unroll 1
                         for (int s = max(s0, 0); s < min(s1, Cap); ++s)
                             ns.of[s] = (unsigned char)(lane * kRowRuns + k);
                     }
