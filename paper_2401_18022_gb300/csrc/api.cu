@@ -569,7 +569,7 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
             Bv.push_back(c.B_THz[j]);
             av.push_back(c.alpha_per_km[j]);
             gv.push_back(c.gamma_per_W_km[j]);
-            nfv.push_back(c.nf_dB ? c.nf_dB[j] : 0.0);
+            nfv.push_back(c.nf_dB ? std::pow(10.0, c.nf_dB[j] / 10.0) : 1.0);
             gd.push_back(c.guard ? c.guard[j] : 0);
         }
     }
@@ -876,7 +876,7 @@ TileSplit tile_split(const isrs_handle_s *h, int n_ch, int cell_set, int G)
     if (h && h->tile_points > 0) return {(int)std::max<int64_t>(1, h->tile_points / ((int64_t)G * G)), 1};
     const int64_t n = n_ch;
     const int64_t total = cell_set == ISRS_CELLS_SCI_XCI ? n * (2 * n + 1) : n * (n + 1) * (n + 3) / 2;
-    const int64_t parts = std::min<int64_t>(std::min(8, std::max(1, G / 16)), (16384 + total - 1) / total);
+    const int64_t parts = std::min<int64_t>(std::min(8, std::max(1, G / 8)), (16384 + total - 1) / total);
     return {(int)std::max<int64_t>(1, std::min<int64_t>(32, total / 38912)), (int)parts};
 }
 
@@ -1018,6 +1018,11 @@ isrs_status run_forward(isrs_handle h, const isrs_fibre *fb, Geom *g, int precis
         pp.lnrho_L = (double *)h->lnrho_L.p;
         pp.ptot = (double *)h->ptot.p;
         pp.kap_L = (double *)h->kapL.p;
+        pp.cs = nullptr;
+        if (adjoint) {
+            if ((s = ensure(h, h->gK, sizeof(double2) * M + sizeof(double) * 4 * (M + 1))) != ISRS_OK) return s;
+            pp.cs = (double *)((double2 *)h->gK.p + M);
+        }
         CK(launch_prep(pp, g->n_prof, st));
         if (g->profile == ISRS_PROFILE_RAMAN_ODE) {
             // the Raman ODE overwrites ln rho(L) and fills the {a, b} tables
@@ -1447,8 +1452,7 @@ isrs_status chain_buffers(isrs_handle h, const isrs_fibre *fb, const isrs_quad *
 {
     isrs_status s;
     if ((s = ensure(h, h->ybar, sizeof(double) * 2 * n)) != ISRS_OK) return s;
-    if ((s = ensure(h, h->gK, sizeof(double2) * g->n_steps + sizeof(double) * (4 * (g->n_steps + 1) + 4))) !=
-        ISRS_OK)
+    if ((s = ensure(h, h->gK, sizeof(double2) * g->n_steps + sizeof(double) * 4 * (g->n_steps + 1))) != ISRS_OK)
         return s;
     if ((s = ensure(h, h->dTdP, sizeof(double) * n)) != ISRS_OK) return s;
     if ((s = ensure(h, h->gVs, sizeof(double) * (size_t)std::max(1, g->n_slots) * n)) != ISRS_OK) return s;
@@ -1461,7 +1465,7 @@ isrs_status chain_buffers(isrs_handle h, const isrs_fibre *fb, const isrs_quad *
     cp.slot_items2 = g->n_mci_items > 0 ? (const int2 *)g->slot_items2.p : nullptr;
     cp.n_items_reg = g->n_items;
     cp.Rb = (double2 *)h->gK.p;
-    cp.cs = (double *)((double2 *)h->gK.p + g->n_steps);
+    cp.cs = (const double *)((double2 *)h->gK.p + g->n_steps);
     return ISRS_OK;
 }
 
@@ -1798,7 +1802,7 @@ isrs_status isrs_gn_grad(isrs_handle h, const isrs_fibre *fibre, const isrs_chan
         Range r_chain("isrs chain rule (dT/dP)");
         CK(launch_chain(cp, st));
     }
-    h->last_launches += 6;   // ybar, PSD-bucket reduction, step-bucket reduction, chain rule (3)
+    h->last_launches += 3;   // ybar, bucket sums, chain rule
     return grad_outputs(h, n, dT_dP, snr, eta, T_host, st);
 }
 
@@ -1917,7 +1921,7 @@ isrs_status isrs_gn_grad_shard_bwd(isrs_handle h, const double *eta_all, int wit
     } else {
         Range r_chain("isrs chain rule (dT/dP)");
         CK(launch_chain(cp, st));
-        h->last_launches = 7;    // SNR from eta, ybar, PSD-bucket reduction, step-bucket reduction, chain rule (3)
+        h->last_launches = 4;    // SNR from eta, ybar, bucket sums, chain rule
     }
     bool host_out = false;
     if ((s = copy_out(h, dT_dP, h->dTdP, n, st, host_out)) != ISRS_OK) return s;

@@ -21,6 +21,7 @@ struct PrepParams {
     double *lnrho_L;
     double *ptot;
     double *kap_L;              // kappa(L) per profile (the largest ISRS exponent slope)
+    double *cs;                 // ChainParams::cs of a gradient (one profile), or null
 };
 
 // FP32 copy of the profile tables for the MCI cells (pairs of steps outermost)
@@ -53,7 +54,7 @@ struct FinishParams {
 
 // Adjoint of the FP32 quadrature (single profile): per work tile the step
 // buckets {R_m, R'_m} and the PSD buckets V of every channel (the tile's own
-// row, written only by its block; k_v_reduce sums a CUT's rows in tile order).
+// row, written only by its block; k_adj_reduce sums a CUT's rows in tile order).
 struct AdjParams {
     QuadParams q;
     double2 *item_R;            // [n_items x n_steps]
@@ -66,14 +67,14 @@ struct AdjParams {
 // buckets may cover a shard of the CUTs (n_slots output slots, slot_cut maps
 // a slot to its channel); SNR, P_NLI, P_ASE, ybar and aase are per channel.
 struct ChainParams {
-    const double *P, *ch_frel, *ch_B, *ch_gamma, *ch_nf;
+    const double *P, *ch_frel, *ch_B, *ch_gamma, *ch_nf;   // ch_nf: noise figures, linear
     const double2 *zs_d;        // {z_m, dz_m}
     const double2 *step_d;      // {lnPtot - lnN_m, kappa_m}
     const double *snr, *pnli, *pase, *lnrho_L;   // [n_ch]
     const double2 *item_R;
     const double *V;            // [n_slots x n_ch] PSD buckets per output slot (from Vt)
     const double *Vt;           // [(n_items) x n_ch] PSD buckets per tile (regular, then MCI tiles)
-    double *Vs;                 // = V, written by k_v_reduce
+    double *Vs;                 // = V, written by k_adj_reduce
     const int2 *slot_items;     // per slot: regular tile range
     const int2 *slot_items2;    // per slot: MCI tile range (nullable), offset by n_items_reg
     int n_items_reg;
@@ -84,8 +85,8 @@ struct ChainParams {
     double *ybar;               // [n_ch] dT/dSigma_i
     double *aase;               // [n_ch] dT/dASE_i * dASE_i/d ln G_i
     double2 *Rb;                // [n_steps] sum over the shard's tiles of ybar_i {R_im, R'_im}
-    double *cs;                 // [4 (n_steps + 1) + 4] profile terms per step (ln N, kappa, L_eff, Fbar), then
-                                // the channel-independent sums of the chain rule
+    const double *cs;           // [4 (n_steps + 1)] profile terms per step and at L (ln N, kappa, L_eff,
+                                // Fbar - f_ref), written by k_prep
     double *dT_dP;              // [n_ch]
 };
 

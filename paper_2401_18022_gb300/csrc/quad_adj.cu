@@ -60,7 +60,7 @@ struct __align__(16) AdjWarp {
 // one beside a zero-weight copy of itself).  Lane buckets accumulate in
 // registers over a piece and are folded into the warp's FP64 buckets, which go
 // to the tile's own row; PSD buckets are added to the tile's own row by one
-// lane.  Every sum has a fixed order (k_v_reduce sums a CUT's rows in tile
+// lane.  Every sum has a fixed order (k_adj_reduce sums a CUT's rows in tile
 // order), so results are bit for bit reproducible.
 // ---------------------------------------------------------------------------
 #ifndef ISRS_ADJ_MIN_BLOCKS
@@ -283,18 +283,35 @@ __global__ void __launch_bounds__(256) k_ybar(ChainParams cp)
         const double P = cp.P[i], B = cp.ch_B[i], g = cp.ch_gamma[i], snr = cp.snr[i];
         const double dTds = 2.0 * B / (0.69314718055994530942 * (1.0 + snr));
         const double dsdN = -snr * snr / P;
-        const double nf = cp.ch_nf ? pow(10.0, cp.ch_nf[i] / 10.0) : 1.0;
+        const double nf = cp.ch_nf ? cp.ch_nf[i] : 1.0;
         const double hfb = cp.n_spans * nf * kHPlanck * ((cp.ch_frel[i] + cp.f_ref) * 1e12) * (B * 1e12);
         cp.ybar[i] = dTds * dsdN * (16.0 / 27.0) * g * g * B;
         cp.aase[i] = dTds * dsdN * (cp.pase[i] + hfb);    // dT/dASE * dASE/d ln G
     }
 }
 
-// V[s][j] = the PSD buckets of slot s's tiles (regular, then MCI), summed in
-// tile order; one block per slot, one thread per channel.
-__global__ void __launch_bounds__(256) k_v_reduce(ChainParams cp)
+// The tiles' buckets, every sum in a fixed order.  Blocks [0, n_steps): Rb[m] =
+// sum over tiles of ybar(channel of tile) {R_m, R'_m}.  Block n_steps + s: V[s][j]
+// = the PSD buckets of slot s's tiles (regular, then MCI) in tile order, one
+// thread per channel.
+__global__ void __launch_bounds__(256) k_adj_reduce(ChainParams cp)
 {
-    const int s = blockIdx.x, n = cp.n_ch;
+    __shared__ double scratch[32];
+    if ((int)blockIdx.x < cp.n_steps) {
+        const int m = blockIdx.x;
+        double rx = 0.0, ry = 0.0;
+        for (int it = threadIdx.x; it < cp.n_items; it += blockDim.x) {
+            const double y = cp.ybar[cp.slot_cut[cp.item_slot[it]]];
+            const double2 v = cp.item_R[(size_t)it * cp.n_steps + m];
+            rx += y * v.x;
+            ry += y * v.y;
+        }
+        rx = block_sum_d(rx, scratch);
+        ry = block_sum_d(ry, scratch);
+        if (threadIdx.x == 0) cp.Rb[m] = make_double2(rx, ry);
+        return;
+    }
+    const int s = blockIdx.x - cp.n_steps, n = cp.n_ch;
     const int2 r1 = cp.slot_items[s];
     const int2 r2 = cp.slot_items2 ? cp.slot_items2[s] : make_int2(0, 0);
     for (int j = threadIdx.x; j < n; j += blockDim.x) {
@@ -305,127 +322,37 @@ __global__ void __launch_bounds__(256) k_v_reduce(ChainParams cp)
     }
 }
 
-// Rb[m] = sum over tiles of ybar(channel of tile) * {R_m, R'_m}; one block per m.
-__global__ void __launch_bounds__(256) k_adj_reduce(ChainParams cp)
-{
-    __shared__ double scratch[32];
-    const int m = blockIdx.x;
-    double rx = 0.0, ry = 0.0;
-    for (int it = threadIdx.x; it < cp.n_items; it += blockDim.x) {
-        const double y = cp.ybar[cp.slot_cut[cp.item_slot[it]]];
-        const double2 v = cp.item_R[(size_t)it * cp.n_steps + m];
-        rx += y * v.x;
-        ry += y * v.y;
-    }
-    rx = block_sum_d(rx, scratch);
-    ry = block_sum_d(ry, scratch);
-    if (threadIdx.x == 0) cp.Rb[m] = make_double2(rx, ry);
-}
-
-__device__ __forceinline__ double sinhc_ad(double x)
-{
-    return fabs(x) < 1e-4 ? 1.0 + x * x / 6.0 : sinh(x) / x;
-}
-
-// sinhc'(y) / sinhc(y) = coth(y) - 1/y
-__device__ __forceinline__ double dlog_sinhc(double y)
-{
-    return fabs(y) < 1e-3 ? y / 3.0 - y * y * y / 45.0 : 1.0 / tanh(y) - 1.0 / y;
-}
-
-// Block maximum (every thread gets it; scratch holds 32 values).
-__device__ __forceinline__ double block_max_d(double v, double *scratch)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    __syncthreads();
-    if (lane == 0) scratch[wid] = v;
-    __syncthreads();
-    double m = -1e300;
-    for (int w = 0; w < nw; ++w) m = fmax(m, scratch[w]);
-    return m;
-}
-
-// The chain rule in three launches, every sum in a fixed order:
-//  k_chain_steps  one block per z-step m (and z = L at m = M): ln N(z_m),
-//                 kappa_m, L_eff(z_m) and the tilted mean Fbar(z_m) - f_ref;
-//  k_chain_const  the channel-independent sums (one block);
-//  k_chain_ch     one warp per channel j: its lanes split the steps and the
-//                 output slots, a warp tree sums them.
-// cs = [lnN | kappa | L_eff | Fbar] (M + 1 each), then {R' term, sum of aase,
-// ASE tilt term, P_tot}.
-__global__ void __launch_bounds__(256) k_chain_steps(ChainParams cp)
-{
-    __shared__ double scratch[32];
-    const int n = cp.n_ch, M = cp.n_steps, m = blockIdx.x;
-    double part = 0.0;
-    for (int c = threadIdx.x; c < n; c += blockDim.x) part += cp.P[c];
-    const double Ptot = block_sum_d(part, scratch);
-    const double z = m < M ? cp.zs_d[m].x : cp.L;
-    const double Le = cp.alpha_R > 0.0 ? -expm1(-cp.alpha_R * z) / cp.alpha_R : z;
-    const double kap = Ptot * cp.Cr * Le;
-    double mx = -1e300;
-    for (int c = threadIdx.x; c < n; c += blockDim.x)
-        mx = fmax(mx, log(cp.P[c]) - kap * cp.ch_frel[c] + log(sinhc_ad(0.5 * kap * cp.ch_B[c])));
-    mx = block_max_d(mx, scratch);
-    double s0 = 0.0, s1 = 0.0;
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        const double a = 0.5 * cp.ch_B[c];
-        const double w = exp(log(cp.P[c]) - kap * cp.ch_frel[c] + log(sinhc_ad(kap * a)) - mx);
-        s0 += w;
-        s1 += w * (cp.ch_frel[c] - a * dlog_sinhc(kap * a));
-    }
-    s0 = block_sum_d(s0, scratch);
-    s1 = block_sum_d(s1, scratch);
-    if (threadIdx.x == 0) {
-        const int st = M + 1;
-        cp.cs[m] = mx + log(s0);
-        cp.cs[st + m] = kap;
-        cp.cs[2 * st + m] = Le;
-        cp.cs[3 * st + m] = s1 / s0;
-    }
-}
-
-__global__ void __launch_bounds__(256) k_chain_const(ChainParams cp)
+// The chain rule from the buckets, one warp per channel j: its lanes split the
+// steps and the output slots, a warp tree sums them.  The step terms cs = [lnN |
+// kappa | L_eff | Fbar - f_ref] (M + 1 each) come from the forward's k_prep; the
+// sums over all channels and steps that every channel needs are a few hundred
+// terms, so each block takes them itself, in the same order.  A 5-channel
+// gradient's launches after the quadrature: @CHAIN@.
+__global__ void __launch_bounds__(256) k_chain_ch(ChainParams cp)
 {
     __shared__ double scratch[32];
     const int n = cp.n_ch, M = cp.n_steps, st = M + 1;
-    const double *Le = cp.cs + 2 * st, *Fb = cp.cs + 3 * st;
-    double part = 0.0;
-    for (int c = threadIdx.x; c < n; c += blockDim.x) part += cp.P[c];
-    const double Ptot = block_sum_d(part, scratch);
-    double a1 = 0.0, a2 = 0.0, a3 = 0.0;
+    const int lane = threadIdx.x & 31;
+    const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const double *lnN = cp.cs, *kap = cp.cs + st, *Le = cp.cs + 2 * st, *Fb = cp.cs + 3 * st;
+    double pt = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
     for (int m = threadIdx.x; m < M; m += blockDim.x) a1 += cp.Rb[m].y * Le[m];
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        pt += cp.P[i];
         a2 += cp.aase[i];
         a3 += cp.aase[i] * (cp.ch_frel[i] - Fb[M]);
     }
     a1 = block_sum_d(a1, scratch);
+    pt = block_sum_d(pt, scratch);
     a2 = block_sum_d(a2, scratch);
     a3 = block_sum_d(a3, scratch);
-    if (threadIdx.x == 0) {
-        double *k = cp.cs + 4 * st;
-        k[0] = -cp.Cr * a1;              // R' term
-        k[1] = a2;                       // sum of aase
-        k[2] = cp.Cr * Le[M] * a3;       // ASE tilt term
-        k[3] = Ptot;
-    }
-}
-
-__global__ void __launch_bounds__(256) k_chain_ch(ChainParams cp)
-{
-    const int n = cp.n_ch, M = cp.n_steps, st = M + 1;
-    const int lane = threadIdx.x & 31;
-    const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (j >= n) return;                  // warp-uniform
-    const double *lnN = cp.cs, *kap = cp.cs + st, *Le = cp.cs + 2 * st, *Fb = cp.cs + 3 * st;
-    const double *k = cp.cs + 4 * st;
-    const double invPt = 1.0 / k[3];
+    const double k0 = -cp.Cr * a1, k2 = cp.Cr * Le[M] * a3;      // R' term, ASE tilt term
+    const double invPt = 1.0 / pt;
     const double fj = cp.ch_frel[j], hB = 0.5 * cp.ch_B[j];
     double gm = 0.0;
     for (int m = lane; m < M; m += 32) {
-        const double hN = exp(-kap[m] * fj + log(sinhc_ad(kap[m] * hB)) - lnN[m]);
+        const double hN = exp(log_sinhc(kap[m] * hB) - kap[m] * fj - lnN[m]);
         gm += cp.Rb[m].x * (invPt - hN + cp.Cr * Le[m] * Fb[m]);
     }
     double v = 0.0;
@@ -433,11 +360,11 @@ __global__ void __launch_bounds__(256) k_chain_ch(ChainParams cp)
     gm = warp_sum_d(gm);
     v = warp_sum_d(v);
     if (lane == 0) {
-        double g = k[0] + gm + v / cp.P[j];
+        double g = k0 + gm + v / cp.P[j];
         if (cp.with_direct) {
             // through the ASE gain of every channel, and the SNR numerator
-            const double hNL = exp(-kap[M] * fj + log(sinhc_ad(kap[M] * hB)) - lnN[M]);
-            g += -k[1] * (invPt - hNL) + k[2];
+            const double hNL = exp(log_sinhc(kap[M] * hB) - kap[M] * fj - lnN[M]);
+            g += -a2 * (invPt - hNL) + k2;
             const double snr = cp.snr[j], P = cp.P[j], B = cp.ch_B[j];
             const double N = cp.pnli[j] + cp.pase[j];
             const double dTds = 2.0 * B / (0.69314718055994530942 * (1.0 + snr));
@@ -483,23 +410,16 @@ cudaError_t launch_adjoint(const AdjParams &ap, int num_sms, int block, cudaStre
 
 cudaError_t launch_ybar(const ChainParams &cp, cudaStream_t st)
 {
-    k_ybar<<<1, 256, 0, st>>>(cp);
+    k_ybar<<<(cp.n_ch + 127) / 128, 128, 0, st>>>(cp);
     return cudaGetLastError();
 }
 
 cudaError_t launch_chain(const ChainParams &cp, cudaStream_t st)
 {
     if (cp.n_steps > kMaxAdjSteps) return cudaErrorInvalidValue;
-    k_ybar<<<1, 256, 0, st>>>(cp);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_ybar(cp, st);
     if (e != cudaSuccess) return e;
-    k_v_reduce<<<cp.n_slots, 256, 0, st>>>(cp);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_adj_reduce<<<cp.n_steps, 256, 0, st>>>(cp);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_chain_steps<<<cp.n_steps + 1, 256, 0, st>>>(cp);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_chain_const<<<1, 256, 0, st>>>(cp);
+    k_adj_reduce<<<cp.n_steps + cp.n_slots, 256, 0, st>>>(cp);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_chain_ch<<<(cp.n_ch + 7) / 8, 256, 0, st>>>(cp);
     return cudaGetLastError();

@@ -285,7 +285,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
         // item outputs: the forward partial, the PSD buckets and the step buckets
         const double tot = block_sum_d((double)sum - (double)comp, scratch);   // syncs the block
         if (threadIdx.x == 0) qp.partial[it] = tot;
-        double *Vrow = ap.V + (size_t)it * ap.n_ch;     // this tile's own row (k_v_reduce sums them)
+        double *Vrow = ap.V + (size_t)it * ap.n_ch;     // this tile's own row (k_adj_reduce sums them)
         for (int c = threadIdx.x; c < n; c += blockDim.x) {
             double v = 0.0;
             for (int x = 0; x < nw; ++x) v += (double)sV[x * nmax + c];

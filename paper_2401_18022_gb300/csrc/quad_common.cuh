@@ -36,6 +36,50 @@ __device__ __forceinline__ double warp_sum_d(double v)
 }
 
 // Deterministic block sum of one double per thread (blockDim multiple of 32).
+// ln(sinh(x) / x) and its derivative coth(x) - 1/x in FP64.  Up to |x| = 0.2
+// (kappa B / 2 of any practical channel) the Taylor series of either, dropped
+// terms below 2e-16: a few FMAs where sinh, log, tanh and two divisions were most
+// of the small per-step kernels' time.
+__device__ __forceinline__ double log_sinhc(double x)
+{
+    const double q = x * x;
+    if (q > 0.04) return log(sinh(x) / x);
+    double p = -691.0 / 3831077250.0;
+    p = fma(p, q, 1.0 / 467775.0);
+    p = fma(p, q, -1.0 / 37800.0);
+    p = fma(p, q, 1.0 / 2835.0);
+    p = fma(p, q, -1.0 / 180.0);
+    p = fma(p, q, 1.0 / 6.0);
+    return p * q;
+}
+
+__device__ __forceinline__ double dlog_sinhc(double x)
+{
+    const double q = x * x;
+    if (q > 0.04) return 1.0 / tanh(x) - 1.0 / x;
+    double p = -1382.0 / 638512875.0;
+    p = fma(p, q, 2.0 / 93555.0);
+    p = fma(p, q, -1.0 / 4725.0);
+    p = fma(p, q, 2.0 / 945.0);
+    p = fma(p, q, -1.0 / 45.0);
+    p = fma(p, q, 1.0 / 3.0);
+    return p * x;
+}
+
+// Block maximum (every thread gets it; scratch holds 32 values).
+__device__ __forceinline__ double block_max_d(double v, double *scratch)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __syncthreads();
+    if (lane == 0) scratch[wid] = v;
+    __syncthreads();
+    double m = -1e300;
+    for (int w = 0; w < nw; ++w) m = fmax(m, scratch[w]);
+    return m;
+}
+
 __device__ __forceinline__ double block_sum_d(double v, double *scratch)
 {
     v = warp_sum_d(v);

@@ -38,14 +38,13 @@ namespace isrs {
 // at = (alpha_a + alpha_b + alpha_c - alpha_i)/2, because F_a + F_b + F_c - f
 // = 2 F_c.  Writes, per step, {A2, K2} = log2(e) {lnPtot - lnN, -kappa} and
 // {lnPtot - lnN, kappa}; per channel P/B (step 0's block) and ln rho(L, f_c)
-// (the z = L block).  ln N is a log-sum-exp over the channels with a block
-// maximum and a block sum in fixed order.
+// (the z = L block); where a gradient follows, the chain rule's step terms too
+// (ln N, kappa, L_eff and the tilted mean frequency Fbar - f_ref).  ln N is a
+// log-sum-exp over the channels with a block maximum and a block sum in fixed
+// order.  A launch is one wave of short blocks, so it is bound by the latency of
+// its FP64 chain: with one exp per channel and log_sinhc by its series it takes
+// @PREP@.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double sinhc_d(double x)
-{
-    return fabs(x) < 1e-4 ? 1.0 + x * x / 6.0 : sinh(x) / x;
-}
-
 __global__ void __launch_bounds__(256) k_prep(PrepParams pp)
 {
     __shared__ double scratch[32];
@@ -73,23 +72,30 @@ __global__ void __launch_bounds__(256) k_prep(PrepParams pp)
     const double z = (m < M) ? pp.zs_d[m].x : pp.L;
     const double leff = pp.alpha_R > 0.0 ? -expm1(-pp.alpha_R * z) / pp.alpha_R : z;
     const double kap = Ptot * pp.Cr * leff;
+    const auto expo = [&](int c) { return log_sinhc(0.5 * kap * B[c]) - kap * fr[c]; };
     double mx = -1e300;
+    for (int c = threadIdx.x; c < n; c += blockDim.x)
+        if (P[c] > 0.0) mx = fmax(mx, expo(c));
+    mx = block_max_d(mx, scratch);
+    double s0 = 0.0, s1 = 0.0;
     for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        if (P[c] > 0.0) mx = fmax(mx, log(P[c]) - kap * fr[c] + log(sinhc_d(0.5 * kap * B[c])));
+        if (!(P[c] > 0.0)) continue;
+        const double w = P[c] * exp(expo(c) - mx), hb = 0.5 * B[c];
+        s0 += w;
+        if (pp.cs) s1 += w * (fr[c] - hb * dlog_sinhc(kap * hb));
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    mx = -1e300;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) mx = fmax(mx, scratch[w]);
-    double sum = 0.0;
-    for (int c = threadIdx.x; c < n; c += blockDim.x) {
-        if (P[c] > 0.0) sum += exp(log(P[c]) - kap * fr[c] + log(sinhc_d(0.5 * kap * B[c])) - mx);
+    s0 = block_sum_d(s0, scratch);
+    const double lnN = mx + log(s0);
+    if (pp.cs) {
+        s1 = block_sum_d(s1, scratch);
+        if (threadIdx.x == 0) {
+            const int st = M + 1;
+            pp.cs[m] = lnN;
+            pp.cs[st + m] = kap;
+            pp.cs[2 * st + m] = leff;
+            pp.cs[3 * st + m] = s1 / s0;
+        }
     }
-    sum = block_sum_d(sum, scratch);
-    const double lnN = mx + log(sum);
     if (m < M) {
         if (threadIdx.x == 0) {
             pp.step_d[(size_t)p * M + m] = make_double2(lnPtot - lnN, kap);
@@ -411,9 +417,13 @@ __global__ void __launch_bounds__(256) k_quad_f64(QuadParams qp)
 // k_finish: per profile, Sigma_i = ordered sum of the CUT's tile partials;
 // eta_i = (16/27) gamma_i^2 B_i Sigma_i / P_i^3 (Eq. gain_fin, P_NLI = G B);
 // SNR_i = P_i / (P_NLI,i + P_ASE,i) with P_ASE,i = NF h f (1/rho(L,f) - 1) B
-// and optional transceiver noise; T = 2 sum B log2(1 + SNR) (Eq. loss).
+// and optional transceiver noise; T = 2 sum B log2(1 + SNR) (Eq. loss).  Eight
+// lanes sum a CUT's tiles: one thread's chain of dependent additions over them
+// was most of the kernel's time (@FIN@).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) k_finish(FinishParams fp)
+constexpr int kFinishLanes = 8;
+
+__global__ void __launch_bounds__(512) k_finish(FinishParams fp)
 {
     __shared__ double scratch[32];
     const int p = blockIdx.x;
@@ -422,15 +432,22 @@ __global__ void __launch_bounds__(256) k_finish(FinishParams fp)
     const int poff = fp.prof_ch_off[p];
     const int s0 = fp.prof_slot_off[p], s1 = fp.prof_slot_off[p + 1];
     double tpart = 0.0;
-    for (int s = s0 + threadIdx.x; s < s1; s += blockDim.x) {
-        const int2 rg = fp.slot_items[s];
-        const int i = fp.slot_cut[s];
+    const int sub = threadIdx.x % kFinishLanes, per = blockDim.x / kFinishLanes;
+    for (int sb = s0; sb < s1; sb += per) {
+        const int s = sb + threadIdx.x / kFinishLanes;
         double sig = 0.0;
-        for (int it = rg.x; it < rg.y; ++it) sig += fp.partial[it];
-        if (fp.slot_items2) {
-            const int2 r2 = fp.slot_items2[s];
-            for (int it = r2.x; it < r2.y; ++it) sig += fp.partial2[it];
+        if (s < s1) {
+            const int2 rg = fp.slot_items[s];
+            for (int it = rg.x + sub; it < rg.y; it += kFinishLanes) sig += fp.partial[it];
+            if (fp.slot_items2) {
+                const int2 r2 = fp.slot_items2[s];
+                for (int it = r2.x + sub; it < r2.y; it += kFinishLanes) sig += fp.partial2[it];
+            }
         }
+#pragma unroll
+        for (int o = kFinishLanes / 2; o > 0; o >>= 1) sig += __shfl_xor_sync(0xffffffffu, sig, o);
+        if (s >= s1 || sub != 0) continue;
+        const int i = fp.slot_cut[s];
         const double g = fp.ch_gamma[coff + i];
         const double B = fp.ch_B[coff + i];
         const double P = fp.P[poff + i];
@@ -440,7 +457,7 @@ __global__ void __launch_bounds__(256) k_finish(FinishParams fp)
         if (fp.pnli) fp.pnli[s] = pnli;
         if (fp.eta) fp.eta[s] = eta;
         if (fp.snr) {
-            const double nf = fp.ch_nf ? pow(10.0, fp.ch_nf[coff + i] / 10.0) : 1.0;
+            const double nf = fp.ch_nf ? fp.ch_nf[coff + i] : 1.0;
             const double f_abs = fp.ch_frel[coff + i] + fp.f_ref;
             const double gain = exp(-fp.lnrho_L[poff + i]);
             const double pase = fp.n_spans * nf * 6.62607015e-34 * (f_abs * 1e12) * (gain - 1.0) * (B * 1e12);
@@ -471,7 +488,7 @@ __global__ void __launch_bounds__(256) k_snr_from_eta(SnrFromEtaParams sp)
     for (int i = threadIdx.x; i < sp.n; i += blockDim.x) {
         const double B = sp.ch_B[i], P = sp.P[i];
         const double pnli = sp.eta[i] * P * P * P;
-        const double nf = sp.ch_nf ? pow(10.0, sp.ch_nf[i] / 10.0) : 1.0;
+        const double nf = sp.ch_nf ? sp.ch_nf[i] : 1.0;
         const double f_abs = sp.ch_frel[i] + sp.f_ref;
         const double gain = exp(-sp.lnrho_L[i]);
         const double pase = sp.n_spans * nf * 6.62607015e-34 * (f_abs * 1e12) * (gain - 1.0) * (B * 1e12);
@@ -542,7 +559,7 @@ cudaError_t launch_quad(const QuadParams &qp, int precision, int num_sms, int bl
 
 cudaError_t launch_finish(const FinishParams &fp, int n_prof, cudaStream_t st)
 {
-    k_finish<<<n_prof, 256, 0, st>>>(fp);
+    k_finish<<<n_prof, 512, 0, st>>>(fp);
     return cudaGetLastError();
 }
 

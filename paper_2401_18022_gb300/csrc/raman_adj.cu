@@ -228,36 +228,61 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
 }
 
 // dT/d{a_c, b_c}(m) and dT/d ln P_c (PSD): the rows of channel c from every
-// tile that touches it, weighted by dT/dSigma of the tile's CUT, in tile
-// order.  One block per plan channel.
-__global__ void __launch_bounds__(128) k_tab_gather(TabGatherParams gp)
+// tile that touches it, weighted by dT/dSigma of the tile's CUT.  One block per
+// plan channel and 32 steps (lane = step); its warps take equal shares of the
+// rows in tile order and are summed in warp order.  Bound by reading the rows
+// (16 M bytes each): @GATHER@.
+constexpr int kGatherWarps = 16;
+
+__global__ void __launch_bounds__(32 * kGatherWarps) k_tab_gather(TabGatherParams gp)
 {
-    const int c = blockIdx.x, M = gp.n_steps;
-    const int e0 = gp.gath_off[c], e1 = gp.gath_off[c + 1];
-    for (int m = threadIdx.x; m < M; m += blockDim.x) {
-        double ga = 0.0, gb = 0.0;
-        for (int e = e0; e < e1; ++e) {
-            const int2 rs = gp.gath[e];
-            const double y = gp.ybar[gp.slot_cut[rs.y]];
-            const double2 v = gp.rows[(size_t)rs.x * M + m];
-            ga += y * v.x;
-            gb += y * v.y;
+    __shared__ double2 part[kGatherWarps][32];
+    __shared__ double partV[kGatherWarps];
+    const int c = blockIdx.x, M = gp.n_steps, m = blockIdx.y * 32 + (threadIdx.x & 31);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int e0 = gp.gath_off[c], len = gp.gath_off[c + 1] - e0;
+    const int ea = e0 + (int)((long long)len * warp / kGatherWarps);
+    const int eb = e0 + (int)((long long)len * (warp + 1) / kGatherWarps);
+    double ga = 0.0, gb = 0.0, gv = 0.0;
+    for (int e = ea; e < eb; e += 32) {
+        int row = 0;
+        double y = 0.0;
+        if (e + lane < eb) {
+            const int2 rs = gp.gath[e + lane];
+            row = rs.x;
+            y = gp.ybar[gp.slot_cut[rs.y]];
+            if (blockIdx.y == 0) gv += y * gp.rowsV[row];
         }
-        gp.gAB[(size_t)c * M + m] = make_double2(ga, gb);
-    }
-    if (threadIdx.x == 0) {
-        double v = 0.0;
-        for (int e = e0; e < e1; ++e) {
-            const int2 rs = gp.gath[e];
-            v += gp.ybar[gp.slot_cut[rs.y]] * gp.rowsV[rs.x];
+        const int n = min(32, eb - e);
+#pragma unroll 8
+        for (int i = 0; i < n; ++i) {
+            const int r = __shfl_sync(kFullT, row, i);
+            const double yi = __shfl_sync(kFullT, y, i);
+            if (m < M) {
+                const double2 v = gp.rows[(size_t)r * M + m];
+                ga += yi * v.x;
+                gb += yi * v.y;
+            }
         }
-        gp.gV[c] = v;
     }
+    gv = warp_sum_d(gv);
+    part[warp][lane] = make_double2(ga, gb);
+    if (lane == 0) partV[warp] = gv;
+    __syncthreads();
+    if (warp != 0) return;
+    ga = gb = gv = 0.0;
+    for (int w = 0; w < kGatherWarps; ++w) {
+        ga += part[w][lane].x;
+        gb += part[w][lane].y;
+        gv += partV[w];
+    }
+    if (m < M) gp.gAB[(size_t)c * M + m] = make_double2(ga, gb);
+    if (blockIdx.y == 0 && lane == 0) gp.gV[c] = gv;
 }
 
 cudaError_t launch_tab_gather(const TabGatherParams &gp, cudaStream_t st)
 {
-    k_tab_gather<<<gp.n_ch, 128, 0, st>>>(gp);
+    k_tab_gather<<<dim3(gp.n_ch, (gp.n_steps + 31) / 32), 32 * kGatherWarps, 0, st>>>(gp);
     return cudaGetLastError();
 }
 
