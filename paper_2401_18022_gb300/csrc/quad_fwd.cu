@@ -42,8 +42,8 @@ namespace isrs {
 // (ln N, kappa, L_eff and the tilted mean frequency Fbar - f_ref).  ln N is a
 // log-sum-exp over the channels with a block maximum and a block sum in fixed
 // order.  A launch is one wave of short blocks, so it is bound by the latency of
-// its FP64 chain: with one exp per channel and log_sinhc by its series it takes
-// @PREP@.
+// its FP64 chain: one exp per channel, log_sinhc by its series (two logs, two
+// sinhs and a log more took 20 us at 5 channels).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_prep(PrepParams pp)
 {
@@ -419,7 +419,8 @@ __global__ void __launch_bounds__(256) k_quad_f64(QuadParams qp)
 // SNR_i = P_i / (P_NLI,i + P_ASE,i) with P_ASE,i = NF h f (1/rho(L,f) - 1) B
 // and optional transceiver noise; T = 2 sum B log2(1 + SNR) (Eq. loss).  Eight
 // lanes sum a CUT's tiles: one thread's chain of dependent additions over them
-// was most of the kernel's time (@FIN@).
+// was most of the kernel's time (15 us at 5
+// channels, 64 us at 589).
 // ---------------------------------------------------------------------------
 constexpr int kFinishLanes = 8;
 

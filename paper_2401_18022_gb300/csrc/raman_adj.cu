@@ -231,7 +231,8 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
 // tile that touches it, weighted by dT/dSigma of the tile's CUT.  One block per
 // plan channel and 32 steps (lane = step); its warps take equal shares of the
 // rows in tile order and are summed in warp order.  Bound by reading the rows
-// (16 M bytes each): @GATHER@.
+// (16 M bytes each); one block per channel in one
+// chain over its rows left a 41-channel plan on 41 SMs (1.95 ms).
 constexpr int kGatherWarps = 16;
 
 __global__ void __launch_bounds__(32 * kGatherWarps) k_tab_gather(TabGatherParams gp)
