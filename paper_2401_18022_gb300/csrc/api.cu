@@ -812,7 +812,7 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
         UP(tab_gath, gath);
     }
 #undef UP
-    CK(launch_piece_logs((DevPiece *)g->pieces.p, (int)g->n_pieces, st));
+    CK(launch_piece_logs((DevPiece *)g->pieces.p, (int)g->n_pieces, q->G, -std::log(q->eps_v1), st));
     CK(cudaStreamSynchronize(st));   // host vectors die at return
 
     h->cache.insert(h->cache.begin(), std::move(g));
@@ -929,6 +929,8 @@ QuadParams quad_params(isrs_handle h, const isrs_fibre *fb, Geom *g)
     qp.beta2 = fb->beta2;
     qp.beta3 = fb->beta3;
     qp.beta4 = fb->beta4;
+    qp.c3 = kPi * qp.beta3;
+    qp.c4 = 2.0 * kPi * kPi / 3.0 * qp.beta4;
     qp.ch_frel = (const double *)g->ch_frel.p;
     qp.ch_B = (const double *)g->ch_B.p;
     qp.ch_alpha = (const double *)g->ch_alpha.p;
@@ -2151,7 +2153,9 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     pp.lnrho_L = (double *)(base + o_lnL);
     pp.ptot = (double *)(base + o_ptot);
     pp.kap_L = (double *)(base + o_kapL);
-    if (launch_piece_logs((DevPiece *)(base + o_pieces), (int)pieces.size(), st) != cudaSuccess) return ISRS_ERR_CUDA;
+    if (launch_piece_logs((DevPiece *)(base + o_pieces), (int)pieces.size(), quad->G, -std::log(quad->eps_v1), st) !=
+        cudaSuccess)
+        return ISRS_ERR_CUDA;
     if (launch_prep(pp, 1, st) != cudaSuccess) return ISRS_ERR_CUDA;
 
     QuadParams qp;
@@ -2167,6 +2171,8 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     qp.beta2 = fibre->beta2;
     qp.beta3 = fibre->beta3;
     qp.beta4 = fibre->beta4;
+    qp.c3 = kPi * qp.beta3;
+    qp.c4 = 2.0 * kPi * kPi / 3.0 * qp.beta4;
     qp.ch_frel = pp.ch_frel;
     qp.ch_B = pp.ch_B;
     qp.ch_alpha = pp.ch_alpha;

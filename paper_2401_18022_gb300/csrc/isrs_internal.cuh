@@ -31,7 +31,8 @@ constexpr double kLog2e = 1.44269504088896340736;
 // piece (f1 <-> f2) is folded in.  Channel indices are plan-local.
 struct DevPiece {
     double xlo, xhi, ylo, yhi;
-    double lnx, lny;              // ln(xhi / xlo), ln(yhi / ylo), 1e30 for a zero limit (k_piece_logs)
+    float lnx, lny;               // ln(xhi / xlo), ln(yhi / ylo), 1e30 for a zero limit (k_piece_logs)
+    float2 ds2;                   // row pitch in log2 upsilon1, float-float (k_piece_logs)
     int cut, a, b, c_lo;
     int c_hi, flags, plan;        // flags bit0: s1 < 0, bit1: s2 < 0
     float mult;
@@ -62,6 +63,7 @@ struct QuadParams {
     double ln_eps;              // -ln(eps_v1)
     // fibre
     double beta2, beta3, beta4;
+    double c3, c4;              // pi beta3, 2 pi^2 / 3 beta4
     // per plan channel tables (concatenated, index plan_ch_off[plan] + c)
     const double *ch_frel;      // f_c - f_ref
     const double *ch_B;

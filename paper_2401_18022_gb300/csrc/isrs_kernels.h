@@ -172,8 +172,8 @@ cudaError_t launch_raman(const RamanParams &rp, int n_prof, int max_n, cudaStrea
 // Gauss rules of the row sums: the module's array on the current device, and its fill
 cudaError_t gauss_array(void **out);
 cudaError_t launch_gauss(float2 *out, cudaStream_t st);
-// fills DevPiece::lnx, lny
-cudaError_t launch_piece_logs(DevPiece *pieces, int n, cudaStream_t st);
+// fills DevPiece::lnx, lny, ds2
+cudaError_t launch_piece_logs(DevPiece *pieces, int n, int G, double ln_eps, cudaStream_t st);
 cudaError_t launch_prep(const PrepParams &pp, int n_prof, cudaStream_t st);
 cudaError_t launch_quad(const QuadParams &qp, int precision, int num_sms, int block, cudaStream_t st);
 // the same quadratures with the tabulated profile (qp.ab set)

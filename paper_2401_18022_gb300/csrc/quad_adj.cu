@@ -112,7 +112,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
 #pragma unroll
             for (int k = 0; k < K2; ++k) R[k] = Rp[k] = dup2(0.0f);
             double ptot = 0.0;
-            const PieceBlocks pb = row_blocks(ns, G);
+            const PieceBlocks pb = row_blocks(ns, qp.gauss, G);
             n_small += lane == 0 && part == 0 ? pb.R1 * G : 0;
             for (int ca = 0; ca < g.nc; ca += kAdjCand) {
                 const int cb = min(g.nc, ca + kAdjCand);

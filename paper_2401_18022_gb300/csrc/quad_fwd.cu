@@ -124,7 +124,13 @@ __global__ void __launch_bounds__(256) k_prep(PrepParams pp)
 __global__ void __launch_bounds__(128) k_gauss(float2 *out)
 {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= kGaussEntries) return;
+    if (e >= kGaussEntries) {
+        const int j = e - kGaussEntries;
+        if (j >= kExp2Entries) return;
+        const double v = exp2(-(double)j / kExp2Entries);
+        out[e] = make_float2((float)v, (float)(v - (double)(float)v));
+        return;
+    }
     const int N = e / kGaussPerN + 1, o = e - (N - 1) * kGaussPerN;
     int m = 0;
     while (m + 1 < kGaussMenu && gauss_offset(m + 1) <= o) ++m;
@@ -174,26 +180,31 @@ __global__ void __launch_bounds__(128) k_gauss(float2 *out)
 
 cudaError_t launch_gauss(float2 *out, cudaStream_t st)
 {
-    k_gauss<<<(kGaussEntries + 127) / 128, 128, 0, st>>>(out);
+    k_gauss<<<(kGaussEntries + kExp2Entries + 127) / 128, 128, 0, st>>>(out);
     return cudaGetLastError();
 }
 
-__device__ float2 g_isrs_gauss[kGaussEntries];
+__device__ float2 g_isrs_gauss[kGaussEntries + kExp2Entries];
 
-// ln(xhi / xlo) and ln(yhi / ylo) of every piece, once per plan (the quadrature
-// would otherwise take two FP64 logarithms per piece and launch).
-__global__ void __launch_bounds__(256) k_piece_logs(DevPiece *pieces, int n)
+// ln(xhi / xlo), ln(yhi / ylo) and the row pitch of every piece, once per plan (the
+// quadrature would otherwise take two FP64 logarithms and a division per piece and
+// launch).
+__global__ void __launch_bounds__(256) k_piece_logs(DevPiece *pieces, int n, int G, double ln_eps)
 {
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         DevPiece &p = pieces[k];
-        p.lnx = p.xlo > 0.0 ? log(p.xhi / p.xlo) : 1e30;
-        p.lny = p.ylo > 0.0 ? log(p.yhi / p.ylo) : 1e30;
+        const double lx = p.xlo > 0.0 ? log(p.xhi / p.xlo) : 1e30, ly = p.ylo > 0.0 ? log(p.yhi / p.ylo) : 1e30;
+        // upsilon1 runs from max(xlo ylo, eps xhi yhi) to xhi yhi
+        const double ds2 = fmin(lx + ly, ln_eps) / G * kLog2e;
+        p.lnx = (float)lx;
+        p.lny = (float)ly;
+        p.ds2 = make_float2((float)ds2, (float)(ds2 - (double)(float)ds2));
     }
 }
 
-cudaError_t launch_piece_logs(DevPiece *pieces, int n, cudaStream_t st)
+cudaError_t launch_piece_logs(DevPiece *pieces, int n, int G, double ln_eps, cudaStream_t st)
 {
-    if (n > 0) k_piece_logs<<<std::min(2048, (n + 255) / 256), 256, 0, st>>>(pieces, n);
+    if (n > 0) k_piece_logs<<<std::min(2048, (n + 255) / 256), 256, 0, st>>>(pieces, n, G, ln_eps);
     return cudaGetLastError();
 }
 
@@ -253,7 +264,7 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
             __syncwarp();
             const PieceGeo &g = ns.geo;
             float sum = 0.0f, comp = 0.0f;
-            const PieceBlocks pb = row_blocks(ns, G);
+            const PieceBlocks pb = row_blocks(ns, qp.gauss, G);
             n_small += lane == 0 && part == 0 ? pb.R1 * G : 0;
 #pragma unroll 1
             for (int ca = 0; ca < g.nc; ca += kFwdCand) {

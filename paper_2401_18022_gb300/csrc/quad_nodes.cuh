@@ -27,7 +27,12 @@
 // Coordinates are carried relative to a corner of the piece, U = s1 xhi +
 // s2 yhi, so that an FP32 point is located to ~1e-8 THz also where F_c - f_i
 // is tens of THz, and phi is split per row into its value at the row's centre
-// (FP64, kept as a float-float pair) and an increment quadratic in u.
+// (a float-float pair) and an increment quadratic in u.
+//
+// FP64 is used once per piece (node_geo, one warp instruction for several values
+// where that goes): an SM takes 16 clocks for an FP64 warp instruction, and with
+// ~30 of them per row and row test the set-up was bound by that pipe (half of a
+// 589-channel call at G = 64).
 //
 // One warp works on one piece: lane = row while rows are set up and their runs
 // listed, lane = node (or half-warp = node) afterwards.  Blocks working on one
@@ -49,6 +54,8 @@ constexpr int kGaussMenu = 18;
 constexpr int kGaussPerN = 297;                        // nodes of all rules of one N
 constexpr int kGaussEntries = kGaussMaxN * kGaussPerN;
 constexpr int kRowRuns = 4;                            // runs of a row listed at a time
+// behind the rules: 2^(-j / kExp2Entries) as float-float pairs (node_row)
+constexpr int kExp2Entries = 256;
 
 __host__ __device__ constexpr int gauss_nodes(int k)
 {
@@ -87,9 +94,10 @@ constexpr float kBlkPhiLow = 0.15f;      // ... and up to which they join the lo
 // One piece's geometry, |f1| the longer axis (f1 and f2 enter symmetrically,
 // so swapping them only reverses the columns).
 struct PieceGeo {
-    double u1hi;                // xhi yhi
-    double br0;                 // bracket of Eq. phi: br0 + br1 u + c4 u^2 - c4/2 f1 f2, u from the corner
-    double ds2;                 // row pitch in log2 upsilon1
+    float2 vC;                  // -4 pi^2 f1 f2 at the corner, float-float
+    float2 br0;                 // bracket of Eq. phi: br0 + br1 u + c4 u^2 - c4/2 f1 f2, u from the corner
+    float2 ds2;                 // row pitch in log2 upsilon1
+    float u1hi;                 // xhi yhi
     float br1, c4;
     float ds;                   // row pitch in ln upsilon1
     float xhi, yhi;             // corner of the piece
@@ -142,77 +150,77 @@ __device__ __forceinline__ bool node_geo(const QuadParams &qp, const DevPiece &p
     const int lane = threadIdx.x & 31;
     const bool sw = pc.yhi > pc.xhi;
     const double xhi = sw ? pc.yhi : pc.xhi, yhi = sw ? pc.xhi : pc.yhi;
-    const double R = sw ? pc.lny : pc.lnx, Rb = sw ? pc.lnx : pc.lny;
     const bool n1 = pc.flags & (sw ? 2 : 1), n2 = pc.flags & (sw ? 1 : 2);
-    const double s1 = n1 ? -1.0 : 1.0, s2 = n2 ? -1.0 : 1.0;
     const int coff = qp.plan_ch_off[pc.plan], poff = qp.prof_ch_off[prof];
     const double fi = qp.ch_frel[coff + pc.cut];
-    const double U = s1 * xhi + s2 * yhi;
+    const double U = (n1 ? -xhi : xhi) + (n2 ? -yhi : yhi);
     const int nc = min(pc.c_hi - pc.c_lo + 1, kMaxCand);
     if (lane < nc) {
-        const double fc = qp.ch_frel[coff + pc.c_lo + lane], hb = 0.5 * qp.ch_B[coff + pc.c_lo + lane];
-        g.lo[lane] = (float)(((fc - hb) - fi) - U);
-        g.hi[lane] = (float)(((fc + hb) - fi) - U);
+        const double e = (qp.ch_frel[coff + pc.c_lo + lane] - fi) - U, B = qp.ch_B[coff + pc.c_lo + lane];
+        g.lo[lane] = (float)fma(-0.5, B, e);
+        g.hi[lane] = (float)fma(0.5, B, e);
         g.pd[lane] = pdv[poff + pc.c_lo + lane];
-        g.hat[lane] = (float)(0.5 * qp.ch_alpha[coff + pc.c_lo + lane]) * at_scale;
+        g.hat[lane] = 0.5f * (float)qp.ch_alpha[coff + pc.c_lo + lane] * at_scale;
     }
+    // lane k takes the k-th value apart
+    const double t = 3.0 * qp.c4 * fi, b1 = qp.c3 + t;
+    const double b0 = fma(fi, qp.c3 + b1, qp.beta2), u1 = xhi * yhi;
+    double v = u1;
+    if (lane == 1) v = (n1 == n2 ? -4.0 : 4.0) * kPi * kPi * u1;
+    if (lane == 2) v = fma(U, fma(qp.c4, U, b1), b0);
+    if (lane == 3) v = fma(2.0 * qp.c4, U, b1);
+    if (lane == 4) v = fi + U;
+    if (lane == 5) v = xhi;
+    if (lane == 6) v = yhi;
+    if (lane == 7)
+        v = 0.5 * (qp.ch_alpha[coff + pc.a] + qp.ch_alpha[coff + pc.b] - qp.ch_alpha[coff + pc.cut]);
+    const float vh = (float)v, vl = (float)(v - (double)vh);
+    if (lane == 1) g.vC = make_float2(vh, vl);
+    if (lane == 2) g.br0 = make_float2(vh, vl);
+    if (lane == 3) g.br1 = vh;
+    if (lane == 4) g.Fc0 = vh;
+    if (lane == 5) g.xhi = vh;
+    if (lane == 6) g.yhi = vh;
+    if (lane == 7) g.at_ab = vh * at_scale;
     if (lane == 0) {
-        const double c3 = kPi * qp.beta3, c4 = 2.0 * kPi * kPi / 3.0 * qp.beta4;
-        const double ds = fmin(R + Rb, qp.ln_eps) / qp.G;     // upsilon1 from max(xlo ylo, eps xhi yhi)
-        g.u1hi = xhi * yhi;
-        g.br0 = qp.beta2 + c3 * (U + 2.0 * fi) + c4 * (U * U + 3.0 * fi * U + 3.0 * fi * fi);
-        g.br1 = (float)(c3 + c4 * (2.0 * U + 3.0 * fi));
-        g.c4 = (float)c4;
-        g.ds = (float)ds;
-        g.ds2 = ds * kLog2e;
-        g.xhi = (float)xhi;
-        g.yhi = (float)yhi;
-        g.s1 = (float)s1;
-        g.s2 = (float)s2;
-        g.R = (float)R;
-        g.Rb = (float)Rb;
+        const float2 ds2 = pc.ds2;
+        g.u1hi = vh;
+        g.c4 = (float)qp.c4;
+        g.ds2 = ds2;
+        g.ds = fmaf(ds2.x, 0.693147182f, fmaf(ds2.x, -1.90465421e-9f, ds2.y * 0.693147182f));   // times ln 2
+        g.s1 = n1 ? -1.0f : 1.0f;
+        g.s2 = n2 ? -1.0f : 1.0f;
+        g.R = sw ? pc.lny : pc.lnx;
+        g.Rb = sw ? pc.lnx : pc.lny;
         g.band = qp.L * (float)qp.n_spans;
         g.tilt = tilt;
-        g.Fc0 = (float)(fi + U);
         g.wab = pdv[poff + pc.a] * pdv[poff + pc.b];
-        g.at_ab = (float)(0.5 * (qp.ch_alpha[coff + pc.a] + qp.ch_alpha[coff + pc.b] -
-                                 qp.ch_alpha[coff + pc.cut])) * at_scale;
         g.mult = pc.mult;
         g.nc = nc;
     }
     return sw;
 }
 
-// 2^-t for t >= 0 in FP64 to ~1e-11 relative: the Taylor series of e^x on |x|
-// <= ln 2 / 2 to x^9 (remainder (0.347)^10 / 10! = 7e-12), exponent by its bits.
-__device__ __forceinline__ double exp2_neg(double t)
-{
-    const double n = rint(t);
-    const double x = (n - t) * 0.69314718055994530942;
-    double p = 1.0 / 362880.0;
-    p = fma(p, x, 1.0 / 40320.0);
-    p = fma(p, x, 1.0 / 5040.0);
-    p = fma(p, x, 1.0 / 720.0);
-    p = fma(p, x, 1.0 / 120.0);
-    p = fma(p, x, 1.0 / 24.0);
-    p = fma(p, x, 1.0 / 6.0);
-    p = fma(p, x, 0.5);
-    p = fma(p, x, 1.0);
-    p = fma(p, x, 1.0);
-    if (n > 1000.0) return 0.0;
-    return __hiloint2double(__double2hiint(p) - ((int)n << 20), __double2loint(p));
-}
-
-// The row k = G - 1/2 - r pitches below the corner (r real-valued in a block).
-// In logarithms relative to the corner, l = ln(upsilon1 / (xhi yhi)), |f2| runs
+// The row k + k_lo = G - 1/2 - r pitches below the corner (r real-valued in a
+// block).  upsilon1 / (xhi yhi) = 2^-t, t = k ds2, is taken in FP32 pairs to ~1e-10
+// relative: t = n + j / 256 + rest, a table of 2^(-j/256) and the Taylor series of
+// 2^-rest - 1 (|rest| <= 1/512; to the third power, remainder below 2e-13).  In logarithms relative to the corner, l = ln(upsilon1 / (xhi yhi)), |f2| runs
 // over [max(-Rb, l), min(0, l + R)] and the row's centre lies at ln(xc / xhi) =
 // gx, ln(yc / yhi) = gy.  Returns which limits hold: bit 0 the one set by xhi,
 // bit 1 by xlo (else by ylo, yhi); -1 for an empty row.
-__device__ __forceinline__ int node_row(const PieceGeo &g, int G, double k, NodeRow &o)
+__device__ __forceinline__ int node_row(const PieceGeo &g, const float2 *gauss, int G, float k, float k_lo,
+                                        NodeRow &o)
 {
-    const double u1d = g.u1hi * exp2_neg(k * g.ds2);
-    const float u1 = (float)u1d;
-    const float l = -(float)k * g.ds;
+    const float t = k * g.ds2.x, tl = fmaf(k, g.ds2.x, -t) + fmaf(k, g.ds2.y, k_lo * g.ds2.x);
+    const float mf = __fadd_rn(fmaf(t, (float)kExp2Entries, 12582912.0f), -12582912.0f);
+    const float y = (fmaf(mf, -1.0f / kExp2Entries, t) + tl) * -0.6931471806f;
+    const float q = fmaf(y * y, fmaf(y, 1.0f / 6.0f, 0.5f), y);
+    const int mi = (int)mf, n = mi / kExp2Entries;
+    const float2 T = __ldg(gauss + kGaussEntries + (mi & (kExp2Entries - 1)));
+    const float eh = fmaf(T.x, q, T.x), el = fmaf(T.x, q, __fadd_rn(T.x, -eh)) + fmaf(T.y, q, T.y);
+    const float sc = n < 127 ? __int_as_float((127 - n) << 23) : 0.0f;
+    const float u1 = fmaf(g.u1hi, eh, g.u1hi * el) * sc;
+    const float l = -k * g.ds;
     const bool a = l > -g.Rb, b = l + g.R < 0.0f;
     const float D = a ? (b ? g.R : -l) : (b ? l + g.R + g.Rb : g.Rb);
     const float gx = a ? (b ? -0.5f * g.R : 0.5f * l) : (b ? 0.5f * (l + g.Rb - g.R) : l + 0.5f * g.Rb);
@@ -228,11 +236,13 @@ __device__ __forceinline__ int node_row(const PieceGeo &g, int G, double k, Node
     o.x0 = g.s1 * g.xhi * expm1f(gx);
     o.y0 = g.s2 * g.yhi * expm1f(gy);
     const float u0 = o.x0 + o.y0;
-    const double v = (double)(g.s1 * g.s2) * u1d;
-    const double br = g.br0 + (double)(u0 * fmaf(g.c4, u0, g.br1)) - (double)(0.5f * g.c4) * v;
-    const double phi = (-4.0 * kPi * kPi) * v * br;
-    o.phi0 = (float)phi;
-    o.phi0_lo = (float)(phi - (double)o.phi0);
+    const float db = fmaf(-0.5f * g.c4 * g.s1 * g.s2, u1, u0 * fmaf(g.c4, u0, g.br1));
+    const float bh = __fadd_rn(g.br0.x, db), bb = __fadd_rn(bh, -g.br0.x);        // two-sum
+    const float bl = __fadd_rn(__fadd_rn(g.br0.x, -__fadd_rn(bh, -bb)), __fadd_rn(db, -bb)) + g.br0.y;
+    const float vh = g.vC.x * eh, vl = fmaf(g.vC.x, eh, -vh) + fmaf(g.vC.x, el, g.vC.y * eh);
+    const float ph = vh * bh;
+    o.phi0 = ph * sc;
+    o.phi0_lo = (fmaf(vh, bh, -ph) + fmaf(vh, bl, vl * bh)) * sc;
     return (a ? 1 : 0) | (b ? 2 : 0);
 }
 
@@ -417,7 +427,7 @@ struct PieceBlocks {
 };
 
 template <int Cap>
-__device__ __forceinline__ PieceBlocks row_blocks(WarpNodes<Cap> &ns, int G)
+__device__ __forceinline__ PieceBlocks row_blocks(WarpNodes<Cap> &ns, const float2 *gauss, int G)
 {
     PieceBlocks pb = {0, 0, 0, -1};
     int &R1 = pb.R1, &nblk = pb.nblk, &cand = pb.cand, &units = pb.units;
@@ -427,7 +437,7 @@ __device__ __forceinline__ PieceBlocks row_blocks(WarpNodes<Cap> &ns, int G)
     // candidate and limits of row r (-1: not in one candidate), |phi| band
     const auto test = [&](int r, float &ph) {
         NodeRow o;
-        const int lim = node_row(g, G, (double)(G - r) - 0.5, o);
+        const int lim = node_row(g, gauss, G, (float)(G - r) - 0.5f, 0.0f, o);
         ph = 0.0f;
         const int c = lim >= 0 ? row_whole(g, o, G, ph) : -1;
         return c >= 0 ? (c << 2 | lim) : -1;
@@ -493,7 +503,7 @@ template <int Cap>
 __device__ __forceinline__ void unit_row(const WarpNodes<Cap> &ns, const float2 *gauss, int G, int q, int nv, int R1,
                                          int nblk, NodeRow &o)
 {
-    double k = (double)(G - (R1 + q - nv)) - 0.5;
+    float k = (float)(G - (R1 + q - nv)) - 0.5f, k_lo = 0.0f;
     float wt = 1.0f;
     if (q < nv) {
         int b = 0;
@@ -502,13 +512,15 @@ __device__ __forceinline__ void unit_row(const WarpNodes<Cap> &ns, const float2 
         const RowBlock bl = ns.blk[b];
         if (bl.toff >= 0) {
             const float2 e = __ldg(gauss + bl.toff + (q - bl.unit0));
-            k = (double)(G - bl.r0) - 0.5 * (double)bl.N - 0.5 * (double)bl.N * (double)e.x;
+            const float h = -0.5f * (float)bl.N, kc = (float)(G - bl.r0) + h, kt = h * e.x;
+            k = __fadd_rn(kc, kt);                            // |kt| <= kc
+            k_lo = __fadd_rn(__fadd_rn(kc, -k), kt) + fmaf(h, e.x, -kt);
             wt = e.y;
         } else {
-            k = (double)(G - (bl.r0 + q - bl.unit0)) - 0.5;
+            k = (float)(G - (bl.r0 + q - bl.unit0)) - 0.5f;
         }
     }
-    node_row(ns.geo, G, k, o);
+    node_row(ns.geo, gauss, G, k, k_lo, o);
     o.w *= wt;
 }
 

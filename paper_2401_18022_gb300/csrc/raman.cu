@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(256, ISRS_TAB_MIN_BLOCKS) k_quad_f32_tab(QuadP
             __syncwarp();
             PieceGeo &g = ns.geo;
             float sum = 0.0f, comp = 0.0f;
-            const PieceBlocks pb = row_blocks(ns, G);
+            const PieceBlocks pb = row_blocks(ns, qp.gauss, G);
             n_small += lane == 0 && part == 0 ? pb.R1 * G : 0;
             for (int ca = 0; ca < g.nc; ca += kTabCand) {
                 const int cb = min(g.nc, ca + kTabCand);

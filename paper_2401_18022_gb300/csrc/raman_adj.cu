@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
             const int4 pr = ap.prow[kp];
             __syncwarp();
             PieceGeo &g = ns.geo;
-            const PieceBlocks pb = row_blocks(ns, G);
+            const PieceBlocks pb = row_blocks(ns, qp.gauss, G);
             for (int cc = 0; cc < g.nc; ++cc) {
                 const double fc = qp.ch_frel[coff + pc.c_lo + cc];
                 float tilt = 0.0f;
