@@ -214,14 +214,23 @@ cudaError_t gauss_array(void **out) { return cudaGetSymbolAddress(out, g_isrs_ga
 // k_quad_f32: persistent FP32 quadrature.
 // ---------------------------------------------------------------------------
 constexpr int kFwdSlots = 512;       // node slots of a chunk
-constexpr int kFwdCand = 3;          // F_c candidates swept together (most pieces have two)
 using FwdNodes = WarpNodes<kFwdSlots>;
 
+// The nodes a warp has yet to sum, by form of the z-sum (direct, telescoped).  A
+// queue is drained 32 at a time, and what a tile leaves at its end shares the
+// lanes, several to a node: a piece's ~250 nodes at G = 64 taken as they come
+// filled 23 of 32 lanes, by the rows' tails and by rounds that held both forms and
+// so took both.
+struct FwdQueue {
+    float4 a[2][64];            // {phi, phi_lo, F_c - f_i, attenuation part of log2 p}
+    float w[2][64];             // weight
+};
+
 // Dynamic shared memory of k_quad_f32: eB and zD (pair_tables), then per warp the
-// nodes and the candidates' step rows.
+// nodes, the queues and the step rows {A2, A2', K2, K2'} about the CUT's frequency.
 __host__ __device__ constexpr size_t fwd_warp_bytes(int n_steps)
 {
-    return sizeof(FwdNodes) + sizeof(float4) * kFwdCand * (size_t)step_pairs(n_steps);
+    return sizeof(FwdNodes) + sizeof(FwdQueue) + sizeof(float4) * (size_t)step_pairs(n_steps);
 }
 #ifndef ISRS_FWD_MIN_BLOCKS
 #define ISRS_FWD_MIN_BLOCKS 3   // resident blocks per SM the register budget is sized for
@@ -236,7 +245,8 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
     float4 *eB = smem_f4, *zD = eB + M2;
     unsigned char *mine = reinterpret_cast<unsigned char *>(zD + M2) + fwd_warp_bytes(M) * warp;
     FwdNodes &ns = *reinterpret_cast<FwdNodes *>(mine);
-    float4 *ek = reinterpret_cast<float4 *>(mine + sizeof(FwdNodes));   // [kFwdCand][M2] {log2 p at f_c (2), K2 (2)}
+    FwdQueue &qu = *reinterpret_cast<FwdQueue *>(mine + sizeof(FwdNodes));
+    float4 *sp = reinterpret_cast<float4 *>(mine + sizeof(FwdNodes) + sizeof(FwdQueue));
 
     pair_tables(qp, eB, zD);
     __syncthreads();
@@ -245,17 +255,56 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
     const float log2e = (float)kLog2e;
     unsigned long long n_small = 0;
     unsigned n_direct = 0, n_tele = 0;
-
     for (;;) {
         int it = 0;
         if (lane == 0) it = atomicAdd(qp.counter, 1);
         it = __shfl_sync(0xffffffffu, it, 0);
         if (it >= qp.n_items) break;
         const DevItem item = qp.items[it];
-        const float2 *st = qp.step_f + (size_t)item.prof * M;
         const float tilt = (float)qp.kap_L[item.prof];
         const int part = item.part & 0xffff, parts = item.part >> 16;
-        double acc = 0.0;
+        // log2 p at F_c = f_i: taken about f_ref, a plan tens of THz away from it would
+        // lose the last digits to the difference of two large terms
+        {
+            const double fi = qp.ch_frel[qp.plan_ch_off[qp.prof_plan[item.prof]] + item.cut];
+            const double2 *sd = qp.step_d + (size_t)item.prof * M;
+            const float2 *st = qp.step_f + (size_t)item.prof * M;
+            for (int k = lane; k < M2; k += 32) {
+                const int k1 = min(2 * k + 1, M - 1);
+                const double2 v = sd[2 * k], u = sd[k1];
+                sp[k] = make_float4((float)(kLog2e * fma(-v.y, fi, v.x)),
+                                    2 * k + 1 < M ? (float)(kLog2e * fma(-u.y, fi, u.x)) : -1000.0f,
+                                    st[2 * k].y, st[k1].y);
+            }
+        }
+        float sum = 0.0f, comp = 0.0f;
+        int nd_q = 0, nt_q = 0;              // nodes in the queues
+        // entries [first, first + n) of a queue, 32 / n lanes (a power of two) to a node
+        const auto drain = [&](int form, int first, int n) {
+            const int lg = n > 16 ? 0 : n > 8 ? 1 : n > 4 ? 2 : n > 2 ? 3 : n > 1 ? 4 : 5;
+            const int node = lane >> lg, sub = lane - (node << lg);
+            const int k0 = (M2 * sub) >> lg, k1 = (M2 * (sub + 1)) >> lg;
+            const float4 a = qu.a[form][first + min(node, n - 1)];
+            const float w = node < n && sub == 0 ? qu.w[form][first + node] : 0.0f;
+            const f32x2 F2 = dup2(a.z), nat = dup2(-a.w);
+            const auto lp = [&](int k) {
+                const float4 x = sp[k], z = zD[k];
+                return fma2(pack2(x.z, x.w), F2, fma2(nat, pack2(z.x, z.y), pack2(x.x, x.y)));
+            };
+            float2 S = form == 0 ? zsum_direct_part(a.x, lp, zD, k0, k1)
+                                 : zsum_tele_part<false>(a.x, a.y, lp, eB, k0, k1);
+            for (int o = (1 << lg) >> 1; o > 0; o >>= 1) {
+                S.x += __shfl_xor_sync(0xffffffffu, S.x, o);
+                S.y += __shfl_xor_sync(0xffffffffu, S.y, o);
+            }
+            const float S2 = S.x * S.x + S.y * S.y;
+            // compensated accumulation over this lane's nodes
+            const float y = w * (form == 0 ? S2 : __fdividef(S2, a.x * a.x)) * array_factor_f(a.x, qp, a.y) - comp;
+            const float t = sum + y;
+            comp = (t - sum) - y;
+            sum = t;
+            __syncwarp();
+        };
 #pragma unroll 1
         for (int k = item.piece0; k < item.piece1; ++k) {
             const DevPiece &pc = qp.pieces[dbg_clamp(k, qp.n_pieces, kDbgPiece, qp.dbg)];
@@ -263,57 +312,40 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
             node_geo(qp, pc, item.prof, log2e, qp.pd_f, tilt, ns.geo);
             __syncwarp();
             const PieceGeo &g = ns.geo;
-            float sum = 0.0f, comp = 0.0f;
             const PieceBlocks pb = row_blocks(ns, qp.gauss, G);
             n_small += lane == 0 && part == 0 ? pb.R1 * G : 0;
+            const float wp = g.mult * g.wab;
+            piece_nodes(ns, pb, qp.gauss, G, 0, g.nc, [&](int c0, int nq) {
 #pragma unroll 1
-            for (int ca = 0; ca < g.nc; ca += kFwdCand) {
-                const int cb = min(g.nc, ca + kFwdCand);
-                // step rows of the candidates: ln p at the channel's centre
-#pragma unroll 1
-                for (int c = ca; c < cb; ++c) {
-                    const float at = g.at_ab + g.hat[c], F = g.Fc0 + 0.5f * (g.lo[c] + g.hi[c]);
-#pragma unroll 2
-                    for (int k = lane; k < M2; k += 32) {
-                        const float2 v = st[2 * k], u = st[min(2 * k + 1, M - 1)];
-                        const float4 z = zD[k];
-                        ek[(c - ca) * M2 + k] =
-                            make_float4(fmaf(v.y, F, fmaf(-at, z.x, v.x)),
-                                        2 * k + 1 < M ? fmaf(u.y, F, fmaf(-at, z.y, u.x)) : -1000.0f, v.y, u.y);
-                    }
-                }
-                __syncwarp();
-                piece_nodes(ns, pb, qp.gauss, G, ca, cb, [&](int c0, int nq) {
-#pragma unroll 1
-                    for (int q = lane + 32 * part; q < nq; q += 32 * parts) {
-                        Node nd;
-                        node_get(ns, qp.gauss, c0, q, nd);
-                        const int ci = dbg_clamp(nd.ci, g.nc, kDbgCand, qp.dbg);
-                        const float aphi = fabsf(nd.phi);
-                        const float dF = (nd.x + nd.y) - 0.5f * (g.lo[ci] + g.hi[ci]);
-                        const float4 *e = ek + (ci - ca) * M2;
-                        const f32x2 dF2 = dup2(dF);
-                        const auto lp = [&](int k) {
-                            const float4 x = e[k];
-                            return fma2(pack2(x.z, x.w), dF2, pack2(x.x, x.y));
-                        };
-                        const bool direct = aphi <= phi_direct;
-                        const float S2 = direct ? zsum_direct_n(nd.phi, lp, zD, M2)
-                                                : zsum_tele_n<false>(nd.phi, nd.phi_lo, lp, eB, M2);
+                for (int q0 = 32 * part; q0 < nq; q0 += 32 * parts) {
+                    const bool on = q0 + lane < nq;
+                    Node nd;
+                    node_get(ns, qp.gauss, c0, on ? q0 + lane : nq - 1, nd);
+                    const int ci = dbg_clamp(nd.ci, g.nc, kDbgCand, qp.dbg);
+                    const float aphi = fabsf(nd.phi);
+                    const int form = aphi <= phi_direct ? 0 : 1;
+                    const unsigned tele = __ballot_sync(0xffffffffu, on && form == 1);
+                    const unsigned direct = __ballot_sync(0xffffffffu, on && form == 0);
+                    const unsigned below = (1u << lane) - 1u;
+                    if (on) {
+                        const int d = (form ? nt_q : nd_q) + __popc((form ? tele : direct) & below);
+                        qu.a[form][d] = make_float4(nd.phi, nd.phi_lo, g.Fi + (nd.x + nd.y), g.at_ab + g.hat[ci]);
+                        qu.w[form][d] = wp * (nd.wq * g.pd[ci]);
                         n_small += aphi <= phi_small ? nd.N : 0;
-                        n_direct += aphi > phi_small && direct ? nd.N : 0;
-                        n_tele += direct ? 0 : nd.N;
-                        // compensated accumulation over this lane's nodes
-                        const float y = nd.wq * g.pd[ci] * S2 * array_factor_f(nd.phi, qp, nd.phi_lo) - comp;
-                        const float t = sum + y;
-                        comp = (t - sum) - y;
-                        sum = t;
+                        n_direct += aphi > phi_small && form == 0 ? nd.N : 0;
+                        n_tele += form ? nd.N : 0;
                     }
-                });
-            }
-            acc += (double)(g.mult * g.wab) * ((double)sum - (double)comp);
+                    nd_q += __popc(direct);
+                    nt_q += __popc(tele);
+                    __syncwarp();
+                    if (nd_q >= 32) drain(0, nd_q -= 32, 32);
+                    if (nt_q >= 32) drain(1, nt_q -= 32, 32);
+                }
+            });
         }
-        const double tot = warp_sum_d(acc);
+        if (nd_q > 0) drain(0, 0, nd_q);
+        if (nt_q > 0) drain(1, 0, nt_q);
+        const double tot = warp_sum_d((double)sum - (double)comp);
         if (lane == 0) qp.partial[it] = tot;
     }
     if (qp.path_count) {
@@ -545,7 +577,7 @@ size_t fwd_smem(int n_steps, int block)
 
 // Persistent launch of the quadrature.  FP32: the warps of a block work alone,
 // so a block is any number of them: as many as fit in shared memory (fewer than
-// asked only past ~900 z-steps), one where there are too few tiles to give every
+// asked only past ~1,800 z-steps), one where there are too few tiles to give every
 // SM a full block (a 5-channel plan's ~90 tiles then run on as many SMs).
 cudaError_t launch_quad(const QuadParams &qp, int precision, int num_sms, int block, cudaStream_t st)
 {

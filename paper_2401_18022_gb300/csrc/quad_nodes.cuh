@@ -105,7 +105,7 @@ struct PieceGeo {
     float R, Rb;                // ln(xhi / xlo), ln(yhi / ylo) (1e30 where the lower limit is 0)
     float band;                 // n_spans L: phase swing per |d phi|
     float tilt;                 // bound of |d ln p / dF|
-    float Fc0;                  // F_c - f_ref at the corner
+    float Fc0, Fi;              // F_c - f_ref and F_c - f_i at the corner
     float wab, at_ab, mult;     // P_a P_b / (B_a B_b), attenuation part of ln p, mirror weight
     int nc;                     // F_c candidates: edges from the corner, P/B, half attenuation
     float lo[kMaxCand], hi[kMaxCand], pd[kMaxCand], hat[kMaxCand];
@@ -170,6 +170,7 @@ __device__ __forceinline__ bool node_geo(const QuadParams &qp, const DevPiece &p
     if (lane == 2) v = fma(U, fma(qp.c4, U, b1), b0);
     if (lane == 3) v = fma(2.0 * qp.c4, U, b1);
     if (lane == 4) v = fi + U;
+    if (lane == 8) v = U;
     if (lane == 5) v = xhi;
     if (lane == 6) v = yhi;
     if (lane == 7)
@@ -179,6 +180,7 @@ __device__ __forceinline__ bool node_geo(const QuadParams &qp, const DevPiece &p
     if (lane == 2) g.br0 = make_float2(vh, vl);
     if (lane == 3) g.br1 = vh;
     if (lane == 4) g.Fc0 = vh;
+    if (lane == 8) g.Fi = vh;
     if (lane == 5) g.xhi = vh;
     if (lane == 6) g.yhi = vh;
     if (lane == 7) g.at_ab = vh * at_scale;

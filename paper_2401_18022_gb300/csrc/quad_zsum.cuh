@@ -105,15 +105,17 @@ __device__ __forceinline__ float zsum_tele_f(float phi, float Fc, float at, cons
 // of weight 2^-1000 with the same edge.  phi is float-float (the direct form's
 // phases need only its head).  Packed, a step takes ~13 instructions where the
 // scalar form took ~19; bound by the XU pipe (20 cycles per warp and step).
+// The _part forms give Re S and Im S (times phi for the telescoped one) of the
+// pairs [k0, k1), so that a few lanes can share a node.
 template <typename LP>
-__device__ __forceinline__ float zsum_direct_n(float phi, const LP &lp, const float4 *zD, int M2)
+__device__ __forceinline__ float2 zsum_direct_part(float phi, const LP &lp, const float4 *zD, int k0, int k1)
 {
     const f32x2 hph = dup2(0.5f * phi), phr = dup2(phi * 0.15915494309189535f),
                 nphr = dup2(-phi * 0.15915494309189535f);
     const f32x2 mg = dup2(12582912.0f), nm = dup2(-12582912.0f);
     f32x2 Sr = dup2(0.0f), Si = dup2(0.0f);
 #pragma unroll 2
-    for (int k = 0; k < M2; ++k) {
+    for (int k = k0; k < k1; ++k) {
         const float4 z = zD[k];
         const f32x2 zz = pack2(z.x, z.y), dz = pack2(z.z, z.w);
         float s0, c0, s1, c1, l0, l1;
@@ -132,18 +134,30 @@ __device__ __forceinline__ float zsum_direct_n(float phi, const LP &lp, const fl
     float r0, r1, i0, i1;
     unpack2(Sr, r0, r1);
     unpack2(Si, i0, i1);
-    const float sr = r0 + r1, si = i0 + i1;
-    return sr * sr + si * si;
+    return make_float2(r0 + r1, i0 + i1);
+}
+
+template <typename LP>
+__device__ __forceinline__ float zsum_direct_n(float phi, const LP &lp, const float4 *zD, int M2)
+{
+    const float2 s = zsum_direct_part(phi, lp, zD, 0, M2);
+    return s.x * s.x + s.y * s.y;
 }
 
 template <bool Wide, typename LP>
-__device__ __forceinline__ float zsum_tele_n(float phi, float phi_lo, const LP &lp, const float4 *eB, int M2)
+__device__ __forceinline__ float2 zsum_tele_part(float phi, float phi_lo, const LP &lp, const float4 *eB, int k0,
+                                                 int k1)
 {
     const f32x2 ph = dup2(phi), nph = dup2(-phi), pl = dup2(phi_lo);
     float Er = 1.0f, Ei = 0.0f;
+    if (k0 > 0) {                        // phasor at the edge before
+        const float4 e = eB[k0 - 1];
+        float s0, c0;
+        sincos_turn2(rev_fraction2<Wide>(ph, nph, pl, pack2(e.x, e.y), pack2(e.z, e.w)), s0, c0, Ei, Er);
+    }
     f32x2 Sr = dup2(0.0f), Si = dup2(0.0f);
 #pragma unroll 4
-    for (int k = 0; k < M2; ++k) {
+    for (int k = k0; k < k1; ++k) {
         const float4 e = eB[k];
         float s0, c0, s1, c1, l0, l1;
         sincos_turn2(rev_fraction2<Wide>(ph, nph, pl, pack2(e.x, e.y), pack2(e.z, e.w)), s0, c0, s1, c1);
@@ -157,8 +171,14 @@ __device__ __forceinline__ float zsum_tele_n(float phi, float phi_lo, const LP &
     float r0, r1, i0, i1;
     unpack2(Sr, r0, r1);
     unpack2(Si, i0, i1);
-    const float sr = r0 + r1, si = i0 + i1;
-    return __fdividef(sr * sr + si * si, phi * phi);
+    return make_float2(r0 + r1, i0 + i1);
+}
+
+template <bool Wide, typename LP>
+__device__ __forceinline__ float zsum_tele_n(float phi, float phi_lo, const LP &lp, const float4 *eB, int M2)
+{
+    const float2 s = zsum_tele_part<Wide>(phi, phi_lo, lp, eB, 0, M2);
+    return __fdividef(s.x * s.x + s.y * s.y, phi * phi);
 }
 
 // Steps in pairs: pair k holds steps 2k, 2k + 1.
