@@ -24,7 +24,7 @@ struct PrepParams {
     double *cs;                 // ChainParams::cs of a gradient (one profile), or null
 };
 
-// FP32 copy of the profile tables for the MCI cells (pairs of steps outermost)
+// FP32 copy of the profile tables for the MCI cells (pairs of steps)
 struct TabHalfParams {
     const double2 *ab;
     float4 *abf;

@@ -32,25 +32,23 @@ namespace isrs {
 namespace {
 
 constexpr int kMciCells = 6;       // cells of a group at most
-constexpr int kMciUnits = 6;       // step rows of a group: one per cell and F_c channel
+constexpr int kMciUnits = 4;       // step rows of a group: one per cell and F_c channel
 constexpr int kMciList = 96;       // points waiting: telescoped from the front, direct from the back (31 + 31 + 32)
 constexpr int kMciRows = 32;       // rows of a group
 
 // Cells a warp takes together: at most 32 grid rows (and kMciUnits step rows).
 __host__ __device__ constexpr int mci_group(int G) { return G >= 32 ? 1 : (32 / G < kMciCells ? 32 / G : kMciCells); }
 
-// {1/2 log2(e) a_c, 1/2 log2(e) b_c} in FP32, steps outermost: float4 {a, a', b,
-// b'} of pair k and channel c at prof_ch_off[p] pairs + k n + c.  Neighbouring
-// points of a group have F_c in neighbouring channels, so a warp's 32 rows of one
-// pair lie in a few lines; with the channel outermost (as qp.ab) every lane read
-// its own sector and the loads bound the kernel.  One block row per profile.
+// {1/2 log2(e) a_c, 1/2 log2(e) b_c} in FP32: float4 {a, a', b, b'} of channel c and
+// pair k at (prof_ch_off[p] + c) pairs + k, the order in which a warp reads them for
+// its step rows.  One block row per profile.
 __global__ void __launch_bounds__(256) k_tab_half_log2(TabHalfParams hp)
 {
     const int p = blockIdx.y, n = hp.plan_n[hp.prof_plan[p]], M = hp.n_steps, M2 = step_pairs(M);
     const double2 *ab = hp.ab + (size_t)hp.prof_ch_off[p] * M;
     float4 *out = hp.abf + (size_t)hp.prof_ch_off[p] * M2;
     for (int t = threadIdx.x + blockIdx.x * blockDim.x; t < n * M2; t += blockDim.x * gridDim.x) {
-        const int k = t / n, c = t - k * n;
+        const int c = t / M2, k = t - c * M2;
         const double2 v = ab[(size_t)c * M + 2 * k], w = ab[(size_t)c * M + min(2 * k + 1, M - 1)];
         const double h = 0.5 * kLog2e;
         out[t] = make_float4((float)(h * v.x), (float)(h * w.x), (float)(h * v.y), (float)(h * w.y));
@@ -85,7 +83,11 @@ __host__ __device__ constexpr size_t mci_warp_bytes(int n_steps)
 // are summed 32 at a time, one per lane.  Bound by the XU pipe (20 cycles per warp
 // and step) and the issue of the other ~14 instructions.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256, 2) k_quad_mci_f32_tab(QuadParams qp)
+#ifndef ISRS_MCI_TAB_MIN_BLOCKS
+#define ISRS_MCI_TAB_MIN_BLOCKS 3   // resident blocks per SM the register budget is sized for
+#endif
+
+__global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_tab(QuadParams qp)
 {
     extern __shared__ float4 smem_f4[];
     const int M = qp.n_steps, G = qp.G, M2 = step_pairs(M), MS = M2 | 1, GC = mci_group(G);
@@ -111,6 +113,7 @@ __global__ void __launch_bounds__(256, 2) k_quad_mci_f32_tab(QuadParams qp)
     const float phi_direct = 3.14159265f / qp.dz_max;
     const float eps = (float)qp.eps_v1;
     const unsigned lt_mask = (1u << lane) - 1u;
+    const float inv_G = 1.0f / (float)G;               // (q + 1/2) inv_G floors to q / G: q < 1,024
     int cur_prof = -1, cur_cut = -1;
 
     for (;;) {
@@ -141,12 +144,16 @@ __global__ void __launch_bounds__(256, 2) k_quad_mci_f32_tab(QuadParams qp)
         const float three_fi2 = 3.0f * fi * fi;
         float sum = 0.0f, comp = 0.0f;
         int nl[2] = {0, 0};                              // list lengths (direct, telescoped)
-        // one list's first 32 points (or what is left), one per lane
+        // one list's first 32 points, one per lane; of what is left at a group's end, 32 /
+        // cnt lanes (a power of two) share a point's steps
         const auto flush = [&](int f) {
             const int cnt = min(nl[f], 32);
+            const int lg = cnt > 16 ? 0 : cnt > 8 ? 1 : cnt > 4 ? 2 : cnt > 2 ? 3 : cnt > 1 ? 4 : 5;
+            const int pt = lane >> lg, sub = lane - (pt << lg);
+            const int k0 = (M2 * sub) >> lg, k1 = (M2 * (sub + 1)) >> lg;
             __syncwarp();
-            const int at = f ? lane : kMciList - 1 - lane, step = f ? cnt : -cnt;
-            if (lane < cnt) {
+            {
+                const int e = min(pt, cnt - 1), at = f ? e : kMciList - 1 - e;
                 const float4 v = w.Lp[at];
                 const int u = w.Lu[at] * MS;
                 const f32x2 da = dup2(v.y), db = dup2(v.z);
@@ -155,14 +162,20 @@ __global__ void __launch_bounds__(256, 2) k_quad_mci_f32_tab(QuadParams qp)
                     const float2 y = Qb[u + k];
                     return fma2(pack2(y.x, y.y), db, fma2(pack2(x.z, x.w), da, pack2(x.x, x.y)));
                 };
-                const float S2 = f ? zsum_tele_n<true>(v.x, 0.0f, lp, eB, M2) : zsum_direct_n(v.x, lp, zD, M2);
-                const float y = v.w * S2 * array_factor_f(v.x, qp) - comp;
+                float2 S = f ? zsum_tele_part<true>(v.x, 0.0f, lp, eB, k0, k1) : zsum_direct_part(v.x, lp, zD, k0, k1);
+                for (int o = (1 << lg) >> 1; o > 0; o >>= 1) {
+                    S.x += __shfl_xor_sync(0xffffffffu, S.x, o);
+                    S.y += __shfl_xor_sync(0xffffffffu, S.y, o);
+                }
+                const float S2 = S.x * S.x + S.y * S.y, wt = pt < cnt && sub == 0 ? v.w : 0.0f;
+                const float y = wt * (f ? __fdividef(S2, v.x * v.x) : S2) * array_factor_f(v.x, qp) - comp;
                 const float t = sum + y;
                 comp = (t - sum) - y;
                 sum = t;
             }
             __syncwarp();
             nl[f] -= cnt;
+            const int at = f ? lane : kMciList - 1 - lane, step = f ? cnt : -cnt;
             if (lane < nl[f]) {                          // at most 31 stay
                 w.Lp[at] = w.Lp[at + step];
                 w.Lu[at] = w.Lu[at + step];
@@ -190,22 +203,24 @@ __global__ void __launch_bounds__(256, 2) k_quad_mci_f32_tab(QuadParams qp)
                 __syncwarp();
                 // step rows: ln p at da = db = 0 of the cell with F_c in channel c, dc
                 // = da + db + D
-                for (int e = lane; e < nu * M2; e += 32) {
-                    const int k = e / nu, u = e - k * nu;
+#pragma unroll 1
+                for (int u = 0; u < nu; ++u) {
                     const int2 un = w.unit[u];
                     const int ab = w.cell[un.x].x, a = ab & 0xffff, b = ab >> 16;
                     const float D = (rel[a] + rel[b]) - rel[un.y];
-                    const float4 *Tk = T + (size_t)k * n;
-                    const float4 ta = Tk[a], tb = Tk[b], ti = Tk[i], tc = Tk[un.y];
-                    float4 q = make_float4(fmaf(tc.z, D, (ta.x + tb.x) + (tc.x - ti.x)),
-                                           fmaf(tc.w, D, (ta.y + tb.y) + (tc.y - ti.y)), ta.z + tc.z, ta.w + tc.w);
-                    if (2 * k + 1 >= M) q.y = -1000.0f;
-                    Qa[u * MS + k] = q;
-                    Qb[u * MS + k] = make_float2(tb.z + tc.z, tb.w + tc.w);
+                    const float4 *Ta = T + a * M2, *Tb = T + b * M2, *Tc = T + un.y * M2, *Ti = T + i * M2;
+                    for (int k = lane; k < M2; k += 32) {
+                        const float4 ta = Ta[k], tb = Tb[k], ti = Ti[k], tc = Tc[k];
+                        float4 q = make_float4(fmaf(tc.z, D, (ta.x + tb.x) + (tc.x - ti.x)),
+                                               fmaf(tc.w, D, (ta.y + tb.y) + (tc.y - ti.y)), ta.z + tc.z, ta.w + tc.w);
+                        if (2 * k + 1 >= M) q.y = -1000.0f;
+                        Qa[u * MS + k] = q;
+                        Qb[u * MS + k] = make_float2(tb.z + tc.z, tb.w + tc.w);
+                    }
                 }
                 // grid rows
                 for (int e = lane; e < ncc * G; e += 32) {
-                    const int cc = e / G, r = e - cc * G;
+                    const int cc = (int)(((float)e + 0.5f) * inv_G), r = e - cc * G;
                     const int4 cl = w.cell[cc];
                     const int a = cl.x & 0xffff, b = cl.x >> 16;
                     const float mult = a == b ? 1.0f : 2.0f;
@@ -227,15 +242,19 @@ __global__ void __launch_bounds__(256, 2) k_quad_mci_f32_tab(QuadParams qp)
                     w.row[e] = o;
                 }
                 __syncwarp();
-                for (int q0 = 0; q0 < ncc * G * G; q0 += 32) {
+                // the last turn, without points, sums what is left: the next group
+                // replaces the step rows
+#pragma unroll 1
+                for (int q0 = 0, more = 1; more; q0 += 32) {
                     const int q = q0 + lane;
+                    more = q0 < ncc * G * G;
                     int cls = -1, ci = -1, un = 0;
                     float phi = 0.0f, da = 0.0f, db = 0.0f, W = 0.0f;
                     if (q < ncc * G * G) {
-                        const int rr = q / G, j = q - rr * G;
+                        const int rr = (int)(((float)q + 0.5f) * inv_G), j = q - rr * G;
                         const float4 o = w.row[rr];
                         if (o.w != 0.0f) {
-                            const int4 cl = w.cell[rr / G];
+                            const int4 cl = w.cell[(int)(((float)rr + 0.5f) * inv_G)];
                             const float ra = rel[cl.x & 0xffff], rb = rel[cl.x >> 16];
                             const float s1 = ra > 0.0f ? 1.0f : -1.0f, s2 = rb > 0.0f ? 1.0f : -1.0f;
                             const float d = ((float)j + 0.5f - 0.5f * (float)G) * o.z;
@@ -265,12 +284,9 @@ __global__ void __launch_bounds__(256, 2) k_quad_mci_f32_tab(QuadParams qp)
                             w.Lu[at] = un;
                         }
                         nl[f] += __popc(m);
-                        if (nl[f] >= 32) flush(f);
+                        if (nl[f] >= (more ? 32 : 1)) flush(f);
                     }
                 }
-                // the next group replaces the step rows
-                for (int f = 0; f < 2; ++f)
-                    if (nl[f] > 0) flush(f);
             }
         }
         const double tot = block_sum_d((double)sum - (double)comp, scratch);
