@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
                 return fma2(pack2(x.z, x.w), F2, fma2(nat, pack2(z.x, z.y), pack2(x.x, x.y)));
             };
             float2 S = form == 0 ? zsum_direct_part(a.x, lp, zD, k0, k1)
-                                 : zsum_tele_part<false>(a.x, a.y, lp, eB, k0, k1);
+                                 : zsum_tele_part<0>(a.x, a.y, lp, eB, k0, k1);
             for (int o = (1 << lg) >> 1; o > 0; o >>= 1) {
                 S.x += __shfl_xor_sync(0xffffffffu, S.x, o);
                 S.y += __shfl_xor_sync(0xffffffffu, S.y, o);

@@ -111,6 +111,7 @@ __global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_t
     const float b2 = (float)qp.beta2;
     const float m4pi2 = (float)(-4.0 * kPi * kPi);
     const float phi_direct = 3.14159265f / qp.dz_max;
+    const float phi_wide = 6.28318531f * 1048576.0f / qp.L;     // 2^20 revolutions over the span: one rounding does
     const float eps = (float)qp.eps_v1;
     const unsigned lt_mask = (1u << lane) - 1u;
     const float inv_G = 1.0f / (float)G;               // (q + 1/2) inv_G floors to q / G: q < 1,024
@@ -162,7 +163,11 @@ __global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_t
                     const float2 y = Qb[u + k];
                     return fma2(pack2(y.x, y.y), db, fma2(pack2(x.z, x.w), da, pack2(x.x, x.y)));
                 };
-                float2 S = f ? zsum_tele_part<true>(v.x, 0.0f, lp, eB, k0, k1) : zsum_direct_part(v.x, lp, zD, k0, k1);
+                float2 S;
+                if (f == 0) S = zsum_direct_part(v.x, lp, zD, k0, k1);
+                else if (__any_sync(0xffffffffu, fabsf(v.x) > phi_wide))
+                    S = zsum_tele_part<1>(v.x, 0.0f, lp, eB, k0, k1);
+                else S = zsum_tele_part<2>(v.x, 0.0f, lp, eB, k0, k1);
                 for (int o = (1 << lg) >> 1; o > 0; o >>= 1) {
                     S.x += __shfl_xor_sync(0xffffffffu, S.x, o);
                     S.y += __shfl_xor_sync(0xffffffffu, S.y, o);

@@ -489,7 +489,7 @@ __global__ void __launch_bounds__(256, ISRS_TAB_MIN_BLOCKS) k_quad_f32_tab(QuadP
                         };
                         const bool direct = aphi <= phi_direct;
                         const float S2 = direct ? zsum_direct_n(nd.phi, lp, zD, M2)
-                                                : zsum_tele_n<false>(nd.phi, nd.phi_lo, lp, eB, M2);
+                                                : zsum_tele_n<0>(nd.phi, nd.phi_lo, lp, eB, M2);
                         n_small += aphi <= phi_small ? nd.N : 0;
                         n_direct += aphi > phi_small && direct ? nd.N : 0;
                         n_tele += direct ? 0 : nd.N;
