@@ -183,7 +183,7 @@ size_t quad_tab_limit_bytes(int precision, int n_steps, int G, int nc_max);
 cudaError_t launch_quad_tab(const QuadParams &qp, int precision, int num_sms, int block, cudaStream_t st);
 cudaError_t launch_finish(const FinishParams &fp, int n_prof, cudaStream_t st);
 // MCI cells with their own grid (closed-form profile)
-size_t quad_mci_smem_bytes(int precision, int n_steps, int n_max);
+size_t quad_mci_smem_bytes(int precision, int n_steps, int n_max, int block);
 int quad_mci_blocks_per_sm(int precision, int n_steps, int n_max, int block);
 cudaError_t launch_quad_mci(const QuadParams &qp, int precision, int grid, int block, cudaStream_t st);
 // ... with the tabulated (Raman-ODE) profile: qp.ab (FP64 kernel) or qp.ab_f

@@ -1,5 +1,4 @@
-// Cell decoding of the multi-channel-interference (MCI) grid, shared by the
-// MCI quadrature and its adjoint: a work item is a range of cells (a, b),
+// Cells and grid points of the multi-channel-interference (MCI) grid: a work item is a range of cells (a, b),
 // a <= b, a, b != CUT, in triangular order over the other N - 1 channels.
 #pragma once
 #include <cuda_runtime.h>
@@ -84,5 +83,47 @@ __device__ __forceinline__ int cell_round(CellRound &cr, int t0, int t1, int n, 
     __syncthreads();
     return tot;
 }
+
+// Row r of a cell's hyperbolic grid (ra, rb: |f_a - f_i|, |f_b - f_i|; P: the
+// powers' product with the mirror weight): {xc, yc, du2, weight}, 0 if empty.
+__device__ __forceinline__ float4 mci_row(float ra, float rb, float hba, float hbb, float eps, int G, int r, float P)
+{
+    const float xlo = ra - hba, xhi = ra + hba;
+    const float ylo = rb - hbb, yhi = rb + hbb;
+    const float u1hi = xhi * yhi;
+    const float llo = logf(fmaxf(xlo * ylo, eps * u1hi));
+    const float ds = (logf(u1hi) - llo) / (float)G;
+    const float u1 = expf(fmaf((float)r + 0.5f, ds, llo));
+    const float ymin = fmaxf(ylo, u1 / xhi), ymax = fminf(yhi, u1 / xlo);
+    float4 o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    if (ymax > ymin) {
+        o.z = log1pf((ymax - ymin) / ymin) / (float)G;
+        o.y = sqrtf(ymin * ymax);
+        o.x = u1 / o.y;
+        o.w = u1 * ds * o.z * P;
+    }
+    return o;
+}
+
+// f1 and f2 at column j of a row (sa, sb: f_a - f_i, f_b - f_i)
+__device__ __forceinline__ float2 mci_point(const float4 &o, float sa, float sb, int j, int G)
+{
+    const float d = ((float)j + 0.5f - 0.5f * (float)G) * o.z;
+    const float ex = expf(d);
+    const float s1 = sa > 0.0f ? 1.0f : -1.0f, s2 = sb > 0.0f ? 1.0f : -1.0f;
+    return make_float2(s1 * (o.x * ex), s2 * (o.y * __frcp_rn(ex)));
+}
+
+// Coefficients of phi (Eq. phi) at the CUT's frequency
+struct MciPhase {
+    float b2, c3, c4, fi, three_fi2;
+    __device__ __forceinline__ float at(float f1, float f2) const
+    {
+        const float u = f1 + f2;
+        const float br = b2 + c3 * (u + 2.0f * fi) +
+                         c4 * (f1 * f1 + 1.5f * f1 * f2 + 3.0f * fi * u + f2 * f2 + three_fi2);
+        return -39.4784176f * f1 * f2 * br;
+    }
+};
 
 }  // namespace isrs

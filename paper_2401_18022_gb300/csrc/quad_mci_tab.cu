@@ -106,10 +106,6 @@ __global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_t
     __shared__ int s_item;
 
     pair_tables(qp, eB, zD);
-    const float c3 = (float)(kPi * qp.beta3);
-    const float c4 = (float)(2.0 * kPi * kPi / 3.0 * qp.beta4);
-    const float b2 = (float)qp.beta2;
-    const float m4pi2 = (float)(-4.0 * kPi * kPi);
     const float phi_direct = 3.14159265f / qp.dz_max;
     const float phi_wide = 6.28318531f * 1048576.0f / qp.L;     // 2^20 revolutions over the span: one rounding does
     const float eps = (float)qp.eps_v1;
@@ -142,7 +138,7 @@ __global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_t
         const float4 *T = qp.ab_f + (size_t)poff * M2;   // this profile's channel rows
         const float *pd = qp.pd_f + poff;                // [n] P/B
         const float fi = (float)qp.ch_frel[coff + i];
-        const float three_fi2 = 3.0f * fi * fi;
+        const MciPhase ph = {(float)qp.beta2, (float)qp.c3, (float)qp.c4, fi, 3.0f * fi * fi};
         float sum = 0.0f, comp = 0.0f;
         int nl[2] = {0, 0};                              // list lengths (direct, telescoped)
         // one list's first 32 points, one per lane; of what is left at a group's end, 32 /
@@ -228,23 +224,8 @@ __global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_t
                     const int cc = (int)(((float)e + 0.5f) * inv_G), r = e - cc * G;
                     const int4 cl = w.cell[cc];
                     const int a = cl.x & 0xffff, b = cl.x >> 16;
-                    const float mult = a == b ? 1.0f : 2.0f;
-                    const float ra = fabsf(rel[a]), rb = fabsf(rel[b]);
-                    const float xlo = ra - hb[a], xhi = ra + hb[a];
-                    const float ylo = rb - hb[b], yhi = rb + hb[b];
-                    const float u1hi = xhi * yhi;
-                    const float llo = logf(fmaxf(xlo * ylo, eps * u1hi));
-                    const float ds = (logf(u1hi) - llo) / (float)G;
-                    const float u1 = expf(fmaf((float)r + 0.5f, ds, llo));
-                    const float ymin = fmaxf(ylo, u1 / xhi), ymax = fminf(yhi, u1 / xlo);
-                    float4 o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                    if (ymax > ymin) {
-                        o.z = log1pf((ymax - ymin) / ymin) / (float)G;
-                        o.y = sqrtf(ymin * ymax);
-                        o.x = u1 / o.y;
-                        o.w = u1 * ds * o.z * mult * (pd[a] * pd[b]);
-                    }
-                    w.row[e] = o;
+                    w.row[e] = mci_row(fabsf(rel[a]), fabsf(rel[b]), hb[a], hb[b], eps, G, r,
+                                       (a == b ? 1.0f : 2.0f) * (pd[a] * pd[b]));
                 }
                 __syncwarp();
                 // the last turn, without points, sums what is left: the next group
@@ -261,21 +242,16 @@ __global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_t
                         if (o.w != 0.0f) {
                             const int4 cl = w.cell[(int)(((float)rr + 0.5f) * inv_G)];
                             const float ra = rel[cl.x & 0xffff], rb = rel[cl.x >> 16];
-                            const float s1 = ra > 0.0f ? 1.0f : -1.0f, s2 = rb > 0.0f ? 1.0f : -1.0f;
-                            const float d = ((float)j + 0.5f - 0.5f * (float)G) * o.z;
-                            const float ex = expf(d);
-                            const float f1 = s1 * (o.x * ex), f2 = s2 * (o.y * __frcp_rn(ex));
-                            const float u = f1 + f2;
+                            const float2 f = mci_point(o, ra, rb, j, G);
+                            const float u = f.x + f.y;
                             for (int c = cl.y; c <= cl.z; ++c)
                                 if (rel[c] - hb[c] <= u && u < rel[c] + hb[c]) ci = c;
                             if (ci >= 0) {
                                 W = o.w * pd[ci];
-                                da = f1 - ra;
-                                db = f2 - rb;
+                                da = f.x - ra;
+                                db = f.y - rb;
                                 un = cl.w + (ci - cl.y);
-                                const float br = b2 + c3 * (u + 2.0f * fi) +
-                                                 c4 * (f1 * f1 + 1.5f * f1 * f2 + 3.0f * fi * u + f2 * f2 + three_fi2);
-                                phi = m4pi2 * f1 * f2 * br;
+                                phi = ph.at(f.x, f.y);
                                 if (W != 0.0f) cls = fabsf(phi) <= phi_direct ? 0 : 1;
                             }
                         }
