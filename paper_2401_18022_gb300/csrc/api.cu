@@ -47,7 +47,7 @@ struct Geom {
     std::vector<int> prof_ch_off, plan_ch_off, plan_n, prof_plan;
     int total_prof_ch = 0, total_plan_ch = 0;
     DevBuf pieces, items, slot_items, slot_cut, prof_slot_off, plan_ch_off_d, plan_n_d, prof_ch_off_d,
-        prof_plan_d, ch_frel, ch_B, ch_alpha, ch_gamma, ch_nf, guard, zs_a, zs_b, zs_d, zs_g, item_slot;
+        prof_plan_d, ch_frel, ch_B, ch_alpha, ch_gamma, ch_nf, guard, zs_a, zs_b, zs_d, item_slot;
     bool has_nf = false, has_guard = false;
     // Raman-ODE profile: partner windows and gain scale per plan channel, RK4
     // steps per half z-step, largest candidate count of a piece
@@ -442,7 +442,7 @@ isrs_status cut_pieces(isrs_handle h, const isrs_channels *c, int plan, int i, i
 // positions in revolutions (z / 2 pi) as float-float pairs.
 // ----------------------------------------------------------------------------
 void zgrid_tables(double L, double a, int n_edges, std::vector<float4> &za, std::vector<float4> &zb,
-                  std::vector<double2> &zd, float &dz_max, std::vector<float4> *zg = nullptr)
+                  std::vector<double2> &zd, float &dz_max)
 {
     std::vector<double> ze(n_edges);
     const double drop = a > 0.0 ? -std::expm1(-a * L) : 0.0;
@@ -467,23 +467,6 @@ void zgrid_tables(double L, double a, int n_edges, std::vector<float4> &za, std:
         zb[m] = make_float4(reh, (float)(re - (double)reh), (float)rm, 0.f);
     }
     dz_max = (float)dmax;
-    if (zg) {
-        // centred step moments g_n(m) = mean of (zeta - L/2)^n over [ze_m, ze_{m+1}]
-        // = (b^{n+1} - a^{n+1}) / ((n + 1)(b - a)), n = 0..18, and g_19 = 0
-        zg->assign(5 * (size_t)M, make_float4(0.f, 0.f, 0.f, 0.f));
-        for (int m = 0; m < M; ++m) {
-            const double lo = ze[m] - 0.5 * L, hi = ze[m + 1] - 0.5 * L;
-            float g[20] = {0.f};
-            double pa = lo, pb = hi;
-            for (int n = 0; n <= 18; ++n) {
-                g[n] = (float)((pb - pa) / ((n + 1) * (hi - lo)));
-                pa *= lo;
-                pb *= hi;
-            }
-            for (int q = 0; q < 5; ++q)
-                (*zg)[5 * m + q] = make_float4(g[4 * q], g[4 * q + 1], g[4 * q + 2], g[4 * q + 3]);
-        }
-    }
 }
 
 // ----------------------------------------------------------------------------
@@ -687,9 +670,9 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
     g->n_slots = (int)slot_items.size();
     g->n_mci_items = (int)mitems.size();
 
-    std::vector<float4> za, zb, zg;
+    std::vector<float4> za, zb;
     std::vector<double2> zd;
-    zgrid_tables(fb->L_km, fb->alpha_R_per_km, q->n_edges, za, zb, zd, g->dz_max, &zg);
+    zgrid_tables(fb->L_km, fb->alpha_R_per_km, q->n_edges, za, zb, zd, g->dz_max);
 
     // Raman-ODE profile: the partners of channel i are the k != i with
     // |f_k - f_i| <= raman_max_THz, one index window of the sorted plan; the
@@ -792,7 +775,6 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
     UP(zs_a, za);
     UP(zs_b, zb);
     UP(zs_d, zd);
-    UP(zs_g, zg);
     UP(item_slot, item_slot);
     if (mci) {
         UP(mci_items, mitems);
@@ -831,7 +813,7 @@ void free_geom(Geom *g)
     DevBuf *bufs[] = {&g->pieces, &g->items, &g->slot_items, &g->slot_cut, &g->prof_slot_off,
                       &g->plan_ch_off_d, &g->plan_n_d, &g->prof_ch_off_d, &g->prof_plan_d,
                       &g->ch_frel, &g->ch_B, &g->ch_alpha, &g->ch_gamma, &g->ch_nf,
-                      &g->guard, &g->zs_a, &g->zs_b, &g->zs_d, &g->zs_g, &g->item_slot,
+                      &g->guard, &g->zs_a, &g->zs_b, &g->zs_d, &g->item_slot,
                       &g->win_lo, &g->win_hi, &g->ch_scale, &g->half_steps, &g->mci_items, &g->slot_items2,
                       &g->item_slot_all, &g->tab_row_off, &g->tab_prow, &g->tab_gath_off, &g->tab_gath};
     for (DevBuf *b : bufs) release(*b);
@@ -879,12 +861,6 @@ TileSplit tile_split(const isrs_handle_s *h, int n_ch, int cell_set, int G)
     const int64_t parts = std::min<int64_t>(std::min(8, std::max(1, G / 8)), (16384 + total - 1) / total);
     return {(int)std::max<int64_t>(1, std::min<int64_t>(32, total / 38912)), (int)parts};
 }
-
-struct Launch {
-    Geom *g = nullptr;
-    int precision = 0;
-    int block = 256;
-};
 
 RamanParams raman_params(isrs_handle h, const isrs_fibre *fb, Geom *g, bool keep_nodes)
 {
@@ -944,7 +920,6 @@ QuadParams quad_params(isrs_handle h, const isrs_fibre *fb, Geom *g)
     qp.zs_a = (const float4 *)g->zs_a.p;
     qp.zs_b = (const float4 *)g->zs_b.p;
     qp.zs_d = (const double2 *)g->zs_d.p;
-    qp.zs_g = (const float4 *)g->zs_g.p;
     qp.gauss = h->gauss;
     qp.dz_max = g->dz_max;
     qp.kap_L = (const double *)h->kapL.p;
@@ -2068,10 +2043,10 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
         av[k] = ch->alpha_per_km[k];
         gv[k] = ch->gamma_per_W_km[k];
     }
-    std::vector<float4> za, zb, zg;
+    std::vector<float4> za, zb;
     std::vector<double2> zd;
     float dz_max = 0.f;
-    zgrid_tables(fibre->L_km, fibre->alpha_R_per_km, quad->n_edges, za, zb, zd, dz_max, &zg);
+    zgrid_tables(fibre->L_km, fibre->alpha_R_per_km, quad->n_edges, za, zb, zd, dz_max);
     const int M = quad->n_edges - 1;
     if (quad->precision == ISRS_PREC_FP32) {
         const double pi = 3.14159265358979323846;
@@ -2099,7 +2074,6 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     const size_t o_alpha = L.take(sizeof(double) * n), o_gamma = L.take(sizeof(double) * n);
     const size_t o_za = L.take(sizeof(float4) * M), o_zb = L.take(sizeof(float4) * M);
     const size_t o_zd = L.take(sizeof(double2) * M);
-    const size_t o_zg = L.take(sizeof(float4) * zg.size());   // centred step moments (contracted small phase)
     const size_t o_kapL = L.take(sizeof(double));
     const size_t o_P = L.take(sizeof(double) * n);
     const size_t o_pdd = L.take(sizeof(double) * n), o_pdf = L.take(sizeof(float) * n);
@@ -2122,8 +2096,7 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
         {o_plan_n, plan_n.data(), sizeof(int)}, {o_frel, frel.data(), sizeof(double) * n},
         {o_B, Bv.data(), sizeof(double) * n}, {o_alpha, av.data(), sizeof(double) * n},
         {o_gamma, gv.data(), sizeof(double) * n}, {o_za, za.data(), sizeof(float4) * M},
-        {o_zb, zb.data(), sizeof(float4) * M}, {o_zd, zd.data(), sizeof(double2) * M},
-        {o_zg, zg.data(), sizeof(float4) * zg.size()}};
+        {o_zb, zb.data(), sizeof(float4) * M}, {o_zd, zd.data(), sizeof(double2) * M}};
     for (const Up &u : ups)
         if (u.bytes && cudaMemcpyAsync(base + u.off, u.src, u.bytes, cudaMemcpyHostToDevice, st) != cudaSuccess)
             return ISRS_ERR_CUDA;
@@ -2184,7 +2157,6 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     qp.zs_a = (const float4 *)(base + o_za);
     qp.zs_b = (const float4 *)(base + o_zb);
     qp.zs_d = pp.zs_d;
-    qp.zs_g = (const float4 *)(base + o_zg);
     qp.gauss = gauss;
     qp.kap_L = pp.kap_L;
     qp.n_spans = 1;

@@ -55,8 +55,8 @@ __device__ __forceinline__ void sincos_turn2(f32x2 x, float &s0, float &c0, floa
     __sincosf(b, &s1, &c1);
 }
 
-// As rev_fraction, phasor_rev_ff and phasor_rev_ff_wide (quad_common.cuh,
-// quad_zsum.cuh): the fraction of (phi + phi_lo)(hi + lo) in revolutions; nphi =
+// As rev_fraction and phasor_rev_ff (quad_common.cuh): the fraction of (phi +
+// phi_lo)(hi + lo) in revolutions; nphi =
 // -phi.  Form 0: as written.  1: phi_lo = 0 and phases up to 2^29 revolutions, rounded
 // twice.  2: phi_lo = 0, up to 2^20 revolutions.
 template <int Form>

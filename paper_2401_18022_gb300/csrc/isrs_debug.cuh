@@ -12,7 +12,6 @@ enum DbgCode : unsigned {
     kDbgPiece = 1,      // piece index of a work tile outside the piece list
     kDbgRow = 2,        // grid row outside [0, G)
     kDbgCand = 3,       // F_c candidate outside the piece's candidates
-    kDbgList = 4,       // per-warp point list overflow
     kDbgVrow = 5,       // PSD bucket channel outside the plan
     kDbgCell = 6,       // MCI cell decoded outside the plan
 };

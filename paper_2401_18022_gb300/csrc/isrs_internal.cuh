@@ -5,8 +5,7 @@
 //   pieces        DevPiece[], plans concatenated; per CUT contiguous
 //   items         DevItem[]: work queue of (profile, piece range) tiles, ordered by
 //                 (profile, CUT) so that each CUT owns a contiguous item range
-//   z tables      per step m: z_m, dz_m, log2 dz_m, the centred step moments and
-//                 the edge phase z_{m+1}/2pi (float-float)
+//   z tables      per step m: z_m, dz_m and the edge phase z_{m+1}/2pi (float-float)
 //   profile tabs  per profile and step: float2 {A2_m, K2_m}; per profile and
 //                 channel: P/B (float, double), lnrho(L, f_c)
 //   partials      one double per item
@@ -81,7 +80,6 @@ struct QuadParams {
     const float4 *zs_a;         // {z_m, z_m^2 + dz_m^2/12, log2 dz_m, dz_m}
     const float4 *zs_b;         // {z_{m+1}/2pi hi, lo (float-float), z_m/2pi, 0}
     const double2 *zs_d;        // {z_m, dz_m}
-    const float4 *zs_g;         // [5 per step] g_0..g_19: mean of (zeta - L/2)^n over step m (g_19 = 0)
     const float2 *gauss;        // Gauss rules of the row sums (quad_nodes.cuh): {t, weight}
     const double *kap_L;        // per profile: kappa(L) [1/THz]
     float dz_max;

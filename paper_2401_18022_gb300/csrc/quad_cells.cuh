@@ -20,24 +20,6 @@ __device__ __forceinline__ void tri_decode(int t, int n2, int &ap, int &bp)
     bp = a + (t - a * (2 * n2 - a + 1) / 2);
 }
 
-// index of the channel containing offset u from the CUT, or -1
-// (lo[c] = rel[c] - hb[c] ascending, channels disjoint)
-template <typename T>
-__device__ __forceinline__ int channel_of(const T *rel, const T *hb, int n, T u)
-{
-    int lo = 0, hi = n - 1, c = -1;
-    while (lo <= hi) {
-        const int mid = (lo + hi) >> 1;
-        if (rel[mid] - hb[mid] <= u) {
-            c = mid;
-            lo = mid + 1;
-        } else {
-            hi = mid - 1;
-        }
-    }
-    return (c >= 0 && u < rel[c] + hb[c]) ? c : -1;
-}
-
 // The cells of one round of a block (blockDim cells from t0, one per thread) whose
 // F_c can fall in a channel, compacted in order: {a, b, first and last channel}.
 struct CellRound {

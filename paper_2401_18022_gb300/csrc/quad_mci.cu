@@ -214,6 +214,7 @@ __global__ void __launch_bounds__(256) k_quad_mci_f64(QuadParams qp)
     __shared__ int s_item;
 
     for (int m = threadIdx.x; m < M; m += blockDim.x) sz[m] = qp.zs_d[m];
+    const double phi_f64 = kF64Direct / qp.dz_max;
     const double c3 = kPi * qp.beta3;
     const double c4 = 2.0 * kPi * kPi / 3.0 * qp.beta4;
     int cur_prof = -1;
@@ -285,18 +286,11 @@ __global__ void __launch_bounds__(256) k_quad_mci_f64(QuadParams qp)
                 const double br = qp.beta2 + c3 * (u + 2.0 * fi) +
                                   c4 * (f1 * f1 + 1.5 * f1 * f2 + 3.0 * fi * u + f2 * f2 + 3.0 * fi * fi);
                 const double phi = -4.0 * kPi * kPi * f1 * f2 * br;
-                double Sr = 0.0, Si = 0.0;
-                for (int m = 0; m < M; ++m) {
-                    const double2 zz = sz[m];
+                const double S2 = zsum_f64(phi, phi_f64, sz, M, [&](int m) {
                     const double2 tt = st[m];
-                    const double p = exp(tt.x - tt.y * Fc - at * zz.x);
-                    const double amp = p * zz.y * sinc_d(0.5 * phi * zz.y);
-                    double sn, cs;
-                    sincos(phi * zz.x, &sn, &cs);
-                    Sr += amp * cs;
-                    Si += amp * sn;
-                }
-                sum += w * W * (Sr * Sr + Si * Si) * array_factor_d(phi, qp);
+                    return exp(tt.x - tt.y * Fc - at * sz[m].x);
+                });
+                sum += w * W * S2 * array_factor_d(phi, qp);
             }
         }
         const double tot = block_sum_d(sum, scratch);

@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_t
 }
 
 // Plain FP64 reference kernel: every step reads the profile rows of a, b, c
-// and the CUT from the FP64 tables; the z-sum as written (Eq. slow_vary).
+// and the CUT from the FP64 tables; the z-sum by zsum_f64.
 __global__ void __launch_bounds__(256) k_quad_mci_f64_tab(QuadParams qp)
 {
     extern __shared__ double2 smem_d2[];
@@ -287,6 +287,7 @@ __global__ void __launch_bounds__(256) k_quad_mci_f64_tab(QuadParams qp)
     __shared__ int s_item;
 
     for (int m = threadIdx.x; m < M; m += blockDim.x) sz[m] = qp.zs_d[m];
+    const double phi_f64 = kF64Direct / qp.dz_max;
     const double c3 = kPi * qp.beta3;
     const double c4 = 2.0 * kPi * kPi / 3.0 * qp.beta4;
 
@@ -355,18 +356,11 @@ __global__ void __launch_bounds__(256) k_quad_mci_f64_tab(QuadParams qp)
                                   c4 * (f1 * f1 + 1.5 * f1 * f2 + 3.0 * fi * u + f2 * f2 + 3.0 * fi * fi);
                 const double phi = -4.0 * kPi * kPi * f1 * f2 * br;
                 const double2 *Tc = T + (size_t)c * M;
-                double Sr = 0.0, Si = 0.0;
-                for (int m = 0; m < M; ++m) {
-                    const double2 zz = sz[m];
+                const double S2 = zsum_f64(phi, phi_f64, sz, M, [&](int m) {
                     const double2 ta = Ta[m], tb = Tb[m], tc = Tc[m];
-                    const double p = exp(0.5 * (ta.x + tb.x + tc.x - sti[m] + ta.y * da + tb.y * db + tc.y * dc));
-                    const double amp = p * zz.y * sinc_d(0.5 * phi * zz.y);
-                    double sn, cs;
-                    sincos(phi * zz.x, &sn, &cs);
-                    Sr += amp * cs;
-                    Si += amp * sn;
-                }
-                sum += w * W * (Sr * Sr + Si * Si) * array_factor_d(phi, qp);
+                    return exp(0.5 * (ta.x + tb.x + tc.x - sti[m] + ta.y * da + tb.y * db + tc.y * dc));
+                });
+                sum += w * W * S2 * array_factor_d(phi, qp);
             }
         }
         const double tot = block_sum_d(sum, scratch);

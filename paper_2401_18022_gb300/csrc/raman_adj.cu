@@ -182,7 +182,6 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
                 });
                 double vtot = (double)sum - (double)comp;
                 vtot += __shfl_down_sync(kFullT, vtot, 16);
-                const int c = pc.c_lo + cc;
                 const double D = tp.Dl - fc;
                 // the tile's rows, written by this warp alone: one lane per step, in
                 // program order, so rows that coincide (a = CUT, c = b) add in a
