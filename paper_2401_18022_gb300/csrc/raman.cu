@@ -56,8 +56,8 @@ namespace {
 // channel.  A right-hand side is a chain of short FP64 steps (exp, prefix sums,
 // combination), ~1,800 of them one after another over 80 km.  On one SM the
 // FP64 pipe (2 lanes a clock) and the block barriers of a 1,024-thread scan took
-// 18 us each on the 557-channel plan (12.5 us on 41 channels); two warps to an
-// SM and one cluster barrier a stage bring that down (DESIGN table).
+// 18 us each on the 557-channel plan (12.5 us on 41 channels); with two warps to an
+// SM and one cluster barrier a stage they take 3.5 us (2.7 us).
 constexpr int kOdeWarps = 2;             // warps of a block at most 32 warps of channels
 constexpr int kOdeMaxCluster = 16;
 constexpr int kOdeMaxWarps = kMaxRamanCh / 32;
@@ -75,6 +75,8 @@ struct OdeWindow {
 struct OdeLane {
     int n, i, wpc;                // channels, this lane's, warps per block
     bool live;
+    bool one;                     // the cluster is one block: its own barrier and shared memory do
+    int jhi, jlo;                 // hi and lo - 1
     int wi, whi, wlo;             // warps of i, of the window's last, of the one before its first
     bool has_lo;                  // the window does not start at channel 0
     const double2 *xhi, *xlo;     // remote prefixes at hi and lo - 1 (buffer 0, pair 0)
@@ -95,6 +97,9 @@ __device__ __forceinline__ OdeLane ode_lane(cg::cluster_group &cl, OdeWindow &wi
         const int r = j / (32 * L.wpc);
         return cl.map_shared_rank(&win.x[0][0][0], r) + (j - r * 32 * L.wpc);
     };
+    L.one = cl.num_blocks() == 1;
+    L.jhi = hi;
+    L.jlo = max(lo - 1, 0);
     L.wi = L.i >> 5;
     L.has_lo = lo > 0;
     L.xhi = at(hi);
@@ -133,15 +138,24 @@ __device__ __forceinline__ void ode_window(cg::cluster_group &cl, OdeWindow &win
     // totals of this warp to every block: lane r (r + 16) takes pair 0 (1) of block r
     const double2 t0 = make_double2(__shfl_sync(0xffffffffu, x0, 31), __shfl_sync(0xffffffffu, x1, 31));
     const double2 t1 = make_double2(__shfl_sync(0xffffffffu, x2, 31), __shfl_sync(0xffffffffu, x3, 31));
-    const int r = lane & 15;
-    if (r < (int)cl.num_blocks()) {
-        double2 *dst = cl.map_shared_rank(&win.tot[buf][lane >> 4][0], r);
-        dst[L.wi] = lane < 16 ? t0 : t1;
+    double2 h, l;
+    if (L.one) {
+        if ((lane & 15) == 0) win.tot[buf][lane >> 4][L.wi] = lane < 16 ? t0 : t1;
+        __syncthreads();
+        h = win.x[buf][pu][L.jhi];
+        l = win.x[buf][pd][L.jlo];
+    } else {
+        const int r = lane & 15;
+        if (r < (int)cl.num_blocks()) {
+            double2 *dst = cl.map_shared_rank(&win.tot[buf][lane >> 4][0], r);
+            dst[L.wi] = lane < 16 ? t0 : t1;
+        }
+        cl.sync();
+        const int per = 2 * (int)(sizeof(win.x[0][0]) / sizeof(double2));      // entries of one buffer
+        const int one = per / 2;
+        h = L.xhi[buf * per + pu * one];
+        l = L.xlo[buf * per + pd * one];
     }
-    cl.sync();
-    const int per = 2 * (int)(sizeof(win.x[0][0]) / sizeof(double2));      // entries of one buffer
-    const int one = per / 2;
-    const double2 h = L.xhi[buf * per + pu * one], l = L.xlo[buf * per + pd * one];
     const double2 iu = pu ? make_double2(x2, x3) : make_double2(x0, x1);
     const double2 id = pd ? make_double2(x2, x3) : make_double2(x0, x1);
     up = make_double2(h.x - iu.x, h.y - iu.y);
