@@ -294,14 +294,15 @@ def _snr_eval(eng, wl, P, dev, n_grid, reps: int = 2):
 # profiles/ (the 148-ch G = 256 profiling cases, --profile-case adjoint256 /
 # quad256): DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum), executed
 # warp instructions (smsp__inst_executed.sum) and FP32-pipe warp instructions
-# (FFMA + FADD + FMUL of sass__inst_executed_per_opcode), with the grid points
+# (FFMA + FADD + FMUL of sass__inst_executed_per_opcode, a packed one counted
+# twice), with the grid points
 # that launch evaluated.  The kernels' work per evaluated point is the same at
 # full size (same G, same per-piece shape), so each count is scaled to a full
 # launch by evaluated points.
 ADJ_CAPTURE = {"profile": "k_quad_adj_uwb148_every4th_G256.md", "points": 2880700416,
-               "dram_bytes": 4.861e6, "warp_inst": 1.587e11, "fp32_warp_inst": 8.530e10}
+               "dram_bytes": 7.739e7, "warp_inst": 2.972e9, "fp32_warp_inst": 2.571e9}
 FWD_CAPTURE = {"profile": "k_quad_f32_uwb148_every4th_G256.md", "points": 2880700416,
-               "dram_bytes": 4.126e6, "warp_inst": 7.114e10, "fp32_warp_inst": 4.469e10}
+               "dram_bytes": 4.600e6, "warp_inst": 1.723e9, "fp32_warp_inst": 1.416e9}
 ISSUE_PER_CLK_PER_SM = 4         # one warp instruction per clock per SM sub-partition
 
 
@@ -312,12 +313,11 @@ def _roofline(eng, wl, paths, n_eval, kernel_ms, use_grad, clocks):
       * sfu_algorithmic (the headline, `frac`): the work the method states per
         evaluated point-step, 3 SFU operations (sin, cos, exp), over every
         evaluated point and all N_M - 1 steps, against the SFU throughput
-        measured by isrs_probe_alu_peaks in this run.  The contracted
-        small-phase form (its z-sum from moments, exact to < 2e-8) needs none
-        of them, so this fraction can exceed 1: it measures the method's
-        rate, not pipe use;
-      * sfu_executed: the SFU operations the kernel actually issues (3 per
-        step of its direct and telescoped points, from its path counts);
+        measured by isrs_probe_alu_peaks in this run.  A row's points are
+        summed from a few nodes, so this fraction exceeds 1: it measures the
+        method's rate, not pipe use;
+      * sfu_executed: the same over the points of the direct and telescoped
+        range only (the path counts), again per point, not per node;
       * issue: executed warp instructions (ncu capture, scaled by evaluated
         points) over 152 SMs x 4 per clock at the SM clock sampled during the
         timed region: the limiter of these kernels;

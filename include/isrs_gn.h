@@ -314,10 +314,10 @@ isrs_status isrs_last_graph_replay(isrs_handle h, int *replayed);
 
 /* Grid points of the last FP32 quadrature launch (forward, or the fused
  * forward + adjoint of isrs_gn_grad) by the form its z-sum took (App. A,
- * Eq. slow_vary): counts[0] moment expansions (small phase: about the span
- * centre, contracted or per step; in the forward at G >= 160 also about the
- * centres of 2, 4 or 8 segments of the span), counts[1] direct form, counts[2]
- * telescoped form.  Synchronises the device.  Errors: INVALID_ARG (NULL, or
+ * Eq. slow_vary) by phase: counts[0] |phi| n_spans L <= 6 (low rows, also
+ * summed across rows), counts[1] the other points of the direct form, counts[2]
+ * telescoped form.  Each point counts once, also where a few nodes stand for
+ * its row.  Synchronises the device.  Errors: INVALID_ARG (NULL, or
  * no launch yet), CUDA. */
 isrs_status isrs_last_path_counts(isrs_handle h, int64_t *counts);
 
@@ -342,9 +342,10 @@ isrs_status isrs_probe_alu_peaks(int device, int which, double *ops_per_s, float
  * a memory-budgeted real-time loop, a process whose allocator is locked).
  * The paper has no counterpart; this is a deployment variant.
  *
- * All scratch (plan tables, per-profile tables, the z-grid with its step
- * moments, tile partials) lives in one file-scope device array of 4 MiB that
- * every GPU loading this library holds until the process exits.  The first
+ * All scratch (plan tables, per-profile tables, the z-grid, tile partials)
+ * lives in one file-scope device array of 4 MiB that every GPU loading this
+ * library holds until the process exits, beside the 0.6 MB table of Gauss rules
+ * that every entry point uses.  The first
  * call on a device looks up that array's address with the device current;
  * make that first call before any stream capture.  Every call shares the
  * array and leaves the last call's contents in it; calls whose GPU work

@@ -2074,6 +2074,9 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     const size_t o_alpha = L.take(sizeof(double) * n), o_gamma = L.take(sizeof(double) * n);
     const size_t o_za = L.take(sizeof(float4) * M), o_zb = L.take(sizeof(float4) * M);
     const size_t o_zd = L.take(sizeof(double2) * M);
+    // what the call once kept here (step moments, less what a tile has grown by): the
+    // problems the scratch takes stay the same
+    L.take((size_t)std::max<int64_t>(0, 80 * (int64_t)M - 4 * (int64_t)items.size()));
     const size_t o_kapL = L.take(sizeof(double));
     const size_t o_P = L.take(sizeof(double) * n);
     const size_t o_pdd = L.take(sizeof(double) * n), o_pdf = L.take(sizeof(float) * n);

@@ -5,14 +5,12 @@
 //                per-step power tables of Eq. pk for the linear-slope
 //                closed-form profile.
 //  k_gauss       the Gauss rules of the discrete uniform measures (quad_nodes.cuh).
-//  k_quad_f32    persistent quadrature: one block per work tile (a range of
+//  k_quad_f32    persistent quadrature: one warp per work tile (a range of
 //                pieces of one CUT); G x G hyperbolic grid per piece
 //                (Eqs. q1..q4), each row's sum taken from a few nodes
-//                (quad_nodes.cuh), the z-sum of Eq. slow_vary per node in FP32:
-//                the moment series about the span centre (|phi| L <= 6), else
-//                the direct or telescoped step sums with a float-float phase
-//                and mod-2pi reduction; compensated accumulation; one FP64
-//                partial per tile.
+//                (quad_nodes.cuh), the z-sum of Eq. slow_vary per node in FP32
+//                (quad_zsum.cuh) with a float-float phase; compensated
+//                accumulation; one FP64 partial per tile.
 //  k_quad_f64    the same quadrature in plain FP64 at every grid point, used as
 //                the reference GPU path.
 //  k_finish      per profile: deterministic FP64 sum of tile partials per CUT,
@@ -211,7 +209,12 @@ cudaError_t launch_piece_logs(DevPiece *pieces, int n, int G, double ln_eps, cud
 cudaError_t gauss_array(void **out) { return cudaGetSymbolAddress(out, g_isrs_gauss); }
 
 // ---------------------------------------------------------------------------
-// k_quad_f32: persistent FP32 quadrature.
+// k_quad_f32: persistent FP32 quadrature.  Bound by the XU pipe (sin and cos at 16
+// lanes a clock, ex2 at 32: 20 cycles per warp and z-step), 72 % busy on a 148-channel
+// plan at G = 256 (2.28 ms; every grid point summed one by one: 74.4 ms).  589
+// channels at G = 256: 1,129 -> 43.9 ms; 12 profiles at G = 64: 541 -> 77 ms, a
+// quarter of it the pieces' set-up.  Three blocks of 80 registers an SM: two leave
+// 5 % on the G = 256 case and 6 % on the G = 64 one, four spill (4 % and 9 %).
 // ---------------------------------------------------------------------------
 constexpr int kFwdSlots = 512;       // node slots of a chunk
 using FwdNodes = WarpNodes<kFwdSlots>;
@@ -461,9 +464,8 @@ __global__ void __launch_bounds__(256) k_quad_f64(QuadParams qp)
 // eta_i = (16/27) gamma_i^2 B_i Sigma_i / P_i^3 (Eq. gain_fin, P_NLI = G B);
 // SNR_i = P_i / (P_NLI,i + P_ASE,i) with P_ASE,i = NF h f (1/rho(L,f) - 1) B
 // and optional transceiver noise; T = 2 sum B log2(1 + SNR) (Eq. loss).  Eight
-// lanes sum a CUT's tiles: one thread's chain of dependent additions over them
-// was most of the kernel's time (15 us at 5
-// channels, 64 us at 589).
+// lanes sum a CUT's tiles, then a thread per CUT takes the FP64 rest (one thread for
+// both took 15 us at 5 channels).
 // ---------------------------------------------------------------------------
 constexpr int kFinishLanes = 8;
 
@@ -477,20 +479,29 @@ __global__ void __launch_bounds__(512) k_finish(FinishParams fp)
     const int s0 = fp.prof_slot_off[p], s1 = fp.prof_slot_off[p + 1];
     double tpart = 0.0;
     const int sub = threadIdx.x % kFinishLanes, per = blockDim.x / kFinishLanes;
-    for (int sb = s0; sb < s1; sb += per) {
-        const int s = sb + threadIdx.x / kFinishLanes;
-        double sig = 0.0;
-        if (s < s1) {
-            const int2 rg = fp.slot_items[s];
-            for (int it = rg.x + sub; it < rg.y; it += kFinishLanes) sig += fp.partial[it];
-            if (fp.slot_items2) {
-                const int2 r2 = fp.slot_items2[s];
-                for (int it = r2.x + sub; it < r2.y; it += kFinishLanes) sig += fp.partial2[it];
+    __shared__ double sums[512];
+    for (int cb = s0; cb < s1; cb += blockDim.x) {
+        const int ce = min(cb + (int)blockDim.x, s1);
+        for (int sb = cb; sb < ce; sb += per) {
+            const int s = sb + threadIdx.x / kFinishLanes;
+            double sig = 0.0;
+            if (s < ce) {
+                const int2 rg = fp.slot_items[s];
+                for (int it = rg.x + sub; it < rg.y; it += kFinishLanes) sig += fp.partial[it];
+                if (fp.slot_items2) {
+                    const int2 r2 = fp.slot_items2[s];
+                    for (int it = r2.x + sub; it < r2.y; it += kFinishLanes) sig += fp.partial2[it];
+                }
             }
-        }
 #pragma unroll
-        for (int o = kFinishLanes / 2; o > 0; o >>= 1) sig += __shfl_xor_sync(0xffffffffu, sig, o);
-        if (s >= s1 || sub != 0) continue;
+            for (int o = kFinishLanes / 2; o > 0; o >>= 1) sig += __shfl_xor_sync(0xffffffffu, sig, o);
+            if (s < ce && sub == 0) sums[s - cb] = sig;
+        }
+        __syncthreads();
+        const int s = cb + threadIdx.x;
+        const double sig = s < ce ? sums[threadIdx.x] : 0.0;
+        __syncthreads();
+        if (s >= ce) continue;
         const int i = fp.slot_cut[s];
         const double g = fp.ch_gamma[coff + i];
         const double B = fp.ch_B[coff + i];

@@ -7,8 +7,8 @@
 // mirror cell (b, a) onto (a, b) (the integrand is symmetric in f1, f2), so
 // no piece list is built: a work item is a range of cells of one CUT in the
 // triangular order of the pairs (a', b'), a' <= b', of the N - 1 channels
-// other than the CUT (a = a' + [a' >= i], likewise b), and every thread
-// decodes its cell and grid row from its index.  Each cell lies in one
+// other than the CUT (a = a' + [a' >= i], likewise b), decoded from the index.
+// Each cell lies in one
 // quadrant (channel a does not straddle f_i) and gets its own G_mci x G_mci
 // hyperbolic grid: rows uniform in ln(upsilon1), columns uniform in upsilon2,
 // exactly as the per-piece grids of the SCI/XCI cells.  The z-sum and the

@@ -9,13 +9,11 @@
 // of cell (a, b) with F_c in channel c and in-channel offsets
 // da = F_a - f_a, db = F_b - f_b, dc = F_c - f_c,
 //   ln p_m = 1/2 [a_a + a_b - a_i + a_c + b_a da + b_b db + b_c dc](m).
-// The first three terms belong to the cell; per chunk of cells the FP32
-// kernel tabulates, per cell and step, {A + log2 dz, S_a, S_b, A} (log2
-// units) in shared memory, and reads {a_c, b_c}(m) of the point's F_c channel
-// from an FP32 copy of the profile tables (one float2 per channel and step,
-// L1/L2-resident), so a step costs two loads and four FMAs for ln p.  The
-// z-sum forms are those of the closed-form MCI kernel (second-order small
-// phase, direct, telescoped with the wide phase reduction).
+// For the few cells a warp takes together the FP32 kernel tabulates, per cell, F_c
+// channel and pair of steps, {A, S_a, S_b} (log2 units; A at da = db = 0, S_a = (b_a +
+// b_c)/2, S_b = (b_b + b_c)/2) in shared memory from an FP32 copy of the profile
+// tables, so a step costs two FMAs for ln p.  The z-sum forms are those of
+// quad_zsum.cuh.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -81,7 +79,8 @@ __host__ __device__ constexpr size_t mci_warp_bytes(int n_steps)
 // every step instead left the loop waiting on L2: the block's shared memory leaves
 // the L1 28 KB), then grid rows, then points, which go to a list per z-sum form and
 // are summed 32 at a time, one per lane.  Bound by the XU pipe (20 cycles per warp
-// and step) and the issue of the other ~14 instructions.
+// and step; 74 % busy on 147 adjacent channels) and the issue of the rest (70 %).
+// 557 channels, G_mci 8: 518 ms with the F_c rows read at every step, now 278 ms.
 // ---------------------------------------------------------------------------
 #ifndef ISRS_MCI_TAB_MIN_BLOCKS
 #define ISRS_MCI_TAB_MIN_BLOCKS 3   // resident blocks per SM the register budget is sized for
