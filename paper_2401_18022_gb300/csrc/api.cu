@@ -846,10 +846,10 @@ cudaError_t gauss_rules(int dev, cudaStream_t st, const float2 **out)
 // Work tiles of a plan: `chunk` pieces per tile, each piece shared by `parts`
 // tiles.  A warp takes a tile (FP64: a block), so a small plan wants many: below
 // ~16,000 pieces every piece is its own tile, and below that its nodes are
-// shared by up to 8 (a 5-channel plan has 90 pieces for 4,864 resident warps;
+// shared by up to 8 (a 5-channel plan has 90 pieces for 3,648 resident warps;
 // every share repeats the piece's set-up, which only pays on an idle chip: at G 64 4
 // shares take 40 us forward and 57 us with the adjoint, 8 take 35 and 45, 16 take 41
-// and 46).  A large plan takes up to 32 pieces a tile, ~8 tiles per resident warp, so that a
+// and 46).  A large plan takes up to 32 pieces a tile, ~10 tiles per resident warp, so that a
 // tile's fixed cost (queue, bucket rows) stays small and the last wave short.
 // The split depends on the plan and grid alone, never on the CUT list or the
 // number of profiles, so a CUT's tiles and the order of its sum are the same in
