@@ -92,10 +92,6 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
 
     walk_tables<K2>(qp, ze, zd);
     for (int t = lane; t < 2 * K2 * 16; t += 32) w.B[t] = make_double2(0.0, 0.0);
-    const float c3 = (float)(kPi * qp.beta3);
-    const float c4 = (float)(2.0 * kPi * kPi / 3.0 * qp.beta4);
-    const float b2 = (float)qp.beta2;
-    const float m4pi2 = (float)(-4.0 * kPi * kPi);
     const float phi_direct = 3.14159265f / qp.dz_max;
     const float phi_small = 0.02f / qp.L;
     const float eps = (float)qp.eps_v1;
@@ -139,7 +135,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
         __syncthreads();
         float *myV = sV + warp * nmax;
         const float fi = (float)qp.ch_frel[coff + i];
-        const float three_fi2 = 3.0f * fi * fi;
+        const MciPhase ph = {(float)qp.beta2, (float)qp.c3, (float)qp.c4, fi};
         const float ha_i = ha[i];
         float sum = 0.0f, comp = 0.0f;
         f32x2 R[K2], Rp[K2];
@@ -227,24 +223,11 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
                     const int4 cl = cr.cell[v0 + tl];
                     a = cl.x;
                     b = cl.y;
-                    const float mult = a == b ? 1.0f : 2.0f;
                     const float ra = rel[a], rb = rel[b];
-                    const float s1 = ra > 0.0f ? 1.0f : -1.0f, s2 = rb > 0.0f ? 1.0f : -1.0f;
-                    const float xlo = fabsf(ra) - hb[a], xhi = fabsf(ra) + hb[a];
-                    const float ylo = fabsf(rb) - hb[b], yhi = fabsf(rb) + hb[b];
-                    const float u1hi = xhi * yhi;
-                    const float llo = logf(fmaxf(xlo * ylo, eps * u1hi));
-                    const float ds = (logf(u1hi) - llo) / (float)G;
-                    const float u1 = expf(fmaf((float)r + 0.5f, ds, llo));
-                    const float ymin = fmaxf(ylo, u1 / xhi), ymax = fminf(yhi, u1 / xlo);
-                    if (ymax > ymin) {
-                        const float du2 = log1pf((ymax - ymin) / ymin) / (float)G;
-                        const float yc = sqrtf(ymin * ymax), xc = u1 / yc;
-                        const float wt = u1 * ds * du2 * mult;
-                        const float d = ((float)j + 0.5f - 0.5f * (float)G) * du2;
-                        const float e = expf(d);
-                        const float f1 = s1 * (xc * e), f2 = s2 * (yc * __frcp_rn(e));
-                        const float u = f1 + f2;
+                    const float4 row = mci_row(fabsf(ra), fabsf(rb), hb[a], hb[b], eps, G, r, a == b ? 1.0f : 2.0f);
+                    if (row.w != 0.0f) {
+                        const float2 f = mci_point(row, ra, rb, j, G);
+                        const float u = f.x + f.y;
                         for (int x = cl.z; x <= cl.w; ++x)
                             if (rel[x] - hb[x] <= u && u < rel[x] + hb[x]) c = x;
                         if (c >= 0) {
@@ -252,10 +235,8 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
                             if (W != 0.0f) {
                                 at = ha[a] + ha[b] - ha_i + ha[c];
                                 Fc = fi + u;
-                                const float br = b2 + c3 * (u + 2.0f * fi) +
-                                                 c4 * (f1 * f1 + 1.5f * f1 * f2 + 3.0f * fi * u + f2 * f2 + three_fi2);
-                                phi = m4pi2 * f1 * f2 * br;
-                                wwa = wt * W * array_factor_f(phi, qp);
+                                phi = ph.at<true>(f.x, f.y);
+                                wwa = row.w * W * array_factor_f(phi, qp);
                                 cls = fabsf(phi) <= phi_direct ? 0 : 1;
                             }
                         }

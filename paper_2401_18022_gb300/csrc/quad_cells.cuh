@@ -96,15 +96,26 @@ __device__ __forceinline__ float2 mci_point(const float4 &o, float sa, float sb,
     return make_float2(s1 * (o.x * ex), s2 * (o.y * __frcp_rn(ex)));
 }
 
-// Coefficients of phi (Eq. phi) at the CUT's frequency
+// phi (Eq. phi) of a point from its FP32 f1 and f2.  The bracket is a small
+// difference of large terms near the zero-dispersion wavelength: the rounding of a far
+// cell's phi there is radians of |phi| L, the phase is a sample of its rounding, and a
+// multiply-add fused elsewhere moved eta by up to 2.1e-4 (404 channels, 10 spans) and
+// by 7e-5 between the forward and the adjoint of one plan.  So every operation is
+// written with its rounding, in one place for all kernels; what a compiler makes of the
+// code around it no longer shows in the result.  Fused: the last term of the sum as a
+// multiply-add (closed-form profile) or rounded by itself (Raman ODE): the orders these
+// results have always had.
 struct MciPhase {
-    float b2, c3, c4, fi, three_fi2;
+    float b2, c3, c4, fi;
+    template <bool Fused>
     __device__ __forceinline__ float at(float f1, float f2) const
     {
-        const float u = f1 + f2;
-        const float br = b2 + c3 * (u + 2.0f * fi) +
-                         c4 * (f1 * f1 + 1.5f * f1 * f2 + 3.0f * fi * u + f2 * f2 + three_fi2);
-        return -39.4784176f * f1 * f2 * br;
+        const float u = __fadd_rn(f1, f2), fi3 = __fmul_rn(3.0f, fi);
+        float q = __fmaf_rn(f1, f1, __fmul_rn(__fmul_rn(1.5f, f1), f2));
+        q = __fmaf_rn(f2, f2, __fmaf_rn(fi3, u, q));
+        q = Fused ? __fmaf_rn(fi3, fi, q) : __fadd_rn(q, __fmul_rn(fi3, fi));
+        const float br = __fmaf_rn(c4, q, __fmaf_rn(c3, __fmaf_rn(2.0f, fi, u), b2));
+        return __fmul_rn(__fmul_rn(__fmul_rn(-39.4784176f, f1), f2), br);     // -4 pi^2 f1 f2
     }
 };
 

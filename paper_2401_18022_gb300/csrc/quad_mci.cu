@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32(QuadParams qp)
         __syncthreads();
         const float *pd = qp.pd_f + qp.prof_ch_off[item.prof];     // [n] P/B
         const float fi = (float)qp.ch_frel[coff + i], ha_i = ha[i];
-        const MciPhase ph = {(float)qp.beta2, (float)qp.c3, (float)qp.c4, fi, 3.0f * fi * fi};
+        const MciPhase ph = {(float)qp.beta2, (float)qp.c3, (float)qp.c4, fi};
         float sum = 0.0f, comp = 0.0f;
         int nl[2] = {0, 0};                              // list lengths (direct, telescoped)
         // one list's first 32 points, one per lane; of what is left at the item's end,
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(256, 3) k_quad_mci_f32(QuadParams qp)
                             for (int c = cl.z; c <= cl.w; ++c)
                                 if (rel[c] - hb[c] <= pt.y && pt.y < rel[c] + hb[c]) ci = c;
                             if (ci >= 0) {
-                                pt.x = ph.at(f.x, f.y);
+                                pt.x = ph.at<true>(f.x, f.y);
                                 pt.z = (ha[cl.x] + ha[cl.y] - ha_i) + ha[ci];
                                 pt.w = o.w * pd[ci];
                                 if (pt.w != 0.0f) cls = fabsf(pt.x) <= phi_direct ? 0 : 1;

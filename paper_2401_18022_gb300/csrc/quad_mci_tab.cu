@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_t
         const float4 *T = qp.ab_f + (size_t)poff * M2;   // this profile's channel rows
         const float *pd = qp.pd_f + poff;                // [n] P/B
         const float fi = (float)qp.ch_frel[coff + i];
-        const MciPhase ph = {(float)qp.beta2, (float)qp.c3, (float)qp.c4, fi, 3.0f * fi * fi};
+        const MciPhase ph = {(float)qp.beta2, (float)qp.c3, (float)qp.c4, fi};
         float sum = 0.0f, comp = 0.0f;
         int nl[2] = {0, 0};                              // list lengths (direct, telescoped)
         // one list's first 32 points, one per lane; of what is left at a group's end, 32 /
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_t
                                 da = f.x - ra;
                                 db = f.y - rb;
                                 un = cl.w + (ci - cl.y);
-                                phi = ph.at(f.x, f.y);
+                                phi = ph.at<false>(f.x, f.y);
                                 if (W != 0.0f) cls = fabsf(phi) <= phi_direct ? 0 : 1;
                             }
                         }
