@@ -66,7 +66,8 @@ constexpr int kOdeMaxWarps = kMaxRamanCh / 32;
 // 32 channels; the in-warp inclusive prefixes stay in their block's shared
 // memory (read remotely at the window's two ends), the warps' totals are pushed
 // to every block.  Double-buffered, so one cluster barrier per call suffices: a
-// buffer is written again two calls later, after the barrier in between.
+// buffer is written again two calls later, after the barrier in between.  (The first
+// stores wait for the cluster at the end of ode_lane.)
 struct OdeWindow {
     double2 x[2][2][32 * kOdeMaxWarps / 8];      // [buffer][pair][channel of the block]
     double2 tot[2][2][kOdeMaxWarps];             // [buffer][pair][warp of the plan]
@@ -112,6 +113,9 @@ __device__ __forceinline__ OdeLane ode_lane(cg::cluster_group &cl, OdeWindow &wi
     L.alpha = rp.ch_alpha[coff + i];
     L.sc = rp.ch_scale[coff + i];
     L.P0 = L.live ? rp.P[poff + i] : 0.0;
+    // the first ode_window stores into every block of the cluster: only once all of
+    // them run is their shared memory theirs
+    if (!L.one) cl.sync();
     return L;
 }
 
