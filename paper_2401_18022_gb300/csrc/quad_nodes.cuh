@@ -421,8 +421,15 @@ __device__ __forceinline__ int row_whole(const PieceGeo &g, const NodeRow &o, in
 // The blocks of low rows: the rows [0, R1) whose columns all lie in one
 // candidate, with one set of limits and |phi| band <= kBlkPhiL, cut at |phi|
 // band = kBlkPhiLow and into parts of kGaussMaxN rows.  Along t in [-1, 1] over
-// N rows upsilon1 (so the weight and phi) is exp-like with D = N ds / 2, and the
-// phase swings by at most |phi| band D.  Whole warp; writes ns.blk.
+// N rows upsilon1 (so the weight and phi) is exp-like with D = N ds / 2.  phi is
+// upsilon1 times the bracket of Eq. phi, and the bracket may vanish towards the block's
+// last row (the (+,-) quadrant of a CUT near the zero-dispersion wavelength, where rows
+// shrink to f1 = -f2): neither |phi| there nor the largest one bounds the swing then.
+// q_last, the block's largest bracket at the last row's upsilon1, does: |phi| band of
+// row r is below q_last e^{-(R1 - 1 - r) ds} and swings by at most q_last D.  (Rows of
+// the CUT's own cell at 1310 nm, 96 GBaud, G 256, 20 spans: with |phi| of the last row
+// 1.9e-5 of Sigma, with the largest 6.7e-7, with q_last 2.6e-8, 739 / 759 / 766 nodes.)
+// Whole warp; writes ns.blk.
 struct PieceBlocks {
     int units;                  // rows of the rules, all blocks
     int R1, nblk, cand;         // rows covered, blocks, their F_c candidate
@@ -435,7 +442,8 @@ __device__ __forceinline__ PieceBlocks row_blocks(WarpNodes<Cap> &ns, const floa
     int &R1 = pb.R1, &nblk = pb.nblk, &cand = pb.cand, &units = pb.units;
     const PieceGeo &g = ns.geo;
     const int lane = threadIdx.x & 31;
-    float ph_last = 0.0f;
+    float q_max = 0.0f;              // largest |phi| band at the middle row's upsilon1
+    const float k_mid = 0.5f * (float)G;
     // candidate and limits of row r (-1: not in one candidate), |phi| band
     const auto test = [&](int r, float &ph) {
         NodeRow o;
@@ -472,14 +480,17 @@ __device__ __forceinline__ PieceBlocks row_blocks(WarpNodes<Cap> &ns, const floa
         } else {
             R1 += n;
         }
-        if (n > 0) ph_last = __shfl_sync(0xffffffffu, ph, n - 1);
+        // (between two rows tested the bracket lies between theirs)
+        const float q = lane < n ? ph * ex2_approx(((float)(G - r) - 0.5f - k_mid) * g.ds2.x) : 0.0f;
+        q_max = fmaxf(q_max, __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(q))));
         if (!coarse && n < 32) break;
         r0 = R1;
     }
     cand = key0 >> 2;
+    const float q_last = q_max * ex2_approx((k_mid - (float)(G - R1) - 0.5f) * g.ds2.x);
     // rows from the block's top down to |phi| band = kBlkPhiLow
-    int top = ph_last > kBlkPhiLow ? (int)ceilf(__fdividef(__logf(ph_last / kBlkPhiLow), g.ds)) : 0;
-    top = min(top, R1);
+    const float tops = q_last > kBlkPhiLow ? ceilf(__fdividef(__logf(q_last / kBlkPhiLow), g.ds)) : 0.0f;
+    const int top = (int)fminf(tops, (float)R1);
 #pragma unroll 1
     for (int low = 1; low >= 0; --low) {
         const int n_rows = low ? R1 - top : top, parts = (n_rows + kGaussMaxN - 1) / kGaussMaxN;
@@ -487,7 +498,7 @@ __device__ __forceinline__ PieceBlocks row_blocks(WarpNodes<Cap> &ns, const floa
         for (int s = 0; s < parts; ++s) {
             const int a = n_rows * s / parts, b = n_rows * (s + 1) / parts, N = b - a;
             const float D = 0.5f * (float)N * g.ds;
-            const int need = gauss_need(fminf(ph_last, low ? kBlkPhiLow : kBlkPhiL) * D, D);
+            const int need = gauss_need((low ? fminf(q_last, kBlkPhiLow) : q_last) * D, D);
             const int n = need <= kGaussMaxNodes ? gauss_nodes(gauss_pick(need)) : N;
             if (lane == 0)
                 ns.blk[nblk] = RowBlock{units, (low ? 0 : R1 - top) + a, N,
