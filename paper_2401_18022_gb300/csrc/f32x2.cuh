@@ -57,13 +57,15 @@ __device__ __forceinline__ void sincos_turn2(f32x2 x, float &s0, float &c0, floa
 
 // As rev_fraction and phasor_rev_ff (quad_common.cuh): the fraction of (phi +
 // phi_lo)(hi + lo) in revolutions; nphi =
-// -phi.  Form 0: as written.  1: phi_lo = 0 and phases up to 2^29 revolutions, rounded
-// twice.  2: phi_lo = 0, up to 2^20 revolutions.
+// -phi.  Form 0: as written.  1: phi_lo = 0 and phases up to 2^30 revolutions, rounded
+// twice, first to what `magic` (turn_magic) leaves.  2: phi_lo = 0, up to 2^20 revolutions.
 template <int Form>
-__device__ __forceinline__ f32x2 rev_fraction2(f32x2 phi, f32x2 nphi, f32x2 phi_lo, f32x2 hi, f32x2 lo)
+__device__ __forceinline__ f32x2 rev_fraction2(f32x2 phi, f32x2 nphi, f32x2 phi_lo, f32x2 hi, f32x2 lo,
+                                               float magic = 12582912.0f)
 {
     const f32x2 mg = dup2(12582912.0f), nm = dup2(-12582912.0f);
-    f32x2 fr = fma2(phi, hi, add2(fma2(nphi, hi, mg), nm));
+    f32x2 fr = Form == 1 ? fma2(phi, hi, add2(fma2(nphi, hi, dup2(magic)), dup2(-magic)))
+                         : fma2(phi, hi, add2(fma2(nphi, hi, mg), nm));
     fr = fma2(phi, lo, fr);
     if constexpr (Form == 1) fr = add2(fr, add2(fma2(fr, dup2(-1.0f), mg), nm));
     if constexpr (Form == 0) fr = fma2(phi_lo, hi, fr);

@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
                 f32x2 tr[K2], ti[K2];
                 float sr, si, sq = p + half < cnt ? v.x : 0.0f;
                 if (tele) {
-                    walk_tele<K2, true>(ze + l16, l16, v.y, 0.0f, lp, tr, ti, sr, si);
+                    walk_tele<K2, true>(ze + l16, l16, v.y, 0.0f, lp, tr, ti, sr, si, turn_magic(v.y * qp.Lrev_hi));
                     sq *= __fdividef(1.0f, v.y * v.y);
                 } else {
                     walk_direct<K2>(zd + l16, v.y, lp, tr, ti, sr, si);
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
                                 at = ha[a] + ha[b] - ha_i + ha[c];
                                 Fc = fi + u;
                                 phi = ph.at<true>(f.x, f.y);
-                                wwa = row.w * W * array_factor_f(phi, qp);
+                                wwa = row.w * W * array_factor_f<true>(phi, qp);
                                 cls = fabsf(phi) <= phi_direct ? 0 : 1;
                             }
                         }

@@ -171,11 +171,30 @@ __device__ __forceinline__ void piece_consts(const QuadParams &qp, const DevPiec
     }
 }
 
-// e^{j phi z}: the phase (phi + phi_lo)(hi + lo) in revolutions, |.| < 2^22
+// Beyond 2^21 revolutions (the MCI cells) the constant 1.5 2^23 is too small: past 2^22
+// the sum with it leaves the binade whose spacing is 1, and "the nearest integer" becomes a
+// half-integer.  With 1.5 2^31 it is a multiple of 256 (up to 2^30 revolutions), and a
+// second rounding takes the rest.
+constexpr float kTurnMagic = 12582912.0f, kTurnMagicWide = 3221225472.0f;
+constexpr float kTurnsWide = 2097152.0f;
+__device__ __forceinline__ float turn_magic(float revs)
+{
+    return fabsf(revs) > kTurnsWide ? kTurnMagicWide : kTurnMagic;
+}
+
+// e^{j phi z}: the phase (phi + phi_lo)(hi + lo) in revolutions, |.| < 2^22 (Wide: 2^30)
+template <bool Wide = false>
 __device__ __forceinline__ void phasor_rev_ff(float phi, float hi, float lo, float &sn, float &cs,
                                               float phi_lo = 0.0f)
 {
-    const float fr = fmaf(phi_lo, hi, fmaf(phi, lo, rev_fraction(phi, hi)));
+    float fr;
+    if constexpr (Wide) {
+        const float mg = turn_magic(phi * hi);
+        fr = fmaf(phi, lo, __fmaf_rn(phi, hi, __fadd_rn(__fmaf_rn(-phi, hi, mg), -mg)));
+        fr = rev_fraction(fr, 1.0f);
+    } else {
+        fr = fmaf(phi_lo, hi, fmaf(phi, lo, rev_fraction(phi, hi)));
+    }
     __sincosf(fr * 6.283185307179586f, &sn, &cs);
 }
 
@@ -251,12 +270,13 @@ __device__ __forceinline__ double zsum_f64(double phi, double phi_direct, const 
 
 // Phased-array factor of n identical spans (Eq. new_gn_model with
 // L-tilde_k = (k-1) L): |sum_{k<n} e^{j k phi L}|^2, by rotation from the
-// float-float phase phi L / 2pi.
+// float-float phase phi L / 2pi (Wide: as phasor_rev_ff).
+template <bool Wide = false>
 __device__ __forceinline__ float array_factor_f(float phi, const QuadParams &qp, float phi_lo = 0.0f)
 {
     if (qp.n_spans <= 1) return 1.0f;
     float sn, cs;
-    phasor_rev_ff(phi, qp.Lrev_hi, qp.Lrev_lo, sn, cs, phi_lo);
+    phasor_rev_ff<Wide>(phi, qp.Lrev_hi, qp.Lrev_lo, sn, cs, phi_lo);
     float sr = 0.0f, si = 0.0f, zr = 1.0f, zi = 0.0f;
     for (int k = 0; k < qp.n_spans; ++k) {
         sr += zr;

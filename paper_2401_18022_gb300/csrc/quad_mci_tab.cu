@@ -161,14 +161,14 @@ __global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_t
                 float2 S;
                 if (f == 0) S = zsum_direct_part(v.x, lp, zD, k0, k1);
                 else if (__any_sync(0xffffffffu, fabsf(v.x) > phi_wide))
-                    S = zsum_tele_part<1>(v.x, 0.0f, lp, eB, k0, k1);
+                    S = zsum_tele_part<1>(v.x, 0.0f, lp, eB, k0, k1, turn_magic(v.x * qp.Lrev_hi));
                 else S = zsum_tele_part<2>(v.x, 0.0f, lp, eB, k0, k1);
                 for (int o = (1 << lg) >> 1; o > 0; o >>= 1) {
                     S.x += __shfl_xor_sync(0xffffffffu, S.x, o);
                     S.y += __shfl_xor_sync(0xffffffffu, S.y, o);
                 }
                 const float S2 = S.x * S.x + S.y * S.y, wt = pt < cnt && sub == 0 ? v.w : 0.0f;
-                const float y = wt * (f ? __fdividef(S2, v.x * v.x) : S2) * array_factor_f(v.x, qp) - comp;
+                const float y = wt * (f ? __fdividef(S2, v.x * v.x) : S2) * array_factor_f<true>(v.x, qp) - comp;
                 const float t = sum + y;
                 comp = (t - sum) - y;
                 sum = t;

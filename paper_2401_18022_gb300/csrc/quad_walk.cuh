@@ -101,10 +101,11 @@ __device__ __forceinline__ void walk_direct(const float4 *zd, float ph, const LP
 
 // Telescoped: terms p_m (E_{m+1} - E_m), E_e = e^{j phi z_e}, and their sum U,
 // |S|^2 = |U|^2 / phi^2 (ze offset by the lane; phi float-float, or Wide: up to
-// 2^29 revolutions).
+// 2^30 revolutions, magic by turn_magic).
 template <int K2, bool Wide, typename LP>
 __device__ __forceinline__ void walk_tele(const float4 *ze, int l16, float ph, float ph_lo, const LP &lp,
-                                          f32x2 (&tr)[K2], f32x2 (&ti)[K2], float &ur, float &ui)
+                                          f32x2 (&tr)[K2], f32x2 (&ti)[K2], float &ur, float &ui,
+                                          float magic = kTurnMagic)
 {
     const f32x2 p2 = dup2(ph), np2 = dup2(-ph), pl2 = dup2(ph_lo);
     float Er = 0.0f, Ei = 0.0f, f0r = 0.0f, f0i = 0.0f, f1r = 0.0f, f1i = 0.0f;
@@ -113,7 +114,7 @@ __device__ __forceinline__ void walk_tele(const float4 *ze, int l16, float ph, f
     for (int k = 0; k < K2; ++k) {
         const float4 e = ze[k * 16];
         float s0, c0, s1, c1;
-        sincos_turn2(rev_fraction2<Wide>(p2, np2, pl2, pack2(e.x, e.y), pack2(e.z, e.w)), s0, c0, s1, c1);
+        sincos_turn2(rev_fraction2<Wide>(p2, np2, pl2, pack2(e.x, e.y), pack2(e.z, e.w), magic), s0, c0, s1, c1);
         const f32x2 p = ex2_pair(lp(k));
         if (k == 0) {
             p0 = p;

@@ -66,21 +66,21 @@ __device__ __forceinline__ float zsum_direct_n(float phi, const LP &lp, const fl
 // sum (p_m - p_{m-1}) E_m: two differences per pair of steps instead of four.
 template <int Form, typename LP>
 __device__ __forceinline__ float2 zsum_tele_part(float phi, float phi_lo, const LP &lp, const float4 *eB, int k0,
-                                                 int k1)
+                                                 int k1, float magic = kTurnMagic)
 {
     const f32x2 ph = dup2(phi), nph = dup2(-phi), pl = dup2(phi_lo);
     float Er = 1.0f, Ei = 0.0f, pp = 0.0f;
     if (k0 > 0) {                        // phasor at the edge before
         const float4 e = eB[k0 - 1];
         float s0, c0;
-        sincos_turn2(rev_fraction2<Form>(ph, nph, pl, pack2(e.x, e.y), pack2(e.z, e.w)), s0, c0, Ei, Er);
+        sincos_turn2(rev_fraction2<Form>(ph, nph, pl, pack2(e.x, e.y), pack2(e.z, e.w), magic), s0, c0, Ei, Er);
     }
     f32x2 Sr = dup2(0.0f), Si = dup2(0.0f);
 #pragma unroll 4
     for (int k = k0; k < k1; ++k) {
         const float4 e = eB[k];
         float s0, c0, s1, c1, l0, l1;
-        sincos_turn2(rev_fraction2<Form>(ph, nph, pl, pack2(e.x, e.y), pack2(e.z, e.w)), s0, c0, s1, c1);
+        sincos_turn2(rev_fraction2<Form>(ph, nph, pl, pack2(e.x, e.y), pack2(e.z, e.w), magic), s0, c0, s1, c1);
         unpack2(lp(k), l0, l1);
         const float p0 = ex2_approx(l0), p1 = ex2_approx(l1);
         const f32x2 d = pack2(pp - p0, p0 - p1);
