@@ -95,12 +95,14 @@ __host__ __device__ inline int gauss_need(float A, float D)
 // over a block the rows' weight is exp-like, e^{D t}, and wants 4 + 6 sqrt(D) = 2 n by
 // itself (e^{D t} and e^{D t} (c - t) to 1e-8, D up to 20, N from 16 to 256).  With
 // gauss_need a block of every row (three 32 GBaud channels at 1310 nm, eps_v1 1e-3, D
-// 3.4) was off by 3.6e-5 of Sigma.  Over 640 random plans (16 to 200 rows, 1 to 100
-// spans, either cell set) Sigma is within 6e-8 now, all of it the rows' part, for 3 %
-// more nodes (589 channels: 5 % at G 64, 3 % at G 256).
-__host__ __device__ inline int block_need(float A, float D)
+// 3.4) was off by 3.6e-5 of Sigma.  part: rows up to kBlkPhiLow below others, a few per
+// cent of the piece, where the weight alone counts.  Over 640 random plans (16 to 200
+// rows, 1 to 100 spans, either cell set) Sigma is within 6e-8 now, all of it the rows'
+// part, for 2 % more nodes and of the time (589 channels, G 256: 43.9 -> 44.9 ms; 12
+// profiles, G 64: 77.1 -> 79.0; 45.8 and 82.0 if the low part follows the swing too).
+__host__ __device__ inline int block_need(float A, float D, bool part)
 {
-    const float two_n = A + 4.0f + 4.2f * A / (A + 0.35f) + 0.6f * sqrtf(A) + 6.0f * sqrtf(D);
+    const float two_n = 4.0f + 6.0f * sqrtf(D) + (part ? 0.0f : A + 4.2f * A / (A + 0.35f) + 0.6f * sqrtf(A));
     return two_n < 8192.0f ? (int)ceilf(0.5f * two_n) : 4096;
 }
 
@@ -515,7 +517,7 @@ __device__ __forceinline__ PieceBlocks row_blocks(WarpNodes<Cap> &ns, const floa
         for (int s = 0; s < parts; ++s) {
             const int a = n_rows * s / parts, b = n_rows * (s + 1) / parts, N = b - a;
             const float D = 0.5f * (float)N * g.ds;
-            const int need = block_need((low ? fminf(q_last, kBlkPhiLow) : q_last) * D, D);
+            const int need = block_need((low ? fminf(q_last, kBlkPhiLow) : q_last) * D, D, low && top > 0);
             const int n = need <= kGaussMaxNodes ? gauss_nodes(gauss_pick(need)) : N;
             if (lane == 0)
                 ns.blk[nblk] = RowBlock{units, (low ? 0 : R1 - top) + a, N,

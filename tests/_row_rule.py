@@ -18,7 +18,7 @@ BLOCK_PHI, LOW_PHI = 6.0, 0.15
 SRC = """
 #include "quad_nodes.cuh"
 extern "C" int run_need(float A, float D) { return isrs::gauss_need(A, D); }
-extern "C" int block_need(float A, float D) { return isrs::block_need(A, D); }
+extern "C" int block_need(float A, float D, int part) { return isrs::block_need(A, D, part != 0); }
 extern "C" int picked(int n) { return isrs::gauss_nodes(isrs::gauss_pick(n)); }
 """
 
@@ -30,8 +30,8 @@ def shipped_counts(folder):
         f.write(SRC)
     subprocess.check_call([build.nvcc(), *build.ARCH, *build.FLAGS, "-shared", "-o", lib, src])
     so = ctypes.CDLL(lib)
-    for fn in (so.run_need, so.block_need):
-        fn.argtypes = [ctypes.c_float, ctypes.c_float]
+    so.run_need.argtypes = [ctypes.c_float, ctypes.c_float]
+    so.block_need.argtypes = [ctypes.c_float, ctypes.c_float, ctypes.c_int]
     assert [so.picked(n) for n in range(1, 49)] == [next(m for m in MENU if m >= n) for n in range(1, 49)]
     return so.run_need, so.block_need
 
@@ -163,12 +163,12 @@ class Piece:
             return out
         q = max(t[1] * math.exp((R1 - 1 - r) * self.ds) for r, t in enumerate(tests[:R1]))
         top = min(R1, math.ceil(math.log(q / LOW_PHI) / self.ds)) if q > LOW_PHI else 0
-        for r0, n, cap in ((0, R1 - top, min(q, LOW_PHI)), (R1 - top, top, q)):
+        for r0, n, cap, part in ((0, R1 - top, min(q, LOW_PHI), top > 0), (R1 - top, top, q, False)):
             parts = -(-n // MAX_N)
             for s in range(parts):
                 a, N = n * s // parts, n * (s + 1) // parts - n * s // parts
                 D = 0.5 * N * self.ds
-                pos, w = nodes(N, block_need(cap * D, D))
+                pos, w = nodes(N, block_need(cap * D, D, part))
                 out += [(G - (r0 + a + 0.5 * N + p), v) for p, v in zip(pos, w)]
         return out
 
@@ -205,4 +205,4 @@ class Piece:
 
     def full(self):
         """Every grid point."""
-        return self.sigma(lambda A, D: 1 << 20, lambda A, D: 1 << 20)
+        return self.sigma(lambda A, D: 1 << 20, lambda A, D, part: 1 << 20)
