@@ -238,8 +238,9 @@ def run_gpu(args):
     value = (1 if split else world) * n_grid * args.steps / t_total
 
     quad_ms = float(np.mean(quad_ms))
-    paths = eng.last_path_counts()          # z-sum forms of the last timed launch (both kernels count)
-    roof = _roofline(eng, wl, paths, n_eval, quad_ms, use_grad, clocks)
+    # z-sums of the last timed launch by form (both kernels count): every one is direct or telescoped
+    nodes = {"small": 0, **eng.last_node_counts()}
+    roof = _roofline(eng, wl, nodes, n_eval, quad_ms, use_grad, clocks)
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": 1e3 * t_total / args.steps, "higher_is_better": True,
             "scaling": "strong" if split else "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
@@ -306,7 +307,7 @@ FWD_CAPTURE = {"profile": "k_quad_f32_uwb148_every4th_G256.md", "points": 288070
 ISSUE_PER_CLK_PER_SM = 4         # one warp instruction per clock per SM sub-partition
 
 
-def _roofline(eng, wl, paths, n_eval, kernel_ms, use_grad, clocks):
+def _roofline(eng, wl, nodes, n_eval, kernel_ms, use_grad, clocks):
     """Roofline of the dominant kernel (k_quad_adj for the gradient step,
     k_quad_f32 for the SNR evaluation): plain ALU work, no tensor cores, not
     memory-bound.  Four fractions, each with its own peak:
@@ -316,8 +317,8 @@ def _roofline(eng, wl, paths, n_eval, kernel_ms, use_grad, clocks):
         measured by isrs_probe_alu_peaks in this run.  A row's points are
         summed from a few nodes, so this fraction exceeds 1: it measures the
         method's rate, not pipe use;
-      * sfu_executed: the same over the points of the direct and telescoped
-        range only (the path counts), again per point, not per node;
+      * sfu_executed: the SFU operations the kernel issues, 3 per step of every
+        node it sums (the launch's own node counts, direct and telescoped);
       * issue: executed warp instructions (ncu capture, scaled by evaluated
         points) over 152 SMs x 4 per clock at the SM clock sampled during the
         timed region: the limiter of these kernels;
@@ -327,7 +328,7 @@ def _roofline(eng, wl, paths, n_eval, kernel_ms, use_grad, clocks):
     n_steps = wl.n_edges - 1
     t = kernel_ms / 1e3
     sfu_alg = 3.0 * n_eval * n_steps
-    sfu_exec = 3.0 * n_steps * (paths["direct"] + paths["telescoped"])
+    sfu_exec = 3.0 * n_steps * (nodes["direct"] + nodes["telescoped"])
     cap = ADJ_CAPTURE if use_grad else FWD_CAPTURE
     scale = n_eval / cap["points"]
     warp_inst = cap["warp_inst"] * scale
@@ -336,7 +337,7 @@ def _roofline(eng, wl, paths, n_eval, kernel_ms, use_grad, clocks):
     issue_peak = N_SMS * ISSUE_PER_CLK_PER_SM * mhz * 1e6
     sfu_peak = peaks["sfu_ops_per_s"]
     fp32_peak = peaks["fp32_ops_per_s"]
-    tot_pts = max(1, sum(paths.values()))
+    tot = max(1, sum(nodes.values()))
     return {"bound": "alu", "unit": "Tops/s (SFU ops of the method: 3 per evaluated point-step)",
             "achieved": sfu_alg / t / 1e12, "peak": sfu_peak / 1e12, "frac": sfu_alg / t / sfu_peak,
             "traffic": cap["dram_bytes"] * scale,
@@ -351,7 +352,7 @@ def _roofline(eng, wl, paths, n_eval, kernel_ms, use_grad, clocks):
             "kernel": "k_quad_adj" if use_grad else "k_quad_f32", "kernel_ms": kernel_ms,
             "sfu_ops_per_launch": {"algorithmic": sfu_alg, "executed": sfu_exec},
             "warp_inst_per_launch": warp_inst,
-            "path_fraction": {k: v / tot_pts for k, v in paths.items()}}
+            "path_fraction": {k: v / tot for k, v in nodes.items()}}
 
 
 def _batched_record(eng, dev_index, reps: int = 1):

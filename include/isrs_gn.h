@@ -312,14 +312,20 @@ isrs_status isrs_last_kernel_ms(isrs_handle h, int which, float *ms);
  * possible).  Errors: INVALID_ARG (NULL). */
 isrs_status isrs_last_graph_replay(isrs_handle h, int *replayed);
 
-/* Grid points of the last FP32 quadrature launch (forward, or the fused
- * forward + adjoint of isrs_gn_grad) by the form its z-sum took (App. A,
- * Eq. slow_vary) by phase: counts[0] |phi| n_spans L <= 6 (low rows, also
- * summed across rows), counts[1] the other points of the direct form, counts[2]
- * telescoped form.  Each point counts once, also where a few nodes stand for
- * its row.  Synchronises the device.  Errors: INVALID_ARG (NULL, or
- * no launch yet), CUDA. */
+/* Grid points of the last FP32 quadrature launch by the form of their z-sum (App.
+ * A, Eq. slow_vary), low ones apart: counts[0] |phi| n_spans L <= 6 (the range of
+ * the rows that are also summed across rows), counts[1] direct, counts[2]
+ * telescoped.  Each point whose F_c lies in a channel counts once, a run of a row
+ * by its first node.  Counted: the forward of the pieces (also with the Raman-ODE
+ * profile) and the closed-form gradient with its MCI cells; not the forward of
+ * separate MCI cells nor the Raman-ODE gradient.  Synchronises the device.
+ * Errors: INVALID_ARG (NULL, or no launch yet), CUDA. */
 isrs_status isrs_last_path_counts(isrs_handle h, int64_t *counts);
+
+/* Z-sums of the same launch, counts[0] direct, counts[1] telescoped: the nodes
+ * that stood for the points of isrs_last_path_counts (each of n_edges - 1 steps,
+ * 3 special-function operations a step).  Errors as there. */
+isrs_status isrs_last_node_counts(isrs_handle h, int64_t *counts);
 
 /* Measured throughput of the ALU pipes that bound the quadrature kernels
  * (a measurement utility; the paper has no counterpart).  which = 0: the SFU

@@ -95,6 +95,8 @@ def load(build_if_missing: bool = True):
     lib.isrs_last_graph_replay.restype = ctypes.c_int
     lib.isrs_last_path_counts.argtypes = [vp, P(ctypes.c_int64)]
     lib.isrs_last_path_counts.restype = ctypes.c_int
+    lib.isrs_last_node_counts.argtypes = [vp, P(ctypes.c_int64)]
+    lib.isrs_last_node_counts.restype = ctypes.c_int
     lib.isrs_last_kernel_ms.argtypes = [vp, ctypes.c_int, ctypes.POINTER(ctypes.c_float)]
     lib.isrs_probe_alu_peaks.argtypes = [ctypes.c_int, ctypes.c_int, c_double_p, ctypes.POINTER(ctypes.c_float)]
     lib.isrs_probe_alu_peaks.restype = ctypes.c_int

@@ -158,6 +158,12 @@ class Engine:
         check(self.lib.isrs_last_path_counts(self.h, c), self.h)
         return {"small": c[0], "direct": c[1], "telescoped": c[2]}
 
+    def last_node_counts(self):
+        """Z-sums of the last FP32 launch per form: the nodes that stood for its points."""
+        c = (ctypes.c_int64 * 2)()
+        check(self.lib.isrs_last_node_counts(self.h, c), self.h)
+        return {"direct": c[0], "telescoped": c[1]}
+
     # ---- calls -----------------------------------------------------------
     def eta(self, wl, P=None, cuts: Optional[Sequence[int]] = None, precision: int = PREC_FP32,
             want_sigma: bool = True):

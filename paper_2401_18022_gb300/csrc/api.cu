@@ -1011,7 +1011,7 @@ isrs_status run_forward(isrs_handle h, const isrs_fibre *fb, Geom *g, int precis
             CK(launch_raman(raman_params(h, fb, g, keep_nodes), g->n_prof, g->max_plan_n, st));
         }
     }
-    if ((s = ensure(h, h->paths, sizeof(unsigned long long) * 4)) != ISRS_OK) return s;
+    if ((s = ensure(h, h->paths, sizeof(unsigned long long) * kPathCounts)) != ISRS_OK) return s;
     if (prep_only) {
         h->last_launches = g->profile == ISRS_PROFILE_RAMAN_ODE ? 2 : 1;
         return ISRS_OK;
@@ -1019,7 +1019,7 @@ isrs_status run_forward(isrs_handle h, const isrs_fibre *fb, Geom *g, int precis
     Range r_quad(adjoint ? "isrs quadrature + adjoint" : "isrs quadrature");
     QuadParams qp = quad_params(h, fb, g);
     CK(cudaMemsetAsync(h->counter.p, 0, sizeof(int) * 4, st));
-    CK(cudaMemsetAsync(h->paths.p, 0, sizeof(unsigned long long) * 4, st));
+    CK(cudaMemsetAsync(h->paths.p, 0, sizeof(unsigned long long) * kPathCounts, st));
     const int block = h->tile_threads > 0 ? h->tile_threads : 256;
     if (adjoint) {
         const int n_ch = g->plan_n[0];
@@ -1605,16 +1605,20 @@ isrs_status isrs_last_kernel_ms(isrs_handle h, int which, float *ms)
     return ISRS_OK;
 }
 
-isrs_status isrs_last_path_counts(isrs_handle h, int64_t *counts)
+static isrs_status read_counts(isrs_handle h, int first, int n, int64_t *counts)
 {
     if (!h || !counts) return ISRS_ERR_INVALID_ARG;
     if (!h->paths.p) return fail(h, ISRS_ERR_INVALID_ARG, "no launch recorded");
-    unsigned long long c[4] = {0, 0, 0, 0};
+    unsigned long long c[kPathCounts];
     CK(cudaSetDevice(h->device));
     CK(cudaMemcpy(c, h->paths.p, sizeof(c), cudaMemcpyDeviceToHost));
-    for (int k = 0; k < 3; ++k) counts[k] = (int64_t)c[k];
+    for (int k = 0; k < n; ++k) counts[k] = (int64_t)c[first + k];
     return ISRS_OK;
 }
+
+isrs_status isrs_last_path_counts(isrs_handle h, int64_t *counts) { return read_counts(h, 0, 3, counts); }
+
+isrs_status isrs_last_node_counts(isrs_handle h, int64_t *counts) { return read_counts(h, 3, 2, counts); }
 
 isrs_status isrs_gn_eta(isrs_handle h, const isrs_fibre *fibre, const isrs_channels *ch, const double *P_W,
                         const isrs_quad *quad, const int *cuts, int n_cuts, double *eta, double *pnli,
@@ -2085,7 +2089,7 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     const size_t o_stepd = L.take(sizeof(double2) * M), o_stepf = L.take(sizeof(float2) * M);
     const size_t o_partial = L.take(sizeof(double) * std::max<size_t>(1, items.size()));
     const size_t o_counter = L.take(sizeof(int) * 4), o_T = L.take(sizeof(double));
-    const size_t o_paths = L.take(sizeof(unsigned long long) * 4);
+    const size_t o_paths = L.take(sizeof(unsigned long long) * kPathCounts);
     if (L.off > kNoAllocBytes) return ISRS_ERR_UNSUPPORTED;
 
     unsigned char *base = nullptr;
@@ -2106,7 +2110,7 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
             return ISRS_ERR_CUDA;
     if (cudaMemcpyAsync(base + o_P, P_W, sizeof(double) * n, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
         cudaMemsetAsync(base + o_counter, 0, sizeof(int) * 4, st) != cudaSuccess ||
-        cudaMemsetAsync(base + o_paths, 0, sizeof(unsigned long long) * 4, st) != cudaSuccess ||
+        cudaMemsetAsync(base + o_paths, 0, sizeof(unsigned long long) * kPathCounts, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)      // the host tables are freed at return
         return ISRS_ERR_CUDA;
 

@@ -20,6 +20,7 @@ constexpr int kMaxSteps = 2048;     // max z-steps (n_edges - 1)
 constexpr int kMaxG = 4096;         // max grid points per dimension
 constexpr int kMaxRamanCh = 2048;   // max channels of a plan with the Raman-ODE profile
 constexpr int kMaxRamanGradCh = 1536;   // ... and of its gradient (shared memory of the ODE adjoint)
+constexpr int kPathCounts = 5;      // entries of QuadParams::path_count
 constexpr double kPi = 3.14159265358979323846;
 constexpr double kLog2e = 1.44269504088896340736;
 
@@ -91,7 +92,7 @@ struct QuadParams {
     double *partial;            // one per item
     int *counter;               // persistent work counter (zeroed before launch)
     int *err_flag;
-    unsigned long long *path_count;   // [3] grid points per z-sum form (small, direct, telescoped)
+    unsigned long long *path_count;   // [kPathCounts] grid points (low, direct, telescoped), z-sums (direct, telescoped)
     // tabulated profile (Raman ODE): per profile, channel and step {a, b} with
     // ln rho(z_m, F) = a + b (F - f_c) inside channel c; index
     // (prof_ch_off[prof] + c) * n_steps + m.  Null for the closed-form profile.

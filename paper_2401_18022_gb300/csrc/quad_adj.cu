@@ -84,11 +84,10 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
     walk_tables<K2>(qp, ze, zd);
     __syncthreads();
     const float phi_direct = 3.14159265f / qp.dz_max;
-    const float phi_small = kBlkPhiL / qp.L;
+    const float phi_small = kSmallPhiL / (qp.L * (float)qp.n_spans);
     const float log2e = (float)kLog2e;
     const unsigned lt_mask = (1u << lane) - 1u;
-    unsigned long long n_small = 0;
-    unsigned n_direct = 0, n_tele = 0;
+    PathCount count;
 
     for (;;) {
         int it = 0;
@@ -115,7 +114,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
             for (int k = 0; k < K2; ++k) R[k] = Rp[k] = dup2(0.0f);
             double ptot = 0.0;
             const PieceBlocks pb = row_blocks(ns, qp.gauss, G);
-            n_small += lane == 0 && part == 0 ? pb.R1 * G : 0;
+            if (lane == 0 && part == 0) count.small += pb.R1 * G;
             for (int ca = 0; ca < g.nc; ca += kAdjCand) {
                 const int cb = min(g.nc, ca + kAdjCand);
                 for (int c = ca; c < cb; ++c) {
@@ -157,9 +156,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
                             node_get(ns, qp.gauss, c0, q0 + lane, nd);
                             const float aphi = fabsf(nd.phi);
                             cls = aphi <= phi_direct ? 0 : 1;
-                            n_small += aphi <= phi_small ? nd.N : 0;
-                            n_direct += aphi > phi_small && cls == 0 ? nd.N : 0;
-                            n_tele += cls == 0 ? 0 : nd.N;
+                            count.points(aphi, phi_small, cls == 1, nd.N);
                         }
                         const unsigned bd = __ballot_sync(kFull, cls == 0), bt = __ballot_sync(kFull, cls == 1);
                         if (cls >= 0) {
@@ -173,6 +170,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
                         const int nd0 = __popc(bd), nt0 = __popc(bt);
                         for (int f = 0; f < 2; ++f) {
                             const int cnt = f ? nt0 : nd0;
+                            if (lane == 0) count.sums(f, cnt);
                             for (int p = 0; p < cnt; p += 2) {
                                 const int e = min(p + half, cnt - 1), at = f ? 31 - e : e;
                                 const float4 v = w.L[at];
@@ -251,20 +249,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
         }
         __syncwarp();
     }
-    if (qp.path_count) {
-        unsigned long long c0 = n_small, c1 = n_direct, c2 = n_tele;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            c0 += __shfl_xor_sync(kFull, c0, o);
-            c1 += __shfl_xor_sync(kFull, c1, o);
-            c2 += __shfl_xor_sync(kFull, c2, o);
-        }
-        if (lane == 0) {
-            atomicAdd(&qp.path_count[0], c0);
-            atomicAdd(&qp.path_count[1], c1);
-            atomicAdd(&qp.path_count[2], c2);
-        }
-    }
+    if (qp.path_count) count.store(qp.path_count);
 }
 
 // ---------------------------------------------------------------------------

@@ -93,10 +93,10 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
     walk_tables<K2>(qp, ze, zd);
     for (int t = lane; t < 2 * K2 * 16; t += 32) w.B[t] = make_double2(0.0, 0.0);
     const float phi_direct = 3.14159265f / qp.dz_max;
-    const float phi_small = 0.02f / qp.L;
+    const float phi_small = kSmallPhiL / (qp.L * (float)qp.n_spans);
     const float eps = (float)qp.eps_v1;
     const unsigned lt_mask = (1u << lane) - 1u;
-    unsigned n_small = 0, n_direct = 0, n_tele = 0;
+    PathCount count;
     int cur_prof = -1, cur_cut = -1;
 
     for (;;) {
@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
         // walks a list's first 32 points (or what is left)
         const auto flush = [&](bool tele) {
             const int len = tele ? nt : nd, cnt = min(len, 32);
+            if (lane == 0) count.sums(tele, cnt);
             __syncwarp();
             for (int p = 0; p < cnt; p += 2) {
                 const int e = min(p + half, cnt - 1), at = tele ? e : kMciList - 1 - e;
@@ -242,17 +243,12 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
                         }
                     }
                 }
-                const unsigned bs = __ballot_sync(kWarpAll, cls == 0 && fabsf(phi) <= phi_small);
                 const unsigned bd = __ballot_sync(kWarpAll, cls == 0), bt = __ballot_sync(kWarpAll, cls == 1);
                 if (cls >= 0) {
                     const int pos = cls ? nt + __popc(bt & lt_mask) : kMciList - 1 - (nd + __popc(bd & lt_mask));
                     w.L[pos] = make_float4(wwa, phi, Fc, at);
                     w.ch[pos] = make_int2(a | b << 16, c);
-                }
-                if (lane == 0) {
-                    n_small += __popc(bs);
-                    n_direct += __popc(bd & ~bs);
-                    n_tele += __popc(bt);
+                    count.points(fabsf(phi), phi_small, cls, 1);
                 }
                 nd += __popc(bd);
                 nt += __popc(bt);
@@ -285,11 +281,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
         __syncthreads();
         for (int t = lane; t < 2 * K2 * 16; t += 32) w.B[t] = make_double2(0.0, 0.0);
     }
-    if (qp.path_count && lane == 0) {
-        atomicAdd(&qp.path_count[0], (unsigned long long)n_small);
-        atomicAdd(&qp.path_count[1], (unsigned long long)n_direct);
-        atomicAdd(&qp.path_count[2], (unsigned long long)n_tele);
-    }
+    if (qp.path_count) count.store(qp.path_count);
 }
 
 // ---------------------------------------------------------------------------

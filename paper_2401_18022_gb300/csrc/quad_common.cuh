@@ -98,6 +98,40 @@ __device__ __forceinline__ double block_sum_d(double v, double *scratch)
     return r;
 }
 
+// Grid points and z-sums of a launch (QuadParams::path_count, isrs_last_path_counts and
+// isrs_last_node_counts).  A point counts by its phase, the low ones first, so that each
+// counts once also where the z-grid is so coarse that low points are telescoped.
+constexpr float kSmallPhiL = 6.0f;       // |phi| n_spans L of the low points
+
+struct PathCount {                       // of one lane
+    unsigned long long small = 0;
+    unsigned direct = 0, tele = 0, sums_direct = 0, sums_tele = 0;
+    // a z-sum that stands for n points
+    __device__ __forceinline__ void points(float aphi, float phi_small, bool telescoped, int n)
+    {
+        const bool low = aphi <= phi_small;
+        small += low ? n : 0;
+        direct += low || telescoped ? 0 : n;
+        tele += !low && telescoped ? n : 0;
+    }
+    __device__ __forceinline__ void sums(bool telescoped, int n)
+    {
+        if (telescoped) sums_tele += n;
+        else sums_direct += n;
+    }
+    // whole warp
+    __device__ __forceinline__ void store(unsigned long long *out) const
+    {
+        unsigned long long c[5] = {small, direct, tele, sums_direct, sums_tele};
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) c[k] += __shfl_xor_sync(0xffffffffu, c[k], o);
+            if ((threadIdx.x & 31) == 0) atomicAdd(out + k, c[k]);
+        }
+    }
+};
+
 // ---------------------------------------------------------------------------
 // Piece set-up of the FP64 kernels, once per piece.
 // Row r (uniform in s = ln upsilon1): upsilon1 = exp(s_r); the |f2| range

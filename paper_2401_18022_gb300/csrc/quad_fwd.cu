@@ -254,10 +254,9 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
     pair_tables(qp, eB, zD);
     __syncthreads();
     const float phi_direct = 3.14159265f / qp.dz_max;
-    const float phi_small = kBlkPhiL / qp.L;
+    const float phi_small = kSmallPhiL / (qp.L * (float)qp.n_spans);
     const float log2e = (float)kLog2e;
-    unsigned long long n_small = 0;
-    unsigned n_direct = 0, n_tele = 0;
+    PathCount count;
     for (;;) {
         int it = 0;
         if (lane == 0) it = atomicAdd(qp.counter, 1);
@@ -300,6 +299,7 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
                 S.x += __shfl_xor_sync(0xffffffffu, S.x, o);
                 S.y += __shfl_xor_sync(0xffffffffu, S.y, o);
             }
+            if (lane == 0) count.sums(form, n);
             const float S2 = S.x * S.x + S.y * S.y;
             // compensated accumulation over this lane's nodes
             const float y = w * (form == 0 ? S2 : __fdividef(S2, a.x * a.x)) * array_factor_f(a.x, qp, a.y) - comp;
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
             __syncwarp();
             const PieceGeo &g = ns.geo;
             const PieceBlocks pb = row_blocks(ns, qp.gauss, G);
-            n_small += lane == 0 && part == 0 ? pb.R1 * G : 0;
+            if (lane == 0 && part == 0) count.small += pb.R1 * G;
             const float wp = g.mult * g.wab;
             piece_nodes(ns, pb, qp.gauss, G, 0, g.nc, [&](int c0, int nq) {
 #pragma unroll 1
@@ -334,9 +334,7 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
                         const int d = (form ? nt_q : nd_q) + __popc((form ? tele : direct) & below);
                         qu.a[form][d] = make_float4(nd.phi, nd.phi_lo, g.Fi + (nd.x + nd.y), g.at_ab + g.hat[ci]);
                         qu.w[form][d] = wp * (nd.wq * g.pd[ci]);
-                        n_small += aphi <= phi_small ? nd.N : 0;
-                        n_direct += aphi > phi_small && form == 0 ? nd.N : 0;
-                        n_tele += form ? nd.N : 0;
+                        count.points(aphi, phi_small, form, nd.N);
                     }
                     nd_q += __popc(direct);
                     nt_q += __popc(tele);
@@ -351,20 +349,7 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
         const double tot = warp_sum_d((double)sum - (double)comp);
         if (lane == 0) qp.partial[it] = tot;
     }
-    if (qp.path_count) {
-        unsigned long long c0 = n_small, c1 = n_direct, c2 = n_tele;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            c0 += __shfl_xor_sync(0xffffffffu, c0, o);
-            c1 += __shfl_xor_sync(0xffffffffu, c1, o);
-            c2 += __shfl_xor_sync(0xffffffffu, c2, o);
-        }
-        if (lane == 0) {
-            atomicAdd(&qp.path_count[0], c0);
-            atomicAdd(&qp.path_count[1], c1);
-            atomicAdd(&qp.path_count[2], c2);
-        }
-    }
+    if (qp.path_count) count.store(qp.path_count);
 }
 
 // ---------------------------------------------------------------------------

@@ -107,7 +107,7 @@ __host__ __device__ inline int block_need(float A, float D, bool part)
 }
 
 constexpr int kBlkMax = 18;              // row blocks of a piece at most (kMaxG / 256 + 2)
-constexpr float kBlkPhiL = 6.0f;         // |phi| n_spans L up to which rows join a block ...
+constexpr float kBlkPhiL = kSmallPhiL;   // |phi| n_spans L up to which rows join a block ...
 constexpr float kBlkPhiLow = 0.15f;      // ... and up to which they join the low ones
 
 // One piece's geometry, |f1| the longer axis (f1 and f2 enter symmetrically,

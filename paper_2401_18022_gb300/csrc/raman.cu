@@ -449,9 +449,8 @@ __global__ void __launch_bounds__(256, ISRS_TAB_MIN_BLOCKS) k_quad_f32_tab(QuadP
     pair_tables(qp, eB, zD);
     __syncthreads();
     const float phi_direct = 3.14159265f / qp.dz_max;
-    const float phi_small = kBlkPhiL / qp.L;
-    unsigned long long n_small = 0;
-    unsigned n_direct = 0, n_tele = 0;
+    const float phi_small = kSmallPhiL / (qp.L * (float)qp.n_spans);
+    PathCount count;
 
     for (;;) {
         int it = 0;
@@ -471,7 +470,7 @@ __global__ void __launch_bounds__(256, ISRS_TAB_MIN_BLOCKS) k_quad_f32_tab(QuadP
             PieceGeo &g = ns.geo;
             float sum = 0.0f, comp = 0.0f;
             const PieceBlocks pb = row_blocks(ns, qp.gauss, G);
-            n_small += lane == 0 && part == 0 ? pb.R1 * G : 0;
+            if (lane == 0 && part == 0) count.small += pb.R1 * G;
             for (int ca = 0; ca < g.nc; ca += kTabCand) {
                 const int cb = min(g.nc, ca + kTabCand);
                 float tilt = 0.0f;
@@ -507,9 +506,8 @@ __global__ void __launch_bounds__(256, ISRS_TAB_MIN_BLOCKS) k_quad_f32_tab(QuadP
                         const bool direct = aphi <= phi_direct;
                         const float S2 = direct ? zsum_direct_n(nd.phi, lp, zD, M2)
                                                 : zsum_tele_n<0>(nd.phi, nd.phi_lo, lp, eB, M2);
-                        n_small += aphi <= phi_small ? nd.N : 0;
-                        n_direct += aphi > phi_small && direct ? nd.N : 0;
-                        n_tele += direct ? 0 : nd.N;
+                        count.points(aphi, phi_small, !direct, nd.N);
+                        count.sums(!direct, 1);
                         const float y = nd.wq * g.pd[ci] * S2 * array_factor_f(nd.phi, qp, nd.phi_lo) - comp;
                         const float t = sum + y;
                         comp = (t - sum) - y;
@@ -522,20 +520,7 @@ __global__ void __launch_bounds__(256, ISRS_TAB_MIN_BLOCKS) k_quad_f32_tab(QuadP
         const double tot = warp_sum_d(acc);
         if (lane == 0) qp.partial[it] = tot;
     }
-    if (qp.path_count) {
-        unsigned long long c0 = n_small, c1 = n_direct, c2 = n_tele;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            c0 += __shfl_xor_sync(0xffffffffu, c0, o);
-            c1 += __shfl_xor_sync(0xffffffffu, c1, o);
-            c2 += __shfl_xor_sync(0xffffffffu, c2, o);
-        }
-        if (lane == 0) {
-            atomicAdd(&qp.path_count[0], c0);
-            atomicAdd(&qp.path_count[1], c1);
-            atomicAdd(&qp.path_count[2], c2);
-        }
-    }
+    if (qp.path_count) count.store(qp.path_count);
 }
 
 // Plain FP64 quadrature with the tabulated profile (direct form, libm).

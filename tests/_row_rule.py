@@ -152,13 +152,13 @@ class Piece:
         return (4 * c[0] + r["lim"] if c else -1), self.band * (abs(self.phi(r, r["u0"])) + sw * (p1 + p2 * sw))
 
     def units(self, block_need):
-        """(k, weight) of the rows that stand for all G."""
+        """(k, weight, whether it is a block's, so in one channel) of the rows that stand for all G."""
         G = self.G
         tests = [self.test(r) for r in self.rows(G - np.arange(G) - 0.5)]
         key0, R1 = tests[0][0], 0
         while R1 < G and key0 >= 0 and tests[R1][0] == key0 and tests[R1][1] <= BLOCK_PHI:
             R1 += 1
-        out = [(G - r - 0.5, 1.0) for r in range(R1, G)]
+        out = [(G - r - 0.5, 1.0, False) for r in range(R1, G)]
         if R1 == 0:
             return out
         q = max(t[1] * math.exp((R1 - 1 - r) * self.ds) for r, t in enumerate(tests[:R1]))
@@ -169,13 +169,13 @@ class Piece:
                 a, N = n * s // parts, n * (s + 1) // parts - n * s // parts
                 D = 0.5 * N * self.ds
                 pos, w = nodes(N, block_need(cap * D, D, part))
-                out += [(G - (r0 + a + 0.5 * N + p), v) for p, v in zip(pos, w)]
+                out += [(G - (r0 + a + 0.5 * N + p), v, True) for p, v in zip(pos, w)]
         return out
 
     def sigma(self, run_need, block_need):
         phi, at, wt = [], [], []
         units = self.units(block_need)
-        for r, (_, wr) in zip(self.rows([k for k, _ in units]), units):
+        for r, (_, wr, whole) in zip(self.rows([k for k, _, _ in units]), units):
             if r["w"] == 0:
                 continue
             G = self.G
@@ -184,7 +184,7 @@ class Piece:
             E, hd = math.exp(0.5 * r["D"]), 0.5 * r["D"] / G
             x, y = self.s1 * r["xc"], self.s2 * r["yc"]
             e = max(abs(x * E - y / E), abs(x / E - y * E)) * hd
-            per, jm = e * self.band * (p1 + 2 * p2 * e * G), self.turn(r)
+            per, jm = e * self.band * (p1 + 2 * p2 * e * G), 0 if whole else self.turn(r)
             for ja, jb in ((0, jm), (jm, G)):
                 for c in range(len(self.lo)):
                     j = np.flatnonzero((u[ja:jb] >= self.lo[c]) & (u[ja:jb] < self.hi[c])) + ja
@@ -201,7 +201,18 @@ class Piece:
                         phi.append(self.phi(r, v))
                         at.append(np.full(len(v), self.at[c]))
                         wt.append(w * (r["w"] * wr * self.pd[c]))
+        self.nodes = sum(len(v) for v in phi)
         return float(np.sum(np.concatenate(wt) * self.fib.s2(np.concatenate(phi), np.concatenate(at)))) if wt else 0.0
+
+    def points(self):
+        """|phi| of every grid point whose F_c lies in a channel."""
+        out = []
+        for r in self.rows(self.G - np.arange(self.G) - 0.5):
+            if r["w"] > 0:
+                u = self.u(r, np.arange(self.G) + 0.5 - 0.5 * self.G)
+                ok = ((u[:, None] >= self.lo) & (u[:, None] < self.hi)).any(1)
+                out.append(np.abs(self.phi(r, u[ok])))
+        return np.concatenate(out) if out else np.zeros(0)
 
     def full(self):
         """Every grid point."""
