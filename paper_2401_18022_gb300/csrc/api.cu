@@ -1978,6 +1978,34 @@ struct NoAllocLayout {
     }
 };
 
+// Tiles of `chunk` pieces, none of two CUTs (cut_end: one past each CUT's pieces).
+size_t n_tiles(const std::vector<int> &cut_end, int64_t chunk)
+{
+    size_t t = 0;
+    int64_t p0 = 0;
+    for (const int p1 : cut_end) {
+        t += (size_t)((p1 - p0 + chunk - 1) / chunk);
+        p0 = p1;
+    }
+    return t;
+}
+
+// What a problem counts against the 4 MiB: a limit of the interface, not the layout of
+// the present tables (which need less), so that what is taken and what is UNSUPPORTED
+// stays the same for a caller.  80 bytes a piece, 24 a tile of 2^20 grid points, 392 a
+// z-step, 76 a channel, in slots of 256 bytes.
+size_t noalloc_need(const std::vector<DevPiece> &pieces, const std::vector<int> &cut_end, size_t n, size_t M,
+                    int64_t G2)
+{
+    const size_t tiles = n_tiles(cut_end, std::max<int64_t>(1, ((int64_t)1 << 20) / G2));
+    NoAllocLayout L;
+    for (const size_t b : {80 * pieces.size(), 16 * tiles, 8 * std::max<size_t>(1, tiles)}) L.take(b);
+    for (const size_t b : {16, 16, 16, 80, 240, 16, 8}) L.take(b * M);
+    for (const size_t b : {8, 4, 8, 8, 8, 8, 8, 8, 4, 8}) L.take(b * n);
+    for (const size_t b : {8, 4, 4, 224, 8, 8, 16, 8, 32}) L.take(b);
+    return L.off;
+}
+
 }  // namespace
 
 extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_channels *ch, const double *P_W,
@@ -2025,22 +2053,6 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
         if ((s = cut_pieces(nullptr, ch, 0, i, quad->cell_set, pieces)) != ISRS_OK) return s;
         cut_end.push_back((int)pieces.size());
     }
-    // tiles as in the handle calls; where the scratch is nearly full of pieces,
-    // larger ones, so that the tile tables never make a plan too large
-    const TileSplit ts = sizeof(DevPiece) * pieces.size() < kNoAllocBytes / 4
-                             ? tile_split(nullptr, n, quad->cell_set, quad->G)
-                             : TileSplit{(int)std::max<int64_t>(1, (int64_t)(1 << 20) / G2), 1};
-    for (int i = 0; i < n; ++i) {
-        const int p0 = i > 0 ? cut_end[i - 1] : 0, p1 = cut_end[i];
-        const int it0 = (int)items.size();
-        for (int a = p0; a < p1; a += ts.chunk)
-            for (int t = 0; t < ts.parts; ++t) {
-                items.push_back(DevItem{0, a, std::min(a + ts.chunk, p1), i, t | ts.parts << 16});
-                item_slot.push_back(i);
-            }
-        slot_items.push_back(make_int2(it0, (int)items.size()));
-        slot_cut.push_back(i);
-    }
     std::vector<double> frel(n), Bv(n), av(n), gv(n);
     for (int k = 0; k < n; ++k) {
         frel[k] = ch->f_THz[k] - fibre->f_ref_THz;
@@ -2066,10 +2078,11 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     }
     const std::vector<int> zero1{0}, plan_n{n}, slot_off{0, n};
 
-    // layout in the scratch array; anything beyond its size is rejected
+    if (noalloc_need(pieces, cut_end, n, M, G2) > kNoAllocBytes) return ISRS_ERR_UNSUPPORTED;
+
+    // layout in the scratch array: the tile tables last, in what room is left
     NoAllocLayout L;
     const size_t o_pieces = L.take(sizeof(DevPiece) * pieces.size());
-    const size_t o_items = L.take(sizeof(DevItem) * items.size());
     const size_t o_slot_items = L.take(sizeof(int2) * n);
     const size_t o_slot_cut = L.take(sizeof(int) * n);
     const size_t o_slot_off = L.take(sizeof(int) * 2);
@@ -2079,18 +2092,40 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     const size_t o_alpha = L.take(sizeof(double) * n), o_gamma = L.take(sizeof(double) * n);
     const size_t o_za = L.take(sizeof(float4) * M), o_zb = L.take(sizeof(float4) * M);
     const size_t o_zd = L.take(sizeof(double2) * M);
-    // what the call once kept here (step moments, less what a tile has grown by): the
-    // problems the scratch takes stay the same
-    L.take((size_t)std::max<int64_t>(0, 80 * (int64_t)M - 4 * (int64_t)items.size()));
     const size_t o_kapL = L.take(sizeof(double));
     const size_t o_P = L.take(sizeof(double) * n);
     const size_t o_pdd = L.take(sizeof(double) * n), o_pdf = L.take(sizeof(float) * n);
     const size_t o_lnL = L.take(sizeof(double) * n), o_ptot = L.take(sizeof(double));
     const size_t o_stepd = L.take(sizeof(double2) * M), o_stepf = L.take(sizeof(float2) * M);
-    const size_t o_partial = L.take(sizeof(double) * std::max<size_t>(1, items.size()));
     const size_t o_counter = L.take(sizeof(int) * 4), o_T = L.take(sizeof(double));
     const size_t o_paths = L.take(sizeof(unsigned long long) * kPathCounts);
-    if (L.off > kNoAllocBytes) return ISRS_ERR_UNSUPPORTED;
+
+    // tiles as in the handle calls, larger ones where their tables would not fit
+    TileSplit ts = tile_split(nullptr, n, quad->cell_set, quad->G);
+    const auto room_for = [&](size_t tiles) {
+        NoAllocLayout t = L;
+        t.take(sizeof(DevItem) * tiles);
+        t.take(sizeof(double) * std::max<size_t>(1, tiles));
+        return t.off <= kNoAllocBytes;
+    };
+    while (!room_for(n_tiles(cut_end, ts.chunk) * ts.parts)) {
+        if (ts.parts > 1) ts.parts = 1;
+        else if ((size_t)ts.chunk < pieces.size()) ts.chunk *= 2;
+        else return ISRS_ERR_UNSUPPORTED;
+    }
+    for (int i = 0; i < n; ++i) {
+        const int p0 = i > 0 ? cut_end[i - 1] : 0, p1 = cut_end[i];
+        const int it0 = (int)items.size();
+        for (int a = p0; a < p1; a += ts.chunk)
+            for (int t = 0; t < ts.parts; ++t) {
+                items.push_back(DevItem{0, a, std::min(a + ts.chunk, p1), i, t | ts.parts << 16});
+                item_slot.push_back(i);
+            }
+        slot_items.push_back(make_int2(it0, (int)items.size()));
+        slot_cut.push_back(i);
+    }
+    const size_t o_items = L.take(sizeof(DevItem) * items.size());
+    const size_t o_partial = L.take(sizeof(double) * std::max<size_t>(1, items.size()));
 
     unsigned char *base = nullptr;
     if ((s = noalloc_scratch(dev, (void **)&base)) != ISRS_OK) return s;
