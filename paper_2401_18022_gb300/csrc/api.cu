@@ -438,10 +438,10 @@ isrs_status cut_pieces(isrs_handle h, const isrs_channels *c, int plan, int i, i
 // ----------------------------------------------------------------------------
 // z-grid (Sec. III-A, App. A): equal power drop per step,
 //   exp(-a z_e) = 1 - (e/(N_M - 1)) (1 - exp(-a L)),  z-tilde_m = z_m (midpoint)
-// Stored per step as FP64 {z_m, dz_m}, FP32 {z_m, dz_m} and the phase
-// positions in revolutions (z / 2 pi) as float-float pairs.
+// Stored per step as FP64 {z_m, dz_m}, FP32 {z_m, dz_m} and the upper edge's
+// phase position in revolutions (z_{m+1} / 2 pi) as a float-float pair.
 // ----------------------------------------------------------------------------
-void zgrid_tables(double L, double a, int n_edges, std::vector<float4> &za, std::vector<float4> &zb,
+void zgrid_tables(double L, double a, int n_edges, std::vector<float2> &za, std::vector<float2> &zb,
                   std::vector<double2> &zd, float &dz_max)
 {
     std::vector<double> ze(n_edges);
@@ -460,11 +460,10 @@ void zgrid_tables(double L, double a, int n_edges, std::vector<float4> &za, std:
         const double dz = ze[m + 1] - ze[m];
         dmax = std::max(dmax, dz);
         zd[m] = make_double2(zm, dz);
-        // {z_m, z_m^2 + dz_m^2/12 (second moment incl. the sinc term), log2 dz_m, dz_m}
-        za[m] = make_float4((float)zm, (float)(zm * zm + dz * dz / 12.0), (float)std::log2(dz), (float)dz);
-        const double re = ze[m + 1] * inv2pi, rm = zm * inv2pi;
+        za[m] = make_float2((float)zm, (float)dz);
+        const double re = ze[m + 1] * inv2pi;
         const float reh = (float)re;
-        zb[m] = make_float4(reh, (float)(re - (double)reh), (float)rm, 0.f);
+        zb[m] = make_float2(reh, (float)(re - (double)reh));
     }
     dz_max = (float)dmax;
 }
@@ -670,7 +669,7 @@ isrs_status get_geom(isrs_handle h, const isrs_fibre *fb, int n_plans, const isr
     g->n_slots = (int)slot_items.size();
     g->n_mci_items = (int)mitems.size();
 
-    std::vector<float4> za, zb;
+    std::vector<float2> za, zb;
     std::vector<double2> zd;
     zgrid_tables(fb->L_km, fb->alpha_R_per_km, q->n_edges, za, zb, zd, g->dz_max);
 
@@ -918,8 +917,8 @@ QuadParams quad_params(isrs_handle h, const isrs_fibre *fb, Geom *g)
     qp.prof_plan = (const int *)g->prof_plan_d.p;
     qp.step_f = (const float2 *)h->step_f.p;
     qp.step_d = (const double2 *)h->step_d.p;
-    qp.zs_a = (const float4 *)g->zs_a.p;
-    qp.zs_b = (const float4 *)g->zs_b.p;
+    qp.zs_a = (const float2 *)g->zs_a.p;
+    qp.zs_b = (const float2 *)g->zs_b.p;
     qp.zs_d = (const double2 *)g->zs_d.p;
     qp.gauss = h->gauss;
     qp.dz_max = g->dz_max;
@@ -2046,7 +2045,7 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     std::vector<DevPiece> pieces;
     std::vector<DevItem> items;
     std::vector<int2> slot_items;
-    std::vector<int> slot_cut, item_slot;
+    std::vector<int> slot_cut;
     const int64_t G2 = (int64_t)quad->G * quad->G;
     std::vector<int> cut_end;
     for (int i = 0; i < n; ++i) {
@@ -2060,7 +2059,7 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
         av[k] = ch->alpha_per_km[k];
         gv[k] = ch->gamma_per_W_km[k];
     }
-    std::vector<float4> za, zb;
+    std::vector<float2> za, zb;
     std::vector<double2> zd;
     float dz_max = 0.f;
     zgrid_tables(fibre->L_km, fibre->alpha_R_per_km, quad->n_edges, za, zb, zd, dz_max);
@@ -2090,7 +2089,7 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     const size_t o_plan_n = L.take(sizeof(int));
     const size_t o_frel = L.take(sizeof(double) * n), o_B = L.take(sizeof(double) * n);
     const size_t o_alpha = L.take(sizeof(double) * n), o_gamma = L.take(sizeof(double) * n);
-    const size_t o_za = L.take(sizeof(float4) * M), o_zb = L.take(sizeof(float4) * M);
+    const size_t o_za = L.take(sizeof(float2) * M), o_zb = L.take(sizeof(float2) * M);
     const size_t o_zd = L.take(sizeof(double2) * M);
     const size_t o_kapL = L.take(sizeof(double));
     const size_t o_P = L.take(sizeof(double) * n);
@@ -2117,10 +2116,8 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
         const int p0 = i > 0 ? cut_end[i - 1] : 0, p1 = cut_end[i];
         const int it0 = (int)items.size();
         for (int a = p0; a < p1; a += ts.chunk)
-            for (int t = 0; t < ts.parts; ++t) {
+            for (int t = 0; t < ts.parts; ++t)
                 items.push_back(DevItem{0, a, std::min(a + ts.chunk, p1), i, t | ts.parts << 16});
-                item_slot.push_back(i);
-            }
         slot_items.push_back(make_int2(it0, (int)items.size()));
         slot_cut.push_back(i);
     }
@@ -2138,8 +2135,8 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
         {o_slot_off, slot_off.data(), sizeof(int) * 2}, {o_zero, zero1.data(), sizeof(int)},
         {o_plan_n, plan_n.data(), sizeof(int)}, {o_frel, frel.data(), sizeof(double) * n},
         {o_B, Bv.data(), sizeof(double) * n}, {o_alpha, av.data(), sizeof(double) * n},
-        {o_gamma, gv.data(), sizeof(double) * n}, {o_za, za.data(), sizeof(float4) * M},
-        {o_zb, zb.data(), sizeof(float4) * M}, {o_zd, zd.data(), sizeof(double2) * M}};
+        {o_gamma, gv.data(), sizeof(double) * n}, {o_za, za.data(), sizeof(float2) * M},
+        {o_zb, zb.data(), sizeof(float2) * M}, {o_zd, zd.data(), sizeof(double2) * M}};
     for (const Up &u : ups)
         if (u.bytes && cudaMemcpyAsync(base + u.off, u.src, u.bytes, cudaMemcpyHostToDevice, st) != cudaSuccess)
             return ISRS_ERR_CUDA;
@@ -2197,8 +2194,8 @@ extern "C" isrs_status isrs_gn_eta_noalloc(const isrs_fibre *fibre, const isrs_c
     qp.pd_d = pp.pd_d;
     qp.step_f = pp.step_f;
     qp.step_d = pp.step_d;
-    qp.zs_a = (const float4 *)(base + o_za);
-    qp.zs_b = (const float4 *)(base + o_zb);
+    qp.zs_a = (const float2 *)(base + o_za);
+    qp.zs_b = (const float2 *)(base + o_zb);
     qp.zs_d = pp.zs_d;
     qp.gauss = gauss;
     qp.kap_L = pp.kap_L;

@@ -78,8 +78,8 @@ struct QuadParams {
     const float2 *step_f;       // {A2_m, K2_m}: log2 p = A2 + K2 (F_c - f_ref) - at2 z_m
     const double2 *step_d;      // {ln Ptot - ln N_m, kappa_m}
     // z tables (per step m)
-    const float4 *zs_a;         // {z_m, z_m^2 + dz_m^2/12, log2 dz_m, dz_m}
-    const float4 *zs_b;         // {z_{m+1}/2pi hi, lo (float-float), z_m/2pi, 0}
+    const float2 *zs_a;         // {z_m, dz_m}
+    const float2 *zs_b;         // z_{m+1}/2pi, float-float
     const double2 *zs_d;        // {z_m, dz_m}
     const float2 *gauss;        // Gauss rules of the row sums (quad_nodes.cuh): {t, weight}
     const double *kap_L;        // per profile: kappa(L) [1/THz]

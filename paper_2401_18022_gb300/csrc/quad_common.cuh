@@ -35,7 +35,6 @@ __device__ __forceinline__ double warp_sum_d(double v)
     return v;
 }
 
-// Deterministic block sum of one double per thread (blockDim multiple of 32).
 // ln(sinh(x) / x) and its derivative coth(x) - 1/x in FP64.  Up to |x| = 0.2
 // (kappa B / 2 of any practical channel) the Taylor series of either, dropped
 // terms below 2e-16: a few FMAs where sinh, log, tanh and two divisions were most
@@ -80,6 +79,7 @@ __device__ __forceinline__ double block_max_d(double v, double *scratch)
     return m;
 }
 
+// Deterministic block sum of one double per thread (blockDim multiple of 32).
 __device__ __forceinline__ double block_sum_d(double v, double *scratch)
 {
     v = warp_sum_d(v);

@@ -35,9 +35,9 @@ __device__ __forceinline__ void walk_tables(const QuadParams &qp, float4 *ze, fl
     for (int t = threadIdx.x; t < K2 * 16; t += blockDim.x) {
         const int m0 = min(walk_step<K2>(t >> 4, t & 15, 0), qp.n_steps - 1);
         const int m1 = min(walk_step<K2>(t >> 4, t & 15, 1), qp.n_steps - 1);
-        const float4 b0 = qp.zs_b[m0], b1 = qp.zs_b[m1], a0 = qp.zs_a[m0], a1 = qp.zs_a[m1];
+        const float2 b0 = qp.zs_b[m0], b1 = qp.zs_b[m1], a0 = qp.zs_a[m0], a1 = qp.zs_a[m1];
         ze[t] = make_float4(b0.x, b1.x, b0.y, b1.y);
-        zd[t] = make_float4(a0.x, a1.x, a0.w, a1.w);
+        zd[t] = make_float4(a0.x, a1.x, a0.y, a1.y);
     }
 }
 

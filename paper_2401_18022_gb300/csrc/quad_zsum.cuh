@@ -112,9 +112,9 @@ __device__ __forceinline__ void pair_tables(const QuadParams &qp, float4 *eB, fl
     const int M = qp.n_steps;
     for (int k = threadIdx.x; k < step_pairs(M); k += blockDim.x) {
         const int m0 = 2 * k, m1 = min(2 * k + 1, M - 1);
-        const float4 b0 = qp.zs_b[m0], b1 = qp.zs_b[m1], a0 = qp.zs_a[m0], a1 = qp.zs_a[m1];
+        const float2 b0 = qp.zs_b[m0], b1 = qp.zs_b[m1], a0 = qp.zs_a[m0], a1 = qp.zs_a[m1];
         eB[k] = make_float4(b0.x, b1.x, b0.y, b1.y);
-        zD[k] = make_float4(a0.x, a1.x, a0.w, a1.w);
+        zD[k] = make_float4(a0.x, a1.x, a0.y, a1.y);
     }
 }
 
