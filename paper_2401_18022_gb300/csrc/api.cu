@@ -848,8 +848,12 @@ cudaError_t gauss_rules(int dev, cudaStream_t st, const float2 **out)
 // shared by up to 8 (a 5-channel plan has 90 pieces for 3,648 resident warps;
 // every share repeats the piece's set-up, which only pays on an idle chip: at G 64 4
 // shares take 40 us forward and 57 us with the adjoint, 8 take 35 and 45, 16 take 41
-// and 46).  A large plan takes up to 32 pieces a tile, ~10 tiles per resident warp, so that a
-// tile's fixed cost (queue, bucket rows) stays small and the last wave short.
+// and 46).  A large plan takes 1 / 38,912 of its pieces a tile, ~10 tiles per resident warp, so that a
+// tile's fixed cost (queue, bucket rows) stays small and the last wave short.  The number of
+// tiles is also what a gradient's buckets take: n_ch x 8 + n_steps x 16 bytes a tile
+// (closed form; 0.25 GB at 557 channels), n_steps x 16 for every channel that it
+// touches (Raman ODE).  With tiles of 32 pieces at most, every cell of 500 narrow
+// channels had two million tiles and up to 225 GB of Raman rows (39 GB now).
 // The split depends on the plan and grid alone, never on the CUT list or the
 // number of profiles, so a CUT's tiles and the order of its sum are the same in
 // every call.
@@ -859,7 +863,7 @@ TileSplit tile_split(const isrs_handle_s *h, int n_ch, int cell_set, int G)
     const int64_t n = n_ch;
     const int64_t total = cell_set == ISRS_CELLS_SCI_XCI ? n * (2 * n + 1) : n * (n + 1) * (n + 3) / 2;
     const int64_t parts = std::min<int64_t>(std::min(8, std::max(1, G / 8)), (16384 + total - 1) / total);
-    return {(int)std::max<int64_t>(1, std::min<int64_t>(32, total / 38912)), (int)parts};
+    return {(int)std::max<int64_t>(1, total / 38912), (int)parts};
 }
 
 RamanParams raman_params(isrs_handle h, const isrs_fibre *fb, Geom *g, bool keep_nodes)
