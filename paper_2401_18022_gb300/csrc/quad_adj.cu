@@ -186,9 +186,10 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
                                 float sr, si, sq = wq;
                                 if (f) {
                                     walk_tele<K2, false>(ze + l16, l16, v.y, v.z, lp, tr, ti, sr, si);
-                                    sq *= __fdividef(1.0f, v.y * v.y);
+                                    sq *= __fdividef(zsum_gain(true), v.y * v.y);
                                 } else {
                                     walk_direct<K2>(zd + l16, v.y, lp, tr, ti, sr, si);
+                                    sq *= zsum_gain(false);
                                 }
                                 const f32x2 c2 = dup2(2.0f * mult * sq), cF = dup2(2.0f * mult * sq * (g.Fc0 + v.w));
                                 const f32x2 sr2 = dup2(sr), si2 = dup2(si);

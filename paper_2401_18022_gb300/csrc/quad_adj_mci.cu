@@ -177,9 +177,10 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MCI_MIN_BLOCKS) k_quad_adj_mci(A
                 float sr, si, sq = p + half < cnt ? v.x : 0.0f;
                 if (tele) {
                     walk_tele<K2, true>(ze + l16, l16, v.y, 0.0f, lp, tr, ti, sr, si, turn_magic(v.y * qp.Lrev_hi));
-                    sq *= __fdividef(1.0f, v.y * v.y);
+                    sq *= __fdividef(zsum_gain(true), v.y * v.y);
                 } else {
                     walk_direct<K2>(zd + l16, v.y, lp, tr, ti, sr, si);
+                    sq *= zsum_gain(false);
                 }
                 const f32x2 c2 = dup2(2.0f * sq), cF = dup2(2.0f * sq * v.z), sr2 = dup2(sr), si2 = dup2(si);
 #pragma unroll

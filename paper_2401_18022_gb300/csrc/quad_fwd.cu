@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(256, ISRS_FWD_MIN_BLOCKS) k_quad_f32(QuadParam
                     if (on) {
                         const int d = (form ? nt_q : nd_q) + __popc((form ? tele : direct) & below);
                         qu.a[form][d] = make_float4(nd.phi, nd.phi_lo, g.Fi + (nd.x + nd.y), g.at_ab + g.hat[ci]);
-                        qu.w[form][d] = wp * (nd.wq * g.pd[ci]);
+                        qu.w[form][d] = wp * (nd.wq * g.pd[ci]) * zsum_gain(form);
                         count.points(aphi, phi_small, form, nd.N);
                     }
                     nd_q += __popc(direct);

@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(256, ISRS_MCI_TAB_MIN_BLOCKS) k_quad_mci_f32_t
                     S.x += __shfl_xor_sync(0xffffffffu, S.x, o);
                     S.y += __shfl_xor_sync(0xffffffffu, S.y, o);
                 }
-                const float S2 = S.x * S.x + S.y * S.y, wt = pt < cnt && sub == 0 ? v.w : 0.0f;
+                const float S2 = S.x * S.x + S.y * S.y, wt = pt < cnt && sub == 0 ? v.w * zsum_gain(f) : 0.0f;
                 const float y = wt * (f ? __fdividef(S2, v.x * v.x) : S2) * array_factor_f<true>(v.x, qp) - comp;
                 const float t = sum + y;
                 comp = (t - sum) - y;

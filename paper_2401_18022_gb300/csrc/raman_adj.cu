@@ -163,9 +163,10 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_TAB_MIN_BLOCKS) k_quad_adj_tab(A
                                 float sr, si, cp = p + half < cnt ? v.x : 0.0f;
                                 if (f) {
                                     walk_tele<K2, false>(ze + l16, l16, v.y, v.z, lp, tr, ti, sr, si);
-                                    cp *= __fdividef(1.0f, v.y * v.y);
+                                    cp *= __fdividef(zsum_gain(true), v.y * v.y);
                                 } else {
                                     walk_direct<K2>(zd + l16, v.y, lp, tr, ti, sr, si);
+                                    cp *= zsum_gain(false);
                                 }
                                 const f32x2 c2 = dup2(2.0f * cp), cl = dup2(2.0f * cp * v.w), cd = dup2(2.0f * cp * dd);
                                 const f32x2 sr2 = dup2(sr), si2 = dup2(si);
