@@ -117,7 +117,7 @@ __global__ void __launch_bounds__(256) k_prep(PrepParams pp)
 // p_{i+1} = t p_i - b_i p_{i-1} with b_i = i^2 (N^2 - i^2) / (N^2 (4 i^2 - 1)).
 // One thread per node: the k-th smallest zero by bisection on the sign changes
 // of the sequence p_0..p_n (Sturm), then Newton; weight N / sum of the squared
-// orthonormal polynomials.  FP64, run once per device (about 1 ms).
+// orthonormal polynomials.  FP64, run once per device (4 ms).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(128) k_gauss(float2 *out)
 {
@@ -210,9 +210,9 @@ cudaError_t gauss_array(void **out) { return cudaGetSymbolAddress(out, g_isrs_ga
 
 // ---------------------------------------------------------------------------
 // k_quad_f32: persistent FP32 quadrature.  Bound by the XU pipe (sin and cos at 16
-// lanes a clock, ex2 at 32: 20 cycles per warp and z-step), 72 % busy on a 148-channel
-// plan at G = 256 (2.28 ms; every grid point summed one by one: 74.4 ms).  589
-// channels at G = 256: 1,129 -> 43.9 ms; 12 profiles at G = 64: 541 -> 77 ms, a
+// lanes a clock, ex2 at 32: 20 cycles per warp and z-step), 71 % busy on a 148-channel
+// plan at G = 256 (2.40 ms; every grid point summed one by one: 74.4 ms).  589
+// channels at G = 256: 1,129 -> 45.0 ms; 12 profiles at G = 64: 541 -> 79.8 ms, a
 // quarter of it the pieces' set-up.  Three blocks of 80 registers an SM: two leave
 // 5 % on the G = 256 case and 6 % on the G = 64 one, four spill (4 % and 9 %).
 // ---------------------------------------------------------------------------
