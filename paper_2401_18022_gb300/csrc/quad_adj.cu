@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
             for (int ca = 0; ca < g.nc; ca += kAdjCand) {
                 const int cb = min(g.nc, ca + kAdjCand);
                 for (int c = ca; c < cb; ++c) {
-                    const float at = g.at_ab + g.hat[c], F = g.Fc0 + 0.5f * (g.lo[c] + g.hi[c]);
+                    const float at = g.at_ab + g.hat[c], F = g.Fc0 + (0.5f * (g.lo[c] + g.hi[c]) - g.Fi);
                     for (int t = lane; t < K2 * 16; t += 32) {
                         const int m = walk_step<K2>(t >> 4, t & 15, 0);
                         float4 e = make_float4(kPadLog2, kPadLog2, 0.0f, 0.0f);
@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(256, ISRS_ADJ_MIN_BLOCKS) k_quad_adj(AdjParams
                                 const float4 v = w.L[at];
                                 const int c = w.Lc[at];
                                 const float wq = p + half < cnt ? v.x : 0.0f;
-                                const f32x2 dF = dup2(v.w - 0.5f * (g.lo[ca + c] + g.hi[ca + c]));
+                                const f32x2 dF = dup2(v.w - (0.5f * (g.lo[ca + c] + g.hi[ca + c]) - g.Fi));
                                 const float4 *ek = w.ek[c] + l16;
                                 const auto lp = [&](int k) {
                                     const float4 x = ek[k * 16];

@@ -116,17 +116,21 @@ struct PieceGeo {
     float2 vC;                  // -4 pi^2 f1 f2 at the corner, float-float
     float2 br0;                 // bracket of Eq. phi: br0 + br1 u + c4 u^2 - c4/2 f1 f2, u from the corner
     float2 ds2;                 // row pitch in log2 upsilon1
-    float u1hi;                 // xhi yhi
+    float2 u1hi;                // xhi yhi, float-float
+    float2 k[3];                // of a row's centre, float-float: yhi / xhi, ylo / xlo and the root of
+                                // xlo xhi (R < Rb) or ylo yhi
     float br1, c4;
     float ds;                   // row pitch in ln upsilon1
     float xhi, yhi;             // corner of the piece
     float s1, s2;               // signs of f1, f2
     float R, Rb;                // ln(xhi / xlo), ln(yhi / ylo) (1e30 where the lower limit is 0)
+    float off;                  // bound of |row_u - point_u|
     float band;                 // n_spans L: phase swing per |d phi|
     float tilt;                 // bound of |d ln p / dF|
     float Fc0, Fi;              // F_c - f_ref and F_c - f_i at the corner
     float wab, at_ab, mult;     // P_a P_b / (B_a B_b), attenuation part of ln p, mirror weight
-    int nc;                     // F_c candidates: edges from the corner, P/B, half attenuation
+    bool sw;                    // the longer axis belongs to F_b
+    int nc;                     // F_c candidates: edges from the CUT, P/B, half attenuation
     float lo[kMaxCand], hi[kMaxCand], pd[kMaxCand], hat[kMaxCand];
 };
 
@@ -161,6 +165,31 @@ struct WarpNodes {
     PieceGeo geo;
 };
 
+// float-float product, quotient and square root (~2^-45; a, b > 0)
+__device__ __forceinline__ float2 ff_sum(float a, float b)            // |a| >= |b|
+{
+    const float h = __fadd_rn(a, b);
+    return make_float2(h, __fadd_rn(b, -__fadd_rn(h, -a)));
+}
+
+__device__ __forceinline__ float2 ff_mul(float2 a, float2 b)
+{
+    const float h = __fmul_rn(a.x, b.x);
+    return ff_sum(h, fmaf(a.x, b.x, -h) + fmaf(a.x, b.y, a.y * b.x));
+}
+
+__device__ __forceinline__ float2 ff_div(float2 a, float2 b)
+{
+    const float r = __fdividef(1.0f, b.x), q = __fmul_rn(a.x, r);
+    return ff_sum(q, (fmaf(-q, b.x, a.x) + fmaf(-q, b.y, a.y)) * r);
+}
+
+__device__ __forceinline__ float2 ff_sqrt(float2 a)
+{
+    const float r = rsqrtf(a.x), q = __fmul_rn(a.x, r);
+    return ff_sum(q, (fmaf(-q, q, a.x) + a.y) * (0.5f * r));
+}
+
 // The piece's geometry (whole warp; the caller syncs the warp).  sw: the
 // longer axis belongs to F_b.
 __device__ __forceinline__ bool node_geo(const QuadParams &qp, const DevPiece &pc, int prof, float at_scale,
@@ -175,9 +204,9 @@ __device__ __forceinline__ bool node_geo(const QuadParams &qp, const DevPiece &p
     const double U = (n1 ? -xhi : xhi) + (n2 ? -yhi : yhi);
     const int nc = min(pc.c_hi - pc.c_lo + 1, kMaxCand);
     if (lane < nc) {
-        const double e = (qp.ch_frel[coff + pc.c_lo + lane] - fi) - U, B = qp.ch_B[coff + pc.c_lo + lane];
-        g.lo[lane] = (float)fma(-0.5, B, e);
-        g.hi[lane] = (float)fma(0.5, B, e);
+        const double fc = qp.ch_frel[coff + pc.c_lo + lane], hb = 0.5 * qp.ch_B[coff + pc.c_lo + lane];
+        g.lo[lane] = (float)((fc - hb) - fi);
+        g.hi[lane] = (float)((fc + hb) - fi);
         g.pd[lane] = pdv[poff + pc.c_lo + lane];
         g.hat[lane] = 0.5f * (float)qp.ch_alpha[coff + pc.c_lo + lane] * at_scale;
     }
@@ -192,6 +221,8 @@ __device__ __forceinline__ bool node_geo(const QuadParams &qp, const DevPiece &p
     if (lane == 8) v = U;
     if (lane == 5) v = xhi;
     if (lane == 6) v = yhi;
+    if (lane == 9) v = sw ? pc.ylo : pc.xlo;
+    if (lane == 10) v = sw ? pc.xlo : pc.ylo;
     if (lane == 7)
         v = 0.5 * (qp.ch_alpha[coff + pc.a] + qp.ch_alpha[coff + pc.b] - qp.ch_alpha[coff + pc.cut]);
     const float vh = (float)v, vl = (float)(v - (double)vh);
@@ -203,9 +234,17 @@ __device__ __forceinline__ bool node_geo(const QuadParams &qp, const DevPiece &p
     if (lane == 5) g.xhi = vh;
     if (lane == 6) g.yhi = vh;
     if (lane == 7) g.at_ab = vh * at_scale;
+    // lanes 0..2: yhi / xhi, ylo / xlo, the mean of the limits of the shorter range (what
+    // a lower limit of 0 leaves undefined no row takes)
+    const bool cx = (sw ? pc.lny : pc.lnx) < (sw ? pc.lnx : pc.lny);
+    const int la = lane == 0 ? 6 : lane == 1 ? 10 : cx ? 5 : 6, lb = lane == 0 ? 5 : lane == 1 || cx ? 9 : 10;
+    const float2 ka = make_float2(__shfl_sync(0xffffffffu, vh, la), __shfl_sync(0xffffffffu, vl, la));
+    const float2 kb = make_float2(__shfl_sync(0xffffffffu, vh, lb), __shfl_sync(0xffffffffu, vl, lb));
+    if (lane < 3) g.k[lane] = lane == 2 ? ff_sqrt(ff_mul(ka, kb)) : ff_div(ka, kb);
     if (lane == 0) {
         const float2 ds2 = pc.ds2;
-        g.u1hi = vh;
+        g.u1hi = make_float2(vh, vl);
+        g.sw = sw;
         g.c4 = (float)qp.c4;
         g.ds2 = ds2;
         g.ds = fmaf(ds2.x, 0.693147182f, fmaf(ds2.x, -1.90465421e-9f, ds2.y * 0.693147182f));   // times ln 2
@@ -213,6 +252,9 @@ __device__ __forceinline__ bool node_geo(const QuadParams &qp, const DevPiece &p
         g.s2 = n2 ? -1.0f : 1.0f;
         g.R = sw ? pc.lny : pc.lnx;
         g.Rb = sw ? pc.lnx : pc.lny;
+        // 2.4e-7 of |f1| and 3e-7 of |f2| by point_u's rounding, 6e-8 |d| by d's (|d| is at
+        // most half the shorter range, 20 for any epsilon), as much again by row_u's
+        g.off = 8e-7f * (float)(xhi + yhi) * (1.0f + fminf(20.0f, fminf(pc.lnx, pc.lny)));
         g.band = qp.L * (float)qp.n_spans;
         g.tilt = tilt;
         g.wab = pdv[poff + pc.a] * pdv[poff + pc.b];
@@ -240,7 +282,9 @@ __device__ __forceinline__ int node_row(const PieceGeo &g, const float2 *gauss, 
     const float2 T = __ldg(gauss + kGaussEntries + (mi & (kExp2Entries - 1)));
     const float eh = fmaf(T.x, q, T.x), el = fmaf(T.x, q, __fadd_rn(T.x, -eh)) + fmaf(T.y, q, T.y);
     const float sc = n < 127 ? __int_as_float((127 - n) << 23) : 0.0f;
-    const float u1 = fmaf(g.u1hi, eh, g.u1hi * el) * sc;
+    const float uh = __fmul_rn(g.u1hi.x, eh);
+    const float ul = fmaf(g.u1hi.x, eh, -uh) + fmaf(g.u1hi.x, el, g.u1hi.y * eh);
+    const float u1 = (uh + ul) * sc;
     const float l = -k * g.ds;
     const bool a = l > -g.Rb, b = l + g.R < 0.0f;
     const float D = a ? (b ? g.R : -l) : (b ? l + g.R + g.Rb : g.Rb);
@@ -250,9 +294,16 @@ __device__ __forceinline__ int node_row(const PieceGeo &g, const float2 *gauss, 
         o.xc = o.yc = o.du2 = o.w = o.x0 = o.y0 = o.phi0 = o.phi0_lo = 0.0f;
         return -1;
     }
-    o.xc = g.xhi * expf(gx);
-    o.yc = __fdividef(u1, o.xc);
-    o.du2 = __fdividef(D, (float)G);
+    // The centre lies at |f2| = sqrt(ymin ymax): sqrt(u1 yhi / xhi), sqrt(u1 ylo / xlo), or
+    // one of f1 and f2 is the mean of its limits.  Rounded once, for point_u.
+    const bool mid = a == b;
+    const float2 U = make_float2(uh * sc, ul * sc);
+    const float2 p = mid ? g.k[2] : ff_sqrt(ff_mul(U, a ? g.k[0] : g.k[1]));
+    const float qc = ff_div(U, p).x;
+    o.xc = mid && a ? p.x : qc;
+    o.yc = mid && a ? qc : p.x;
+    const float rG = __fdividef(1.0f, (float)G), du2 = D * rG;
+    o.du2 = fmaf(fmaf(-du2, (float)G, D), rG, du2);
     o.w = u1 * g.ds * o.du2;
     o.x0 = g.s1 * g.xhi * expm1f(gx);
     o.y0 = g.s2 * g.yhi * expm1f(gy);
@@ -304,6 +355,23 @@ __device__ __forceinline__ float row_u(const PieceGeo &g, const NodeRow &o, floa
     return (o.x0 + o.y0) + fmaf(g.s1 * o.xc, ep, g.s2 * o.yc * em);
 }
 
+// F_c - f_i at column j of a grid row, as the sum of the point's FP32 f1 and f2: what
+// decides its F_c channel.  A point next to a channel's edge falls on the side where this
+// rounding puts it (a few 1e-6 THz in the far cells).  From the corner's coordinates,
+// which are finer, others fall otherwise, each worth up to 1e-3 of a channel's eta on a
+// coarse grid: 148 neighbouring channels around the zero-dispersion wavelength at G 40
+// came out 5.3e-5 (2-norm of eta) from the sum over single points, 8.3e-7 now.  So every
+// factor is rounded as that sum rounds it: the row's centre and pitch once to FP32, e^d,
+// its reciprocal, the products.  Costs 1 to 5 % of the time (589 channels, G 256: 44.9 ->
+// 45.4 ms; 12 profiles, G 64: 79.7 -> 83.3); taking it only within g.off of an edge costs
+// more (46.9 and 93.7), some row of a warp nearly always is.
+__device__ __forceinline__ float point_u(const PieceGeo &g, const NodeRow &o, int G, int j)
+{
+    const float d = __fmul_rn((float)j + 0.5f - 0.5f * (float)G, o.du2);
+    const float e = expf(g.sw ? -d : d), er = __frcp_rn(e);
+    return __fadd_rn(g.s1 * __fmul_rn(o.xc, g.sw ? er : e), g.s2 * __fmul_rn(o.yc, g.sw ? e : er));
+}
+
 // first column of the row past |f1| = |f2|, where u turns if both have one sign
 __device__ __forceinline__ int row_turn(const PieceGeo &g, const NodeRow &o, int G)
 {
@@ -321,8 +389,7 @@ template <typename F>
 __device__ __forceinline__ void row_runs(const PieceGeo &g, const NodeRow &o, int G, int ca, int cb, int whole,
                                          const F &f)
 {
-    const float c0 = 0.5f - 0.5f * (float)G;
-    const auto u_at = [&](int j) { return row_u(g, o, ((float)j + c0) * o.du2); };
+    const auto u_at = [&](int j) { return point_u(g, o, G, j); };
     const int jm = whole >= 0 ? 0 : row_turn(g, o, G);
     if (whole >= 0) {
         ca = whole;
@@ -333,7 +400,7 @@ __device__ __forceinline__ void row_runs(const PieceGeo &g, const NodeRow &o, in
         const int ja = part == 0 ? 0 : jm, jb = part == 0 ? jm : G;
         if (jb <= ja) continue;
         const bool up = (g.s1 > 0.0f) == (part == 1 || g.s1 != g.s2);
-        const float ua = u_at(ja), ub = u_at(jb - 1);
+        const float ua = whole < 0 ? u_at(ja) : 0.0f, ub = whole < 0 ? u_at(jb - 1) : 0.0f;
         // first column of [ja, jb) at or past edge e in the direction of travel (ja
         // is before it, jb - 1 at or past it or nothing is): the column a straight
         // line between the ends gives and a neighbour of it usually bracket it (u
@@ -413,8 +480,8 @@ __device__ __forceinline__ void run_parts(const PieceGeo &g, const NodeRow &o, i
     }
 }
 
-// The F_c candidate that holds every column of the row, or -1; ph: bound of
-// |phi| band over the row's columns.
+// The F_c candidate that holds every column of the row with room for point_u's rounding,
+// or -1; ph: bound of |phi| band over the row's columns.
 __device__ __forceinline__ int row_whole(const PieceGeo &g, const NodeRow &o, int G, float &ph)
 {
     const float c0 = 0.5f - 0.5f * (float)G;
@@ -430,6 +497,8 @@ __device__ __forceinline__ int row_whole(const PieceGeo &g, const NodeRow &o, in
     row_slopes(g, o, p1, p2);
     const float r = mx - mn;
     ph = g.band * (fabsf(o.phi0) + r * (fabsf(p1) + fabsf(p2) * r));
+    mn = (mn + g.Fi) - g.off;
+    mx = (mx + g.Fi) + g.off;
     int c = -1;
 #pragma unroll 1
     for (int q = 0; q < g.nc; ++q)
