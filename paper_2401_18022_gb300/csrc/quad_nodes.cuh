@@ -400,7 +400,13 @@ __device__ __forceinline__ void row_runs(const PieceGeo &g, const NodeRow &o, in
         const int ja = part == 0 ? 0 : jm, jb = part == 0 ? jm : G;
         if (jb <= ja) continue;
         const bool up = (g.s1 > 0.0f) == (part == 1 || g.s1 != g.s2);
-        const float ua = whole < 0 ? u_at(ja) : 0.0f, ub = whole < 0 ? u_at(jb - 1) : 0.0f;
+        float ua = 0.0f, ub = 0.0f;
+        if (whole < 0)
+#pragma unroll 1
+            for (int side = 0; side < 2; ++side) {
+                ua = ub;
+                ub = u_at(side == 0 ? ja : jb - 1);
+            }
         // first column of [ja, jb) at or past edge e in the direction of travel (ja
         // is before it, jb - 1 at or past it or nothing is): the column a straight
         // line between the ends gives and a neighbour of it usually bracket it (u
@@ -485,13 +491,15 @@ __device__ __forceinline__ void run_parts(const PieceGeo &g, const NodeRow &o, i
 __device__ __forceinline__ int row_whole(const PieceGeo &g, const NodeRow &o, int G, float &ph)
 {
     const float c0 = 0.5f - 0.5f * (float)G;
-    const float ua = row_u(g, o, c0 * o.du2), ub = row_u(g, o, -c0 * o.du2);
-    float mn = fminf(ua, ub), mx = fmaxf(ua, ub);
     const int jm = row_turn(g, o, G);
-    if (jm > 0 && jm < G) {
-        const float um = row_u(g, o, ((float)jm + c0) * o.du2), un = row_u(g, o, ((float)jm - 1.0f + c0) * o.du2);
-        mn = fminf(mn, fminf(um, un));
-        mx = fmaxf(mx, fmaxf(um, un));
+    float mn = 1e30f, mx = -1e30f;
+    const int n = jm > 0 && jm < G ? 4 : 2;
+#pragma unroll 1
+    for (int k = 0; k < n; ++k) {                         // both ends, both sides of the turn
+        const int j = k == 0 ? 0 : k == 1 ? G - 1 : jm + k - 3;
+        const float u = row_u(g, o, ((float)j + c0) * o.du2);
+        mn = fminf(mn, u);
+        mx = fmaxf(mx, u);
     }
     float p1, p2;
     row_slopes(g, o, p1, p2);
