@@ -301,9 +301,9 @@ def _snr_eval(eng, wl, P, dev, n_grid, reps: int = 2):
 # full size (same G, same per-piece shape), so each count is scaled to a full
 # launch by evaluated points.
 ADJ_CAPTURE = {"profile": "k_quad_adj_uwb148_every4th_G256.md", "points": 2880700416,
-               "dram_bytes": 7.829e7, "warp_inst": 3.069e9, "fp32_warp_inst": 2.647e9}
+               "dram_bytes": 7.935e7, "warp_inst": 3.107e9, "fp32_warp_inst": 2.663e9}
 FWD_CAPTURE = {"profile": "k_quad_f32_uwb148_every4th_G256.md", "points": 2880700416,
-               "dram_bytes": 4.596e6, "warp_inst": 1.756e9, "fp32_warp_inst": 1.461e9}
+               "dram_bytes": 4.596e6, "warp_inst": 1.817e9, "fp32_warp_inst": 1.463e9}
 ISSUE_PER_CLK_PER_SM = 4         # one warp instruction per clock per SM sub-partition
 
 

@@ -21,7 +21,7 @@
 // same registers give d|S|^2/d ln p_m = 2 Re(conj(S) t_m) for the lane's own step
 // buckets, which stay in registers between FP64 folds.  Those registers (128) leave
 // 16 warps an SM, so the chain phase -> sin, cos -> term -> half sum -> bucket bounds
-// it: issue 62 %, XU pipe 48 %.  557 channels at G = 128: 610 -> 41.4 ms.
+// it: issue 61 %, XU pipe 47 %.  557 channels at G = 128: 610 -> 42.6 ms.
 #include <cuda_runtime.h>
 
 #include "isrs_internal.cuh"

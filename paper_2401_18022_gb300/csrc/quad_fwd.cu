@@ -210,9 +210,9 @@ cudaError_t gauss_array(void **out) { return cudaGetSymbolAddress(out, g_isrs_ga
 
 // ---------------------------------------------------------------------------
 // k_quad_f32: persistent FP32 quadrature.  Bound by the XU pipe (sin and cos at 16
-// lanes a clock, ex2 at 32: 20 cycles per warp and z-step), 71 % busy on a 148-channel
-// plan at G = 256 (2.40 ms; every grid point summed one by one: 74.4 ms).  589
-// channels at G = 256: 1,129 -> 45.0 ms; 12 profiles at G = 64: 541 -> 79.8 ms, a
+// lanes a clock, ex2 at 32: 20 cycles per warp and z-step), 70 % busy on a 148-channel
+// plan at G = 256 (2.41 ms; every grid point summed one by one: 74.4 ms).  589
+// channels at G = 256: 1,129 -> 45.6 ms; 12 profiles at G = 64: 541 -> 81.8 ms, a
 // quarter of it the pieces' set-up.  Three blocks of 80 registers an SM: two leave
 // 5 % on the G = 256 case and 6 % on the G = 64 one, four spill (4 % and 9 %).
 // ---------------------------------------------------------------------------

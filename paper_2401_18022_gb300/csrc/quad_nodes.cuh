@@ -363,8 +363,9 @@ __device__ __forceinline__ float row_u(const PieceGeo &g, const NodeRow &o, floa
 // came out 5.3e-5 (2-norm of eta) from the sum over single points, 8.3e-7 now.  So every
 // factor is rounded as that sum rounds it: the row's centre and pitch once to FP32, e^d,
 // its reciprocal, the products.  Costs 1 to 5 % of the time (589 channels, G 256: 44.9 ->
-// 45.4 ms; 12 profiles, G 64: 79.7 -> 83.3); taking it only within g.off of an edge costs
-// more (46.9 and 93.7), some row of a warp nearly always is.
+// 45.5 ms; 12 profiles, G 64: 79.7 -> 83.8, 81.8 with row_whole's ends in a loop); taking
+// it only within g.off of an edge costs more (46.9 and 93.7), some row of a warp nearly
+// always is.
 __device__ __forceinline__ float point_u(const PieceGeo &g, const NodeRow &o, int G, int j)
 {
     const float d = __fmul_rn((float)j + 0.5f - 0.5f * (float)G, o.du2);

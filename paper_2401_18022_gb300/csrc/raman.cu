@@ -428,7 +428,7 @@ __host__ __device__ constexpr size_t tab_warp_bytes(int n_steps)
 }
 
 // As k_quad_f32 (quad_fwd.cu: one warp per tile, row sums from nodes), with the
-// step rows of the tabulated profile.  148 channels at G = 256: 112.3 -> 2.56 ms, XU
+// step rows of the tabulated profile.  148 channels at G = 256: 112.3 -> 2.57 ms, XU
 // pipe 71 % busy.
 #ifndef ISRS_TAB_MIN_BLOCKS
 #define ISRS_TAB_MIN_BLOCKS 3   // resident blocks per SM the register budget is sized for
